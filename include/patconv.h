@@ -375,7 +375,9 @@ typedef struct {
     double  covered;            /* output pixels / pixel slots of all tiles (lanes x pixels each)  */
     int32_t last_arriver;       /* split items are added up by the block that arrives last (nobody
                                    waits) rather than by all of their blocks after a wait         */
-    int32_t reserved;
+    int32_t matrix_path;        /* 1: a run takes the matrix units instead (dense taps, pruned weights as
+                                   zeros), because the caller's tuning names no parameter of the
+                                   command-stream kernel; the fields above describe that kernel's plan */
 } xgen_patconv_plan_stats;
 
 /* Fill *stats for the shape.  No CUDA work is enqueued.  Errors: INVALID_ARG, SHAPE, UNSUPPORTED. */

@@ -67,7 +67,7 @@ class PlanStats(ctypes.Structure):
                 ("lanes_n", ctypes.c_int32), ("pixels_per_lane", ctypes.c_int32), ("stages", ctypes.c_int32),
                 ("uses_copy_engine", ctypes.c_int32), ("shared_bytes", ctypes.c_int64),
                 ("workspace_bytes", ctypes.c_int64), ("covered", ctypes.c_double),
-                ("last_arriver", ctypes.c_int32), ("reserved", ctypes.c_int32)]
+                ("last_arriver", ctypes.c_int32), ("matrix_path", ctypes.c_int32)]
 
 
 class ProbeResult(ctypes.Structure):
@@ -246,7 +246,7 @@ class Packed:
     def plan_info(self, n, h, w) -> dict:
         s = PlanStats()
         _check(lib().xgen_patconv_plan_info(self._h, n, h, w, ctypes.byref(s)), "xgen_patconv_plan_info")
-        return {k: getattr(s, k) for k, _ in PlanStats._fields_ if k != "reserved"}
+        return {k: getattr(s, k) for k, _ in PlanStats._fields_}
 
     def test_expect_arrivals(self, extra):
         _check(lib().xgen_patconv_test_expect_arrivals(self._h, int(extra)), "xgen_patconv_test_expect_arrivals")

@@ -28,6 +28,7 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <mutex>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -38,6 +39,7 @@
 #include "blockgemm.h"
 #include "blockgemm_core.inc"
 #include "patconv_internal.h"
+#include "tapgemm.h"
 
 namespace blockgemm {
 
@@ -67,6 +69,12 @@ struct xgen_blockgemm_packed {
     uint32_t *d_stream = nullptr;
     int32_t *d_seg = nullptr;
     std::atomic<bool> attr_set{false};
+    // the dense product on the matrix units (tapgemm.cu): what a run takes unless the caller named
+    // warps_per_block, a parameter of the kernel below
+    patconv::TapWeights tap;
+    std::mutex tap_mu;
+    struct Entry { int64_t m = 0; patconv::TapPlan plan; uint64_t stamp = 0; } tap_cache[4];
+    uint64_t tap_stamp = 0;
 };
 
 namespace blockgemm {
@@ -433,6 +441,23 @@ static const void *kernel_for(xgen_dtype dt, int ks) {
                                                                                       : (const void *)blockgemm_kernel<XGEN_F16_F32ACC, 8>;
 }
 
+// The matrix path's plan for a row count, from the handle's small cache or made now.
+static bool tap_plan_of(xgen_blockgemm_packed *h, const patconv::TapShape &s, patconv::TapPlan &plan) {
+    std::lock_guard<std::mutex> lock(h->tap_mu);
+    auto *victim = &h->tap_cache[0];
+    for (auto &e : h->tap_cache) {
+        if (e.stamp && e.m == s.rows) {
+            e.stamp = ++h->tap_stamp;
+            plan = e.plan;
+            return true;
+        }
+        if (e.stamp < victim->stamp) victim = &e;
+    }
+    if (!patconv::tap_choose(h->tap, s, h->device, plan)) return false;
+    victim->m = s.rows; victim->plan = plan; victim->stamp = ++h->tap_stamp;
+    return true;
+}
+
 }  // namespace blockgemm
 
 using namespace blockgemm;
@@ -501,6 +526,8 @@ xgen_status xgen_blockgemm_pack(const xgen_blockgemm_desc *d, const void *dense_
         if (st == XGEN_OK && (cudaMalloc(&h->d_stream, sb) != cudaSuccess || cudaMalloc(&h->d_seg, gb) != cudaSuccess)) st = XGEN_ERR_ALLOC;
         if (st == XGEN_OK && ((!H.stream.empty() && cudaMemcpy(h->d_stream, H.stream.data(), H.stream.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) ||
                               cudaMemcpy(h->d_seg, H.seg_off.data(), gb, cudaMemcpyHostToDevice) != cudaSuccess)) st = XGEN_ERR_CUDA;
+        if (st == XGEN_OK && d->warps_per_block == 0)
+            st = patconv::tap_upload_dense(h->tap, d->dtype, d->k, d->c_out, dense_w, row_keep, col_keep, d->block_rows, d->block_cols);
         cudaSetDevice(prev);
         if (st != XGEN_OK) {
             cudaGetLastError();
@@ -525,6 +552,23 @@ xgen_status xgen_blockgemm_run(const xgen_blockgemm_packed *hc, const void *x, i
         if (xa < ye && ya < xe) return XGEN_ERR_INVALID_ARG;
     }
     if (h->device < 0) return XGEN_ERR_CUDA;
+    if (h->tap.dev) {
+        patconv::TapShape ts;
+        ts.n = 1; ts.w = 8; ts.h = (int)((m + 7) / 8); ts.rows = m;
+        int prev = 0;
+        cudaGetDevice(&prev);
+        if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
+        patconv::TapPlan plan;
+        const bool fits = tap_plan_of(h, ts, plan);
+        cudaError_t e = cudaSuccess;
+        if (fits) {
+            const patconv::TapCall call{x, y, bias, nullptr, nullptr, 0, relu, 0, nullptr, 2000000u, true};
+            e = patconv::tap_launch(h->tap, ts, plan, call, (cudaStream_t)stream);
+            if (e != cudaSuccess) cudaGetLastError();
+        }
+        if (prev != h->device) cudaSetDevice(prev);
+        if (fits) return e == cudaSuccess ? XGEN_OK : XGEN_ERR_CUDA;
+    }
     GParams P{};
     P.x = x; P.y = y; P.bias = static_cast<const float *>(bias);
     P.stream = reinterpret_cast<const uint4 *>(h->d_stream); P.seg_off = h->d_seg;
@@ -583,6 +627,7 @@ void xgen_blockgemm_free(xgen_blockgemm_packed *h) {
         if (cudaSetDevice(h->device) == cudaSuccess) {
             if (h->d_stream) cudaFree(h->d_stream);
             if (h->d_seg) cudaFree(h->d_seg);
+            patconv::tap_free(h->tap);
         }
         cudaSetDevice(prev);
     }

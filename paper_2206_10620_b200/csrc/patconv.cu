@@ -40,6 +40,8 @@
 
 #include "core_gen.inc"
 #include "patconv_internal.h"
+#include "ptx.cuh"
+#include "tapgemm.h"
 
 namespace patconv {
 
@@ -115,67 +117,6 @@ struct KParams {
     int last_reduces;                    // nobody waits: the block that arrives last adds up the whole item
     uint32_t wait_us;                    // bound of every device-side wait, microseconds
 };
-
-// ---- small PTX wrappers -----------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void tmem_ld8(uint32_t ta, uint32_t (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(ta) : "memory");
-}
-__device__ __forceinline__ void tmem_ld4(uint32_t ta, uint32_t (&r)[4]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(ta) : "memory");
-}
-__device__ __forceinline__ void tmem_st8(uint32_t ta, const uint32_t (&r)[8]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
-                 ::"r"(ta), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mbar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t mbar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ uint64_t global_ns() {
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Wait for an mbarrier phase with a bound in time (limit_us microseconds, plus a cap on the
-// polls in case the timer stands still): on expiry the block-wide abort flag and the device
-// status word are set and every later wait returns at once; the warps then leave their
-// loops, so the kernel still runs to its end (releasing tensor memory) with results the
-// host can tell are invalid.
-__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, volatile int *abort_flag, int *status,
-                                          uint32_t limit_us) {
-    uint64_t t0 = 0;
-    for (uint32_t it = 0; it < 40000000u; ++it) {
-        uint32_t ok;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(ok) : "r"(mbar), "r"(parity), "r"(2000u) : "memory");
-        if (ok) return true;
-        if (*abort_flag) return false;
-        if ((it & 7u) == 7u) {
-            const uint64_t t = global_ns();
-            if (t0 == 0) t0 = t;
-            else if (t - t0 > (uint64_t)limit_us * 1000ull) break;
-        }
-    }
-    *abort_flag = 1;
-    if (status) atomicExch(status, 1);
-    return false;
-}
 
 template <int STRIDE, int NP, int BH>
 __device__ __forceinline__ void run_commands(uint32_t sp, uint32_t base_a, uint32_t plane_bytes,
@@ -1155,6 +1096,9 @@ struct LaunchEntry {
 };
 constexpr int kLaunchCache = 4;
 
+// A plan of the matrix path for one shape.
+struct TapEntry { TapShape shape; TapPlan plan; uint64_t stamp = 0; };
+
 }  // namespace patconv
 
 using namespace patconv;
@@ -1180,6 +1124,13 @@ struct xgen_patconv_packed {
     xgen_patconv_tuning tuning{};       // caller's overrides (xgen_patconv_plan_tuned)
     uint32_t wait_us = 2000000;         // bound of every device-side wait
     int hook_extra_arrivals = 0;        // testing aid: arrivals a planned split waits for beyond its own
+    // the layer as dense taps on the matrix units (tapgemm.cu): what a run takes unless the caller
+    // has asked for parameters of the command-stream kernel
+    TapWeights tap;
+    bool stream_asked = false;
+    mutable std::mutex tap_mu;
+    mutable TapEntry tap_cache[kLaunchCache];
+    mutable uint64_t tap_stamp = 0;
     // prepared launches (shape, input address)
     mutable std::mutex cache_mu;
     mutable LaunchEntry cache[kLaunchCache];
@@ -1241,11 +1192,9 @@ static cudaError_t log_cuda(cudaError_t e, const char *what) {
     return e;
 }
 
+namespace patconv {
 // cuTensorMapEncodeTiled, fetched through the runtime so the library does not link libcuda.
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-static EncodeTiledFn encode_tiled_fn() {
+EncodeTiledFn encode_tiled_fn() {
     static EncodeTiledFn fn = nullptr;
     static std::once_flag once;
     std::call_once(once, [] {
@@ -1259,6 +1208,7 @@ static EncodeTiledFn encode_tiled_fn() {
     });
     return fn;
 }
+}  // namespace patconv
 
 template <int DT, int STRIDE, bool FUSED, int BH>
 static const void *kernel_np(int np) {
@@ -1469,6 +1419,26 @@ static void forget_prepared_launches(xgen_patconv_packed *h) {
     for (LaunchEntry &e : h->cache) e.stamp = 0;
 }
 
+// Whether a run takes the matrix path.
+static bool on_matrix_units(const xgen_patconv_packed *h) { return h->tap.dev && !h->stream_asked; }
+
+// The matrix path's plan of a shape, from the handle's small cache or made now.
+static bool tap_plan_of(const xgen_patconv_packed *h, const TapShape &s, TapPlan &plan) {
+    std::lock_guard<std::mutex> lock(h->tap_mu);
+    TapEntry *victim = &h->tap_cache[0];
+    for (TapEntry &e : h->tap_cache) {
+        if (e.stamp && e.shape.n == s.n && e.shape.h == s.h && e.shape.w == s.w && e.shape.pool == s.pool) {
+            e.stamp = ++h->tap_stamp;
+            plan = e.plan;
+            return true;
+        }
+        if (e.stamp < victim->stamp) victim = &e;
+    }
+    if (!tap_choose(h->tap, s, h->device, plan)) return false;
+    victim->shape = s; victim->plan = plan; victim->stamp = ++h->tap_stamp;
+    return true;
+}
+
 // Where a run keeps the partial sums of a split, when the caller (not the plan) decides.
 struct SplitChoice { int splits, chunks_per_split; uint32_t *partial; };
 
@@ -1505,6 +1475,27 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
             const char *re = ra + (size_t)n * ho * wo * p.c_out * rb;
             if (ra < ye && ya < re) return XGEN_ERR_INVALID_ARG;
         }
+    }
+    if (!forced && on_matrix_units(h)) {
+        TapShape ts;
+        ts.n = n; ts.h = hh; ts.w = ww; ts.stride = p.stride; ts.pool = pool == 2;
+        int prev = 0;
+        if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
+        if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
+        TapPlan plan;
+        const bool fits = tap_plan_of(h, ts, plan);
+        cudaError_t e = cudaSuccess;
+        if (fits) {
+            const TapCall call{x, y, bias, residual, rq_scale, ep ? ep->requant_zero_point : 0, relu, pool,
+                               h->d_status, h->wait_us, !h->tuning.no_launch_overlap};
+            if (log_enabled())
+                fprintf(stderr, "libpatconv: matrix path, %d blocks = %d items (%d row tiles x %d columns x %d filter tiles of %d) x %d splits, %d x 128 pixels%s, %d planes x %d stages, %d + %d buffers%s, %zu bytes shared, %.0f cycles expected\n",
+                        plan.grid, plan.items, plan.row_tiles, plan.segs, plan.nblk, plan.nt, plan.splits, plan.mt, plan.pair ? " (block pairs)" : "", plan.pl, plan.stages,
+                        plan.a_stages, plan.b_slots, plan.resident ? " (resident weights)" : "", plan.smem, plan.cycles);
+            e = log_cuda(tap_launch(h->tap, ts, plan, call, (cudaStream_t)stream), "matrix kernel launch");
+        }
+        if (prev != h->device) cudaSetDevice(prev);
+        if (fits) return e == cudaSuccess ? XGEN_OK : XGEN_ERR_CUDA;
     }
     Layout L;
     CUtensorMap tm;
@@ -1664,6 +1655,13 @@ xgen_status xgen_patconv_pack(const xgen_patconv_desc *desc, const void *dense_w
         int prev = 0;
         if (cudaGetDevice(&prev) != cudaSuccess || cudaSetDevice(device) != cudaSuccess) { delete h; return XGEN_ERR_CUDA; }
         xgen_status us = upload_layout(h);
+        // Three input channels fill a fifth of the 16 that a matrix instruction takes: such first layers
+        // stay on the command-stream kernel (3 -> 64 at 224x224, fp32: 12.7 us against 15.8 us).
+        if (us == XGEN_OK && desc->c_in >= 8) {
+            const PackedHost &p = h->host;
+            us = tap_upload_patterns(h->tap, p.dtype, p.c_in, p.c_out, p.kpat.data(), p.kw4.data(), p.masks.data(), (int)p.masks.size());
+            if (us != XGEN_OK) free_device_layout(h);
+        }
         cudaSetDevice(prev);
         if (us != XGEN_OK) { delete h; return us; }
         h->device = device;
@@ -1675,6 +1673,7 @@ xgen_status xgen_patconv_pack(const xgen_patconv_desc *desc, const void *dense_w
 void xgen_patconv_free(xgen_patconv_packed *h) {
     if (!h) return;
     free_device_layout(h);
+    tap_free(h->tap);
     if (h->d_partial) cudaFree(h->d_partial);
     if (h->d_counters) cudaFree(h->d_counters);
     if (h->d_hx) cudaFree(h->d_hx);
@@ -1763,7 +1762,7 @@ xgen_status xgen_patconv_plan_info(const xgen_patconv_packed *h, int32_t n, int3
     out->uses_copy_engine = L.kp.use_tma;
     out->shared_bytes = (int64_t)L.smem;
     out->last_arriver = planned && h->plan_last ? 1 : 0;
-    out->reserved = 0;
+    out->matrix_path = on_matrix_units(h) ? 1 : 0;
     out->workspace_bytes = planned ? (int64_t)((size_t)(L.items - h->plan_whole) * (size_t)h->plan_splits * rows_per_item(p) * 1024) : 0;
     return XGEN_OK;
 }
@@ -1951,6 +1950,7 @@ xgen_status xgen_patconv_plan_tuned(xgen_patconv_packed *h, int32_t n, int32_t h
     forget_prepared_launches(h);
     if (rs != XGEN_OK) { h->plan_splits = 1; h->plan_n = 0; return rs; }
     h->tuning = tn;
+    h->stream_asked = tn.splits || tn.no_copy_engine || tn.reduce_mode || tn.channels_per_chunk || tn.groups_per_block;
     h->wait_us = tn.wait_limit_ms > 0 ? (uint32_t)std::min<int64_t>((int64_t)tn.wait_limit_ms * 1000, 60000000) : 2000000u;
     h->plan_n = n; h->plan_h = hh; h->plan_w = ww;
     h->plan_splits = (int)splits; h->plan_cps = cps; h->plan_whole = (int)whole; h->plan_last = last;

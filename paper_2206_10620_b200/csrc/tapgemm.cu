@@ -1,0 +1,1137 @@
+// The pattern-pruned convolution and the block-pruned matrix product on the matrix units.
+//
+// What is left of a pruned layer is 4/9 x (1 - prune rate) of a dense one, but the matrix units
+// are 22 times (fp16) to 44 times (int8) the packed-FMA pipe, so the layer is run dense: pruned
+// weights are zeros of the operand.  (0 x infinity is NaN there, as in the definition written out
+// over the masked dense tensor.)
+//
+// A tile is 8 pixels wide and 16 (or 32) rows high.  Its input with the halo is staged once per
+// group of channels, as planes of 16 bytes of channels per pixel, and serves all nine taps: in
+// shared memory a tap is only another start address.  The operand layout without swizzle (8 rows
+// of 16 contiguous bytes, groups of rows a free pitch apart) allows any start that is a multiple
+// of 16 bytes, so a row of 8 output pixels is one group, the pitch of the staged rows the distance
+// of groups.  Measured: full rate (64 cycles for 128 x 128 x 16) at every shift.  The other choice,
+// one copy-engine load per tap (im2col), moves the tile nine times through L2.
+//
+// A matrix instruction of 128 x 128 x 16 reads 8 KB of shared memory in its 64 cycles, all that
+// shared memory delivers; the weights that stream in slow it down.  So where there are two tiles,
+// two blocks work as a pair (cta_group::2): each reads its own rows and half of the filters.
+//
+// fp32: every operand is split into three bf16 parts (8 + 8 + 8 significand bits, the sum is
+// exact) and six of the nine products are taken; what is left out is below 2^-24 of the product.
+// The matrix unit truncates when it adds to its accumulator (measured: a chain of 288 steps ends
+// 1.5e-5 low, one of 9 steps 1.6e-7), so the leading product is accumulated for one stage only
+// (at most 18 steps) and then added, rounded, to sums in registers; the five small products have
+// an accumulator of their own, where truncation is 2^-8 of that, and are added the same way.
+//
+// Roles: 8 epilogue warps (tensor memory -> registers -> y), 6 producer warps (x -> planes), one
+// warp that issues the matrix instructions, one that fetches weights with tensor copies.  Blocks are
+// persistent; a block keeps its range of filters, and where all of its weights fit they are
+// fetched once.  Items that would leave the GPU idle share one reduction between the blocks of a
+// cluster, which add their sums through distributed shared memory in a fixed order.
+#include <cuda.h>
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <mutex>
+#include <utility>
+#include <vector>
+
+#include "patconv_internal.h"
+#include "ptx.cuh"
+#include "tapgemm.h"
+
+namespace patconv {
+
+// 16 warps: four a scheduler, so that a thread may hold 128 registers (fp32 keeps 64 sums)
+constexpr int kEpiWarps = 8, kProdWarps = 6;
+constexpr int kTapThreads = (kEpiWarps + kProdWarps + 2) * 32;
+constexpr int kProdThreads = kProdWarps * 32;
+constexpr int kMaxA = 4, kMaxB = 64;
+constexpr int kTapSmemMax = 232448 - 4096;      // 227 KB less static shared memory
+constexpr int kMaxFilterTile = 256;
+
+struct TapParams {
+    const void *x; void *y; const void *bias; const void *residual; const float *rq_scale;
+    int *status;
+    uint32_t wait_us;
+    int rq_zero, relu, pool;
+    int n, h, w, ho, wo, c_in, c_out;
+    int po, pw;                                 // stored extents
+    int64_t npix;                               // product: rows of x
+    int vh, straddle;                           // virtual rows per image; tiles may cross images
+    int segs, nblk, nt, items, splits, per_split, stages;
+    int pl, pl_log, plane_pitch;
+    int a_stages, b_slots, resident, b_bytes;
+    int b_off, tab_off;                         // bytes into dynamic shared memory
+    int tmem_cols, acc_bufs;
+    int vec_x;                                  // 16-byte pieces of x can be copied as they are
+    int vec_y, vec_r, y32;                      // 16-byte (32-byte) pieces of y / the residual can be moved whole
+    uint32_t idesc;
+};
+
+// Elements of x per 16-byte plane entry (K of one matrix instruction = two planes), bf16 parts, bytes.
+template <int DT> struct TapTraits;
+template <> struct TapTraits<XGEN_F32> { static constexpr int cpp = 8, parts = 3, xb = 4; };
+template <> struct TapTraits<XGEN_F16_F32ACC> { static constexpr int cpp = 8, parts = 1, xb = 2; };
+template <> struct TapTraits<XGEN_I8_I32> { static constexpr int cpp = 16, parts = 1, xb = 1; };
+
+// Staged tile: the row pitch in pixels, pixels in all, where a tap starts.  Stride 2 keeps four
+// images of the tile, one per parity of row and column, so that neighbouring output pixels read
+// neighbouring entries there too.
+template <int STRIDE, int TAPS, int MT> struct TapTile {
+    static constexpr int R = 16 * MT;
+    static constexpr int pitch = TAPS == 1 ? 8 : STRIDE == 1 ? 10 : 9;
+    static constexpr int pixels = TAPS == 1 ? 8 * R : STRIDE == 1 ? 10 * (R + 2) : 9 * (4 * R + 2);
+    static __host__ __device__ constexpr int tap_start(int t) {
+        if (TAPS == 1) return 0;
+        const int dy = t / 3, dx = t % 3;
+        if (STRIDE == 1) return dy * 10 + dx;
+        // even rows: even columns, odd columns; odd rows (one more of them): even, odd
+        const int row_part = dy == 1 ? 0 : 2 * R * 9, rows = dy == 1 ? R : R + 1;
+        return row_part + (dx == 1 ? 0 : rows * 9) + (dy == 2 ? 9 : 0) + (dx == 2 ? 1 : 0);
+    }
+    // Staged pixel -> (row of the tile's staged rows, column relative to stride x first output column);
+    // padding entries lie far out.
+    static __device__ void entry(int p, int &row, int &col) {
+        if (TAPS == 1) { row = p / 8; col = p % 8; return; }
+        if (STRIDE == 1) { row = p / 10; col = p % 10 - 1; return; }
+        const bool odd_row = p >= 2 * R * 9;
+        if (odd_row) p -= 2 * R * 9;
+        const int rows = odd_row ? R + 1 : R;
+        const bool odd_col = p >= rows * 9;
+        if (odd_col) p -= rows * 9;
+        const int j = p % 9;
+        row = p / 9 + (odd_row ? R : 0);
+        col = odd_col ? 2 * j - 1 : (j < 8 ? 2 * j : -(1 << 20));
+    }
+};
+
+// ---- results -------------------------------------------------------------------
+// W sums of adjacent channels of one pixel: bias, residual, activation, in fp32 (int32).
+template <int DT, bool FUSED, int W>
+__device__ __forceinline__ void tap_affine(const TapParams &P, const uint32_t *s_bias, uint32_t (&v)[W], int64_t pixel,
+                                           bool valid, int c0, int n0) {
+#pragma unroll
+    for (int q = 0; q < W / 4; ++q) {
+        const uint4 b = *reinterpret_cast<const uint4 *>(s_bias + (c0 - n0) + 4 * q);
+        const uint32_t bb[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            v[4 * q + i] = DT == XGEN_I8_I32 ? v[4 * q + i] + bb[i]
+                                             : __float_as_uint(__uint_as_float(v[4 * q + i]) + __uint_as_float(bb[i]));
+    }
+    if (FUSED && P.residual && valid) {
+        const size_t off = (size_t)pixel * P.c_out + c0;
+        if (DT == XGEN_F16_F32ACC) {
+            const __half *r = static_cast<const __half *>(P.residual) + off;
+            if (P.vec_r && c0 + W <= P.c_out) {
+#pragma unroll
+                for (int q = 0; q < W / 8; ++q) {
+                    const uint4 a = __ldg(reinterpret_cast<const uint4 *>(r) + q);
+                    const uint32_t aa[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&aa[i]));
+                        v[8 * q + 2 * i] = __float_as_uint(__uint_as_float(v[8 * q + 2 * i]) + f.x);
+                        v[8 * q + 2 * i + 1] = __float_as_uint(__uint_as_float(v[8 * q + 2 * i + 1]) + f.y);
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < W; ++i)
+                    if (c0 + i < P.c_out) v[i] = __float_as_uint(__uint_as_float(v[i]) + __half2float(r[i]));
+            }
+        } else {
+            const uint32_t *r = static_cast<const uint32_t *>(P.residual) + off;
+            uint32_t a[W];
+            if (P.vec_r && c0 + W <= P.c_out) {
+#pragma unroll
+                for (int q = 0; q < W / 4; ++q) {
+                    const uint4 t = __ldg(reinterpret_cast<const uint4 *>(r) + q);
+                    a[4 * q] = t.x; a[4 * q + 1] = t.y; a[4 * q + 2] = t.z; a[4 * q + 3] = t.w;
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < W; ++i) a[i] = c0 + i < P.c_out ? r[i] : 0u;
+            }
+#pragma unroll
+            for (int i = 0; i < W; ++i)
+                v[i] = DT == XGEN_I8_I32 ? v[i] + a[i] : __float_as_uint(__uint_as_float(v[i]) + __uint_as_float(a[i]));
+        }
+    }
+    if (P.relu) {
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            if (DT == XGEN_I8_I32) v[i] = (uint32_t)max((int)v[i], 0);
+            else {                                  // NaN stays NaN
+                float f;
+                asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(f) : "f"(__uint_as_float(v[i])));
+                v[i] = __float_as_uint(f);
+            }
+        }
+    }
+}
+
+template <int DT> __device__ __forceinline__ uint32_t tap_max(uint32_t a, uint32_t b) {
+    if (DT == XGEN_I8_I32) return (uint32_t)max((int)a, (int)b);
+    float f;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(f) : "f"(__uint_as_float(a)), "f"(__uint_as_float(b)));
+    return __float_as_uint(f);
+}
+
+// Store W results of one pixel, converted; whole 16- or 32-byte pieces where the tensor allows it.
+template <int DT, bool FUSED, int W>
+__device__ __forceinline__ void tap_store(const TapParams &P, const float *s_scale, const uint32_t (&v)[W], int64_t pixel,
+                                          int c0, int n0) {
+    const size_t off = (size_t)pixel * P.c_out + c0;
+    const bool full = c0 + W <= P.c_out;
+    if (FUSED && DT == XGEN_I8_I32 && P.rq_scale) {
+        uint32_t code[W / 4];
+#pragma unroll
+        for (int q = 0; q < W / 4; ++q) {
+            code[q] = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float f = __fmul_rn((float)(int)v[4 * q + i], s_scale[c0 - n0 + 4 * q + i]);
+                int r;
+                asm("add.sat.s32 %0, %1, %2;" : "=r"(r) : "r"(__float2int_rn(f)), "r"(P.rq_zero));
+                code[q] |= (uint32_t)max(min(r, 255), 0) << (8 * i);
+            }
+        }
+        uint8_t *y = static_cast<uint8_t *>(P.y) + off;
+        if (full && P.vec_y) {
+            if (W == 16) *reinterpret_cast<uint4 *>(y) = make_uint4(code[0], code[1], code[W / 4 - 2], code[W / 4 - 1]);
+            else *reinterpret_cast<uint2 *>(y) = make_uint2(code[0], code[1]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < W; ++i) if (c0 + i < P.c_out) y[i] = (uint8_t)(code[i / 4] >> (8 * (i % 4)));
+        }
+        return;
+    }
+    constexpr int NW = DT == XGEN_F16_F32ACC ? W / 2 : W;
+    uint32_t o[NW];
+    if (DT == XGEN_F16_F32ACC) {
+#pragma unroll
+        for (int i = 0; i < NW; ++i) {
+            const __half2 h = __floats2half2_rn(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+            o[i] = *reinterpret_cast<const uint32_t *>(&h);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < NW; ++i) o[i] = v[i];
+    }
+    if (full && P.vec_y) {
+        uint32_t *y = reinterpret_cast<uint32_t *>(static_cast<char *>(P.y) + off * (DT == XGEN_F16_F32ACC ? 2 : 4));
+        if (P.y32 && NW >= 8) {
+#pragma unroll
+            for (int q = 0; q < NW / 8; ++q)
+                asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                             ::"l"(y + 8 * q), "r"(o[8 * q]), "r"(o[8 * q + 1]), "r"(o[8 * q + 2]), "r"(o[8 * q + 3]),
+                               "r"(o[8 * q + 4]), "r"(o[8 * q + 5]), "r"(o[8 * q + 6]), "r"(o[8 * q + 7]) : "memory");
+        } else {
+#pragma unroll
+            for (int q = 0; q < NW / 4; ++q)
+                reinterpret_cast<uint4 *>(y)[q] = make_uint4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+        }
+    } else if (DT == XGEN_F16_F32ACC) {
+        unsigned short *y = static_cast<unsigned short *>(P.y) + off;
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            if (c0 + i < P.c_out) y[i] = (unsigned short)(o[i / 2] >> (16 * (i % 2)));
+    } else {
+        uint32_t *y = static_cast<uint32_t *>(P.y) + off;
+#pragma unroll
+        for (int i = 0; i < W; ++i)
+            if (c0 + i < P.c_out) y[i] = v[i];
+    }
+}
+
+// ---- operands ------------------------------------------------------------------
+// fp32 -> three bf16 parts.  The first is clamped to the largest bf16 so that a finite value never
+// becomes an infinity; an infinity or NaN survives in the second part.
+__device__ __forceinline__ void split3(const float (&a)[8], uint4 &p0, uint4 &p1, uint4 &p2) {
+    const float big = __uint_as_float(0x7F7F0000u);
+    uint32_t o[3][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float x = a[2 * i], y = a[2 * i + 1];
+        __nv_bfloat162 h = __floats2bfloat162_rn(fminf(fmaxf(x, -big), big), fminf(fmaxf(y, -big), big));
+        o[0][i] = *reinterpret_cast<uint32_t *>(&h);
+#pragma unroll
+        for (int k = 1; k < 3; ++k) {
+            x -= __uint_as_float(o[k - 1][i] << 16);
+            y -= __uint_as_float(o[k - 1][i] & 0xFFFF0000u);
+            h = __floats2bfloat162_rn(x, y);
+            o[k][i] = *reinterpret_cast<uint32_t *>(&h);
+        }
+    }
+    p0 = make_uint4(o[0][0], o[0][1], o[0][2], o[0][3]);
+    p1 = make_uint4(o[1][0], o[1][1], o[1][2], o[1][3]);
+    p2 = make_uint4(o[2][0], o[2][1], o[2][2], o[2][3]);
+}
+
+// 16 bytes from any address, bytes beyond `valid` zero: aligned words, shifted into place.  Only
+// words that hold at least one wanted byte are read.
+__device__ __forceinline__ uint4 gather16(const char *src, int valid) {
+    if (valid <= 0) return make_uint4(0, 0, 0, 0);
+    const uintptr_t a = reinterpret_cast<uintptr_t>(src);
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(a & ~(uintptr_t)3);
+    const int lead = (int)(a & 3), nbytes = min(valid, 16), words = (lead + nbytes + 3) / 4;
+    uint32_t in[5], o[4];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) in[i] = i < words ? __ldg(w + i) : 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        o[i] = __funnelshift_r(in[i], in[i + 1], 8 * lead);
+        const int left = nbytes - 4 * i;                       // wanted bytes of this word
+        if (left < 4) o[i] = left <= 0 ? 0u : (o[i] & ((1u << (8 * left)) - 1u));
+    }
+    return make_uint4(o[0], o[1], o[2], o[3]);
+}
+
+__device__ __forceinline__ void sts128(uint32_t dst, const uint4 &v) {
+    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+
+// Position of a block's work: item = (tile or pair of tiles, range of filters), tile = (rows, 8-pixel
+// column).  The second tile of the last pair may lie past the end: all of its pixels are invalid.
+struct TapItem { int n0, ox0, v0; };
+template <bool PAIR> __device__ __forceinline__ TapItem tap_item(const TapParams &P, int item, int rows, int side) {
+    TapItem t;
+    int tile = item / P.nblk;
+    t.n0 = (item - tile * P.nblk) * P.nt;
+    if (PAIR) tile = 2 * tile + side;
+    const int rt = tile / P.segs;
+    t.ox0 = (tile - rt * P.segs) * 8;
+    t.v0 = rt * rows;
+    return t;
+}
+
+// First pixel (of x) of staged row `i` of a tile, or -1 for a row of zeros.
+template <int STRIDE, int TAPS, int MT>
+__device__ __forceinline__ int tap_origin(const TapParams &P, int v0, int i) {
+    constexpr int R = 16 * MT;
+    if (TAPS == 1) return (int64_t)(v0 + i) * 8 < P.npix ? (v0 + i) * 8 : -1;
+    int img, iy;
+    const int step = STRIDE == 1 ? i - 1 : i < R ? i : i - R;      // output rows from the tile's first
+    if (P.straddle) {
+        const int v = v0 + step;
+        if (v < 0) return -1;
+        img = v / P.vh;
+        iy = v - img * P.vh;
+    } else {
+        img = v0 / P.vh;
+        iy = v0 - img * P.vh + step;
+    }
+    if (STRIDE == 2) iy = i < R ? 2 * iy : 2 * iy - 1;
+    if (img >= P.n || iy < 0 || iy >= P.h) return -1;
+    return (img * P.h + iy) * P.w;
+}
+
+template <int DT, int STRIDE, int TAPS, int MT, bool PAIR>
+__global__ void __launch_bounds__(kTapThreads, 1)
+tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensorMap wmap) {
+    using T = TapTraits<DT>;
+    using TL = TapTile<STRIDE, TAPS, MT>;
+    constexpr int PARTS = T::parts, R = TL::R;
+    constexpr bool kF32 = DT == XGEN_F32, FUSED = TAPS == 9;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_abort;
+    __shared__ __align__(8) uint64_t s_bars[2 * kMaxA + 2 * kMaxB + 5];
+    __shared__ __align__(16) uint32_t s_bias[kMaxFilterTile];
+    __shared__ __align__(16) float s_scale[kMaxFilterTile];
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t sbase = smem_u32(smem), bars = smem_u32(s_bars);
+    auto a_full = [&](int s) { return bars + 8u * s; };
+    auto a_empty = [&](int s) { return bars + 8u * (kMaxA + s); };
+    auto b_full = [&](int s) { return bars + 8u * (2 * kMaxA + s); };
+    auto b_empty = [&](int s) { return bars + 8u * (2 * kMaxA + kMaxB + s); };
+    auto acc_full = [&](int s) { return bars + 8u * (2 * kMaxA + 2 * kMaxB + s); };
+    auto acc_empty = [&](int s) { return bars + 8u * (2 * kMaxA + 2 * kMaxB + 2 + s); };
+    const uint32_t all_done = bars + 8u * (2 * kMaxA + 2 * kMaxB + 4);
+    auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait<PAIR>(bar, parity, &s_abort, P.status, P.wait_us); };
+    // Clusters: a pair of blocks (PAIR), or the blocks (pairs) that split an item's reduction.  The even
+    // block of a pair holds the barriers that say "operands are there" and "sums have been read".
+    const int csize = (PAIR ? 2 : 1) * P.splits;
+    const int crank = csize > 1 ? (int)(blockIdx.x % (unsigned)csize) : 0;
+    const int side = PAIR ? crank & 1 : 0, rank = PAIR ? crank >> 1 : crank;
+    const uint16_t both = (uint16_t)(3u << (crank & ~1));
+    auto arrive_lead = [&](uint32_t bar) {
+        if (PAIR) mbar_arrive_cluster(cluster_addr(bar, (uint32_t)(crank & ~1)));
+        else mbar_arrive(bar);
+    };
+
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (tid == 0) {
+        s_abort = 0;
+        for (int i = 0; i < P.a_stages; ++i) { mbar_init(a_full(i), (PAIR ? 2 : 1) * kProdWarps); mbar_init(a_empty(i), 1); }
+        for (int i = 0; i < P.b_slots; ++i) { mbar_init(b_full(i), 1); mbar_init(b_empty(i), 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(acc_full(i), 1); mbar_init(acc_empty(i), (PAIR ? 2 : 1) * kEpiWarps); }
+        mbar_init(all_done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_async_proxy();
+    }
+    if (warp == kEpiWarps + kProdWarps) tmem_alloc<PAIR>(smem_u32(&s_tmem), (uint32_t)P.tmem_cols);
+    tc_fence_before();
+    __syncthreads();
+    if (PAIR) cluster_meet();            // the other block's barriers stand
+    tc_fence_after();
+    const uint32_t tmem = s_tmem;
+
+    // A block (pair) of an unsplit launch takes items its number, + number of blocks, ... (all of the
+    // same filter range); a cluster of a split launch takes one item, each block a range of stages.
+    const int item0 = (int)(blockIdx.x / (unsigned)csize);
+    const int item_step = P.splits > 1 ? P.items : (int)(gridDim.x / (unsigned)csize);
+    const int k0 = rank * P.per_split, k1 = min(P.stages, k0 + P.per_split);
+    const int n0 = tap_item<PAIR>(P, item0, R, side).n0;
+    const int planes = (P.c_in + T::cpp * 2 - 1) / (T::cpp * 2) * 2;
+    const uint32_t a_part = (uint32_t)P.pl * P.plane_pitch, a_bytes = a_part * PARTS;
+
+    if (warp >= kEpiWarps && warp < kEpiWarps + kProdWarps) {
+        // ---- producers: x -> planes ------------------------------------------------
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        const int pt = tid - kEpiWarps * 32;
+        int s = 0, pending = 0, sp = 0;
+        uint32_t ph = 1;
+        bool ok = true, par = false;
+        const char *const x = static_cast<const char *>(P.x);
+        const int total = TL::pixels << P.pl_log;
+        auto publish = [&]() {           // the oldest unpublished stage has landed
+            fence_async_proxy();
+            __syncwarp();
+            if (lane == 0) arrive_lead(a_full(sp));
+            sp = sp + 1 == P.a_stages ? 0 : sp + 1;
+            --pending;
+        };
+        for (int item = item0; item < P.items && ok; item += item_step, par = !par) {
+            const TapItem t = tap_item<PAIR>(P, item, R, side);
+            // x's pixel of every staged pixel, or -1 for zeros
+            int *const pix = reinterpret_cast<int *>(smem + P.tab_off) + (par ? TL::pixels : 0);
+            for (int p = pt; p < TL::pixels; p += kProdThreads) {
+                int row, col;
+                TL::entry(p, row, col);
+                const int o = tap_origin<STRIDE, TAPS, MT>(P, t.v0, row), ix = t.ox0 * STRIDE + col;
+                const bool in = o >= 0 && (TAPS == 1 ? (int64_t)o + ix < P.npix : (unsigned)ix < (unsigned)P.w);
+                pix[p] = in ? o + ix : -1;
+            }
+            asm volatile("bar.sync 1, %0;" ::"n"(kProdThreads) : "memory");
+            for (int ks = k0; ks < k1; ++ks) {
+                // What was copied earlier is handed over before this warp waits for room.
+                if (pending && !__all_sync(0xFFFFFFFFu, mbar_ready(a_empty(s), ph))) {
+                    copy_wait<0>();
+                    while (pending) publish();
+                }
+                ok = wait(a_empty(s), ph);
+                if (!ok) break;
+                const uint32_t dst = sbase + (uint32_t)s * a_bytes;
+                const int npl = min(P.pl, planes - ks * P.pl);
+                if (!kF32 && P.vec_x) {
+#pragma unroll 4
+                    for (int i = pt; i < total; i += kProdThreads) {
+                        const int pl = i & (P.pl - 1), p = i >> P.pl_log;
+                        const int c = (ks * P.pl + pl) * T::cpp;
+                        const int px = pix[p];
+                        const bool in = px >= 0 && c < P.c_in;
+                        if (pl < npl)
+                            copy16(dst + (uint32_t)(pl * P.plane_pitch + p * 16), in ? x + ((size_t)px * P.c_in + c) * T::xb : x, in ? 16u : 0u);
+                    }
+                    copy_commit();
+                    ++pending;
+                    if (pending == P.a_stages) {            // as many stages in flight as there are
+                        if (P.a_stages == 1) copy_wait<0>();
+                        else if (P.a_stages == 2) copy_wait<1>();
+                        else if (P.a_stages == 3) copy_wait<2>();
+                        else copy_wait<3>();
+                        publish();
+                    }
+                } else {
+                    constexpr int U = kF32 ? 4 : 2;          // pieces of a thread in flight
+                    for (int i0 = pt; i0 < total; i0 += U * kProdThreads) {
+                        float f[kF32 ? U : 1][8];
+                        uint4 g[kF32 ? 1 : U];
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            const int i = i0 + u * kProdThreads;
+                            const int pl = i & (P.pl - 1), p = i >> P.pl_log;
+                            const int c = (ks * P.pl + pl) * T::cpp;
+                            const int px = i < total ? pix[p] : -1;
+                            const char *src = x + ((size_t)(px < 0 ? 0 : px) * P.c_in + c) * T::xb;
+                            const int left = px < 0 ? 0 : P.c_in - c;     // channels there are
+                            if (kF32) {
+                                float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+                                if (P.vec_x) {
+                                    if (left > 0) lo = __ldg(reinterpret_cast<const float4 *>(src));
+                                    if (left > 4) hi = __ldg(reinterpret_cast<const float4 *>(src) + 1);
+                                } else {
+                                    const float *q = reinterpret_cast<const float *>(src);
+                                    if (left > 0) lo.x = __ldg(q);
+                                    if (left > 1) lo.y = __ldg(q + 1);
+                                    if (left > 2) lo.z = __ldg(q + 2);
+                                    if (left > 3) lo.w = __ldg(q + 3);
+                                    if (left > 4) hi.x = __ldg(q + 4);
+                                    if (left > 5) hi.y = __ldg(q + 5);
+                                    if (left > 6) hi.z = __ldg(q + 6);
+                                    if (left > 7) hi.w = __ldg(q + 7);
+                                }
+                                float *const fu = f[kF32 ? u : 0];
+                                fu[0] = lo.x; fu[1] = lo.y; fu[2] = lo.z; fu[3] = lo.w;
+                                fu[4] = hi.x; fu[5] = hi.y; fu[6] = hi.z; fu[7] = hi.w;
+                            } else {
+                                g[kF32 ? 0 : u] = gather16(src, left * T::xb);
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            const int i = i0 + u * kProdThreads;
+                            const int pl = i & (P.pl - 1), p = i >> P.pl_log;
+                            const uint32_t d = dst + (uint32_t)(pl * P.plane_pitch + p * 16);
+                            if (i < total && pl < npl) {
+                                if (kF32) {
+                                    uint4 p0, p1, p2;
+                                    split3(f[kF32 ? u : 0], p0, p1, p2);
+                                    sts128(d, p0);
+                                    sts128(d + a_part, p1);
+                                    sts128(d + 2 * a_part, p2);
+                                } else {
+                                    sts128(d, g[kF32 ? 0 : u]);
+                                }
+                            }
+                        }
+                    }
+                    ++pending;
+                    publish();
+                }
+                if (++s == P.a_stages) { s = 0; ph ^= 1u; }
+            }
+        }
+        copy_wait<0>();
+        while (pending) publish();
+    } else if (warp == kEpiWarps + kProdWarps) {
+        // ---- matrix instructions ---------------------------------------------------
+        const bool leader = elect_one();
+        const uint32_t sbo = TL::pitch * 16;
+        const uint32_t b_rows = (uint32_t)P.nt / (PAIR ? 2 : 1);         // filters whose weights this block holds
+        const uint32_t b_plane = PARTS * b_rows * 16;
+        const uint64_t a0 = operand_desc(sbase, (uint32_t)P.plane_pitch, sbo);
+        const uint64_t b0 = operand_desc(sbase + P.b_off, b_plane, 128);
+        const uint32_t a_k = (uint32_t)P.plane_pitch * 2 / 16, b_k = b_plane * 2 / 16, a_p = a_part / 16, b_p = b_rows;
+        int s = 0, b = 0, buf = 0;
+        uint32_t pha = 0, phb = 0, phc = 1;
+        bool ok = true;
+        for (int item = item0; item < P.items && ok && side == 0; item += item_step) {
+            for (int ks = k0; ks < k1 && ok; ++ks) {
+                if (kF32 || ks == k0) ok = wait(acc_empty(buf), phc);
+                ok = ok && wait(a_full(s), pha);
+                tc_fence_after();
+                const int kk_n = min(P.pl, planes - ks * P.pl) / 2;
+                const uint64_t as = a0 + (uint32_t)s * (a_bytes / 16);
+                const uint32_t d = tmem + (uint32_t)buf * (uint32_t)(MT * P.nt);
+                const uint32_t dc = d + 2u * P.nt;          // fp32: the small products (two buffers behind the two of the sums)
+#pragma unroll
+                for (int tap = 0; tap < TAPS; ++tap) {
+                    ok = ok && wait(b_full(b), P.resident ? 0u : phb);
+                    if (!ok) break;
+                    if (leader) {
+                        const uint64_t at = as + TL::tap_start(tap);
+                        const uint64_t bt = b0 + (uint32_t)b * (uint32_t)(P.b_bytes / 16);
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            if (kk < kk_n) {
+                                const uint64_t ak = at + kk * a_k, bk = bt + kk * b_k;
+                                const uint32_t first_s = tap > 0 || kk > 0 ? 1u : 0u;       // 0: the first of the stage
+                                const uint32_t first_i = first_s | (ks > k0 ? 1u : 0u);     // 0: the first of the item
+                                if (kF32) {
+                                    mma_f16<PAIR>(d, ak, bk, P.idesc, first_s);
+                                    mma_f16<PAIR>(dc, ak, bk + b_p, P.idesc, first_s);
+                                    mma_f16<PAIR>(dc, ak, bk + 2 * b_p, P.idesc, 1u);
+                                    mma_f16<PAIR>(dc, ak + a_p, bk, P.idesc, 1u);
+                                    mma_f16<PAIR>(dc, ak + a_p, bk + b_p, P.idesc, 1u);
+                                    mma_f16<PAIR>(dc, ak + 2 * a_p, bk, P.idesc, 1u);
+                                } else {
+#pragma unroll
+                                    for (int m = 0; m < MT; ++m) {
+                                        const uint64_t am = ak + m * 16 * TL::pitch;
+                                        if (DT == XGEN_I8_I32) mma_i8<PAIR>(d + m * P.nt, am, bk, P.idesc, first_i);
+                                        else mma_f16<PAIR>(d + m * P.nt, am, bk, P.idesc, first_i);
+                                    }
+                                }
+                            }
+                        }
+                        if (!P.resident) tc_commit<PAIR>(b_empty(b), both);
+                    }
+                    __syncwarp();
+                    if (++b == P.b_slots) { b = 0; phb ^= 1u; }
+                }
+                if (!ok) break;
+                if (leader) {
+                    tc_commit<PAIR>(a_empty(s), both);
+                    if (kF32 || ks + 1 == k1) tc_commit<PAIR>(acc_full(buf), both);
+                }
+                __syncwarp();
+                if (++s == P.a_stages) { s = 0; pha ^= 1u; }
+                if (kF32 || ks + 1 == k1) { if (++buf == P.acc_bufs) { buf = 0; phc ^= 1u; } }
+            }
+        }
+        if (leader && side == 0) tc_commit<PAIR>(all_done, both);
+        __syncwarp();
+        for (int it = 0; it < 4000000 && !mbar_ready(all_done, 0); ++it) {}
+    } else if (warp > kEpiWarps + kProdWarps) {
+        // ---- weights ---------------------------------------------------------------
+        const bool leader = elect_one();
+        int b = 0, issued = 0;
+        uint32_t ph = 1;
+        bool ok = true;
+        for (int item = item0; item < P.items && ok; item += item_step) {
+            for (int ks = k0; ks < k1 && ok; ++ks) {
+                for (int tap = 0; tap < TAPS; ++tap) {
+                    if (issued >= P.b_slots) ok = wait(b_empty(b), ph);
+                    if (!ok) break;
+                    if (leader) {
+                        // one copy for a tap: pieces of 2 KB with a copy of their own cost 50 cycles
+                        // of issue apiece and held the whole kernel to 5.5 TB/s of weights
+                        if (side == 0) mbar_expect_tx(b_full(b), (uint32_t)P.b_bytes * (PAIR ? 2 : 1));
+                        tensor_load4<PAIR>(sbase + P.b_off + (uint32_t)(b * P.b_bytes), &wmap, (n0 + side * P.nt / 2) * 2, 0, tap, ks * P.pl,
+                                           PAIR ? cluster_addr(b_full(b), (uint32_t)(crank & ~1)) : b_full(b));
+                    }
+                    __syncwarp();
+                    ++issued;
+                    if (++b == P.b_slots) { b = 0; ph ^= 1u; }
+                }
+            }
+            if (P.resident) break;
+        }
+        // Nothing may land in shared memory after this block has gone (a wait above may have given up).
+        for (int q = max(0, issued - P.b_slots); q < issued && side == 0; ++q)
+            for (int it = 0; it < 1000000 && !mbar_ready(b_full(q % P.b_slots), (uint32_t)(q / P.b_slots) & 1u); ++it) {}
+    } else {
+        // ---- epilogue ----------------------------------------------------------------
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        for (int i = tid; i < P.nt; i += kEpiWarps * 32) {
+            const bool in = n0 + i < P.c_out;
+            s_bias[i] = P.bias && in ? static_cast<const uint32_t *>(P.bias)[n0 + i] : 0u;
+            s_scale[i] = FUSED && P.rq_scale && in ? P.rq_scale[n0 + i] : 0.0f;
+        }
+        asm volatile("bar.sync 2, %0;" ::"n"(kEpiWarps * 32) : "memory");
+        const int quarter = warp & 3, half = warp >> 2;
+        const int sub = MT == 2 ? half : 0;
+        const int cols = MT == 2 ? P.nt : P.nt / 2, col0 = MT == 2 ? 0 : half * cols;   // this warp's filters of the tile
+        const uint32_t lanes = (uint32_t)quarter << 21;
+        const int m = quarter * 32 + lane;                       // pixel of the 128
+        float *const stage = reinterpret_cast<float *>(smem) + (size_t)(sub * 128 + m) * (P.nt + 4);
+        int buf = 0;
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int item = item0; item < P.items && ok; item += item_step) {
+            const TapItem t = tap_item<PAIR>(P, item, R, side);
+            const int v = t.v0 + sub * 16 + (m >> 3), ox = t.ox0 + (m & 7);
+            int64_t pixel;
+            bool valid;
+            int oy = 0, img = 0;
+            if (TAPS == 1) {
+                pixel = (int64_t)v * 8 + ox;
+                valid = pixel < P.npix;
+            } else {
+                img = v / P.vh;
+                oy = v - img * P.vh;
+                valid = img < P.n && oy < P.ho && ox < P.wo;
+                pixel = ((int64_t)img * P.ho + oy) * P.wo + ox;
+            }
+            // 16 sums of this lane's pixel, from column c of the warp's range on.
+            auto finish = [&](uint32_t (&r)[16], int c) {
+                if (P.splits > 1) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        *reinterpret_cast<uint4 *>(stage + col0 + c + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+                    return;
+                }
+                const int c0 = n0 + col0 + c;
+                if (c0 >= P.c_out) return;
+                tap_affine<DT, FUSED, 16>(P, s_bias, r, pixel, valid, c0, n0);
+                if (FUSED && P.pool) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        r[i] = tap_max<DT>(r[i], __shfl_xor_sync(0xFFFFFFFFu, r[i], 1));
+                        r[i] = tap_max<DT>(r[i], __shfl_xor_sync(0xFFFFFFFFu, r[i], 8));
+                    }
+                    if (valid && !(oy & 1) && !(ox & 1))
+                        tap_store<DT, FUSED, 16>(P, s_scale, r, ((int64_t)img * P.po + oy / 2) * P.pw + ox / 2, c0, n0);
+                } else if (valid) {
+                    tap_store<DT, FUSED, 16>(P, s_scale, r, pixel, c0, n0);
+                }
+            };
+            if (kF32) {
+                float sum[64];
+#pragma unroll
+                for (int i = 0; i < 64; ++i) sum[i] = 0.0f;
+                for (int ks = k0; ks < k1 && ok; ++ks) {
+                    ok = wait(acc_full(buf), ph);
+                    tc_fence_after();
+                    const uint32_t ta = tmem + lanes + (uint32_t)(buf * P.nt + col0);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        if (16 * q < cols) {
+                            uint32_t a[16], b[16];
+                            tmem_ld16(ta + 16 * q, a);
+                            tmem_ld16(ta + 2 * P.nt + 16 * q, b);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) sum[16 * q + i] += __uint_as_float(a[i]) + __uint_as_float(b[i]);
+                        }
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) arrive_lead(acc_empty(buf));
+                    if (++buf == P.acc_bufs) { buf = 0; ph ^= 1u; }
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (16 * q < cols && ok) {
+                        uint32_t r[16];
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(sum[16 * q + i]);
+                        finish(r, 16 * q);
+                    }
+                }
+            } else {
+                ok = wait(acc_full(buf), ph);
+                tc_fence_after();
+                const uint32_t ta = tmem + lanes + (uint32_t)((buf * MT + sub) * P.nt + col0);
+                for (int c = 0; c < cols && ok; c += 16) {
+                    uint32_t r[16];
+                    tmem_ld16(ta + c, r);
+                    tmem_wait_ld();
+                    finish(r, c);
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) arrive_lead(acc_empty(buf));
+                if (++buf == P.acc_bufs) { buf = 0; ph ^= 1u; }
+            }
+        }
+    }
+
+    // ---- split items: the blocks of the cluster add their sums, 16 pixels at a time ---------
+    if (P.splits > 1) {
+        __syncwarp();
+        cluster_meet();
+        constexpr int kAdders = (kEpiWarps + kProdWarps) * 32;
+        if (tid < kAdders && !s_abort) {
+            const TapItem t = tap_item<PAIR>(P, item0, R, side);
+            const int groups = P.nt / 8, pitch = (P.nt + 4) * 4;
+            const bool pool = FUSED && P.pool;
+            for (int u = rank; u < 8 * MT; u += P.splits) {
+                for (int w = tid; w < (pool ? 4 : 16) * groups; w += kAdders) {
+                    const int row = w / groups, g = w - row * groups;
+                    const int c0 = n0 + 8 * g;
+                    // pixel(s): a unit is two rows of 8; pooled pixel `row` covers columns 2 row, 2 row + 1 of both
+                    const int m0 = 16 * u + (pool ? 2 * row : row);
+                    const int v = t.v0 + (m0 >> 3), ox = t.ox0 + (m0 & 7);
+                    int64_t pixel;
+                    int img = 0, oy = 0;
+                    bool valid;
+                    if (TAPS == 1) {
+                        pixel = (int64_t)v * 8 + ox;
+                        valid = pixel < P.npix;
+                    } else {
+                        img = v / P.vh;
+                        oy = v - img * P.vh;
+                        valid = img < P.n && oy < P.ho && ox < P.wo;
+                        pixel = ((int64_t)img * P.ho + oy) * P.wo + ox;
+                    }
+                    if (!valid || c0 >= P.c_out) continue;
+                    uint32_t best[8];
+#pragma unroll 1
+                    for (int q = 0; q < (pool ? 4 : 1); ++q) {
+                        const int mm = m0 + (q & 1) + (q >> 1) * 8;
+                        uint32_t v8[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) v8[i] = 0;
+                        const uint32_t own = sbase + (uint32_t)(mm * pitch + g * 32);
+#pragma unroll 4
+                        for (int r = 0; r < P.splits; ++r) {
+                            const uint32_t far = cluster_addr(own, (uint32_t)(PAIR ? 2 * r + side : r));
+                            const uint4 a = lds_cluster(far), b = lds_cluster(far + 16);
+                            const uint32_t ab[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                v8[i] = DT == XGEN_I8_I32 ? v8[i] + ab[i] : __float_as_uint(__uint_as_float(v8[i]) + __uint_as_float(ab[i]));
+                        }
+                        tap_affine<DT, FUSED, 8>(P, s_bias, v8, pixel + (q & 1) + (int64_t)(q >> 1) * P.wo, true, c0, n0);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) best[i] = q == 0 ? v8[i] : tap_max<DT>(best[i], v8[i]);
+                    }
+                    tap_store<DT, FUSED, 8>(P, s_scale, best, pool ? ((int64_t)img * P.po + oy / 2) * P.pw + ox / 2 : pixel, c0, n0);
+                }
+            }
+        }
+    }
+    __syncwarp();
+    if (csize > 1) cluster_meet();       // nobody leaves while the others may still use its memory
+    tc_fence_before();
+    __syncthreads();
+    if (warp == kEpiWarps + kProdWarps) tmem_free<PAIR>(tmem, (uint32_t)P.tmem_cols);
+}
+
+// ---- weight image ----------------------------------------------------------------
+template <int DT> __device__ __forceinline__ void put_weight(uint8_t *img, int taps, int rows, int oc, int ic, int tap, float w) {
+    constexpr int cpp = TapTraits<DT>::cpp, parts = TapTraits<DT>::parts;
+    uint8_t *const p = img + ((size_t)(ic / cpp * taps + tap) * parts * rows + oc) * 16;
+    const int e = ic % cpp;
+    if (DT == XGEN_I8_I32) reinterpret_cast<int8_t *>(p)[e] = (int8_t)(int)w;
+    else if (DT == XGEN_F16_F32ACC) reinterpret_cast<__half *>(p)[e] = __float2half_rn(w);      // exact: it was fp16
+    else {
+        const float big = __uint_as_float(0x7F7F0000u);
+        __nv_bfloat16 b = __float2bfloat16_rn(fminf(fmaxf(w, -big), big));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            reinterpret_cast<__nv_bfloat16 *>(p + (size_t)k * rows * 16)[e] = b;
+            w -= __bfloat162float(b);
+            b = __float2bfloat16_rn(w);
+        }
+    }
+}
+
+template <int DT>
+__global__ void tap_expand_patterns(uint8_t *img, int c_in, int c_out, int rows, const int16_t *kpat, const uint4 *kw4,
+                                    const uint16_t *masks) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= c_in * c_out || kpat[k] < 0) return;
+    const uint4 w = kw4[k];
+    const unsigned mask = masks[kpat[k]];
+    int n = 0;
+    for (int t = 0; t < 9; ++t)
+        if ((mask >> t) & 1) {
+            put_weight<DT>(img, 9, rows, k / c_in, k % c_in, t, __uint_as_float(n == 0 ? w.x : n == 1 ? w.y : n == 2 ? w.z : w.w));
+            ++n;
+        }
+}
+
+template <int DT>
+__global__ void tap_expand_dense(uint8_t *img, int c_in, int c_out, int rows, const void *dense, const uint8_t *row_keep,
+                                 const uint8_t *col_keep, int br, int bc) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= c_in * c_out) return;
+    const int oc = k / c_in, ic = k % c_in;
+    const size_t blk = (size_t)(oc / br) * ((c_in + bc - 1) / bc) + ic / bc;
+    if (!row_keep[blk * br + oc % br] || !col_keep[blk * bc + ic % bc]) return;
+    const float w = DT == XGEN_F32 ? static_cast<const float *>(dense)[k] : __half2float(static_cast<const __half *>(dense)[k]);
+    put_weight<DT>(img, 1, rows, oc, ic, 0, w);
+}
+
+static int tap_cpp(xgen_dtype dt) { return dt == XGEN_I8_I32 ? 16 : 8; }
+static int tap_parts(xgen_dtype dt) { return dt == XGEN_F32 ? 3 : 1; }
+
+// The zeroed image, and `extra` bytes of scratch that tap_done gives back.
+static xgen_status tap_alloc(TapWeights &tw, xgen_dtype dt, int taps, int c_in, int c_out, size_t extra, uint8_t **scratch) {
+    tw.dtype = dt; tw.taps = taps; tw.c_in = c_in; tw.c_out = c_out;
+    tw.planes = (c_in + 2 * tap_cpp(dt) - 1) / (2 * tap_cpp(dt)) * 2;
+    tw.rows = (c_out + 15) / 16 * 16;
+    const size_t bytes = (size_t)tw.planes * taps * tap_parts(dt) * tw.rows * 16;
+    cudaError_t e = cudaMalloc(&tw.dev, bytes);
+    if (e == cudaSuccess) e = cudaMalloc(scratch, extra);
+    if (e == cudaSuccess) e = cudaMemsetAsync(tw.dev, 0, bytes, 0);
+    if (e == cudaSuccess) return XGEN_OK;
+    cudaGetLastError();
+    tap_free(tw);
+    return e == cudaErrorMemoryAllocation ? XGEN_ERR_ALLOC : XGEN_ERR_CUDA;
+}
+
+static xgen_status tap_done(TapWeights &tw, uint8_t *scratch, cudaError_t e) {
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+    cudaFree(scratch);
+    if (e == cudaSuccess) return XGEN_OK;
+    cudaGetLastError();
+    tap_free(tw);
+    return XGEN_ERR_CUDA;
+}
+
+void tap_free(TapWeights &tw) {
+    if (tw.dev) cudaFree(tw.dev);
+    tw.dev = nullptr;
+}
+
+xgen_status tap_upload_patterns(TapWeights &tw, xgen_dtype dt, int c_in, int c_out, const int16_t *kpat, const uint32_t *kw4,
+                                const uint16_t *masks, int n_masks) {
+    const size_t nk = (size_t)c_in * c_out, wb = nk * 16, pb = nk * 2;
+    uint8_t *scratch = nullptr;
+    const xgen_status st = tap_alloc(tw, dt, 9, c_in, c_out, wb + pb + (size_t)n_masks * 2, &scratch);
+    if (st != XGEN_OK) return st;
+    cudaError_t e = cudaMemcpyAsync(scratch, kw4, wb, cudaMemcpyHostToDevice, 0);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(scratch + wb, kpat, pb, cudaMemcpyHostToDevice, 0);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(scratch + wb + pb, masks, (size_t)n_masks * 2, cudaMemcpyHostToDevice, 0);
+    const unsigned blocks = (unsigned)((nk + 255) / 256);
+    const uint4 *w = reinterpret_cast<const uint4 *>(scratch);
+    const int16_t *kp = reinterpret_cast<const int16_t *>(scratch + wb);
+    const uint16_t *mk = reinterpret_cast<const uint16_t *>(scratch + wb + pb);
+    if (e == cudaSuccess) {
+        if (dt == XGEN_F32) tap_expand_patterns<XGEN_F32><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, kp, w, mk);
+        else if (dt == XGEN_F16_F32ACC) tap_expand_patterns<XGEN_F16_F32ACC><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, kp, w, mk);
+        else tap_expand_patterns<XGEN_I8_I32><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, kp, w, mk);
+    }
+    return tap_done(tw, scratch, e);
+}
+
+xgen_status tap_upload_dense(TapWeights &tw, xgen_dtype dt, int c_in, int c_out, const void *dense_w, const uint8_t *row_keep,
+                             const uint8_t *col_keep, int br, int bc) {
+    const size_t n = (size_t)c_in * c_out, wb = (n * (dt == XGEN_F32 ? 4 : 2) + 15) / 16 * 16;
+    const size_t blocks_of = (size_t)((c_out + br - 1) / br) * ((c_in + bc - 1) / bc);
+    uint8_t *scratch = nullptr;
+    const xgen_status st = tap_alloc(tw, dt, 1, c_in, c_out, wb + blocks_of * ((size_t)br + bc), &scratch);
+    if (st != XGEN_OK) return st;
+    uint8_t *rk = scratch + wb, *ck = rk + blocks_of * br;
+    cudaError_t e = cudaMemcpyAsync(scratch, dense_w, n * (dt == XGEN_F32 ? 4 : 2), cudaMemcpyHostToDevice, 0);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(rk, row_keep, blocks_of * br, cudaMemcpyHostToDevice, 0);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(ck, col_keep, blocks_of * bc, cudaMemcpyHostToDevice, 0);
+    const unsigned blocks = (unsigned)((n + 255) / 256);
+    if (e == cudaSuccess) {
+        if (dt == XGEN_F32) tap_expand_dense<XGEN_F32><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, scratch, rk, ck, br, bc);
+        else tap_expand_dense<XGEN_F16_F32ACC><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, scratch, rk, ck, br, bc);
+    }
+    return tap_done(tw, scratch, e);
+}
+
+// ---- plans ---------------------------------------------------------------------
+template <int DT, int TAPS> static const void *tap_kernel_dt(int stride, int mt, bool pair) {
+#define TAP_PICK(S, M) (pair ? (const void *)tap_kernel<DT, S, TAPS, M, true> : (const void *)tap_kernel<DT, S, TAPS, M, false>)
+    constexpr int M2 = DT == XGEN_F32 ? 1 : 2, S2 = TAPS == 1 ? 1 : 2;      // (what there is no instance of is never asked for)
+    if (stride == 1) return mt == 2 ? TAP_PICK(1, M2) : TAP_PICK(1, 1);
+    return mt == 2 ? TAP_PICK(S2, M2) : TAP_PICK(S2, 1);
+#undef TAP_PICK
+}
+static const void *tap_kernel_of(xgen_dtype dt, int stride, int taps, int mt, bool pair) {
+    if (taps == 1) return dt == XGEN_F32 ? tap_kernel_dt<XGEN_F32, 1>(1, mt, pair) : tap_kernel_dt<XGEN_F16_F32ACC, 1>(1, mt, pair);
+    if (dt == XGEN_F32) return tap_kernel_dt<XGEN_F32, 9>(stride, mt, pair);
+    return dt == XGEN_F16_F32ACC ? tap_kernel_dt<XGEN_F16_F32ACC, 9>(stride, mt, pair) : tap_kernel_dt<XGEN_I8_I32, 9>(stride, mt, pair);
+}
+
+// Once per kernel and device: large shared memory, clusters of 16.
+static cudaError_t tap_allow(const void *kern, int device) {
+    static std::mutex mu;
+    static std::vector<std::pair<const void *, int>> done;
+    std::lock_guard<std::mutex> lock(mu);
+    for (auto &d : done)
+        if (d.first == kern && d.second == device) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTapSmemMax);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) done.emplace_back(kern, device);
+    return e;
+}
+
+// How many clusters of `size` blocks (one block per SM) the device holds at once.
+static int tap_clusters(int size, int device, int sms) {
+    static std::mutex mu;
+    static int known[64][17];
+    if (device < 0 || device >= 64) return sms / size;
+    std::lock_guard<std::mutex> lock(mu);
+    int &k = known[device][size];
+    if (k) return k;
+    const void *kern = tap_kernel_of(XGEN_F16_F32ACC, 1, 9, 1, false);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size); cfg.blockDim = dim3(kTapThreads); cfg.dynamicSmemBytes = kTapSmemMax;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)size; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    int n = 0;
+    if (tap_allow(kern, device) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+    k = n > 0 ? n : -1;
+    return k;
+}
+
+static int tap_pixels(int stride, int taps, int mt) {
+    const int R = 16 * mt;
+    return taps == 1 ? 8 * R : stride == 1 ? 10 * (R + 2) : 9 * (4 * R + 2);
+}
+
+bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &best) {
+    static int sm_count[64];
+    int sms = 148;
+    if (device >= 0 && device < 64) {
+        if (!sm_count[device]) cudaDeviceGetAttribute(&sm_count[device], cudaDevAttrMultiProcessorCount, device);
+        if (sm_count[device]) sms = sm_count[device];
+    }
+    const xgen_dtype dt = tw.dtype;
+    const int parts = tap_parts(dt), cpp = tap_cpp(dt), prod = dt == XGEN_F32 ? 6 : 1;
+    const int xb = dt == XGEN_F32 ? 4 : dt == XGEN_F16_F32ACC ? 2 : 1, yb = dt == XGEN_F16_F32ACC ? 2 : 4;
+    const int ho = (s.h - 1) / s.stride + 1, wo = (s.w - 1) / s.stride + 1;
+    best = TapPlan();
+    best.cycles = 1e30;
+    for (int shape = 0; shape < (dt == XGEN_F32 ? 2 : 4); ++shape) {
+        TapPlan p;
+        p.pair = shape & 1;
+        p.mt = 1 + (shape >> 1);
+        const int mt = p.mt, ways = p.pair ? 2 : 1, R = 16 * mt, pixels = tap_pixels(s.stride, tw.taps, mt);
+        int64_t row_tiles;
+        if (tw.taps == 1) {
+            p.segs = 1; p.vh = 1;
+            row_tiles = (s.h + R - 1) / R;
+        } else {
+            // Rows of all images below each other: every image rounded up to whole tiles, or one row of
+            // zeros between images and tiles that cross them, whichever has fewer rows.
+            const int whole = (ho + R - 1) / R * R;
+            const int gap = ho + 1 + (s.pool && (ho + 1) % 2 ? 1 : 0);
+            const int64_t tiles_whole = (int64_t)s.n * whole / R, tiles_gap = ((int64_t)s.n * gap + R - 1) / R;
+            p.straddle = tiles_gap < tiles_whole;
+            p.vh = p.straddle ? gap : whole;
+            row_tiles = p.straddle ? tiles_gap : tiles_whole;
+            p.segs = (wo + 7) / 8;
+        }
+        if (row_tiles * p.segs * ((tw.rows + 31) / 32) > 0x7FFFFFFF / 32) continue;
+        p.row_tiles = (int)row_tiles;
+        const int tiles = (p.row_tiles * p.segs + ways - 1) / ways;
+        if (p.pair && p.row_tiles * p.segs == 1) continue;
+        // fp32 keeps four accumulators of `nt` columns and 64 sums a thread; 512 columns hold all of the others'
+        const int nt_top = dt == XGEN_F32 || !p.pair ? 128 : kMaxFilterTile;
+        for (int nt_max = 32; nt_max <= nt_top; nt_max += 32) {
+            p.nblk = (tw.c_out + nt_max - 1) / nt_max;
+            p.nt = ((tw.c_out + p.nblk - 1) / p.nblk + 31) / 32 * 32;
+            p.nblk = (tw.c_out + p.nt - 1) / p.nt;
+            if (p.nt != nt_max) continue;
+            p.items = tiles * p.nblk;
+            for (int pl = 2; pl <= 8; pl *= 2) {
+                if (pl > 2 && pl / 2 >= tw.planes) continue;
+                if (dt == XGEN_F32 && tw.taps * pl / 2 > 18) continue;      // bounds the chain of the fp32 accumulator
+                p.pl = pl;
+                p.stages = (tw.planes + pl - 1) / pl;
+                // 16-byte accesses of 8 lanes (pl planes x 8 / pl pixels) fall into distinct banks
+                p.plane_pitch = pixels * 16;
+                while (p.plane_pitch % 128 != 128 / pl % 128) p.plane_pitch += 16;
+                const size_t a_bytes = (size_t)parts * pl * p.plane_pitch, b_bytes = (size_t)pl * parts * p.nt * 16 / ways;
+                const size_t tables = ((size_t)pixels * 8 + 127) / 128 * 128;
+                for (int sp = 1; sp * ways <= 16 && sp <= p.stages; ++sp) {
+                    p.per_split = (p.stages + sp - 1) / sp;
+                    p.splits = (p.stages + p.per_split - 1) / p.per_split;
+                    if (p.splits != sp) continue;
+                    int64_t waves;
+                    if (sp == 1) {
+                        const int units = p.pair ? std::max(0, tap_clusters(2, device, sms)) : sms;
+                        if (units == 0) continue;
+                        const int at_once = p.items <= units ? p.items : std::min(p.items, std::max(1, units / p.nblk) * p.nblk);
+                        p.grid = at_once * ways;
+                        waves = (p.items + at_once - 1) / at_once;
+                    } else {
+                        if (p.items * (int64_t)sp * ways > 4 * sms) continue;
+                        const int cl = tap_clusters(sp * ways, device, sms);
+                        if (cl <= 0) continue;
+                        p.grid = p.items * sp * ways;
+                        waves = (p.items + cl - 1) / cl;
+                    }
+                    const int64_t uses = (sp == 1 ? waves : 1) * p.per_split;      // stages one block goes through
+                    // Shared memory: two tiles of x (more for a plain product, whose stages are short), the rest weights.
+                    const int want_a = (int)std::min<int64_t>(uses, tw.taps == 1 ? kMaxA : 2);
+                    const int all_b = p.per_split * tw.taps;
+                    bool fits = false;
+                    for (p.a_stages = want_a; p.a_stages >= 1; --p.a_stages) {
+                        const size_t left_a = p.a_stages * a_bytes + tables;
+                        if (left_a >= (size_t)kTapSmemMax) continue;
+                        const int room = (int)std::min<size_t>(kMaxB, ((size_t)kTapSmemMax - left_a) / b_bytes);
+                        p.resident = all_b <= room;
+                        p.b_slots = std::min(room, all_b);
+                        if (p.b_slots >= std::min(all_b, 3) && p.a_stages >= std::min<int64_t>(2, uses)) { fits = true; break; }
+                    }
+                    if (!fits) continue;
+                    p.smem = p.a_stages * a_bytes + p.b_slots * b_bytes + tables;
+                    if (sp > 1) p.smem = std::max(p.smem, (size_t)mt * 128 * (p.nt + 4) * 4);
+                    if (p.smem > (size_t)kTapSmemMax) continue;
+                    p.acc_bufs = dt == XGEN_F32 || 2 * mt * p.nt <= 512 ? 2 : 1;
+                    const int cols = dt == XGEN_F32 ? 4 * p.nt : p.acc_bufs * mt * p.nt;
+                    for (p.tmem_cols = 32; p.tmem_cols < cols;) p.tmem_cols *= 2;
+                    // Cycles of a stage: the matrix instructions (nt / 2 each), or what they and the copies move
+                    // through shared memory at 128 bytes a cycle (128 rows of x, the block's filters), or
+                    // what comes from L2.  A tap costs about 40 cycles besides, a stage 300.
+                    const double kk = (double)tw.planes / p.stages / 2, taps = tw.taps;
+                    const double b_stage = taps * kk * 2 * parts * p.nt * 16.0 / ways, b_moved = p.resident && sp == 1 ? b_stage / waves : b_stage;
+                    const double x_moved = (double)pixels * kk * 2 * cpp * xb, a_stage = (double)parts * pixels * kk * 2 * 16;
+                    const double instr = taps * kk * mt * prod;
+                    const double mma = instr * std::max(p.nt / 2.0, 40.0);
+                    const double shared = (instr * (4096.0 + p.nt * 32.0 / ways) + b_moved + 2 * a_stage) / 128.0;
+                    const double move = (x_moved + b_moved) / 40.0;
+                    const double stage = std::max(std::max(mma, shared), move) + 300.0 + 40.0 * taps;
+                    const double out = (double)mt * 128 * p.nt * yb / 24.0;
+                    const double item = p.per_split * stage;
+                    double c = 3500.0 + (p.pair ? 2500.0 : 0.0);
+                    if (sp == 1) c += waves * std::max(item, p.acc_bufs == 2 ? out : 0.0) + (p.acc_bufs == 2 ? out : waves * out);
+                    else c += waves * (item + 2500.0 + 40.0 * sp + mt * 128.0 * p.nt * 4 / 48.0 + out / sp);
+                    if (c < best.cycles * 0.999) { best = p; best.cycles = c; }
+                }
+            }
+        }
+    }
+    if (best.cycles >= 1e30) return false;
+    // [plane][tap][part][filter x 16 bytes], in units of 8 bytes; what lies beyond the image reads as zeros
+    EncodeTiledFn encode = encode_tiled_fn();
+    if (!encode) return false;
+    const cuuint64_t dim[4] = {(cuuint64_t)tw.rows * 2, (cuuint64_t)parts, (cuuint64_t)tw.taps, (cuuint64_t)tw.planes};
+    const cuuint64_t row = (cuuint64_t)tw.rows * 16;
+    const cuuint64_t str[3] = {row, row * parts, row * parts * tw.taps};
+    const cuuint32_t box[4] = {(cuuint32_t)(best.pair ? best.nt : best.nt * 2), (cuuint32_t)parts, 1, (cuuint32_t)best.pl};
+    const cuuint32_t one[4] = {1, 1, 1, 1};
+    return encode(&best.wmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4, tw.dev, dim, str, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p, const TapCall &c, cudaStream_t st) {
+    const xgen_dtype dt = tw.dtype;
+    const int parts = tap_parts(dt), xb = dt == XGEN_F32 ? 4 : dt == XGEN_F16_F32ACC ? 2 : 1;
+    const int yb = c.rq_scale ? 1 : dt == XGEN_F16_F32ACC ? 2 : 4, rb = dt == XGEN_F16_F32ACC ? 2 : 4;
+    TapParams P{};
+    P.x = c.x; P.y = c.y; P.bias = c.bias; P.residual = c.residual; P.rq_scale = c.rq_scale;
+    P.status = c.status; P.wait_us = c.wait_us;
+    P.rq_zero = c.rq_zero; P.relu = c.relu ? 1 : 0; P.pool = c.pool;
+    P.n = s.n; P.h = s.h; P.w = s.w;
+    P.ho = (s.h - 1) / s.stride + 1; P.wo = (s.w - 1) / s.stride + 1;
+    P.po = c.pool ? P.ho / 2 : P.ho; P.pw = c.pool ? P.wo / 2 : P.wo;
+    P.npix = s.rows;
+    P.c_in = tw.c_in; P.c_out = tw.c_out;
+    P.vh = p.vh; P.straddle = p.straddle;
+    P.segs = p.segs; P.nblk = p.nblk; P.nt = p.nt; P.items = p.items; P.splits = p.splits; P.per_split = p.per_split; P.stages = p.stages;
+    P.pl = p.pl; P.pl_log = p.pl == 2 ? 1 : p.pl == 4 ? 2 : 3; P.plane_pitch = p.plane_pitch;
+    P.a_stages = p.a_stages; P.b_slots = p.b_slots; P.resident = p.resident;
+    P.b_bytes = p.pl * parts * (p.pair ? p.nt / 2 : p.nt) * 16;
+    P.b_off = p.a_stages * parts * p.pl * p.plane_pitch;
+    P.tab_off = P.b_off + p.b_slots * P.b_bytes;
+    P.tmem_cols = p.tmem_cols; P.acc_bufs = p.acc_bufs;
+    auto aligned = [](const void *q, uintptr_t a) { return ((uintptr_t)q & (a - 1)) == 0; };
+    P.vec_x = aligned(c.x, 16) && (size_t)tw.c_in * xb % 16 == 0;
+    P.vec_y = aligned(c.y, 16) && (size_t)tw.c_out * yb % 16 == 0;
+    P.y32 = aligned(c.y, 32) && (size_t)tw.c_out * yb % 32 == 0;
+    P.vec_r = c.residual && aligned(c.residual, 16) && (size_t)tw.c_out * rb % 16 == 0;
+    // D fp32 (int32), A fp16 / bf16 / u8, B fp16 / bf16 / s8, both K-major, 128 rows (256 of a pair)
+    P.idesc = ((uint32_t)(p.nt >> 3) << 17) | ((p.pair ? 16u : 8u) << 24) |
+              (dt == XGEN_I8_I32 ? (2u << 4) | (1u << 10) : (1u << 4) | (dt == XGEN_F32 ? (1u << 7) | (1u << 10) : 0u));
+    const void *kern = tap_kernel_of(dt, s.stride, tw.taps, p.mt, p.pair);
+    int device = 0;
+    cudaError_t e = cudaGetDevice(&device);
+    if (e == cudaSuccess) e = tap_allow(kern, device);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)p.grid); cfg.blockDim = dim3(kTapThreads); cfg.dynamicSmemBytes = p.smem; cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    unsigned na = 0;
+    if (c.overlap) {
+        at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[na++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    const int cluster = (p.pair ? 2 : 1) * p.splits;
+    if (cluster > 1) {
+        at[na].id = cudaLaunchAttributeClusterDimension;
+        at[na].val.clusterDim.x = (unsigned)cluster; at[na].val.clusterDim.y = at[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    cfg.attrs = at; cfg.numAttrs = na;
+    void *args[2] = {&P, const_cast<CUtensorMap *>(&p.wmap)};
+    e = cudaLaunchKernelExC(&cfg, kern, args);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) count_launch();
+    return e;
+}
+
+}  // namespace patconv
