@@ -554,7 +554,7 @@ xgen_status xgen_blockgemm_run(const xgen_blockgemm_packed *hc, const void *x, i
     if (h->device < 0) return XGEN_ERR_CUDA;
     if (h->tap.dev) {
         patconv::TapShape ts;
-        ts.n = 1; ts.w = 8; ts.h = (int)((m + 7) / 8); ts.rows = m;
+        ts.n = 1; ts.w = 8; ts.h = (int)((m + 7) / 8); ts.rows = m; ts.staged = H.c_out * (int)eb % 16 != 0;
         int prev = 0;
         cudaGetDevice(&prev);
         if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;

@@ -1427,7 +1427,7 @@ static bool tap_plan_of(const xgen_patconv_packed *h, const TapShape &s, TapPlan
     std::lock_guard<std::mutex> lock(h->tap_mu);
     TapEntry *victim = &h->tap_cache[0];
     for (TapEntry &e : h->tap_cache) {
-        if (e.stamp && e.shape.n == s.n && e.shape.h == s.h && e.shape.w == s.w && e.shape.pool == s.pool) {
+        if (e.stamp && e.shape.n == s.n && e.shape.h == s.h && e.shape.w == s.w && e.shape.pool == s.pool && e.shape.staged == s.staged) {
             e.stamp = ++h->tap_stamp;
             plan = e.plan;
             return true;
@@ -1479,6 +1479,7 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
     if (!forced && on_matrix_units(h)) {
         TapShape ts;
         ts.n = n; ts.h = hh; ts.w = ww; ts.stride = p.stride; ts.pool = pool == 2;
+        ts.staged = p.c_out * (rq_scale ? 1 : p.dtype == XGEN_F16_F32ACC ? 2 : 4) % 16 != 0;
         int prev = 0;
         if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
         if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;

@@ -92,6 +92,10 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void copy16(uint32_t dst, const void *src, uint32_t bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
+// Ask for `bytes` (a multiple of 16, from a multiple of 16) to be brought into L2.
+__device__ __forceinline__ void prefetch_l2(const void *src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int PENDING> __device__ __forceinline__ void copy_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
@@ -126,13 +130,17 @@ template <bool PAIR> __device__ __forceinline__ void tc_commit(uint32_t mbar, ui
     else
         asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
 }
+// Operand descriptors as (low word, high word): only the low word, which holds the address, moves.
 #define XGEN_MMA(GROUP, KIND)                                                                                             \
-    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%0], %1, %2, %3, p;\n}" \
-                 ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory")
-template <bool PAIR> __device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+    asm volatile("{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.u32 p, %6, 0;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n" \
+                 " tcgen05.mma.cta_group::" GROUP ".kind::" KIND " [%0], a, b, %5, p;\n}"                                   \
+                 ::"r"(d), "r"(a), "r"(a_hi), "r"(b), "r"(b_hi), "r"(idesc), "r"(acc) : "memory")
+template <bool PAIR>
+__device__ __forceinline__ void mma_f16(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t idesc, uint32_t acc) {
     if (PAIR) XGEN_MMA("2", "f16"); else XGEN_MMA("1", "f16");
 }
-template <bool PAIR> __device__ __forceinline__ void mma_i8(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+template <bool PAIR>
+__device__ __forceinline__ void mma_i8(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t idesc, uint32_t acc) {
     if (PAIR) XGEN_MMA("2", "i8"); else XGEN_MMA("1", "i8");
 }
 #undef XGEN_MMA

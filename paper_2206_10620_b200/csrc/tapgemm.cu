@@ -47,13 +47,17 @@
 
 namespace patconv {
 
-// 16 warps: four a scheduler, so that a thread may hold 128 registers (fp32 keeps 64 sums)
-constexpr int kEpiWarps = 8, kProdWarps = 6;
-constexpr int kTapThreads = (kEpiWarps + kProdWarps + 2) * 32;
+// Epilogue warps wait for tensor memory and y more than they compute: sixteen where the registers
+// allow it; fp32 keeps 64 sums a thread, so eight.
+__host__ __device__ constexpr int epi_warps(int dt) { return dt == XGEN_F32 ? 8 : 16; }
+constexpr int kProdWarps = 6;
+__host__ __device__ constexpr int tap_threads(int dt) { return (epi_warps(dt) + kProdWarps + 2) * 32; }
 constexpr int kProdThreads = kProdWarps * 32;
 constexpr int kMaxA = 4, kMaxB = 64;
 constexpr int kTapSmemMax = 232448 - 4096;      // 227 KB less static shared memory
 constexpr int kMaxFilterTile = 256;
+constexpr int kStagePitch = 20;                 // words of a staged pixel's 16 sums: rows of 16-byte accesses in distinct banks
+constexpr int kStageBytes = 32 * kStagePitch * 4;   // a warp's
 
 struct TapParams {
     const void *x; void *y; const void *bias; const void *residual; const float *rq_scale;
@@ -67,8 +71,9 @@ struct TapParams {
     int segs, nblk, nt, items, splits, per_split, stages;
     int pl, pl_log, plane_pitch;
     int a_stages, b_slots, resident, b_bytes;
-    int b_off, tab_off;                         // bytes into dynamic shared memory
-    int tmem_cols, acc_bufs;
+    int b_off, tab_off, stage_off;              // bytes into dynamic shared memory
+    int tmem_cols, acc_bufs, staged;
+    int tap_start[9];                           // first staged pixel of a tap
     int vec_x;                                  // 16-byte pieces of x can be copied as they are
     int vec_y, vec_r, y32;                      // 16-byte (32-byte) pieces of y / the residual can be moved whole
     uint32_t idesc;
@@ -87,7 +92,7 @@ template <int STRIDE, int TAPS, int MT> struct TapTile {
     static constexpr int R = 16 * MT;
     static constexpr int pitch = TAPS == 1 ? 8 : STRIDE == 1 ? 10 : 9;
     static constexpr int pixels = TAPS == 1 ? 8 * R : STRIDE == 1 ? 10 * (R + 2) : 9 * (4 * R + 2);
-    static __host__ __device__ constexpr int tap_start(int t) {
+    static int tap_start(int t) {
         if (TAPS == 1) return 0;
         const int dy = t / 3, dx = t % 3;
         if (STRIDE == 1) return dy * 10 + dx;
@@ -114,7 +119,7 @@ template <int STRIDE, int TAPS, int MT> struct TapTile {
 // ---- results -------------------------------------------------------------------
 // W sums of adjacent channels of one pixel: bias, residual, activation, in fp32 (int32).
 template <int DT, bool FUSED, int W>
-__device__ __forceinline__ void tap_affine(const TapParams &P, const uint32_t *s_bias, uint32_t (&v)[W], int64_t pixel,
+__device__ __forceinline__ void tap_affine(const TapParams &P, const uint32_t *s_bias, uint32_t (&v)[W], int pixel,
                                            bool valid, int c0, int n0) {
 #pragma unroll
     for (int q = 0; q < W / 4; ++q) {
@@ -184,9 +189,30 @@ template <int DT> __device__ __forceinline__ uint32_t tap_max(uint32_t a, uint32
     return __float_as_uint(f);
 }
 
+// Re-quantisation of an int32 result: scaled, rounded, zero point added (saturating); then clamped to uint8.
+__device__ __forceinline__ int tap_level(const TapParams &P, uint32_t v, float scale) {
+    int r;
+    asm("add.sat.s32 %0, %1, %2;" : "=r"(r) : "r"(__float2int_rn(__fmul_rn((float)(int)v, scale))), "r"(P.rq_zero));
+    return r;
+}
+__device__ __forceinline__ uint32_t tap_code(const TapParams &P, uint32_t v, float scale) {
+    return (uint32_t)max(min(tap_level(P, v, scale), 255), 0);
+}
+__device__ __forceinline__ uint32_t pack_codes(int a, int b, int c, int d) {
+    uint32_t hi, r;
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, 0;" : "=r"(hi) : "r"(d), "r"(c));
+    asm("cvt.pack.sat.u8.s32.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(b), "r"(a), "r"(hi));
+    return r;
+}
+// Two fp32 additions (the packed instruction rounds each like the scalar one).
+__device__ __forceinline__ void add2(uint32_t &a0, uint32_t &a1, uint32_t b0, uint32_t b1) {
+    asm("{\n .reg .b64 a, b;\n mov.b64 a, {%0, %1};\n mov.b64 b, {%2, %3};\n add.rn.f32x2 a, a, b;\n mov.b64 {%0, %1}, a;\n}"
+        : "+r"(a0), "+r"(a1) : "r"(b0), "r"(b1));
+}
+
 // Store W results of one pixel, converted; whole 16- or 32-byte pieces where the tensor allows it.
 template <int DT, bool FUSED, int W>
-__device__ __forceinline__ void tap_store(const TapParams &P, const float *s_scale, const uint32_t (&v)[W], int64_t pixel,
+__device__ __forceinline__ void tap_store(const TapParams &P, const float *s_scale, const uint32_t (&v)[W], int pixel,
                                           int c0, int n0) {
     const size_t off = (size_t)pixel * P.c_out + c0;
     const bool full = c0 + W <= P.c_out;
@@ -196,12 +222,7 @@ __device__ __forceinline__ void tap_store(const TapParams &P, const float *s_sca
         for (int q = 0; q < W / 4; ++q) {
             code[q] = 0;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float f = __fmul_rn((float)(int)v[4 * q + i], s_scale[c0 - n0 + 4 * q + i]);
-                int r;
-                asm("add.sat.s32 %0, %1, %2;" : "=r"(r) : "r"(__float2int_rn(f)), "r"(P.rq_zero));
-                code[q] |= (uint32_t)max(min(r, 255), 0) << (8 * i);
-            }
+            for (int i = 0; i < 4; ++i) code[q] |= tap_code(P, v[4 * q + i], s_scale[c0 - n0 + 4 * q + i]) << (8 * i);
         }
         uint8_t *y = static_cast<uint8_t *>(P.y) + off;
         if (full && P.vec_y) {
@@ -248,6 +269,193 @@ __device__ __forceinline__ void tap_store(const TapParams &P, const float *s_sca
 #pragma unroll
         for (int i = 0; i < W; ++i)
             if (c0 + i < P.c_out) y[i] = v[i];
+    }
+}
+
+// One result, for tensors whose rows are not whole 16-byte pieces.
+template <int DT, bool FUSED>
+__device__ __forceinline__ uint32_t tap_affine1(const TapParams &P, uint32_t bias, uint32_t v, size_t off) {
+    v = DT == XGEN_I8_I32 ? v + bias : __float_as_uint(__uint_as_float(v) + __uint_as_float(bias));
+    if (FUSED && P.residual) {
+        if (DT == XGEN_I8_I32) v += static_cast<const uint32_t *>(P.residual)[off];
+        else if (DT == XGEN_F32) v = __float_as_uint(__uint_as_float(v) + static_cast<const float *>(P.residual)[off]);
+        else v = __float_as_uint(__uint_as_float(v) + __half2float(static_cast<const __half *>(P.residual)[off]));
+    }
+    return P.relu ? tap_max<DT>(v, 0u) : v;
+}
+template <int DT, bool FUSED>
+__device__ __forceinline__ void tap_store1(const TapParams &P, float scale, uint32_t v, size_t off) {
+    if (FUSED && DT == XGEN_I8_I32 && P.rq_scale) static_cast<uint8_t *>(P.y)[off] = (uint8_t)tap_code(P, v, scale);
+    else if (DT == XGEN_F16_F32ACC) static_cast<__half *>(P.y)[off] = __float2half_rn(__uint_as_float(v));
+    else static_cast<uint32_t *>(P.y)[off] = v;
+}
+
+// A warp's 32 pixels x 16 channels, staged as [pixel][kStagePitch] sums: finish and store them, pooled,
+// or with neighbouring lanes on neighbouring elements where rows of y are not whole 16-byte pieces.
+// `pix`: this lane's own pixel of the unpooled result, -1 if there is none; `out`: where it is stored
+// (pooled: of the window whose first pixel it is).
+template <int DT, bool FUSED>
+__device__ __forceinline__ void tap_emit(const TapParams &P, const uint32_t *st, const uint32_t *s_bias, const float *s_scale,
+                                      int pix, int out, int c_base, int n0, int lane) {
+    constexpr uint32_t kAll = 0xFFFFFFFFu;
+    const bool pool = FUSED && P.pool;
+    const int c = c_base + (lane & 15);          // a lane keeps its channel, half-warps take a pixel each
+    const bool in = c < P.c_out;
+    const uint32_t bias = in ? s_bias[c - n0] : 0u;
+    const float scale = FUSED && in ? s_scale[c - n0] : 0.0f;
+#pragma unroll 2
+    for (int it = 0; it < (pool ? 4 : 16); ++it) {
+        const int jp = 2 * it + (lane >> 4);
+        uint32_t best = 0;
+        int to = -1;
+#pragma unroll 1
+        for (int q = 0; q < (pool ? 4 : 1); ++q) {
+            const int j = pool ? (jp >> 2) * 16 + (jp & 3) * 2 + (q & 1) + (q >> 1) * 8 : jp;
+            const int px = __shfl_sync(kAll, pix, j);
+            const int o = __shfl_sync(kAll, out, j);
+            if (q == 0) to = o;
+            if (px >= 0 && in) {
+                const uint32_t v = tap_affine1<DT, FUSED>(P, bias, st[j * kStagePitch + (lane & 15)], (size_t)px * P.c_out + c);
+                best = q == 0 ? v : tap_max<DT>(best, v);
+            } else to = -1;
+        }
+        if (to >= 0) tap_store1<DT, FUSED>(P, scale, best, (size_t)to * P.c_out + c);
+    }
+}
+
+// 32 sums of one pixel, from channel c0 on, finished and stored by their own lane: 64 to 128 bytes in
+// whole sectors.
+template <int DT, bool FUSED>
+__device__ __forceinline__ void tap_direct(const TapParams &P, const uint32_t *s_bias, const float *s_scale, uint32_t (&v)[32],
+                                           int pix, int out, int c0, int n0) {
+    if (FUSED && P.pool) {
+        // The four lanes of a 2x2 window share its 32 channels out among them: each sends what the other
+        // needs, 16 and then 8 words, and finishes 8 channels of the pooled pixel.
+        const bool late = P.residual == nullptr;             // bias and activation commute with the maximum
+        if (!late) {
+#pragma unroll 1
+            for (int g = 0; g < 4; ++g) {
+                uint32_t w[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) w[i] = g == 0 ? v[i] : g == 1 ? v[8 + i] : g == 2 ? v[16 + i] : v[24 + i];
+                if (pix >= 0 && c0 + 8 * g < P.c_out) tap_affine<DT, FUSED, 8>(P, s_bias, w, pix, true, c0 + 8 * g, n0);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    if (g == 0) v[i] = w[i]; else if (g == 1) v[8 + i] = w[i]; else if (g == 2) v[16 + i] = w[i]; else v[24 + i] = w[i];
+                }
+            }
+        }
+        const bool odd_x = threadIdx.x & 1, odd_y = threadIdx.x & 8;
+        uint32_t w[8];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const uint32_t got = __shfl_xor_sync(0xFFFFFFFFu, odd_x ? v[i] : v[16 + i], 1);
+            v[i] = tap_max<DT>(odd_x ? v[16 + i] : v[i], got);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const uint32_t got = __shfl_xor_sync(0xFFFFFFFFu, odd_y ? v[i] : v[8 + i], 8);
+            w[i] = tap_max<DT>(odd_y ? v[8 + i] : v[i], got);
+        }
+        const int c = c0 + (odd_x ? 16 : 0) + (odd_y ? 8 : 0);
+        if (pix < 0 || c >= P.c_out) return;
+        if (late) tap_affine<DT, FUSED, 8>(P, s_bias, w, pix, false, c, n0);
+        tap_store<DT, FUSED, 8>(P, s_scale, w, out, c, n0);
+        return;
+    }
+    if (pix < 0) return;
+    if (c0 + 32 > P.c_out || !P.vec_y) {
+#pragma unroll 1
+        for (int g = 0; g < 4; ++g) {
+            if (c0 + 8 * g >= P.c_out) break;
+            uint32_t w[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) w[i] = g == 0 ? v[i] : g == 1 ? v[8 + i] : g == 2 ? v[16 + i] : v[24 + i];
+            tap_affine<DT, FUSED, 8>(P, s_bias, w, pix, true, c0 + 8 * g, n0);
+            tap_store<DT, FUSED, 8>(P, s_scale, w, pix, c0 + 8 * g, n0);
+        }
+        return;
+    }
+    const size_t off = (size_t)pix * P.c_out + c0;
+    const uint32_t *const bias = s_bias + (c0 - n0);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const uint4 b = *reinterpret_cast<const uint4 *>(bias + 4 * q);
+        if (DT == XGEN_I8_I32) { v[4 * q] += b.x; v[4 * q + 1] += b.y; v[4 * q + 2] += b.z; v[4 * q + 3] += b.w; }
+        else { add2(v[4 * q], v[4 * q + 1], b.x, b.y); add2(v[4 * q + 2], v[4 * q + 3], b.z, b.w); }
+    }
+    if (FUSED && P.residual) {
+        if (!P.vec_r) {
+#pragma unroll
+            for (int i = 0; i < 32; ++i) v[i] = tap_affine1<DT, FUSED>(P, 0u, v[i], off + i);
+        } else if (DT == XGEN_F16_F32ACC) {
+            const uint4 *r = reinterpret_cast<const uint4 *>(static_cast<const __half *>(P.residual) + off);
+            uint4 a[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) a[q] = __ldg(r + q);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t aa[4] = {a[q].x, a[q].y, a[q].z, a[q].w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&aa[i]));
+                    add2(v[8 * q + 2 * i], v[8 * q + 2 * i + 1], __float_as_uint(f.x), __float_as_uint(f.y));
+                }
+            }
+        } else {
+            const uint4 *r = reinterpret_cast<const uint4 *>(static_cast<const uint32_t *>(P.residual) + off);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                uint4 a[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) a[q] = __ldg(r + 4 * h + q);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    uint32_t *const w = v + 16 * h + 4 * q;
+                    if (DT == XGEN_I8_I32) { w[0] += a[q].x; w[1] += a[q].y; w[2] += a[q].z; w[3] += a[q].w; }
+                    else { add2(w[0], w[1], a[q].x, a[q].y); add2(w[2], w[3], a[q].z, a[q].w); }
+                }
+            }
+        }
+    }
+    if (P.relu) {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = tap_max<DT>(v[i], 0u);
+    }
+    if (FUSED && DT == XGEN_I8_I32 && P.rq_scale) {
+        uint8_t *const y = static_cast<uint8_t *>(P.y) + off;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t code[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float4 sc = *reinterpret_cast<const float4 *>(s_scale + (c0 - n0) + 16 * h + 4 * q);
+                const uint32_t *const w = v + 16 * h + 4 * q;
+                code[q] = pack_codes(tap_level(P, w[0], sc.x), tap_level(P, w[1], sc.y), tap_level(P, w[2], sc.z), tap_level(P, w[3], sc.w));
+            }
+            *reinterpret_cast<uint4 *>(y + 16 * h) = make_uint4(code[0], code[1], code[2], code[3]);
+        }
+        return;
+    }
+    constexpr int NW = DT == XGEN_F16_F32ACC ? 16 : 32;
+    uint32_t *const y = reinterpret_cast<uint32_t *>(static_cast<char *>(P.y) + off * (DT == XGEN_F16_F32ACC ? 2 : 4));
+    if (DT == XGEN_F16_F32ACC) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const __half2 h = __floats2half2_rn(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+            v[i] = *reinterpret_cast<const uint32_t *>(&h);
+        }
+    }
+    if (P.y32) {
+#pragma unroll
+        for (int q = 0; q < NW / 8; ++q)
+            asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                         ::"l"(y + 8 * q), "r"(v[8 * q]), "r"(v[8 * q + 1]), "r"(v[8 * q + 2]), "r"(v[8 * q + 3]),
+                           "r"(v[8 * q + 4]), "r"(v[8 * q + 5]), "r"(v[8 * q + 6]), "r"(v[8 * q + 7]) : "memory");
+    } else {
+#pragma unroll
+        for (int q = 0; q < NW / 4; ++q)
+            reinterpret_cast<uint4 *>(y)[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     }
 }
 
@@ -334,12 +542,13 @@ __device__ __forceinline__ int tap_origin(const TapParams &P, int v0, int i) {
 }
 
 template <int DT, int STRIDE, int TAPS, int MT, bool PAIR>
-__global__ void __launch_bounds__(kTapThreads, 1)
+__global__ void __launch_bounds__(tap_threads(DT), 1)
 tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensorMap wmap) {
     using T = TapTraits<DT>;
     using TL = TapTile<STRIDE, TAPS, MT>;
     constexpr int PARTS = T::parts, R = TL::R;
     constexpr bool kF32 = DT == XGEN_F32, FUSED = TAPS == 9;
+    constexpr int kEpiWarps = epi_warps(DT);
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
@@ -514,102 +723,93 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
         copy_wait<0>();
         while (pending) publish();
     } else if (warp == kEpiWarps + kProdWarps) {
-        // ---- matrix instructions ---------------------------------------------------
-        const bool leader = elect_one();
-        const uint32_t sbo = TL::pitch * 16;
-        const uint32_t b_rows = (uint32_t)P.nt / (PAIR ? 2 : 1);         // filters whose weights this block holds
-        const uint32_t b_plane = PARTS * b_rows * 16;
-        const uint64_t a0 = operand_desc(sbase, (uint32_t)P.plane_pitch, sbo);
-        const uint64_t b0 = operand_desc(sbase + P.b_off, b_plane, 128);
-        const uint32_t a_k = (uint32_t)P.plane_pitch * 2 / 16, b_k = b_plane * 2 / 16, a_p = a_part / 16, b_p = b_rows;
-        int s = 0, b = 0, buf = 0;
-        uint32_t pha = 0, phb = 0, phc = 1;
-        bool ok = true;
-        for (int item = item0; item < P.items && ok && side == 0; item += item_step) {
-            for (int ks = k0; ks < k1 && ok; ++ks) {
-                if (kF32 || ks == k0) ok = wait(acc_empty(buf), phc);
-                ok = ok && wait(a_full(s), pha);
-                tc_fence_after();
-                const int kk_n = min(P.pl, planes - ks * P.pl) / 2;
-                const uint64_t as = a0 + (uint32_t)s * (a_bytes / 16);
-                const uint32_t d = tmem + (uint32_t)buf * (uint32_t)(MT * P.nt);
-                const uint32_t dc = d + 2u * P.nt;          // fp32: the small products (two buffers behind the two of the sums)
+        // ---- matrix instructions: one thread, which also waits (a warp that meets again at every tap
+        // takes some 600 cycles for a tap's 4 to 8 instructions).  A wait that gives up is not looked at:
+        // nothing per-thread may steer these loops, or every operand is moved to the uniform registers
+        // anew; all later waits then return at once. ------------------------------------------------
+        if (side == 0 && elect_one()) {
+            const uint32_t b_rows = (uint32_t)P.nt / (PAIR ? 2 : 1);         // filters whose weights this block holds
+            const uint32_t b_plane = PARTS * b_rows * 16;
+            const uint64_t a0 = operand_desc(sbase, (uint32_t)P.plane_pitch, TL::pitch * 16);
+            const uint64_t b0 = operand_desc(sbase + P.b_off, b_plane, 128);
+            const uint32_t a_hi = (uint32_t)(a0 >> 32), b_hi = (uint32_t)(b0 >> 32), idesc = P.idesc;
+            const uint32_t a_k = (uint32_t)P.plane_pitch * 2 / 16, b_k = b_plane * 2 / 16, a_p = a_part / 16, b_p = b_rows;
+            const uint32_t b_step = (uint32_t)P.b_bytes / 16;
+            int s = 0, b = 0, buf = 0;
+            uint32_t pha = 0, phb = 0, phc = 1, bt = (uint32_t)b0;
+            for (int item = item0; item < P.items; item += item_step) {
+                for (int ks = k0; ks < k1; ++ks) {
+                    if (kF32 || ks == k0) wait(acc_empty(buf), phc);
+                    wait(a_full(s), pha);
+                    tc_fence_after();
+                    const int kk_n = min(P.pl, planes - ks * P.pl) / 2;
+                    const uint32_t as = (uint32_t)a0 + (uint32_t)s * (a_bytes / 16);
+                    const uint32_t d = tmem + (uint32_t)buf * (uint32_t)(MT * P.nt);
+                    const uint32_t dc = d + 2u * P.nt;      // fp32: the small products (two buffers behind the two of the sums)
+#pragma unroll 1
+                    for (int tap = 0; tap < TAPS; ++tap) {      // (rolled: code that runs once comes from L2, 600 cycles a tap)
+                        wait(b_full(b), P.resident ? 0u : phb);
+                        uint32_t ak = as + (uint32_t)P.tap_start[tap], bk = bt;
+#pragma unroll 1
+                        for (int kk = 0; kk < kk_n; ++kk, ak += a_k, bk += b_k) {
+                            const uint32_t first_s = tap > 0 || kk > 0 ? 1u : 0u;       // 0: the first of the stage
+                            const uint32_t first_i = first_s | (ks > k0 ? 1u : 0u);     // 0: the first of the item
+                            if (kF32) {
+                                mma_f16<PAIR>(d, ak, a_hi, bk, b_hi, idesc, first_s);
+                                mma_f16<PAIR>(dc, ak, a_hi, bk + b_p, b_hi, idesc, first_s);
+                                mma_f16<PAIR>(dc, ak, a_hi, bk + 2 * b_p, b_hi, idesc, 1u);
+                                mma_f16<PAIR>(dc, ak + a_p, a_hi, bk, b_hi, idesc, 1u);
+                                mma_f16<PAIR>(dc, ak + a_p, a_hi, bk + b_p, b_hi, idesc, 1u);
+                                mma_f16<PAIR>(dc, ak + 2 * a_p, a_hi, bk, b_hi, idesc, 1u);
+                            } else {
 #pragma unroll
-                for (int tap = 0; tap < TAPS; ++tap) {
-                    ok = ok && wait(b_full(b), P.resident ? 0u : phb);
-                    if (!ok) break;
-                    if (leader) {
-                        const uint64_t at = as + TL::tap_start(tap);
-                        const uint64_t bt = b0 + (uint32_t)b * (uint32_t)(P.b_bytes / 16);
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
-                            if (kk < kk_n) {
-                                const uint64_t ak = at + kk * a_k, bk = bt + kk * b_k;
-                                const uint32_t first_s = tap > 0 || kk > 0 ? 1u : 0u;       // 0: the first of the stage
-                                const uint32_t first_i = first_s | (ks > k0 ? 1u : 0u);     // 0: the first of the item
-                                if (kF32) {
-                                    mma_f16<PAIR>(d, ak, bk, P.idesc, first_s);
-                                    mma_f16<PAIR>(dc, ak, bk + b_p, P.idesc, first_s);
-                                    mma_f16<PAIR>(dc, ak, bk + 2 * b_p, P.idesc, 1u);
-                                    mma_f16<PAIR>(dc, ak + a_p, bk, P.idesc, 1u);
-                                    mma_f16<PAIR>(dc, ak + a_p, bk + b_p, P.idesc, 1u);
-                                    mma_f16<PAIR>(dc, ak + 2 * a_p, bk, P.idesc, 1u);
-                                } else {
-#pragma unroll
-                                    for (int m = 0; m < MT; ++m) {
-                                        const uint64_t am = ak + m * 16 * TL::pitch;
-                                        if (DT == XGEN_I8_I32) mma_i8<PAIR>(d + m * P.nt, am, bk, P.idesc, first_i);
-                                        else mma_f16<PAIR>(d + m * P.nt, am, bk, P.idesc, first_i);
-                                    }
+                                for (int m = 0; m < MT; ++m) {
+                                    if (DT == XGEN_I8_I32) mma_i8<PAIR>(d + m * P.nt, ak + m * 16 * TL::pitch, a_hi, bk, b_hi, idesc, first_i);
+                                    else mma_f16<PAIR>(d + m * P.nt, ak + m * 16 * TL::pitch, a_hi, bk, b_hi, idesc, first_i);
                                 }
                             }
                         }
                         if (!P.resident) tc_commit<PAIR>(b_empty(b), both);
+                        bt += b_step;
+                        if (++b == P.b_slots) { b = 0; phb ^= 1u; bt = (uint32_t)b0; }
                     }
-                    __syncwarp();
-                    if (++b == P.b_slots) { b = 0; phb ^= 1u; }
-                }
-                if (!ok) break;
-                if (leader) {
                     tc_commit<PAIR>(a_empty(s), both);
-                    if (kF32 || ks + 1 == k1) tc_commit<PAIR>(acc_full(buf), both);
+                    if (++s == P.a_stages) { s = 0; pha ^= 1u; }
+                    if (kF32 || ks + 1 == k1) {
+                        tc_commit<PAIR>(acc_full(buf), both);
+                        if (++buf == P.acc_bufs) { buf = 0; phc ^= 1u; }
+                    }
                 }
-                __syncwarp();
-                if (++s == P.a_stages) { s = 0; pha ^= 1u; }
-                if (kF32 || ks + 1 == k1) { if (++buf == P.acc_bufs) { buf = 0; phc ^= 1u; } }
             }
+            tc_commit<PAIR>(all_done, both);
         }
-        if (leader && side == 0) tc_commit<PAIR>(all_done, both);
         __syncwarp();
         for (int it = 0; it < 4000000 && !mbar_ready(all_done, 0); ++it) {}
     } else if (warp > kEpiWarps + kProdWarps) {
         // ---- weights ---------------------------------------------------------------
-        const bool leader = elect_one();
-        int b = 0, issued = 0;
-        uint32_t ph = 1;
-        bool ok = true;
-        for (int item = item0; item < P.items && ok; item += item_step) {
-            for (int ks = k0; ks < k1 && ok; ++ks) {
-                for (int tap = 0; tap < TAPS; ++tap) {
-                    if (issued >= P.b_slots) ok = wait(b_empty(b), ph);
-                    if (!ok) break;
-                    if (leader) {
+        if (elect_one()) {
+            int b = 0, issued = 0;
+            uint32_t ph = 1;
+            for (int item = item0; item < P.items; item += item_step) {
+                for (int ks = k0; ks < k1; ++ks) {
+                    for (int tap = 0; tap < TAPS; ++tap) {
+                        if (issued >= P.b_slots) wait(b_empty(b), ph);
                         // one copy for a tap: pieces of 2 KB with a copy of their own cost 50 cycles
                         // of issue apiece and held the whole kernel to 5.5 TB/s of weights
                         if (side == 0) mbar_expect_tx(b_full(b), (uint32_t)P.b_bytes * (PAIR ? 2 : 1));
                         tensor_load4<PAIR>(sbase + P.b_off + (uint32_t)(b * P.b_bytes), &wmap, (n0 + side * P.nt / 2) * 2, 0, tap, ks * P.pl,
                                            PAIR ? cluster_addr(b_full(b), (uint32_t)(crank & ~1)) : b_full(b));
+                        ++issued;
+                        if (++b == P.b_slots) { b = 0; ph ^= 1u; }
                     }
-                    __syncwarp();
-                    ++issued;
-                    if (++b == P.b_slots) { b = 0; ph ^= 1u; }
                 }
+                if (P.resident) break;
             }
-            if (P.resident) break;
+            // Nothing may land in shared memory after this block has gone (a wait above may have given up).
+            for (int q = max(0, issued - P.b_slots); q < issued && side == 0; ++q)
+                for (int it = 0; it < 1000000 && !mbar_ready(b_full(q % P.b_slots), (uint32_t)(q / P.b_slots) & 1u); ++it) {}
         }
-        // Nothing may land in shared memory after this block has gone (a wait above may have given up).
-        for (int q = max(0, issued - P.b_slots); q < issued && side == 0; ++q)
-            for (int it = 0; it < 1000000 && !mbar_ready(b_full(q % P.b_slots), (uint32_t)(q / P.b_slots) & 1u); ++it) {}
+        __syncwarp();
     } else {
         // ---- epilogue ----------------------------------------------------------------
         asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -619,100 +819,100 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             s_scale[i] = FUSED && P.rq_scale && in ? P.rq_scale[n0 + i] : 0.0f;
         }
         asm volatile("bar.sync 2, %0;" ::"n"(kEpiWarps * 32) : "memory");
-        const int quarter = warp & 3, half = warp >> 2;
-        const int sub = MT == 2 ? half : 0;
-        const int cols = MT == 2 ? P.nt : P.nt / 2, col0 = MT == 2 ? 0 : half * cols;   // this warp's filters of the tile
+        // a warp's share: a quarter of the lanes, one of the tiles, every kGroups-th chunk of 32 filters
+        constexpr int kGroups = kEpiWarps / 4 / MT;
+        const int quarter = warp & 3, sub = (warp >> 2) % MT, group = (warp >> 2) / MT;
+        const int chunks = P.nt / 32;
         const uint32_t lanes = (uint32_t)quarter << 21;
         const int m = quarter * 32 + lane;                       // pixel of the 128
-        float *const stage = reinterpret_cast<float *>(smem) + (size_t)(sub * 128 + m) * (P.nt + 4);
+        // sums on their way out where they do not go straight from their lanes: the warp's 32 pixels x 16
+        // filters, or (split) the whole tile
+        uint32_t *const st = reinterpret_cast<uint32_t *>(smem + (P.splits > 1 ? 0 : P.stage_off + warp * kStageBytes));
+        uint32_t *const st_own = st + (P.splits > 1 ? (sub * 128 + m) * (P.nt + 4) : lane * kStagePitch);
         int buf = 0;
         uint32_t ph = 0;
         bool ok = true;
         for (int item = item0; item < P.items && ok; item += item_step) {
             const TapItem t = tap_item<PAIR>(P, item, R, side);
             const int v = t.v0 + sub * 16 + (m >> 3), ox = t.ox0 + (m & 7);
-            int64_t pixel;
-            bool valid;
-            int oy = 0, img = 0;
+            int pix = -1, out = -1;              // this lane's pixel: of the result, and where it is stored
             if (TAPS == 1) {
-                pixel = (int64_t)v * 8 + ox;
-                valid = pixel < P.npix;
+                if ((int64_t)v * 8 + ox < P.npix) pix = v * 8 + ox;
+                out = pix;
             } else {
-                img = v / P.vh;
-                oy = v - img * P.vh;
-                valid = img < P.n && oy < P.ho && ox < P.wo;
-                pixel = ((int64_t)img * P.ho + oy) * P.wo + ox;
-            }
-            // 16 sums of this lane's pixel, from column c of the warp's range on.
-            auto finish = [&](uint32_t (&r)[16], int c) {
-                if (P.splits > 1) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        *reinterpret_cast<uint4 *>(stage + col0 + c + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
-                    return;
+                const int img = v / P.vh, oy = v - img * P.vh;
+                if (img < P.n && oy < P.ho && ox < P.wo) {
+                    pix = (img * P.ho + oy) * P.wo + ox;
+                    out = P.pool ? (img * P.po + oy / 2) * P.pw + ox / 2 : pix;
                 }
-                const int c0 = n0 + col0 + c;
-                if (c0 >= P.c_out) return;
-                tap_affine<DT, FUSED, 16>(P, s_bias, r, pixel, valid, c0, n0);
-                if (FUSED && P.pool) {
+            }
+            auto put = [&](const uint32_t *r, int n, int at) {
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        r[i] = tap_max<DT>(r[i], __shfl_xor_sync(0xFFFFFFFFu, r[i], 1));
-                        r[i] = tap_max<DT>(r[i], __shfl_xor_sync(0xFFFFFFFFu, r[i], 8));
+                for (int q = 0; q < n / 4; ++q)
+                    *reinterpret_cast<uint4 *>(st_own + at + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+            };
+            // 32 sums of this lane's pixel, from column c of the tile on
+            auto finish = [&](uint32_t (&r)[32], int c) {
+                if (P.splits > 1) put(r, 32, c);
+                else if (n0 + c >= P.c_out) return;
+                else if (!P.staged) tap_direct<DT, FUSED>(P, s_bias, s_scale, r, pix, out, n0 + c, n0);
+                else {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        __syncwarp();
+                        put(r + 16 * h, 16, 0);
+                        __syncwarp();
+                        tap_emit<DT, FUSED>(P, st, s_bias, s_scale, pix, out, n0 + c + 16 * h, n0, lane);
                     }
-                    if (valid && !(oy & 1) && !(ox & 1))
-                        tap_store<DT, FUSED, 16>(P, s_scale, r, ((int64_t)img * P.po + oy / 2) * P.pw + ox / 2, c0, n0);
-                } else if (valid) {
-                    tap_store<DT, FUSED, 16>(P, s_scale, r, pixel, c0, n0);
                 }
             };
-            if (kF32) {
-                float sum[64];
-#pragma unroll
-                for (int i = 0; i < 64; ++i) sum[i] = 0.0f;
-                for (int ks = k0; ks < k1 && ok; ++ks) {
-                    ok = wait(acc_full(buf), ph);
-                    tc_fence_after();
-                    const uint32_t ta = tmem + lanes + (uint32_t)(buf * P.nt + col0);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        if (16 * q < cols) {
-                            uint32_t a[16], b[16];
-                            tmem_ld16(ta + 16 * q, a);
-                            tmem_ld16(ta + 2 * P.nt + 16 * q, b);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) sum[16 * q + i] += __uint_as_float(a[i]) + __uint_as_float(b[i]);
-                        }
-                    }
-                    tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) arrive_lead(acc_empty(buf));
-                    if (++buf == P.acc_bufs) { buf = 0; ph ^= 1u; }
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (16 * q < cols && ok) {
-                        uint32_t r[16];
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(sum[16 * q + i]);
-                        finish(r, 16 * q);
-                    }
-                }
-            } else {
-                ok = wait(acc_full(buf), ph);
-                tc_fence_after();
-                const uint32_t ta = tmem + lanes + (uint32_t)((buf * MT + sub) * P.nt + col0);
-                for (int c = 0; c < cols && ok; c += 16) {
-                    uint32_t r[16];
-                    tmem_ld16(ta + c, r);
-                    tmem_wait_ld();
-                    finish(r, c);
-                }
+            auto release = [&]() {
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) arrive_lead(acc_empty(buf));
                 if (++buf == P.acc_bufs) { buf = 0; ph ^= 1u; }
+            };
+            if (kF32) {
+                uint32_t sum[2][32];                 // chunks `group` and `group` + kGroups
+#pragma unroll
+                for (int i = 0; i < 64; ++i) sum[i / 32][i % 32] = 0u;
+                for (int ks = k0; ks < k1 && ok; ++ks) {
+                    ok = wait(acc_full(buf), ph);
+                    tc_fence_after();
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const int q = group + h / 2 * kGroups;
+                        if (q < chunks) {
+                            const uint32_t ta = tmem + lanes + (uint32_t)(buf * P.nt + 32 * q + h % 2 * 16);
+                            uint32_t a[16], b[16];
+                            tmem_ld16(ta, a);
+                            tmem_ld16(ta + 2 * P.nt, b);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int i = 0; i < 16; i += 2) {
+                                add2(a[i], a[i + 1], b[i], b[i + 1]);
+                                add2(sum[h / 2][h % 2 * 16 + i], sum[h / 2][h % 2 * 16 + i + 1], a[i], a[i + 1]);
+                            }
+                        }
+                    }
+                    release();
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (group + h * kGroups < chunks && ok) finish(sum[h], 32 * (group + h * kGroups));
+            } else {
+                ok = wait(acc_full(buf), ph);
+                tc_fence_after();
+                const uint32_t ta = tmem + lanes + (uint32_t)((buf * MT + sub) * P.nt);
+#pragma unroll 1
+                for (int q = group; q < chunks && ok; q += kGroups) {
+                    uint32_t r[32];
+                    tmem_ld16(ta + 32 * q, r);
+                    tmem_ld16(ta + 32 * q + 16, r + 16);
+                    tmem_wait_ld();
+                    finish(r, 32 * q);
+                }
+                release();
             }
         }
     }
@@ -726,49 +926,47 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             const TapItem t = tap_item<PAIR>(P, item0, R, side);
             const int groups = P.nt / 8, pitch = (P.nt + 4) * 4;
             const bool pool = FUSED && P.pool;
-            for (int u = rank; u < 8 * MT; u += P.splits) {
-                for (int w = tid; w < (pool ? 4 : 16) * groups; w += kAdders) {
-                    const int row = w / groups, g = w - row * groups;
-                    const int c0 = n0 + 8 * g;
-                    // pixel(s): a unit is two rows of 8; pooled pixel `row` covers columns 2 row, 2 row + 1 of both
-                    const int m0 = 16 * u + (pool ? 2 * row : row);
-                    const int v = t.v0 + (m0 >> 3), ox = t.ox0 + (m0 & 7);
-                    int64_t pixel;
-                    int img = 0, oy = 0;
-                    bool valid;
-                    if (TAPS == 1) {
-                        pixel = (int64_t)v * 8 + ox;
-                        valid = pixel < P.npix;
-                    } else {
-                        img = v / P.vh;
-                        oy = v - img * P.vh;
-                        valid = img < P.n && oy < P.ho && ox < P.wo;
-                        pixel = ((int64_t)img * P.ho + oy) * P.wo + ox;
-                    }
-                    if (!valid || c0 >= P.c_out) continue;
-                    uint32_t best[8];
+            // units of two rows of eight pixels go round the blocks; a thread takes 8 channels of one (pooled) pixel
+            const int units = (8 * MT - rank + P.splits - 1) / P.splits, per_unit = (pool ? 4 : 16) * groups;
 #pragma unroll 1
-                    for (int q = 0; q < (pool ? 4 : 1); ++q) {
-                        const int mm = m0 + (q & 1) + (q >> 1) * 8;
-                        uint32_t v8[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) v8[i] = 0;
-                        const uint32_t own = sbase + (uint32_t)(mm * pitch + g * 32);
-#pragma unroll 4
-                        for (int r = 0; r < P.splits; ++r) {
-                            const uint32_t far = cluster_addr(own, (uint32_t)(PAIR ? 2 * r + side : r));
-                            const uint4 a = lds_cluster(far), b = lds_cluster(far + 16);
-                            const uint32_t ab[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-                            for (int i = 0; i < 8; ++i)
-                                v8[i] = DT == XGEN_I8_I32 ? v8[i] + ab[i] : __float_as_uint(__uint_as_float(v8[i]) + __uint_as_float(ab[i]));
-                        }
-                        tap_affine<DT, FUSED, 8>(P, s_bias, v8, pixel + (q & 1) + (int64_t)(q >> 1) * P.wo, true, c0, n0);
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) best[i] = q == 0 ? v8[i] : tap_max<DT>(best[i], v8[i]);
-                    }
-                    tap_store<DT, FUSED, 8>(P, s_scale, best, pool ? ((int64_t)img * P.po + oy / 2) * P.pw + ox / 2 : pixel, c0, n0);
+            for (int w = tid; w < units * per_unit; w += kAdders) {
+                const int u = w / per_unit, wu = w - u * per_unit, row = wu / groups, g = wu - row * groups;
+                const int c0 = n0 + 8 * g;
+                const int m0 = 16 * (rank + u * P.splits) + (pool ? 2 * row : row);
+                const int v = t.v0 + (m0 >> 3), ox = t.ox0 + (m0 & 7);
+                int pix, out;
+                bool valid;
+                if (TAPS == 1) {
+                    valid = (int64_t)v * 8 + ox < P.npix;
+                    out = pix = v * 8 + ox;
+                } else {
+                    const int img = v / P.vh, oy = v - img * P.vh;
+                    valid = img < P.n && oy < P.ho && ox < P.wo;
+                    pix = (img * P.ho + oy) * P.wo + ox;
+                    out = pool ? (img * P.po + oy / 2) * P.pw + ox / 2 : pix;
                 }
+                if (!valid || c0 >= P.c_out) continue;
+                uint32_t best[8];
+#pragma unroll 1
+                for (int q = 0; q < (pool ? 4 : 1); ++q) {
+                    const uint32_t own = sbase + (uint32_t)((m0 + (q & 1) + (q >> 1) * 8) * pitch + g * 32);
+                    uint32_t v8[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) v8[i] = 0;
+#pragma unroll 4
+                    for (int r = 0; r < P.splits; ++r) {
+                        const uint32_t far = cluster_addr(own, (uint32_t)(PAIR ? 2 * r + side : r));
+                        const uint4 a = lds_cluster(far), b = lds_cluster(far + 16);
+                        const uint32_t ab[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            v8[i] = DT == XGEN_I8_I32 ? v8[i] + ab[i] : __float_as_uint(__uint_as_float(v8[i]) + __uint_as_float(ab[i]));
+                    }
+                    tap_affine<DT, FUSED, 8>(P, s_bias, v8, pix + (q & 1) + (q >> 1) * P.wo, true, c0, n0);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) best[i] = q == 0 ? v8[i] : tap_max<DT>(best[i], v8[i]);
+                }
+                tap_store<DT, FUSED, 8>(P, s_scale, best, out, c0, n0);
             }
         }
     }
@@ -935,7 +1133,7 @@ static int tap_clusters(int size, int device, int sms) {
     if (k) return k;
     const void *kern = tap_kernel_of(XGEN_F16_F32ACC, 1, 9, 1, false);
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)size); cfg.blockDim = dim3(kTapThreads); cfg.dynamicSmemBytes = kTapSmemMax;
+    cfg.gridDim = dim3((unsigned)size); cfg.blockDim = dim3(tap_threads(XGEN_F16_F32ACC)); cfg.dynamicSmemBytes = kTapSmemMax;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)size; at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
@@ -949,6 +1147,12 @@ static int tap_clusters(int size, int device, int sms) {
 static int tap_pixels(int stride, int taps, int mt) {
     const int R = 16 * mt;
     return taps == 1 ? 8 * R : stride == 1 ? 10 * (R + 2) : 9 * (4 * R + 2);
+}
+
+static int tap_start(int stride, int taps, int mt, int t) {
+    if (taps == 1) return 0;
+    if (stride == 1) return TapTile<1, 9, 1>::tap_start(t);
+    return mt == 2 ? TapTile<2, 9, 2>::tap_start(t) : TapTile<2, 9, 1>::tap_start(t);
 }
 
 bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &best) {
@@ -1005,8 +1209,9 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                 p.plane_pitch = pixels * 16;
                 while (p.plane_pitch % 128 != 128 / pl % 128) p.plane_pitch += 16;
                 const size_t a_bytes = (size_t)parts * pl * p.plane_pitch, b_bytes = (size_t)pl * parts * p.nt * 16 / ways;
-                const size_t tables = ((size_t)pixels * 8 + 127) / 128 * 128;
+                const size_t pix_tables = ((size_t)pixels * 8 + 127) / 128 * 128;
                 for (int sp = 1; sp * ways <= 16 && sp <= p.stages; ++sp) {
+                    const size_t tables = pix_tables + (sp == 1 && s.staged ? epi_warps(dt) * kStageBytes : 0);
                     p.per_split = (p.stages + sp - 1) / sp;
                     p.splits = (p.stages + p.per_split - 1) / p.per_split;
                     if (p.splits != sp) continue;
@@ -1098,7 +1303,9 @@ cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p
     P.b_bytes = p.pl * parts * (p.pair ? p.nt / 2 : p.nt) * 16;
     P.b_off = p.a_stages * parts * p.pl * p.plane_pitch;
     P.tab_off = P.b_off + p.b_slots * P.b_bytes;
-    P.tmem_cols = p.tmem_cols; P.acc_bufs = p.acc_bufs;
+    P.stage_off = P.tab_off + (tap_pixels(s.stride, tw.taps, p.mt) * 8 + 127) / 128 * 128;
+    P.tmem_cols = p.tmem_cols; P.acc_bufs = p.acc_bufs; P.staged = s.staged;
+    for (int t = 0; t < tw.taps; ++t) P.tap_start[t] = tap_start(s.stride, tw.taps, p.mt, t);
     auto aligned = [](const void *q, uintptr_t a) { return ((uintptr_t)q & (a - 1)) == 0; };
     P.vec_x = aligned(c.x, 16) && (size_t)tw.c_in * xb % 16 == 0;
     P.vec_y = aligned(c.y, 16) && (size_t)tw.c_out * yb % 16 == 0;
@@ -1113,7 +1320,7 @@ cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p
     if (e == cudaSuccess) e = tap_allow(kern, device);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)p.grid); cfg.blockDim = dim3(kTapThreads); cfg.dynamicSmemBytes = p.smem; cfg.stream = st;
+    cfg.gridDim = dim3((unsigned)p.grid); cfg.blockDim = dim3((unsigned)tap_threads(dt)); cfg.dynamicSmemBytes = p.smem; cfg.stream = st;
     cudaLaunchAttribute at[2];
     unsigned na = 0;
     if (c.overlap) {
