@@ -52,25 +52,29 @@ __device__ __forceinline__ uint64_t global_ns() {
     return t;
 }
 
+template <bool CLUSTER> __device__ __forceinline__ bool mbar_try(uint32_t mbar, uint32_t parity) {
+    uint32_t ok;
+    if (CLUSTER)
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                     : "=r"(ok) : "r"(mbar), "r"(parity) : "memory");
+    else
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                     : "=r"(ok) : "r"(mbar), "r"(parity) : "memory");
+    return ok != 0;
+}
+
 // Wait for an mbarrier phase with a bound in time (limit_us microseconds, plus a cap on the
 // polls in case the timer stands still): on expiry the block-wide abort flag and the device
 // status word are set and every later wait returns at once; the warps then leave their
 // loops, so the kernel still runs to its end (releasing tensor memory) with results the
 // host can tell are invalid.  CLUSTER: what other blocks of the cluster wrote before they
 // arrived is seen too.
-template <bool CLUSTER = false>
-__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, volatile int *abort_flag, int *status,
-                                          uint32_t limit_us) {
+template <bool CLUSTER>
+__device__ __noinline__ bool mbar_wait_long(uint32_t mbar, uint32_t parity, volatile int *abort_flag, int *status,
+                                            uint32_t limit_us) {
     uint64_t t0 = 0;
     for (uint32_t it = 0; it < 40000000u; ++it) {
-        uint32_t ok;
-        if (CLUSTER)
-            asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                         : "=r"(ok) : "r"(mbar), "r"(parity) : "memory");
-        else
-            asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                         : "=r"(ok) : "r"(mbar), "r"(parity) : "memory");
-        if (ok) return true;
+        if (mbar_try<CLUSTER>(mbar, parity)) return true;
         if (*abort_flag) return false;
         if ((it & 7u) == 7u) {
             const uint64_t t = global_ns();
@@ -81,6 +85,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, volati
     *abort_flag = 1;
     if (status) atomicExch(status, 1);
     return false;
+}
+template <bool CLUSTER = false>
+__device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, volatile int *abort_flag, int *status,
+                                          uint32_t limit_us) {
+    return mbar_try<CLUSTER>(mbar, parity) || mbar_wait_long<CLUSTER>(mbar, parity, abort_flag, status, limit_us);
 }
 
 __device__ __forceinline__ bool elect_one() {
@@ -160,6 +169,12 @@ __device__ __forceinline__ void tensor_load4(uint32_t dst, const void *map, int 
     else
         asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
                      ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(mbar) : "memory");
+}
+// The same with rows of 128 bytes of K, 16-byte pieces swizzled by the row (address bits 4..6 xor 7..9):
+// 8 rows are 1024 contiguous bytes, the next 8 follow `sbo` bytes on.  The swizzle is one of addresses,
+// so a start at any row is allowed; K advances by 32 bytes inside the row.
+__device__ __forceinline__ uint64_t operand_desc_swizzled(uint32_t addr, uint32_t sbo) {
+    return (uint64_t)((addr >> 4) & 0x3FFFu) | (1ull << 16) | ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46) | (2ull << 61);
 }
 // Shared-memory operand of a matrix instruction, K-major without swizzle: 8 rows of 16 bytes are
 // contiguous, the next 8 rows follow `sbo` bytes on, the next 16 bytes of K `lbo` bytes on.

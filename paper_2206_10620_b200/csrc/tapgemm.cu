@@ -5,13 +5,19 @@
 // weights are zeros of the operand.  (0 x infinity is NaN there, as in the definition written out
 // over the masked dense tensor.)
 //
-// A tile is 8 pixels wide and 16 (or 32) rows high.  Its input with the halo is staged once per
-// group of channels, as planes of 16 bytes of channels per pixel, and serves all nine taps: in
-// shared memory a tap is only another start address.  The operand layout without swizzle (8 rows
-// of 16 contiguous bytes, groups of rows a free pitch apart) allows any start that is a multiple
-// of 16 bytes, so a row of 8 output pixels is one group, the pitch of the staged rows the distance
-// of groups.  Measured: full rate (64 cycles for 128 x 128 x 16) at every shift.  The other choice,
-// one copy-engine load per tap (im2col), moves the tile nine times through L2.
+// The input of a tile with its halo is staged once per group of channels and serves all nine taps:
+// in shared memory a tap is only another start address.  A tile is 128 (256) output pixels, either
+// 8 wide and 16 (32) high -- a row of 8 pixels is one row group of the operand, the pitch of the
+// staged rows the distance of groups -- or a run of the zero-padded raster of all images (rows one
+// entry longer than the image, one row of zeros between images), which wastes one column in w + 1
+// where 8-pixel columns would waste up to 7.  Measured: the matrix instructions run at full rate (64
+// cycles for 128 x 128 x 16) at every shift.  The other choice, one copy-engine load per tap
+// (im2col), moves the tile nine times through L2.
+//
+// fp16 and int8 pixels are rows of 128 bytes of channels, swizzled; the copy engine delivers them
+// (zeros outside the image), one copy a tile or one a row; layers whose channels it cannot address
+// are gathered by the producer warps.  fp32 goes through the producer warps, which write planes of
+// 16 bytes (8 channels) per pixel and part, unswizzled.
 //
 // A matrix instruction of 128 x 128 x 16 reads 8 KB of shared memory in its 64 cycles, all that
 // shared memory delivers; the weights that stream in slow it down.  So where there are two tiles,
@@ -24,7 +30,7 @@
 // (at most 18 steps) and then added, rounded, to sums in registers; the five small products have
 // an accumulator of their own, where truncation is 2^-8 of that, and are added the same way.
 //
-// Roles: 8 epilogue warps (tensor memory -> registers -> y), 6 producer warps (x -> planes), one
+// Roles: 8 or 16 epilogue warps (tensor memory -> registers -> y), 6 producer warps (x), one
 // warp that issues the matrix instructions, one that fetches weights with tensor copies.  Blocks are
 // persistent; a block keeps its range of filters, and where all of its weights fit they are
 // fetched once.  Items that would leave the GPU idle share one reduction between the blocks of a
@@ -53,7 +59,7 @@ __host__ __device__ constexpr int epi_warps(int dt) { return dt == XGEN_F32 ? 8 
 constexpr int kProdWarps = 6;
 __host__ __device__ constexpr int tap_threads(int dt) { return (epi_warps(dt) + kProdWarps + 2) * 32; }
 constexpr int kProdThreads = kProdWarps * 32;
-constexpr int kMaxA = 4, kMaxB = 64;
+constexpr int kMaxA = 6, kMaxB = 36;
 constexpr int kTapSmemMax = 232448 - 4096;      // 227 KB less static shared memory
 constexpr int kMaxFilterTile = 256;
 constexpr int kStagePitch = 20;                 // words of a staged pixel's 16 sums: rows of 16-byte accesses in distinct banks
@@ -68,53 +74,28 @@ struct TapParams {
     int po, pw;                                 // stored extents
     int64_t npix;                               // product: rows of x
     int vh, straddle;                           // virtual rows per image; tiles may cross images
+    int raster, pitch, rows, pixels, sub_px;    // staged tile: entries of a row, rows (of a parity), entries; of the second sub-tile
     int segs, nblk, nt, items, splits, per_split, stages;
     int pl, pl_log, plane_pitch;
-    int a_stages, b_slots, resident, b_bytes;
+    int a_stages, a_bytes, b_slots, resident, b_bytes, tap_group;
     int b_off, tab_off, stage_off;              // bytes into dynamic shared memory
     int tmem_cols, acc_bufs, staged;
-    int tap_start[9];                           // first staged pixel of a tap
+    int tap_start[9];                           // first staged entry of a tap
+    int tma, row_boxes, a_tx;                        // x comes by tensor copies; a copy per staged row
     int vec_x;                                  // 16-byte pieces of x can be copied as they are
     int vec_y, vec_r, y32;                      // 16-byte (32-byte) pieces of y / the residual can be moved whole
     uint32_t idesc;
 };
 
 // Elements of x per 16-byte plane entry (K of one matrix instruction = two planes), bf16 parts, bytes.
+// `row_ch`: channels of a 128-byte row.
 template <int DT> struct TapTraits;
-template <> struct TapTraits<XGEN_F32> { static constexpr int cpp = 8, parts = 3, xb = 4; };
-template <> struct TapTraits<XGEN_F16_F32ACC> { static constexpr int cpp = 8, parts = 1, xb = 2; };
-template <> struct TapTraits<XGEN_I8_I32> { static constexpr int cpp = 16, parts = 1, xb = 1; };
-
-// Staged tile: the row pitch in pixels, pixels in all, where a tap starts.  Stride 2 keeps four
-// images of the tile, one per parity of row and column, so that neighbouring output pixels read
-// neighbouring entries there too.
-template <int STRIDE, int TAPS, int MT> struct TapTile {
-    static constexpr int R = 16 * MT;
-    static constexpr int pitch = TAPS == 1 ? 8 : STRIDE == 1 ? 10 : 9;
-    static constexpr int pixels = TAPS == 1 ? 8 * R : STRIDE == 1 ? 10 * (R + 2) : 9 * (4 * R + 2);
-    static int tap_start(int t) {
-        if (TAPS == 1) return 0;
-        const int dy = t / 3, dx = t % 3;
-        if (STRIDE == 1) return dy * 10 + dx;
-        // even rows: even columns, odd columns; odd rows (one more of them): even, odd
-        const int row_part = dy == 1 ? 0 : 2 * R * 9, rows = dy == 1 ? R : R + 1;
-        return row_part + (dx == 1 ? 0 : rows * 9) + (dy == 2 ? 9 : 0) + (dx == 2 ? 1 : 0);
-    }
-    // Staged pixel -> (row of the tile's staged rows, column relative to stride x first output column);
-    // padding entries lie far out.
-    static __device__ void entry(int p, int &row, int &col) {
-        if (TAPS == 1) { row = p / 8; col = p % 8; return; }
-        if (STRIDE == 1) { row = p / 10; col = p % 10 - 1; return; }
-        const bool odd_row = p >= 2 * R * 9;
-        if (odd_row) p -= 2 * R * 9;
-        const int rows = odd_row ? R + 1 : R;
-        const bool odd_col = p >= rows * 9;
-        if (odd_col) p -= rows * 9;
-        const int j = p % 9;
-        row = p / 9 + (odd_row ? R : 0);
-        col = odd_col ? 2 * j - 1 : (j < 8 ? 2 * j : -(1 << 20));
-    }
-};
+template <> struct TapTraits<XGEN_F32> { static constexpr int cpp = 8, parts = 3, xb = 4, row_ch = 0; };
+// The kernel instances use `taps` 9 or 1 and stride 1 or 2.  Stride 2 keeps four images of the tile, one per
+// parity of row and column (even rows: even columns, odd columns; odd rows likewise), each with rows of 9
+// and one row more than the tile, so that neighbouring output pixels read neighbouring entries there too.
+template <> struct TapTraits<XGEN_F16_F32ACC> { static constexpr int cpp = 8, parts = 1, xb = 2, row_ch = 64; };
+template <> struct TapTraits<XGEN_I8_I32> { static constexpr int cpp = 16, parts = 1, xb = 1, row_ch = 128; };
 
 // ---- results -------------------------------------------------------------------
 // W sums of adjacent channels of one pixel: bias, residual, activation, in fp32 (int32).
@@ -506,52 +487,99 @@ __device__ __forceinline__ void sts128(uint32_t dst, const uint4 &v) {
     asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
-// Position of a block's work: item = (tile or pair of tiles, range of filters), tile = (rows, 8-pixel
-// column).  The second tile of the last pair may lie past the end: all of its pixels are invalid.
-struct TapItem { int n0, ox0, v0; };
-template <bool PAIR> __device__ __forceinline__ TapItem tap_item(const TapParams &P, int item, int rows, int side) {
+// Position of a block's work: item = (tile or pair of tiles, range of filters).  The second tile of the
+// last pair may lie past the end: all of its pixels are invalid.
+struct TapItem {
+    int n0;                  // first filter
+    int v0, ox0;             // 8-pixel columns: first virtual row, first column; raster: row and column of entry q0
+    int q0;                  // raster: first output entry
+};
+template <int MT, bool PAIR> __device__ __forceinline__ TapItem tap_item(const TapParams &P, int item, int side) {
     TapItem t;
     int tile = item / P.nblk;
     t.n0 = (item - tile * P.nblk) * P.nt;
     if (PAIR) tile = 2 * tile + side;
-    const int rt = tile / P.segs;
-    t.ox0 = (tile - rt * P.segs) * 8;
-    t.v0 = rt * rows;
+    if (P.raster) {
+        t.q0 = tile * 128 * MT;
+        t.v0 = t.q0 / P.pitch;
+        t.ox0 = t.q0 - t.v0 * P.pitch;
+    } else {
+        const int rt = tile / P.segs;
+        t.q0 = 0;
+        t.ox0 = (tile - rt * P.segs) * 8;
+        t.v0 = rt * 16 * MT;
+    }
     return t;
 }
 
-// First pixel (of x) of staged row `i` of a tile, or -1 for a row of zeros.
-template <int STRIDE, int TAPS, int MT>
-__device__ __forceinline__ int tap_origin(const TapParams &P, int v0, int i) {
-    constexpr int R = 16 * MT;
-    if (TAPS == 1) return (int64_t)(v0 + i) * 8 < P.npix ? (v0 + i) * 8 : -1;
-    int img, iy;
-    const int step = STRIDE == 1 ? i - 1 : i < R ? i : i - R;      // output rows from the tile's first
+// Image and input row of staged row `i` (stride 2: i of the parity `odd`); outside the tensor for zeros.
+struct TapRow { int img, y; };
+template <int STRIDE> __device__ __forceinline__ TapRow tap_row(const TapParams &P, const TapItem &t, int i, int odd) {
+    TapRow r;
+    const int step = STRIDE == 1 ? i - 1 : i;                       // output rows from the tile's first
     if (P.straddle) {
-        const int v = v0 + step;
-        if (v < 0) return -1;
-        img = v / P.vh;
-        iy = v - img * P.vh;
+        const int v = t.v0 + step;
+        if (v < 0) return TapRow{0, -1};
+        r.img = v / P.vh;
+        r.y = v - r.img * P.vh;
     } else {
-        img = v0 / P.vh;
-        iy = v0 - img * P.vh + step;
+        r.img = t.v0 / P.vh;
+        r.y = t.v0 - r.img * P.vh + step;
     }
-    if (STRIDE == 2) iy = i < R ? 2 * iy : 2 * iy - 1;
-    if (img >= P.n || iy < 0 || iy >= P.h) return -1;
-    return (img * P.h + iy) * P.w;
+    if (STRIDE == 2) r.y = 2 * r.y - odd;
+    return r;
+}
+
+// x's pixel of staged entry p, or -1 for zeros.
+template <int STRIDE, int TAPS> __device__ __forceinline__ int tap_source(const TapParams &P, const TapItem &t, int p) {
+    if (TAPS == 1) return (int64_t)t.v0 * 8 + p < P.npix ? t.v0 * 8 + p : -1;
+    if (P.raster) p -= P.pitch - 1 - t.ox0;       // (all tiles keep their first output entry at the same place)
+    if (p < 0) return -1;
+    int i = p / P.pitch, ix = p - i * P.pitch, odd = 0;
+    if (STRIDE == 1) ix += (P.raster ? 0 : t.ox0) - 1;
+    else {
+        const int region = i / P.rows;
+        i -= region * P.rows;
+        odd = region >> 1;
+        ix = 2 * (t.ox0 + ix) - (region & 1);
+    }
+    const TapRow r = tap_row<STRIDE>(P, t, i, odd);
+    const bool in = r.img < P.n && (unsigned)r.y < (unsigned)P.h && (unsigned)ix < (unsigned)P.w;
+    return in ? (r.img * P.h + r.y) * P.w + ix : -1;
+}
+
+// Output pixel `m` (0 .. 128 MT - 1) of a tile: of the unpooled result, and where it is stored; -1 if none.
+struct TapPixel { int pix, out; };
+template <int TAPS> __device__ __forceinline__ TapPixel tap_pixel(const TapParams &P, const TapItem &t, int m) {
+    if (TAPS == 1) {
+        const int p = (int64_t)t.v0 * 8 + m < P.npix ? t.v0 * 8 + m : -1;
+        return TapPixel{p, p};
+    }
+    int v, ox;
+    if (P.raster) {
+        v = (t.q0 + m) / P.pitch;
+        ox = t.q0 + m - v * P.pitch;
+    } else {
+        v = t.v0 + (m >> 3);
+        ox = t.ox0 + (m & 7);
+    }
+    const int img = v / P.vh, oy = v - img * P.vh;
+    if (img >= P.n || oy >= P.ho || ox >= P.wo) return TapPixel{-1, -1};
+    const int pix = (img * P.ho + oy) * P.wo + ox;
+    return TapPixel{pix, P.pool ? (img * P.po + oy / 2) * P.pw + ox / 2 : pix};
 }
 
 template <int DT, int STRIDE, int TAPS, int MT, bool PAIR>
 __global__ void __launch_bounds__(tap_threads(DT), 1)
-tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensorMap wmap) {
+tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap) {
     using T = TapTraits<DT>;
-    using TL = TapTile<STRIDE, TAPS, MT>;
-    constexpr int PARTS = T::parts, R = TL::R;
+    constexpr int PARTS = T::parts;
     constexpr bool kF32 = DT == XGEN_F32, FUSED = TAPS == 9;
     constexpr int kEpiWarps = epi_warps(DT);
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
+    __shared__ volatile int s_started;           // items whose x is being fetched
     __shared__ __align__(8) uint64_t s_bars[2 * kMaxA + 2 * kMaxB + 5];
     __shared__ __align__(16) uint32_t s_bias[kMaxFilterTile];
     __shared__ __align__(16) float s_scale[kMaxFilterTile];
@@ -572,15 +600,16 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
     const int crank = csize > 1 ? (int)(blockIdx.x % (unsigned)csize) : 0;
     const int side = PAIR ? crank & 1 : 0, rank = PAIR ? crank >> 1 : crank;
     const uint16_t both = (uint16_t)(3u << (crank & ~1));
+    auto lead = [&](uint32_t bar) { return PAIR ? cluster_addr(bar, (uint32_t)(crank & ~1)) : bar; };
     auto arrive_lead = [&](uint32_t bar) {
-        if (PAIR) mbar_arrive_cluster(cluster_addr(bar, (uint32_t)(crank & ~1)));
+        if (PAIR) mbar_arrive_cluster(lead(bar));
         else mbar_arrive(bar);
     };
 
     asm volatile("griddepcontrol.launch_dependents;");
     if (tid == 0) {
-        s_abort = 0;
-        for (int i = 0; i < P.a_stages; ++i) { mbar_init(a_full(i), (PAIR ? 2 : 1) * kProdWarps); mbar_init(a_empty(i), 1); }
+        s_abort = 0; s_started = 0;
+        for (int i = 0; i < P.a_stages; ++i) { mbar_init(a_full(i), P.tma ? 1 : (PAIR ? 2 : 1) * kProdWarps); mbar_init(a_empty(i), 1); }
         for (int i = 0; i < P.b_slots; ++i) { mbar_init(b_full(i), 1); mbar_init(b_empty(i), 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(acc_full(i), 1); mbar_init(acc_empty(i), (PAIR ? 2 : 1) * kEpiWarps); }
         mbar_init(all_done, 1);
@@ -599,68 +628,83 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
     const int item0 = (int)(blockIdx.x / (unsigned)csize);
     const int item_step = P.splits > 1 ? P.items : (int)(gridDim.x / (unsigned)csize);
     const int k0 = rank * P.per_split, k1 = min(P.stages, k0 + P.per_split);
-    const int n0 = tap_item<PAIR>(P, item0, R, side).n0;
+    const int n0 = tap_item<MT, PAIR>(P, item0, side).n0;
     const int planes = (P.c_in + T::cpp * 2 - 1) / (T::cpp * 2) * 2;
-    const uint32_t a_part = (uint32_t)P.pl * P.plane_pitch, a_bytes = a_part * PARTS;
+    const uint32_t a_part = (uint32_t)P.pl * P.plane_pitch;       // fp32: bytes of one part of a stage
 
     if (warp >= kEpiWarps && warp < kEpiWarps + kProdWarps) {
-        // ---- producers: x -> planes ------------------------------------------------
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        const int pt = tid - kEpiWarps * 32;
-        int s = 0, pending = 0, sp = 0;
-        uint32_t ph = 1;
-        bool ok = true, par = false;
-        const char *const x = static_cast<const char *>(P.x);
-        const int total = TL::pixels << P.pl_log;
-        auto publish = [&]() {           // the oldest unpublished stage has landed
-            fence_async_proxy();
-            __syncwarp();
-            if (lane == 0) arrive_lead(a_full(sp));
-            sp = sp + 1 == P.a_stages ? 0 : sp + 1;
-            --pending;
-        };
-        for (int item = item0; item < P.items && ok; item += item_step, par = !par) {
-            const TapItem t = tap_item<PAIR>(P, item, R, side);
-            // x's pixel of every staged pixel, or -1 for zeros
-            int *const pix = reinterpret_cast<int *>(smem + P.tab_off) + (par ? TL::pixels : 0);
-            for (int p = pt; p < TL::pixels; p += kProdThreads) {
-                int row, col;
-                TL::entry(p, row, col);
-                const int o = tap_origin<STRIDE, TAPS, MT>(P, t.v0, row), ix = t.ox0 * STRIDE + col;
-                const bool in = o >= 0 && (TAPS == 1 ? (int64_t)o + ix < P.npix : (unsigned)ix < (unsigned)P.w);
-                pix[p] = in ? o + ix : -1;
-            }
-            asm volatile("bar.sync 1, %0;" ::"n"(kProdThreads) : "memory");
-            for (int ks = k0; ks < k1; ++ks) {
-                // What was copied earlier is handed over before this warp waits for room.
-                if (pending && !__all_sync(0xFFFFFFFFu, mbar_ready(a_empty(s), ph))) {
-                    copy_wait<0>();
-                    while (pending) publish();
+        if (!kF32 && P.tma) {
+            if (warp == kEpiWarps) {
+                // ---- x by tensor copies, zeros outside the image -------------------------------
+                if (elect_one()) {
+                    int s = 0;
+                    uint32_t ph = 1;
+                    for (int item = item0; item < P.items; item += item_step) {
+                        const TapItem t = tap_item<MT, PAIR>(P, item, side);
+                        s_started = s_started + 1;
+                        for (int ks = k0; ks < k1; ++ks) {
+                            wait(a_empty(s), ph);
+                            const uint32_t bar = lead(a_full(s));
+                            uint32_t dst = sbase + (uint32_t)(s * P.a_bytes) + (P.raster ? (uint32_t)(P.pitch - 1 - t.ox0) * 128u : 0u);
+                            const int c = ks * T::row_ch;
+                            if (side == 0) mbar_expect_tx(a_full(s), (uint32_t)(P.a_tx * (PAIR ? 2 : 1)));
+                            if (TAPS == 1) tensor_load4<PAIR>(dst, &xmap, c, t.v0 * 8, 0, 0, bar);
+                            else {
+                                const int step = (P.row_boxes ? 1 : P.rows) * P.pitch * 128;
+                                for (int region = 0; region < (STRIDE == 1 ? 1 : 4); ++region) {
+                                    const int x0 = STRIDE == 1 ? (P.raster ? 0 : t.ox0) - 1 : 2 * t.ox0 - (region & 1);
+                                    for (int i = 0; i < (P.row_boxes ? P.rows : 1); ++i, dst += step) {
+                                        const TapRow r = tap_row<STRIDE>(P, t, i, region >> 1);
+                                        tensor_load4<PAIR>(dst, &xmap, c, x0, r.y, r.img, bar);
+                                    }
+                                }
+                            }
+                            if (++s == P.a_stages) { s = 0; ph ^= 1u; }
+                        }
+                    }
                 }
-                ok = wait(a_empty(s), ph);
-                if (!ok) break;
-                const uint32_t dst = sbase + (uint32_t)s * a_bytes;
-                const int npl = min(P.pl, planes - ks * P.pl);
-                if (!kF32 && P.vec_x) {
-#pragma unroll 4
-                    for (int i = pt; i < total; i += kProdThreads) {
-                        const int pl = i & (P.pl - 1), p = i >> P.pl_log;
-                        const int c = (ks * P.pl + pl) * T::cpp;
-                        const int px = pix[p];
-                        const bool in = px >= 0 && c < P.c_in;
-                        if (pl < npl)
-                            copy16(dst + (uint32_t)(pl * P.plane_pitch + p * 16), in ? x + ((size_t)px * P.c_in + c) * T::xb : x, in ? 16u : 0u);
+                __syncwarp();
+            } else if (FUSED && P.residual && P.splits == 1) {
+                // ---- the residual into L2, an item ahead of its use --------------------------
+                const int pt = tid - (kEpiWarps + 1) * 32;
+                const int row = min(P.nt, P.c_out - n0) * (DT == XGEN_F16_F32ACC ? 2 : 4), lines = (row + 127) / 128;
+                auto fetch = [&](int item) {
+                    if (item >= P.items) return;
+                    const TapItem t = tap_item<MT, PAIR>(P, item, side);
+                    for (int i = pt; i < 128 * MT * lines; i += kProdThreads - 32) {
+                        const int m = i / lines, at = min((i - m * lines) * 128, row - 4);
+                        const int px = tap_pixel<TAPS>(P, t, m).pix;
+                        if (px >= 0)
+                            asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char *>(P.residual) +
+                                         ((size_t)px * P.c_out + n0) * (DT == XGEN_F16_F32ACC ? 2 : 4) + at));
                     }
-                    copy_commit();
-                    ++pending;
-                    if (pending == P.a_stages) {            // as many stages in flight as there are
-                        if (P.a_stages == 1) copy_wait<0>();
-                        else if (P.a_stages == 2) copy_wait<1>();
-                        else if (P.a_stages == 3) copy_wait<2>();
-                        else copy_wait<3>();
-                        publish();
-                    }
-                } else {
+                };
+                fetch(item0);
+                int done = 0;
+                for (int item = item0; item < P.items; item += item_step, ++done) {
+                    for (int it = 0; it < 100000 && s_started <= done; ++it) __nanosleep(100);     // (a pace, nothing depends on it)
+                    fetch(item + item_step);
+                }
+            }
+        } else {
+            // ---- x through the producer warps ------------------------------------------------------
+            const int pt = tid - kEpiWarps * 32;
+            int s = 0;
+            uint32_t ph = 1;
+            bool ok = true, par = false;
+            const char *const x = static_cast<const char *>(P.x);
+            const int total = kF32 ? P.pixels << P.pl_log : P.pixels * 8;
+            for (int item = item0; item < P.items && ok; item += item_step, par = !par) {
+                const TapItem t = tap_item<MT, PAIR>(P, item, side);
+                int *const pix = reinterpret_cast<int *>(smem + P.tab_off) + (par ? P.pixels : 0);
+                for (int p = pt; p < P.pixels; p += kProdThreads) pix[p] = tap_source<STRIDE, TAPS>(P, t, p);
+                asm volatile("bar.sync 1, %0;" ::"n"(kProdThreads) : "memory");
+                for (int ks = k0; ks < k1; ++ks) {
+                    ok = wait(a_empty(s), ph);
+                    if (!ok) break;
+                    const uint32_t dst = sbase + (uint32_t)(s * P.a_bytes);
+                    const int npl = min(P.pl, planes - ks * P.pl);
                     constexpr int U = kF32 ? 4 : 2;          // pieces of a thread in flight
                     for (int i0 = pt; i0 < total; i0 += U * kProdThreads) {
                         float f[kF32 ? U : 1][8];
@@ -668,9 +712,9 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
                             const int i = i0 + u * kProdThreads;
-                            const int pl = i & (P.pl - 1), p = i >> P.pl_log;
+                            const int pl = kF32 ? i & (P.pl - 1) : i & 7, p = kF32 ? i >> P.pl_log : i >> 3;
                             const int c = (ks * P.pl + pl) * T::cpp;
-                            const int px = i < total ? pix[p] : -1;
+                            const int px = i < total && pl < npl ? pix[p] : -1;
                             const char *src = x + ((size_t)(px < 0 ? 0 : px) * P.c_in + c) * T::xb;
                             const int left = px < 0 ? 0 : P.c_in - c;     // channels there are
                             if (kF32) {
@@ -699,82 +743,100 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
                             const int i = i0 + u * kProdThreads;
-                            const int pl = i & (P.pl - 1), p = i >> P.pl_log;
-                            const uint32_t d = dst + (uint32_t)(pl * P.plane_pitch + p * 16);
+                            const int pl = kF32 ? i & (P.pl - 1) : i & 7, p = kF32 ? i >> P.pl_log : i >> 3;
                             if (i < total && pl < npl) {
                                 if (kF32) {
+                                    const uint32_t d = dst + (uint32_t)(pl * P.plane_pitch + p * 16);
                                     uint4 p0, p1, p2;
                                     split3(f[kF32 ? u : 0], p0, p1, p2);
                                     sts128(d, p0);
                                     sts128(d + a_part, p1);
                                     sts128(d + 2 * a_part, p2);
                                 } else {
-                                    sts128(d, g[kF32 ? 0 : u]);
+                                    sts128(dst + (uint32_t)(p * 128 + ((pl ^ (p & 7)) << 4)), g[kF32 ? 0 : u]);
                                 }
                             }
                         }
                     }
-                    ++pending;
-                    publish();
+                    fence_async_proxy();
+                    __syncwarp();
+                    if (lane == 0) arrive_lead(a_full(s));
+                    if (++s == P.a_stages) { s = 0; ph ^= 1u; }
                 }
-                if (++s == P.a_stages) { s = 0; ph ^= 1u; }
             }
         }
-        copy_wait<0>();
-        while (pending) publish();
     } else if (warp == kEpiWarps + kProdWarps) {
-        // ---- matrix instructions: one thread, which also waits (a warp that meets again at every tap
-        // takes some 600 cycles for a tap's 4 to 8 instructions).  A wait that gives up is not looked at:
+        // ---- matrix instructions: one thread, which also waits.  A wait that gives up is not looked at:
         // nothing per-thread may steer these loops, or every operand is moved to the uniform registers
-        // anew; all later waits then return at once. ------------------------------------------------
+        // anew; all later waits then return at once.  Taps are unrolled, a few share a barrier, and the
+        // next barrier is looked at before the instructions of this one are issued: in a rolled loop with
+        // a wait of its own a tap costs 350 cycles, its four instructions of 128 x 128 x 16 take 256. --
         if (side == 0 && elect_one()) {
             const uint32_t b_rows = (uint32_t)P.nt / (PAIR ? 2 : 1);         // filters whose weights this block holds
-            const uint32_t b_plane = PARTS * b_rows * 16;
-            const uint64_t a0 = operand_desc(sbase, (uint32_t)P.plane_pitch, TL::pitch * 16);
-            const uint64_t b0 = operand_desc(sbase + P.b_off, b_plane, 128);
+            const uint32_t b_tap = PARTS * b_rows;                           // 16-byte units from here on
+            const uint32_t b_plane = b_tap * (uint32_t)P.tap_group;
+            const uint64_t a0 = kF32 ? operand_desc(sbase, (uint32_t)P.plane_pitch, (P.raster ? 8 : P.pitch) * 16)
+                                     : operand_desc_swizzled(sbase, (P.raster ? 8 : P.pitch) * 128);
+            const uint64_t b0 = operand_desc(sbase + P.b_off, b_plane * 16, 128);
             const uint32_t a_hi = (uint32_t)(a0 >> 32), b_hi = (uint32_t)(b0 >> 32), idesc = P.idesc;
-            const uint32_t a_k = (uint32_t)P.plane_pitch * 2 / 16, b_k = b_plane * 2 / 16, a_p = a_part / 16, b_p = b_rows;
-            const uint32_t b_step = (uint32_t)P.b_bytes / 16;
+            const uint32_t a_k = kF32 ? (uint32_t)P.plane_pitch * 2 / 16 : 2u, b_k = b_plane * 2, a_p = a_part / 16, b_p = b_rows;
+            constexpr uint32_t a_px = kF32 ? 1 : 8;
+            const uint32_t a_sub = (uint32_t)P.sub_px * a_px, a_step = (uint32_t)P.a_bytes / 16, b_step = (uint32_t)P.b_bytes / 16;
             int s = 0, b = 0, buf = 0;
-            uint32_t pha = 0, phb = 0, phc = 1, bt = (uint32_t)b0;
+            uint32_t pha = 0, phb = 0, phc = 1, as = (uint32_t)a0, bs = (uint32_t)b0;
+            bool ready = mbar_try<PAIR>(b_full(0), 0);
             for (int item = item0; item < P.items; item += item_step) {
                 for (int ks = k0; ks < k1; ++ks) {
                     if (kF32 || ks == k0) wait(acc_empty(buf), phc);
                     wait(a_full(s), pha);
                     tc_fence_after();
                     const int kk_n = min(P.pl, planes - ks * P.pl) / 2;
-                    const uint32_t as = (uint32_t)a0 + (uint32_t)s * (a_bytes / 16);
                     const uint32_t d = tmem + (uint32_t)buf * (uint32_t)(MT * P.nt);
                     const uint32_t dc = d + 2u * P.nt;      // fp32: the small products (two buffers behind the two of the sums)
-#pragma unroll 1
-                    for (int tap = 0; tap < TAPS; ++tap) {      // (rolled: code that runs once comes from L2, 600 cycles a tap)
-                        wait(b_full(b), P.resident ? 0u : phb);
-                        uint32_t ak = as + (uint32_t)P.tap_start[tap], bk = bt;
-#pragma unroll 1
-                        for (int kk = 0; kk < kk_n; ++kk, ak += a_k, bk += b_k) {
-                            const uint32_t first_s = tap > 0 || kk > 0 ? 1u : 0u;       // 0: the first of the stage
-                            const uint32_t first_i = first_s | (ks > k0 ? 1u : 0u);     // 0: the first of the item
-                            if (kF32) {
-                                mma_f16<PAIR>(d, ak, a_hi, bk, b_hi, idesc, first_s);
-                                mma_f16<PAIR>(dc, ak, a_hi, bk + b_p, b_hi, idesc, first_s);
-                                mma_f16<PAIR>(dc, ak, a_hi, bk + 2 * b_p, b_hi, idesc, 1u);
-                                mma_f16<PAIR>(dc, ak + a_p, a_hi, bk, b_hi, idesc, 1u);
-                                mma_f16<PAIR>(dc, ak + a_p, a_hi, bk + b_p, b_hi, idesc, 1u);
-                                mma_f16<PAIR>(dc, ak + 2 * a_p, a_hi, bk, b_hi, idesc, 1u);
-                            } else {
+                    uint32_t bt = bs;
 #pragma unroll
-                                for (int m = 0; m < MT; ++m) {
-                                    if (DT == XGEN_I8_I32) mma_i8<PAIR>(d + m * P.nt, ak + m * 16 * TL::pitch, a_hi, bk, b_hi, idesc, first_i);
-                                    else mma_f16<PAIR>(d + m * P.nt, ak + m * 16 * TL::pitch, a_hi, bk, b_hi, idesc, first_i);
+                    for (int tap = 0; tap < TAPS; ++tap) {
+                        if ((P.tap_group == 1 || tap % 3 == 0) && !ready)
+                            mbar_wait_long<PAIR>(b_full(b), P.resident ? 0u : phb, &s_abort, P.status, P.wait_us);
+                        const bool last = P.tap_group == 1 || tap % 3 == 2;
+                        if (last) {                         // (of its slot: look at the next one)
+                            const bool wrap = b + 1 == P.b_slots;
+                            ready = mbar_try<PAIR>(b_full(wrap ? 0 : b + 1), P.resident ? 0u : wrap ? phb ^ 1u : phb);
+                        }
+                        const uint32_t at = as + (uint32_t)P.tap_start[tap] * a_px;
+#pragma unroll
+                        for (int kk = 0; kk < 4; ++kk) {
+                            if (kk < kk_n) {
+                                const uint32_t ak = at + kk * a_k, bk = bt + kk * b_k;
+                                const uint32_t first_s = tap > 0 || kk > 0 ? 1u : 0u;       // 0: the first of the stage
+                                const uint32_t first_i = first_s | (ks > k0 ? 1u : 0u);     // 0: the first of the item
+                                if (kF32) {
+                                    mma_f16<PAIR>(d, ak, a_hi, bk, b_hi, idesc, first_s);
+                                    mma_f16<PAIR>(dc, ak, a_hi, bk + b_p, b_hi, idesc, first_s);
+                                    mma_f16<PAIR>(dc, ak, a_hi, bk + 2 * b_p, b_hi, idesc, 1u);
+                                    mma_f16<PAIR>(dc, ak + a_p, a_hi, bk, b_hi, idesc, 1u);
+                                    mma_f16<PAIR>(dc, ak + a_p, a_hi, bk + b_p, b_hi, idesc, 1u);
+                                    mma_f16<PAIR>(dc, ak + 2 * a_p, a_hi, bk, b_hi, idesc, 1u);
+                                } else {
+#pragma unroll
+                                    for (int m = 0; m < MT; ++m) {
+                                        if (DT == XGEN_I8_I32) mma_i8<PAIR>(d + m * P.nt, ak + m * a_sub, a_hi, bk, b_hi, idesc, first_i);
+                                        else mma_f16<PAIR>(d + m * P.nt, ak + m * a_sub, a_hi, bk, b_hi, idesc, first_i);
+                                    }
                                 }
                             }
                         }
-                        if (!P.resident) tc_commit<PAIR>(b_empty(b), both);
-                        bt += b_step;
-                        if (++b == P.b_slots) { b = 0; phb ^= 1u; bt = (uint32_t)b0; }
+                        bt += b_tap;
+                        if (last) {
+                            if (!P.resident) tc_commit<PAIR>(b_empty(b), both);
+                            bs += b_step;
+                            if (++b == P.b_slots) { b = 0; phb ^= 1u; bs = (uint32_t)b0; }
+                            bt = bs;
+                        }
                     }
                     tc_commit<PAIR>(a_empty(s), both);
-                    if (++s == P.a_stages) { s = 0; pha ^= 1u; }
+                    as += a_step;
+                    if (++s == P.a_stages) { s = 0; pha ^= 1u; as = (uint32_t)a0; }
                     if (kF32 || ks + 1 == k1) {
                         tc_commit<PAIR>(acc_full(buf), both);
                         if (++buf == P.acc_bufs) { buf = 0; phc ^= 1u; }
@@ -792,13 +854,13 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             uint32_t ph = 1;
             for (int item = item0; item < P.items; item += item_step) {
                 for (int ks = k0; ks < k1; ++ks) {
-                    for (int tap = 0; tap < TAPS; ++tap) {
+                    for (int tap = 0; tap < TAPS; tap += P.tap_group) {
                         if (issued >= P.b_slots) wait(b_empty(b), ph);
-                        // one copy for a tap: pieces of 2 KB with a copy of their own cost 50 cycles
+                        // one copy for a slot: pieces of 2 KB with a copy of their own cost 50 cycles
                         // of issue apiece and held the whole kernel to 5.5 TB/s of weights
                         if (side == 0) mbar_expect_tx(b_full(b), (uint32_t)P.b_bytes * (PAIR ? 2 : 1));
                         tensor_load4<PAIR>(sbase + P.b_off + (uint32_t)(b * P.b_bytes), &wmap, (n0 + side * P.nt / 2) * 2, 0, tap, ks * P.pl,
-                                           PAIR ? cluster_addr(b_full(b), (uint32_t)(crank & ~1)) : b_full(b));
+                                           lead(b_full(b)));
                         ++issued;
                         if (++b == P.b_slots) { b = 0; ph ^= 1u; }
                     }
@@ -833,19 +895,9 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
         uint32_t ph = 0;
         bool ok = true;
         for (int item = item0; item < P.items && ok; item += item_step) {
-            const TapItem t = tap_item<PAIR>(P, item, R, side);
-            const int v = t.v0 + sub * 16 + (m >> 3), ox = t.ox0 + (m & 7);
-            int pix = -1, out = -1;              // this lane's pixel: of the result, and where it is stored
-            if (TAPS == 1) {
-                if ((int64_t)v * 8 + ox < P.npix) pix = v * 8 + ox;
-                out = pix;
-            } else {
-                const int img = v / P.vh, oy = v - img * P.vh;
-                if (img < P.n && oy < P.ho && ox < P.wo) {
-                    pix = (img * P.ho + oy) * P.wo + ox;
-                    out = P.pool ? (img * P.po + oy / 2) * P.pw + ox / 2 : pix;
-                }
-            }
+            const TapItem t = tap_item<MT, PAIR>(P, item, side);
+            const TapPixel at = tap_pixel<TAPS>(P, t, sub * 128 + m);
+            const int pix = at.pix, out = at.out;
             auto put = [&](const uint32_t *r, int n, int at) {
 #pragma unroll
                 for (int q = 0; q < n / 4; ++q)
@@ -923,7 +975,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
         cluster_meet();
         constexpr int kAdders = (kEpiWarps + kProdWarps) * 32;
         if (tid < kAdders && !s_abort) {
-            const TapItem t = tap_item<PAIR>(P, item0, R, side);
+            const TapItem t = tap_item<MT, PAIR>(P, item0, side);
             const int groups = P.nt / 8, pitch = (P.nt + 4) * 4;
             const bool pool = FUSED && P.pool;
             // units of two rows of eight pixels go round the blocks; a thread takes 8 channels of one (pooled) pixel
@@ -933,19 +985,8 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 const int u = w / per_unit, wu = w - u * per_unit, row = wu / groups, g = wu - row * groups;
                 const int c0 = n0 + 8 * g;
                 const int m0 = 16 * (rank + u * P.splits) + (pool ? 2 * row : row);
-                const int v = t.v0 + (m0 >> 3), ox = t.ox0 + (m0 & 7);
-                int pix, out;
-                bool valid;
-                if (TAPS == 1) {
-                    valid = (int64_t)v * 8 + ox < P.npix;
-                    out = pix = v * 8 + ox;
-                } else {
-                    const int img = v / P.vh, oy = v - img * P.vh;
-                    valid = img < P.n && oy < P.ho && ox < P.wo;
-                    pix = (img * P.ho + oy) * P.wo + ox;
-                    out = pool ? (img * P.po + oy / 2) * P.pw + ox / 2 : pix;
-                }
-                if (!valid || c0 >= P.c_out) continue;
+                const TapPixel px = tap_pixel<TAPS>(P, t, m0);
+                if (px.pix < 0 || c0 >= P.c_out) continue;
                 uint32_t best[8];
 #pragma unroll 1
                 for (int q = 0; q < (pool ? 4 : 1); ++q) {
@@ -962,11 +1003,11 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                         for (int i = 0; i < 8; ++i)
                             v8[i] = DT == XGEN_I8_I32 ? v8[i] + ab[i] : __float_as_uint(__uint_as_float(v8[i]) + __uint_as_float(ab[i]));
                     }
-                    tap_affine<DT, FUSED, 8>(P, s_bias, v8, pix + (q & 1) + (q >> 1) * P.wo, true, c0, n0);
+                    tap_affine<DT, FUSED, 8>(P, s_bias, v8, px.pix + (q & 1) + (q >> 1) * P.wo, true, c0, n0);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) best[i] = q == 0 ? v8[i] : tap_max<DT>(best[i], v8[i]);
                 }
-                tap_store<DT, FUSED, 8>(P, s_scale, best, out, c0, n0);
+                tap_store<DT, FUSED, 8>(P, s_scale, best, px.out, c0, n0);
             }
         }
     }
@@ -1144,17 +1185,6 @@ static int tap_clusters(int size, int device, int sms) {
     return k;
 }
 
-static int tap_pixels(int stride, int taps, int mt) {
-    const int R = 16 * mt;
-    return taps == 1 ? 8 * R : stride == 1 ? 10 * (R + 2) : 9 * (4 * R + 2);
-}
-
-static int tap_start(int stride, int taps, int mt, int t) {
-    if (taps == 1) return 0;
-    if (stride == 1) return TapTile<1, 9, 1>::tap_start(t);
-    return mt == 2 ? TapTile<2, 9, 2>::tap_start(t) : TapTile<2, 9, 1>::tap_start(t);
-}
-
 bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &best) {
     static int sm_count[64];
     int sms = 148;
@@ -1168,30 +1198,48 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
     const int ho = (s.h - 1) / s.stride + 1, wo = (s.w - 1) / s.stride + 1;
     best = TapPlan();
     best.cycles = 1e30;
-    for (int shape = 0; shape < (dt == XGEN_F32 ? 2 : 4); ++shape) {
+    const bool swizzled = dt != XGEN_F32, copied = swizzled && (size_t)tw.c_in * xb % 16 == 0;
+    // Tiles: 8-pixel columns with every image rounded up to whole tiles (0), with one row of zeros between
+    // images and tiles that cross them (1), or runs of the raster (2).
+    for (int shape = 0; shape < 12; ++shape) {
         TapPlan p;
         p.pair = shape & 1;
-        p.mt = 1 + (shape >> 1);
-        const int mt = p.mt, ways = p.pair ? 2 : 1, R = 16 * mt, pixels = tap_pixels(s.stride, tw.taps, mt);
-        int64_t row_tiles;
+        p.mt = 1 + (shape >> 1) % 2;
+        const int form = (shape >> 1) / 2, mt = p.mt, ways = p.pair ? 2 : 1, R = 16 * mt;
+        if (mt == 2 && dt == XGEN_F32) continue;
+        p.raster = form == 2;
+        p.straddle = form >= 1;
+        int64_t tiles_all;
         if (tw.taps == 1) {
-            p.segs = 1; p.vh = 1;
-            row_tiles = (s.h + R - 1) / R;
+            if (form) continue;
+            p.pitch = 8; p.rows = R; p.pixels = 8 * R; p.segs = 1; p.vh = 1;
+            p.row_tiles = (s.h + R - 1) / R;
+            tiles_all = p.row_tiles;
+        } else if (p.raster) {
+            if (s.stride != 1 || s.pool || s.w > 150) continue;
+            p.vh = ho + 1;
+            p.pitch = s.w + 1;
+            p.rows = 3 + (128 * mt + p.pitch - 1) / p.pitch;
+            p.pixels = p.rows * p.pitch + p.pitch - 1;
+            p.segs = 1;
+            tiles_all = ((int64_t)s.n * p.vh * p.pitch + 128 * mt - 1) / (128 * mt);
+            p.row_tiles = (int)std::min<int64_t>(tiles_all, 0x7FFFFFFF);
         } else {
-            // Rows of all images below each other: every image rounded up to whole tiles, or one row of
-            // zeros between images and tiles that cross them, whichever has fewer rows.
-            const int whole = (ho + R - 1) / R * R;
-            const int gap = ho + 1 + (s.pool && (ho + 1) % 2 ? 1 : 0);
-            const int64_t tiles_whole = (int64_t)s.n * whole / R, tiles_gap = ((int64_t)s.n * gap + R - 1) / R;
-            p.straddle = tiles_gap < tiles_whole;
+            const int whole = (ho + R - 1) / R * R, gap = ho + 1 + (s.pool && (ho + 1) % 2 ? 1 : 0);
             p.vh = p.straddle ? gap : whole;
-            row_tiles = p.straddle ? tiles_gap : tiles_whole;
+            if (p.straddle && (int64_t)s.n * gap >= (int64_t)s.n * whole) continue;
+            p.pitch = s.stride == 1 ? 10 : 9;
+            p.rows = s.stride == 1 ? R + 2 : R + 1;
+            p.pixels = p.rows * p.pitch * (s.stride == 1 ? 1 : 4);
             p.segs = (wo + 7) / 8;
+            const int64_t rt = ((int64_t)s.n * p.vh + R - 1) / R;
+            tiles_all = rt * p.segs;
+            p.row_tiles = (int)std::min<int64_t>(rt, 0x7FFFFFFF);
         }
-        if (row_tiles * p.segs * ((tw.rows + 31) / 32) > 0x7FFFFFFF / 32) continue;
-        p.row_tiles = (int)row_tiles;
-        const int tiles = (p.row_tiles * p.segs + ways - 1) / ways;
-        if (p.pair && p.row_tiles * p.segs == 1) continue;
+        if (tiles_all * ((tw.rows + 31) / 32) > 0x7FFFFFFF / 256) continue;
+        if (p.pair && tiles_all == 1) continue;
+        const int tiles = (int)((tiles_all + ways - 1) / ways), pixels = p.pixels;
+        p.table_bytes = copied && tw.taps == 9 ? 0 : (pixels * 8 + 127) / 128 * 128;
         // fp32 keeps four accumulators of `nt` columns and 64 sums a thread; 512 columns hold all of the others'
         const int nt_top = dt == XGEN_F32 || !p.pair ? 128 : kMaxFilterTile;
         for (int nt_max = 32; nt_max <= nt_top; nt_max += 32) {
@@ -1201,17 +1249,17 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
             if (p.nt != nt_max) continue;
             p.items = tiles * p.nblk;
             for (int pl = 2; pl <= 8; pl *= 2) {
-                if (pl > 2 && pl / 2 >= tw.planes) continue;
-                if (dt == XGEN_F32 && tw.taps * pl / 2 > 18) continue;      // bounds the chain of the fp32 accumulator
-                p.pl = pl;
+                if (swizzled && pl != 8) continue;                          // rows of 128 bytes
+                if (!swizzled && pl > 2 && pl / 2 >= tw.planes) continue;
+                if (!swizzled && tw.taps * pl / 2 > 18) continue;           // bounds the chain of the fp32 accumulator
+                p.pl = swizzled ? std::min(8, tw.planes) : pl;
                 p.stages = (tw.planes + pl - 1) / pl;
                 // 16-byte accesses of 8 lanes (pl planes x 8 / pl pixels) fall into distinct banks
                 p.plane_pitch = pixels * 16;
                 while (p.plane_pitch % 128 != 128 / pl % 128) p.plane_pitch += 16;
-                const size_t a_bytes = (size_t)parts * pl * p.plane_pitch, b_bytes = (size_t)pl * parts * p.nt * 16 / ways;
-                const size_t pix_tables = ((size_t)pixels * 8 + 127) / 128 * 128;
+                p.a_bytes = swizzled ? (pixels * 128 + 1023) / 1024 * 1024 : parts * pl * p.plane_pitch;
+                if ((size_t)p.a_bytes > (size_t)kTapSmemMax) continue;
                 for (int sp = 1; sp * ways <= 16 && sp <= p.stages; ++sp) {
-                    const size_t tables = pix_tables + (sp == 1 && s.staged ? epi_warps(dt) * kStageBytes : 0);
                     p.per_split = (p.stages + sp - 1) / sp;
                     p.splits = (p.stages + p.per_split - 1) / p.per_split;
                     if (p.splits != sp) continue;
@@ -1229,42 +1277,47 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                         p.grid = p.items * sp * ways;
                         waves = (p.items + cl - 1) / cl;
                     }
+                    const size_t tables = p.table_bytes + (sp == 1 && s.staged ? epi_warps(dt) * kStageBytes : 0);
                     const int64_t uses = (sp == 1 ? waves : 1) * p.per_split;      // stages one block goes through
-                    // Shared memory: two tiles of x (more for a plain product, whose stages are short), the rest weights.
-                    const int want_a = (int)std::min<int64_t>(uses, tw.taps == 1 ? kMaxA : 2);
-                    const int all_b = p.per_split * tw.taps;
+                    // Shared memory: two tiles of x (more for a plain product, whose stages are short), the rest
+                    // weights, by three taps if at least three such slots fit.
                     bool fits = false;
-                    for (p.a_stages = want_a; p.a_stages >= 1; --p.a_stages) {
-                        const size_t left_a = p.a_stages * a_bytes + tables;
-                        if (left_a >= (size_t)kTapSmemMax) continue;
-                        const int room = (int)std::min<size_t>(kMaxB, ((size_t)kTapSmemMax - left_a) / b_bytes);
-                        p.resident = all_b <= room;
-                        p.b_slots = std::min(room, all_b);
-                        if (p.b_slots >= std::min(all_b, 3) && p.a_stages >= std::min<int64_t>(2, uses)) { fits = true; break; }
+                    for (p.tap_group = tw.taps == 1 ? 1 : 3; p.tap_group >= 1 && !fits; p.tap_group -= 2) {
+                        p.b_bytes = p.tap_group * p.pl * parts * p.nt * 16 / ways;
+                        const int all_b = p.per_split * tw.taps / p.tap_group;
+                        for (p.a_stages = (int)std::min<int64_t>(uses, tw.taps == 1 ? kMaxA : 2); p.a_stages >= 1; --p.a_stages) {
+                            const size_t left_a = (size_t)p.a_stages * p.a_bytes + tables;
+                            if (left_a >= (size_t)kTapSmemMax) continue;
+                            const int room = (int)std::min<size_t>(kMaxB, ((size_t)kTapSmemMax - left_a) / p.b_bytes);
+                            p.resident = all_b <= room;
+                            p.b_slots = std::min(room, all_b);
+                            if (p.b_slots >= std::min(all_b, 3) && p.a_stages >= std::min<int64_t>(2, uses)) { fits = true; break; }
+                        }
+                        if (fits) break;
                     }
                     if (!fits) continue;
-                    p.smem = p.a_stages * a_bytes + p.b_slots * b_bytes + tables;
+                    p.smem = (size_t)p.a_stages * p.a_bytes + (size_t)p.b_slots * p.b_bytes + tables;
                     if (sp > 1) p.smem = std::max(p.smem, (size_t)mt * 128 * (p.nt + 4) * 4);
                     if (p.smem > (size_t)kTapSmemMax) continue;
                     p.acc_bufs = dt == XGEN_F32 || 2 * mt * p.nt <= 512 ? 2 : 1;
                     const int cols = dt == XGEN_F32 ? 4 * p.nt : p.acc_bufs * mt * p.nt;
                     for (p.tmem_cols = 32; p.tmem_cols < cols;) p.tmem_cols *= 2;
-                    // Cycles of a stage: the matrix instructions (nt / 2 each), or what they and the copies move
-                    // through shared memory at 128 bytes a cycle (128 rows of x, the block's filters), or
-                    // what comes from L2.  A tap costs about 40 cycles besides, a stage 300.
+                    // Cycles of a stage: the matrix instructions (nt / 2 each, 45 to issue one), or what they and
+                    // the copies move through shared memory at 128 bytes a cycle (128 rows of x, the block's
+                    // filters), or what comes from L2.  A slot of weights costs 40 cycles besides, a stage 250.
                     const double kk = (double)tw.planes / p.stages / 2, taps = tw.taps;
                     const double b_stage = taps * kk * 2 * parts * p.nt * 16.0 / ways, b_moved = p.resident && sp == 1 ? b_stage / waves : b_stage;
-                    const double x_moved = (double)pixels * kk * 2 * cpp * xb, a_stage = (double)parts * pixels * kk * 2 * 16;
+                    const double x_moved = (double)pixels * kk * 2 * cpp * xb, a_stage = (double)p.a_bytes * (swizzled ? 1 : 2);
                     const double instr = taps * kk * mt * prod;
-                    const double mma = instr * std::max(p.nt / 2.0, 40.0);
-                    const double shared = (instr * (4096.0 + p.nt * 32.0 / ways) + b_moved + 2 * a_stage) / 128.0;
-                    const double move = (x_moved + b_moved) / 40.0;
-                    const double stage = std::max(std::max(mma, shared), move) + 300.0 + 40.0 * taps;
+                    const double mma = instr * std::max(p.nt / 2.0, 45.0);
+                    const double shared = (instr * (4096.0 + p.nt * 32.0 / ways) + b_moved + a_stage) / 128.0;
+                    const double move = (x_moved + b_moved) / 40.0 + (copied && p.straddle ? 60.0 * p.rows * (s.stride == 1 ? 1 : 4) : 0.0) * 0.5;
+                    const double stage = std::max(std::max(mma, shared), move) + 250.0 + 40.0 * taps / p.tap_group;
                     const double out = (double)mt * 128 * p.nt * yb / 24.0;
                     const double item = p.per_split * stage;
                     double c = 3500.0 + (p.pair ? 2500.0 : 0.0);
                     if (sp == 1) c += waves * std::max(item, p.acc_bufs == 2 ? out : 0.0) + (p.acc_bufs == 2 ? out : waves * out);
-                    else c += waves * (item + 2500.0 + 40.0 * sp + mt * 128.0 * p.nt * 4 / 48.0 + out / sp);
+                    else c += waves * (item + 3500.0 + 40.0 * sp + mt * 128.0 * p.nt * 4 / 48.0 + out / sp);
                     if (c < best.cycles * 0.999) { best = p; best.cycles = c; }
                 }
             }
@@ -1277,13 +1330,31 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
     const cuuint64_t dim[4] = {(cuuint64_t)tw.rows * 2, (cuuint64_t)parts, (cuuint64_t)tw.taps, (cuuint64_t)tw.planes};
     const cuuint64_t row = (cuuint64_t)tw.rows * 16;
     const cuuint64_t str[3] = {row, row * parts, row * parts * tw.taps};
-    const cuuint32_t box[4] = {(cuuint32_t)(best.pair ? best.nt : best.nt * 2), (cuuint32_t)parts, 1, (cuuint32_t)best.pl};
+    const cuuint32_t box[4] = {(cuuint32_t)(best.pair ? best.nt : best.nt * 2), (cuuint32_t)parts, (cuuint32_t)best.tap_group, (cuuint32_t)best.pl};
     const cuuint32_t one[4] = {1, 1, 1, 1};
     return encode(&best.wmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 4, tw.dev, dim, str, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The tensor map of x: boxes of 128 bytes of channels of the staged rows (one, or all of a tile).
+static bool x_map(const TapWeights &tw, const TapShape &s, const TapPlan &p, const void *x, CUtensorMap &m) {
+    EncodeTiledFn encode = encode_tiled_fn();
+    if (!encode) return false;
+    const cuuint64_t px = (cuuint64_t)tw.c_in * (tw.dtype == XGEN_I8_I32 ? 1 : 2);
+    const cuuint64_t w = tw.taps == 1 ? (cuuint64_t)s.rows : (cuuint64_t)s.w, h = tw.taps == 1 ? 1 : (cuuint64_t)s.h;
+    const cuuint64_t dim[4] = {(cuuint64_t)tw.c_in, w, h, (cuuint64_t)s.n};
+    const cuuint64_t str[3] = {px, px * w, px * w * h};
+    const cuuint32_t st = (cuuint32_t)s.stride;
+    const cuuint32_t box[4] = {tw.dtype == XGEN_I8_I32 ? 128u : 64u, (cuuint32_t)(tw.taps == 1 ? p.pixels : p.pitch) * st,
+                               (cuuint32_t)(tw.taps == 1 || p.straddle ? 1 : p.rows) * st, 1};
+    const cuuint32_t step[4] = {1, st, st, 1};
+    return encode(&m, tw.dtype == XGEN_I8_I32 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void *>(x), dim, str,
+                  box, step, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p, const TapCall &c, cudaStream_t st) {
+    CUtensorMap xm{};
     const xgen_dtype dt = tw.dtype;
     const int parts = tap_parts(dt), xb = dt == XGEN_F32 ? 4 : dt == XGEN_F16_F32ACC ? 2 : 1;
     const int yb = c.rq_scale ? 1 : dt == XGEN_F16_F32ACC ? 2 : 4, rb = dt == XGEN_F16_F32ACC ? 2 : 4;
@@ -1300,14 +1371,24 @@ cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p
     P.segs = p.segs; P.nblk = p.nblk; P.nt = p.nt; P.items = p.items; P.splits = p.splits; P.per_split = p.per_split; P.stages = p.stages;
     P.pl = p.pl; P.pl_log = p.pl == 2 ? 1 : p.pl == 4 ? 2 : 3; P.plane_pitch = p.plane_pitch;
     P.a_stages = p.a_stages; P.b_slots = p.b_slots; P.resident = p.resident;
-    P.b_bytes = p.pl * parts * (p.pair ? p.nt / 2 : p.nt) * 16;
-    P.b_off = p.a_stages * parts * p.pl * p.plane_pitch;
+    P.b_bytes = p.b_bytes; P.tap_group = p.tap_group;
+    P.a_bytes = p.a_bytes;
+    P.b_off = p.a_stages * p.a_bytes;
     P.tab_off = P.b_off + p.b_slots * P.b_bytes;
-    P.stage_off = P.tab_off + (tap_pixels(s.stride, tw.taps, p.mt) * 8 + 127) / 128 * 128;
+    P.stage_off = P.tab_off + p.table_bytes;
+    P.raster = p.raster; P.pitch = p.pitch; P.rows = p.rows; P.pixels = p.pixels; P.sub_px = p.raster ? 128 : 16 * p.pitch;
+    P.row_boxes = p.straddle; P.a_tx = p.pixels * 128 - (p.raster ? (p.pitch - 1) * 128 : 0);
     P.tmem_cols = p.tmem_cols; P.acc_bufs = p.acc_bufs; P.staged = s.staged;
-    for (int t = 0; t < tw.taps; ++t) P.tap_start[t] = tap_start(s.stride, tw.taps, p.mt, t);
+    for (int t = 0; t < tw.taps; ++t) {
+        const int dy = t / 3, dx = t % 3;
+        if (tw.taps == 1) P.tap_start[t] = 0;
+        else if (s.stride == 1) P.tap_start[t] = (p.raster ? p.pitch - 1 : 0) + dy * p.pitch + dx;
+        else    // of the image of the tap's parities; the third row (column) is the second of the odd ones
+            P.tap_start[t] = ((dy == 1 ? 0 : 2) + (dx == 1 ? 0 : 1)) * p.rows * p.pitch + (dy == 2 ? p.pitch : 0) + (dx == 2 ? 1 : 0);
+    }
     auto aligned = [](const void *q, uintptr_t a) { return ((uintptr_t)q & (a - 1)) == 0; };
     P.vec_x = aligned(c.x, 16) && (size_t)tw.c_in * xb % 16 == 0;
+    P.tma = dt != XGEN_F32 && P.vec_x && x_map(tw, s, p, c.x, xm);
     P.vec_y = aligned(c.y, 16) && (size_t)tw.c_out * yb % 16 == 0;
     P.y32 = aligned(c.y, 32) && (size_t)tw.c_out * yb % 32 == 0;
     P.vec_r = c.residual && aligned(c.residual, 16) && (size_t)tw.c_out * rb % 16 == 0;
@@ -1334,7 +1415,7 @@ cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p
         ++na;
     }
     cfg.attrs = at; cfg.numAttrs = na;
-    void *args[2] = {&P, const_cast<CUtensorMap *>(&p.wmap)};
+    void *args[3] = {&P, const_cast<CUtensorMap *>(&p.wmap), &xm};
     e = cudaLaunchKernelExC(&cfg, kern, args);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) count_launch();

@@ -46,8 +46,9 @@ struct TapPlan {
     int pl = 0, stages = 0;      // planes per stage, stages of the whole reduction
     int splits = 1, per_split = 0;   // blocks that share an item's reduction (one cluster), stages of each
     int vh = 0, straddle = 0, segs = 0, row_tiles = 0, items = 0, grid = 0;
-    int a_stages = 0, b_slots = 0, resident = 0;
-    int plane_pitch = 0;
+    int raster = 0, pitch = 0, rows = 0, pixels = 0;     // staged tile: entries of a row, rows (of a parity), entries
+    int a_stages = 0, a_bytes = 0, b_slots = 0, b_bytes = 0, tap_group = 1, resident = 0;
+    int plane_pitch = 0, table_bytes = 0;
     size_t smem = 0;
     int tmem_cols = 0, acc_bufs = 0;
     double cycles = 0;           // what the cost model expects
