@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libpatconv: argument marshalling only.
+"""Thin binding of libpatconv: argument marshalling only (ctypes; the enqueueing calls through a
+small CPython extension, csrc/calls.cpp).
 
 Every step of the layer runs inside the CUDA library.  There is no CPU
 fallback: if the shared library cannot be loaded the import of this module's
@@ -8,6 +9,7 @@ and streams); this module itself needs numpy and ctypes.
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 
 import numpy as np
@@ -118,11 +120,22 @@ class PatconvError(RuntimeError):
 
 
 _lib = None
+_calls = None           # the extension, its calls bound to the loaded library
+
+
+def _bind_calls(L):
+    path = _build.CALLS_PATH if os.path.exists(_build.CALLS_PATH) else _build.build_calls()
+    spec = importlib.util.spec_from_file_location("_calls", path)
+    m = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(m)
+    m.bind(*(ctypes.cast(getattr(L, "xgen_" + f), ctypes.c_void_p).value
+             for f in ("patconv_run", "patconv_run_fused", "blockgemm_run", "dwconv_run")))
+    return m
 
 
 def lib():
     """Load libpatconv.so (building it first if it is missing or stale)."""
-    global _lib
+    global _lib, _calls
     if _lib is None:
         path = os.environ.get("XGEN_PATCONV_LIB") or _build.LIB_PATH    # another build of the library, if named
         if not os.path.exists(path):
@@ -164,6 +177,7 @@ def lib():
             if name not in ("xgen_patconv_free", "xgen_strerror", "xgen_patconv_launch_count", "xgen_blockgemm_free",
                             "xgen_dwconv_free"):
                 getattr(L, name).restype = ctypes.c_int
+        _calls = _bind_calls(L)
         _lib = L
     return _lib
 
@@ -253,16 +267,18 @@ class Packed:
 
     def run(self, x_ptr, n, h, w, bias_ptr, relu, y_ptr, stream=0):
         """Enqueue the layer; all pointers are device addresses (ints)."""
-        _check(lib().xgen_patconv_run(self._h, x_ptr, n, h, w, bias_ptr or None, int(bool(relu)),
-                                      y_ptr, stream or None), "xgen_patconv_run")
+        status = _calls.conv(self._h.value, x_ptr, n, h, w, bias_ptr, relu, y_ptr, stream)
+        if status:
+            raise PatconvError(status, "xgen_patconv_run")
 
     def run_fused(self, x_ptr, n, h, w, bias_ptr, y_ptr, stream=0, relu=False, pool=0, residual_ptr=0,
                   requant_scale_ptr=0, zero_point=0):
         """xgen_patconv_run_fused: the layer with a residual addition, ReLU, a 2x2 max-pool and
         (integer layers) a re-quantisation to uint8 fused behind it; device addresses as ints."""
-        ep = Epilogue(int(bool(relu)), int(pool), residual_ptr or None, requant_scale_ptr or None, int(zero_point))
-        _check(lib().xgen_patconv_run_fused(self._h, x_ptr, n, h, w, bias_ptr or None, ctypes.byref(ep), y_ptr,
-                                            stream or None), "xgen_patconv_run_fused")
+        status = _calls.fused(self._h.value, x_ptr, n, h, w, bias_ptr, y_ptr, stream, relu, pool, residual_ptr,
+                              requant_scale_ptr, zero_point)
+        if status:
+            raise PatconvError(status, "xgen_patconv_run_fused")
 
     def run_static_scratch(self, x_ptr, n, h, w, bias_ptr, relu, y_ptr, splits, stream=0):
         """Like run(), with the channel chunks split `splits` ways and the partial sums kept
@@ -365,9 +381,9 @@ class BlockGemm:
 
     def run(self, x_ptr, m, bias_ptr, relu, y_ptr, stream=0):
         """Enqueue the layer on a CUDA stream; pointers are device addresses (ints)."""
-        _check(lib().xgen_blockgemm_run(self._h, ctypes.c_void_p(x_ptr), int(m), ctypes.c_void_p(bias_ptr or None),
-                                        int(bool(relu)), ctypes.c_void_p(y_ptr), ctypes.c_void_p(stream or None)),
-               "xgen_blockgemm_run")
+        status = _calls.gemm(self._h.value, x_ptr, m, bias_ptr, relu, y_ptr, stream)
+        if status:
+            raise PatconvError(status, "xgen_blockgemm_run")
 
 
 class Depthwise:
@@ -405,6 +421,6 @@ class Depthwise:
 
     def run(self, x_ptr, n, h, w, bias_ptr, relu, y_ptr, stream=0):
         """Enqueue the layer on a CUDA stream; pointers are device addresses (ints)."""
-        _check(lib().xgen_dwconv_run(self._h, ctypes.c_void_p(x_ptr), n, h, w, ctypes.c_void_p(bias_ptr or None),
-                                     int(bool(relu)), ctypes.c_void_p(y_ptr), ctypes.c_void_p(stream or None)),
-               "xgen_dwconv_run")
+        status = _calls.dw(self._h.value, x_ptr, n, h, w, bias_ptr, relu, y_ptr, stream)
+        if status:
+            raise PatconvError(status, "xgen_dwconv_run")

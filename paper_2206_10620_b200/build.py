@@ -4,11 +4,13 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _CSRC = os.path.join(_HERE, "csrc")
 _INC = os.path.join(os.path.dirname(_HERE), "include")
 LIB_PATH = os.path.join(_HERE, "libpatconv.so")
+CALLS_PATH = os.path.join(_HERE, "_calls.abi3.so")     # the enqueueing calls for Python
 _SOURCES = ["patconv.cu", "tapgemm.cu", "blockgemm.cu", "dwconv.cu", "probe.cu", "pack.cpp"]
 _DEPS = _SOURCES + ["patconv_internal.h", "ptx.cuh", "tapgemm.h", "gen_core.py", "gen_blockgemm.py", os.path.join(_INC, "patconv.h"),
                     os.path.join(_INC, "blockgemm.h"), os.path.join(_INC, "dwconv.h")]
@@ -31,6 +33,18 @@ def _mtime(name: str) -> float:
     return os.path.getmtime(os.path.join(_CSRC, name))
 
 
+def build_calls(force: bool = False) -> str:
+    """Compile the CPython extension that marshals the enqueueing calls (host code only)."""
+    src = os.path.join(_CSRC, "calls.cpp")
+    newest = max(os.path.getmtime(f) for f in [src] + [os.path.join(_INC, h) for h in ("patconv.h", "blockgemm.h", "dwconv.h")])
+    if force or not os.path.exists(CALLS_PATH) or os.path.getmtime(CALLS_PATH) < newest:
+        tmp = CALLS_PATH + ".tmp%d" % os.getpid()
+        subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-I", _INC,
+                               "-I", sysconfig.get_paths()["include"], src, "-o", tmp])
+        os.replace(tmp, CALLS_PATH)
+    return CALLS_PATH
+
+
 def _stale() -> bool:
     if not os.path.exists(LIB_PATH):
         return True
@@ -41,6 +55,7 @@ def _stale() -> bool:
 def build(force: bool = False, verbose: bool = False) -> str:
     """Generate the per-pattern code, compile every source that changed to an object of its
     own, and link the shared library."""
+    build_calls(force)
     if not force and not _stale():
         return LIB_PATH
     gen = os.path.join(_CSRC, "core_gen.inc")
