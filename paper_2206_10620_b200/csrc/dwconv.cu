@@ -2,13 +2,8 @@
 //
 // Every channel has one 3x3 kernel that keeps the 4 weights of its pattern.  The layer moves
 // two activations per 4 useful multiply-adds, so HBM binds it: the kernel's job is to read x
-// once and write y once, in whole 16-byte (fp16: 8-byte) pieces of consecutive channels.
-// A thread owns V consecutive channels of a strip of TX output pixels of one row; it walks the
-// three input rows, keeps the strip's (TX-1)*stride + 3 input columns of the current row in
-// registers and adds their products with the row's three taps.  Pruned taps carry weight 0 in
-// the packed table [9][channels]: all nine taps run, because neighbouring channels need the
-// skipped activations anyway and the arithmetic is far from binding.  Neighbouring strips and
-// rows share input through L1/L2.
+// once and write y once, with enough loads in flight and few instructions for an element (see
+// dwconv_kernel).  Pruned taps carry weight 0 in the packed table [9][channels].
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 

@@ -34,7 +34,7 @@
 // warp that issues the matrix instructions, one that fetches weights with tensor copies.  Blocks are
 // persistent; a block keeps its range of filters, and where all of its weights fit they are
 // fetched once.  Items that would leave the GPU idle share one reduction between the blocks of a
-// cluster, which add their sums through distributed shared memory in a fixed order.
+// cluster, which send each other their sums through distributed shared memory and add them in a fixed order.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -74,11 +74,12 @@ struct TapParams {
     int po, pw;                                 // stored extents
     int64_t npix;                               // product: rows of x
     int vh, straddle;                           // virtual rows per image; tiles may cross images
+    uint32_t mg_vh, mg_pitch, mg_rows;          // division by these as a multiplication (div_by)
     int raster, pitch, rows, pixels, sub_px;    // staged tile: entries of a row, rows (of a parity), entries; of the second sub-tile
     int segs, nblk, nt, items, splits, per_split, stages;
     int pl, pl_log, plane_pitch;
     int a_stages, a_bytes, b_slots, resident, b_bytes, tap_group;
-    int b_off, tab_off, stage_off;              // bytes into dynamic shared memory
+    int b_off, tab_off, stage_off, sum_off;     // bytes into dynamic shared memory
     int tmem_cols, acc_bufs, staged;
     int tap_start[9];                           // first staged entry of a tap
     int tma, row_boxes, a_tx;                        // x comes by tensor copies; a copy per staged row
@@ -271,36 +272,88 @@ __device__ __forceinline__ void tap_store1(const TapParams &P, float scale, uint
     else static_cast<uint32_t *>(P.y)[off] = v;
 }
 
-// A warp's 32 pixels x 16 channels, staged as [pixel][kStagePitch] sums: finish and store them, pooled,
-// or with neighbouring lanes on neighbouring elements where rows of y are not whole 16-byte pieces.
-// `pix`: this lane's own pixel of the unpooled result, -1 if there is none; `out`: where it is stored
-// (pooled: of the window whose first pixel it is).
+// A warp's 32 pixels x 16 channels, staged as rows of kStagePitch words: 16 sums, the pixel of the
+// unpooled result (-1: none), where it is stored (pooled: the window whose first pixel it is).  Finish
+// and store them so that neighbouring lanes hold neighbouring elements: where a residual is read (its
+// 16-byte loads by lanes of different pixels touched 32 lines each, 11000 cycles for 128 x 128), and where
+// rows of y are not whole 16-byte pieces.
 template <int DT, bool FUSED>
 __device__ __forceinline__ void tap_emit(const TapParams &P, const uint32_t *st, const uint32_t *s_bias, const float *s_scale,
-                                      int pix, int out, int c_base, int n0, int lane) {
-    constexpr uint32_t kAll = 0xFFFFFFFFu;
+                                         int c_base, int n0, int lane) {
     const bool pool = FUSED && P.pool;
-    const int c = c_base + (lane & 15);          // a lane keeps its channel, half-warps take a pixel each
-    const bool in = c < P.c_out;
-    const uint32_t bias = in ? s_bias[c - n0] : 0u;
-    const float scale = FUSED && in ? s_scale[c - n0] : 0.0f;
-#pragma unroll 2
-    for (int it = 0; it < (pool ? 4 : 16); ++it) {
-        const int jp = 2 * it + (lane >> 4);
-        uint32_t best = 0;
-        int to = -1;
-#pragma unroll 1
-        for (int q = 0; q < (pool ? 4 : 1); ++q) {
-            const int j = pool ? (jp >> 2) * 16 + (jp & 3) * 2 + (q & 1) + (q >> 1) * 8 : jp;
-            const int px = __shfl_sync(kAll, pix, j);
-            const int o = __shfl_sync(kAll, out, j);
-            if (q == 0) to = o;
-            if (px >= 0 && in) {
-                const uint32_t v = tap_affine1<DT, FUSED>(P, bias, st[j * kStagePitch + (lane & 15)], (size_t)px * P.c_out + c);
-                best = q == 0 ? v : tap_max<DT>(best, v);
-            } else to = -1;
+    if constexpr (FUSED) if (P.vec_y && P.vec_r && !pool) {
+        const int c = c_base + (lane & 3) * 4;
+        if (c >= P.c_out) return;
+        const uint4 b = *reinterpret_cast<const uint4 *>(s_bias + (c - n0));
+        const float4 sc = *reinterpret_cast<const float4 *>(s_scale + (c - n0));
+        const uint32_t *const row0 = st + (lane >> 2) * kStagePitch;
+        uint4 res[4];
+        int px[4];
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            px[it] = (int)row0[it * 8 * kStagePitch + 16];
+            const size_t off = (size_t)max(px[it], 0) * P.c_out + c;
+            if (DT == XGEN_F16_F32ACC) {
+                const uint2 r = __ldg(reinterpret_cast<const uint2 *>(static_cast<const __half *>(P.residual) + off));
+                const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&r.x)), g = __half22float2(*reinterpret_cast<const __half2 *>(&r.y));
+                res[it] = make_uint4(__float_as_uint(f.x), __float_as_uint(f.y), __float_as_uint(g.x), __float_as_uint(g.y));
+            } else res[it] = __ldg(reinterpret_cast<const uint4 *>(static_cast<const uint32_t *>(P.residual) + off));
         }
-        if (to >= 0) tap_store1<DT, FUSED>(P, scale, best, (size_t)to * P.c_out + c);
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            const uint4 a = *reinterpret_cast<const uint4 *>(row0 + it * 8 * kStagePitch + (lane & 3) * 4);
+            uint32_t v[4] = {a.x, a.y, a.z, a.w};
+            if (DT == XGEN_I8_I32) { v[0] += b.x + res[it].x; v[1] += b.y + res[it].y; v[2] += b.z + res[it].z; v[3] += b.w + res[it].w; }
+            else {
+                add2(v[0], v[1], b.x, b.y); add2(v[2], v[3], b.z, b.w);
+                add2(v[0], v[1], res[it].x, res[it].y); add2(v[2], v[3], res[it].z, res[it].w);
+            }
+            if (P.relu) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = tap_max<DT>(v[i], 0u);
+            }
+            if (px[it] < 0) continue;
+            const size_t off = (size_t)px[it] * P.c_out + c;
+            if (DT == XGEN_I8_I32 && P.rq_scale)
+                *reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(P.y) + off) =
+                    pack_codes(tap_level(P, v[0], sc.x), tap_level(P, v[1], sc.y), tap_level(P, v[2], sc.z), tap_level(P, v[3], sc.w));
+            else if (DT == XGEN_F16_F32ACC) {
+                const __half2 f = __floats2half2_rn(__uint_as_float(v[0]), __uint_as_float(v[1])), g = __floats2half2_rn(__uint_as_float(v[2]), __uint_as_float(v[3]));
+                *reinterpret_cast<uint2 *>(static_cast<__half *>(P.y) + off) = make_uint2(*reinterpret_cast<const uint32_t *>(&f), *reinterpret_cast<const uint32_t *>(&g));
+            } else *reinterpret_cast<uint4 *>(static_cast<uint32_t *>(P.y) + off) = make_uint4(v[0], v[1], v[2], v[3]);
+        }
+        return;
+    }
+    const int c = c_base + (lane & 15);          // a lane keeps its channel, half-warps take a pixel each
+    if (c >= P.c_out) return;
+    const uint32_t bias = s_bias[c - n0];
+    const float scale = FUSED ? s_scale[c - n0] : 0.0f;
+    if (!pool) {
+#pragma unroll 4
+        for (int it = 0; it < 16; ++it) {
+            const uint32_t *const row = st + (2 * it + (lane >> 4)) * kStagePitch;
+            const int px = (int)row[16];
+            if (px >= 0) {
+                const size_t off = (size_t)px * P.c_out + c;
+                tap_store1<DT, FUSED>(P, scale, tap_affine1<DT, FUSED>(P, bias, row[lane & 15], off), off);
+            }
+        }
+        return;
+    }
+    if constexpr (FUSED)
+#pragma unroll 1
+    for (int it = 0; it < 4; ++it) {
+        const int jp = 2 * it + (lane >> 4);
+        const uint32_t *const row = st + ((jp >> 2) * 16 + (jp & 3) * 2) * kStagePitch;
+        if ((int)row[16] < 0) continue;
+        uint32_t best = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t *const r = row + ((q & 1) + (q >> 1) * 8) * kStagePitch;
+            const uint32_t v = tap_affine1<DT, FUSED>(P, bias, r[lane & 15], (size_t)(int)r[16] * P.c_out + c);
+            best = q == 0 ? v : tap_max<DT>(best, v);
+        }
+        tap_store1<DT, FUSED>(P, scale, best, (size_t)(int)row[17] * P.c_out + c);
     }
 }
 
@@ -487,6 +540,9 @@ __device__ __forceinline__ void sts128(uint32_t dst, const uint4 &v) {
     asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
+// n / d with the host's multiplier (0: a range for which none is exact).
+__device__ __forceinline__ int div_by(int n, int d, uint32_t mg) { return mg ? (int)__umulhi((uint32_t)n, mg) : n / d; }
+
 // Position of a block's work: item = (tile or pair of tiles, range of filters).  The second tile of the
 // last pair may lie past the end: all of its pixels are invalid.
 struct TapItem {
@@ -501,7 +557,7 @@ template <int MT, bool PAIR> __device__ __forceinline__ TapItem tap_item(const T
     if (PAIR) tile = 2 * tile + side;
     if (P.raster) {
         t.q0 = tile * 128 * MT;
-        t.v0 = t.q0 / P.pitch;
+        t.v0 = div_by(t.q0, P.pitch, P.mg_pitch);
         t.ox0 = t.q0 - t.v0 * P.pitch;
     } else {
         const int rt = tile / P.segs;
@@ -520,10 +576,10 @@ template <int STRIDE> __device__ __forceinline__ TapRow tap_row(const TapParams 
     if (P.straddle) {
         const int v = t.v0 + step;
         if (v < 0) return TapRow{0, -1};
-        r.img = v / P.vh;
+        r.img = div_by(v, P.vh, P.mg_vh);
         r.y = v - r.img * P.vh;
     } else {
-        r.img = t.v0 / P.vh;
+        r.img = div_by(t.v0, P.vh, P.mg_vh);
         r.y = t.v0 - r.img * P.vh + step;
     }
     if (STRIDE == 2) r.y = 2 * r.y - odd;
@@ -535,10 +591,10 @@ template <int STRIDE, int TAPS> __device__ __forceinline__ int tap_source(const 
     if (TAPS == 1) return (int64_t)t.v0 * 8 + p < P.npix ? t.v0 * 8 + p : -1;
     if (P.raster) p -= P.pitch - 1 - t.ox0;       // (all tiles keep their first output entry at the same place)
     if (p < 0) return -1;
-    int i = p / P.pitch, ix = p - i * P.pitch, odd = 0;
+    int i = div_by(p, P.pitch, P.mg_pitch), ix = p - i * P.pitch, odd = 0;
     if (STRIDE == 1) ix += (P.raster ? 0 : t.ox0) - 1;
     else {
-        const int region = i / P.rows;
+        const int region = div_by(i, P.rows, P.mg_rows);
         i -= region * P.rows;
         odd = region >> 1;
         ix = 2 * (t.ox0 + ix) - (region & 1);
@@ -557,13 +613,13 @@ template <int TAPS> __device__ __forceinline__ TapPixel tap_pixel(const TapParam
     }
     int v, ox;
     if (P.raster) {
-        v = (t.q0 + m) / P.pitch;
+        v = div_by(t.q0 + m, P.pitch, P.mg_pitch);
         ox = t.q0 + m - v * P.pitch;
     } else {
         v = t.v0 + (m >> 3);
         ox = t.ox0 + (m & 7);
     }
-    const int img = v / P.vh, oy = v - img * P.vh;
+    const int img = div_by(v, P.vh, P.mg_vh), oy = v - img * P.vh;
     if (img >= P.n || oy >= P.ho || ox >= P.wo) return TapPixel{-1, -1};
     const int pix = (img * P.ho + oy) * P.wo + ox;
     return TapPixel{pix, P.pool ? (img * P.po + oy / 2) * P.pw + ox / 2 : pix};
@@ -619,7 +675,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
     if (warp == kEpiWarps + kProdWarps) tmem_alloc<PAIR>(smem_u32(&s_tmem), (uint32_t)P.tmem_cols);
     tc_fence_before();
     __syncthreads();
-    if (PAIR) cluster_meet();            // the other block's barriers stand
+    if (csize > 1) cluster_meet();       // the other blocks run, their barriers stand
     tc_fence_after();
     const uint32_t tmem = s_tmem;
 
@@ -633,8 +689,8 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
     const uint32_t a_part = (uint32_t)P.pl * P.plane_pitch;       // fp32: bytes of one part of a stage
 
     if (warp >= kEpiWarps && warp < kEpiWarps + kProdWarps) {
-        asm volatile("griddepcontrol.wait;" ::: "memory");
         if (!kF32 && P.tma) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
             if (warp == kEpiWarps) {
                 // ---- x by tensor copies, zeros outside the image -------------------------------
                 if (elect_one()) {
@@ -700,6 +756,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 int *const pix = reinterpret_cast<int *>(smem + P.tab_off) + (par ? P.pixels : 0);
                 for (int p = pt; p < P.pixels; p += kProdThreads) pix[p] = tap_source<STRIDE, TAPS>(P, t, p);
                 asm volatile("bar.sync 1, %0;" ::"n"(kProdThreads) : "memory");
+                if (item == item0) asm volatile("griddepcontrol.wait;" ::: "memory");
                 for (int ks = k0; ks < k1; ++ks) {
                     ok = wait(a_empty(s), ph);
                     if (!ok) break;
@@ -887,10 +944,16 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
         const int chunks = P.nt / 32;
         const uint32_t lanes = (uint32_t)quarter << 21;
         const int m = quarter * 32 + lane;                       // pixel of the 128
-        // sums on their way out where they do not go straight from their lanes: the warp's 32 pixels x 16
-        // filters, or (split) the whole tile
-        uint32_t *const st = reinterpret_cast<uint32_t *>(smem + (P.splits > 1 ? 0 : P.stage_off + warp * kStageBytes));
-        uint32_t *const st_own = st + (P.splits > 1 ? (sub * 128 + m) * (P.nt + 4) : lane * kStagePitch);
+        // Sums on their way out where they do not go straight from their lanes: the warp's 32 pixels x 16
+        // filters, or (split) to the block of the cluster that adds up this pixel's, [source][pixel][filter].
+        uint32_t *const st = reinterpret_cast<uint32_t *>(smem + P.stage_off + warp * kStageBytes);
+        uint32_t *const st_own = st + lane * kStagePitch;
+        uint32_t far = 0;
+        if (P.splits > 1) {
+            const int unit = sub * 8 + m / 16, adder = unit % P.splits, units = (8 * MT + P.splits - 1) / P.splits;
+            far = cluster_addr(sbase + P.sum_off + (uint32_t)((rank * units + unit / P.splits) * 16 + m % 16) * (P.nt + 4) * 4,
+                               (uint32_t)(PAIR ? 2 * adder + side : adder));
+        }
         int buf = 0;
         uint32_t ph = 0;
         bool ok = true;
@@ -898,24 +961,25 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             const TapItem t = tap_item<MT, PAIR>(P, item, side);
             const TapPixel at = tap_pixel<TAPS>(P, t, sub * 128 + m);
             const int pix = at.pix, out = at.out;
-            auto put = [&](const uint32_t *r, int n, int at) {
-#pragma unroll
-                for (int q = 0; q < n / 4; ++q)
-                    *reinterpret_cast<uint4 *>(st_own + at + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
-            };
+            if (P.staged && P.splits == 1) { st_own[16] = (uint32_t)pix; st_own[17] = (uint32_t)out; }
             // 32 sums of this lane's pixel, from column c of the tile on
             auto finish = [&](uint32_t (&r)[32], int c) {
-                if (P.splits > 1) put(r, 32, c);
-                else if (n0 + c >= P.c_out) return;
+                if (P.splits > 1) {
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) sts_cluster(far + (uint32_t)(c + 4 * q) * 4, r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+                } else if (n0 + c >= P.c_out) return;
                 else if (!P.staged) tap_direct<DT, FUSED>(P, s_bias, s_scale, r, pix, out, n0 + c, n0);
                 else {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         __syncwarp();
-                        put(r + 16 * h, 16, 0);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            *reinterpret_cast<uint4 *>(st_own + 4 * q) = make_uint4(r[16 * h + 4 * q], r[16 * h + 4 * q + 1], r[16 * h + 4 * q + 2], r[16 * h + 4 * q + 3]);
                         __syncwarp();
-                        tap_emit<DT, FUSED>(P, st, s_bias, s_scale, pix, out, n0 + c + 16 * h, n0, lane);
+                        tap_emit<DT, FUSED>(P, st, s_bias, s_scale, n0 + c + 16 * h, n0, lane);
                     }
+                    __syncwarp();
                 }
             };
             auto release = [&]() {
@@ -969,7 +1033,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
         }
     }
 
-    // ---- split items: the blocks of the cluster add their sums, 16 pixels at a time ---------
+    // ---- split items: every block adds up its share of the pixels, in the order of the sources -------
     if (P.splits > 1) {
         __syncwarp();
         cluster_meet();
@@ -979,29 +1043,29 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             const int groups = P.nt / 8, pitch = (P.nt + 4) * 4;
             const bool pool = FUSED && P.pool;
             // units of two rows of eight pixels go round the blocks; a thread takes 8 channels of one (pooled) pixel
-            const int units = (8 * MT - rank + P.splits - 1) / P.splits, per_unit = (pool ? 4 : 16) * groups;
+            const int units_all = (8 * MT + P.splits - 1) / P.splits, units = (8 * MT - rank + P.splits - 1) / P.splits;
+            const int per_unit = (pool ? 4 : 16) * groups, source = units_all * 16 * pitch;
 #pragma unroll 1
             for (int w = tid; w < units * per_unit; w += kAdders) {
                 const int u = w / per_unit, wu = w - u * per_unit, row = wu / groups, g = wu - row * groups;
-                const int c0 = n0 + 8 * g;
-                const int m0 = 16 * (rank + u * P.splits) + (pool ? 2 * row : row);
-                const TapPixel px = tap_pixel<TAPS>(P, t, m0);
+                const int c0 = n0 + 8 * g, in_unit = pool ? 2 * row : row;
+                const TapPixel px = tap_pixel<TAPS>(P, t, 16 * (rank + u * P.splits) + in_unit);
                 if (px.pix < 0 || c0 >= P.c_out) continue;
                 uint32_t best[8];
 #pragma unroll 1
                 for (int q = 0; q < (pool ? 4 : 1); ++q) {
-                    const uint32_t own = sbase + (uint32_t)((m0 + (q & 1) + (q >> 1) * 8) * pitch + g * 32);
+                    const unsigned char *own = smem + P.sum_off + (u * 16 + in_unit + (q & 1) + (q >> 1) * 8) * pitch + g * 32;
                     uint32_t v8[8];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) v8[i] = 0;
 #pragma unroll 4
-                    for (int r = 0; r < P.splits; ++r) {
-                        const uint32_t far = cluster_addr(own, (uint32_t)(PAIR ? 2 * r + side : r));
-                        const uint4 a = lds_cluster(far), b = lds_cluster(far + 16);
-                        const uint32_t ab[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            v8[i] = DT == XGEN_I8_I32 ? v8[i] + ab[i] : __float_as_uint(__uint_as_float(v8[i]) + __uint_as_float(ab[i]));
+                    for (int r = 0; r < P.splits; ++r, own += source) {
+                        const uint4 a = *reinterpret_cast<const uint4 *>(own), b = *reinterpret_cast<const uint4 *>(own + 16);
+                        if (DT == XGEN_I8_I32) {
+                            v8[0] += a.x; v8[1] += a.y; v8[2] += a.z; v8[3] += a.w; v8[4] += b.x; v8[5] += b.y; v8[6] += b.z; v8[7] += b.w;
+                        } else {
+                            add2(v8[0], v8[1], a.x, a.y); add2(v8[2], v8[3], a.z, a.w); add2(v8[4], v8[5], b.x, b.y); add2(v8[6], v8[7], b.z, b.w);
+                        }
                     }
                     tap_affine<DT, FUSED, 8>(P, s_bias, v8, px.pix + (q & 1) + (q >> 1) * P.wo, true, c0, n0);
 #pragma unroll
@@ -1012,7 +1076,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
         }
     }
     __syncwarp();
-    if (csize > 1) cluster_meet();       // nobody leaves while the others may still use its memory
+    if (PAIR) cluster_meet();            // nobody leaves while the other may still use its memory
     tc_fence_before();
     __syncthreads();
     if (warp == kEpiWarps + kProdWarps) tmem_free<PAIR>(tmem, (uint32_t)P.tmem_cols);
@@ -1277,7 +1341,8 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                         p.grid = p.items * sp * ways;
                         waves = (p.items + cl - 1) / cl;
                     }
-                    const size_t tables = p.table_bytes + (sp == 1 && s.staged ? epi_warps(dt) * kStageBytes : 0);
+                    const size_t tables = p.table_bytes + (sp > 1 ? (size_t)sp * ((8 * mt + sp - 1) / sp) * 16 * (p.nt + 4) * 4
+                                                                  : s.staged ? (size_t)epi_warps(dt) * kStageBytes : 0);
                     const int64_t uses = (sp == 1 ? waves : 1) * p.per_split;      // stages one block goes through
                     // Shared memory: two tiles of x (more for a plain product, whose stages are short), the rest
                     // weights, by three taps if at least three such slots fit.
@@ -1297,7 +1362,6 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     }
                     if (!fits) continue;
                     p.smem = (size_t)p.a_stages * p.a_bytes + (size_t)p.b_slots * p.b_bytes + tables;
-                    if (sp > 1) p.smem = std::max(p.smem, (size_t)mt * 128 * (p.nt + 4) * 4);
                     if (p.smem > (size_t)kTapSmemMax) continue;
                     p.acc_bufs = dt == XGEN_F32 || 2 * mt * p.nt <= 512 ? 2 : 1;
                     const int cols = dt == XGEN_F32 ? 4 * p.nt : p.acc_bufs * mt * p.nt;
@@ -1317,7 +1381,7 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     const double item = p.per_split * stage;
                     double c = 3500.0 + (p.pair ? 2500.0 : 0.0);
                     if (sp == 1) c += waves * std::max(item, p.acc_bufs == 2 ? out : 0.0) + (p.acc_bufs == 2 ? out : waves * out);
-                    else c += waves * (item + 3500.0 + 40.0 * sp + mt * 128.0 * p.nt * 4 / 48.0 + out / sp);
+                    else c += waves * (item + 3500.0 + 100.0 * sp + mt * 128.0 * p.nt * 4 / 64.0 + out / sp);
                     if (c < best.cycles * 0.999) { best = p; best.cycles = c; }
                 }
             }
@@ -1375,8 +1439,17 @@ cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p
     P.a_bytes = p.a_bytes;
     P.b_off = p.a_stages * p.a_bytes;
     P.tab_off = P.b_off + p.b_slots * P.b_bytes;
-    P.stage_off = P.tab_off + p.table_bytes;
+    P.stage_off = P.sum_off = P.tab_off + p.table_bytes;       // (the one or the other)
     P.raster = p.raster; P.pitch = p.pitch; P.rows = p.rows; P.pixels = p.pixels; P.sub_px = p.raster ? 128 : 16 * p.pitch;
+    {
+        // exact for n < 2^32 / d: the largest n are the rows (raster entries) of all tiles
+        auto magic = [](int64_t most, int d) { return d > 1 && (most + 1) * d < (1ll << 32) ? (uint32_t)((1ull << 32) / (uint64_t)d + 1) : 0u; };
+        const int64_t last_tile = (int64_t)(p.items / p.nblk) * (p.pair ? 2 : 1) * p.mt;
+        const int64_t rows_all = p.raster ? last_tile * 128 / p.pitch + 64 : (int64_t)(p.row_tiles + 2) * 16 * p.mt + 64;
+        P.mg_pitch = magic(p.raster ? last_tile * 128 + 512 : p.pixels, p.pitch);
+        P.mg_vh = magic(rows_all, p.vh);
+        P.mg_rows = magic(p.pixels, p.rows);
+    }
     P.row_boxes = p.straddle; P.a_tx = p.pixels * 128 - (p.raster ? (p.pitch - 1) * 128 : 0);
     P.tmem_cols = p.tmem_cols; P.acc_bufs = p.acc_bufs; P.staged = s.staged;
     for (int t = 0; t < tw.taps; ++t) {

@@ -35,7 +35,7 @@ struct TapShape {
     int stride = 1;
     int64_t rows = 0;            // product: rows of x (0 for a convolution)
     bool pool = false;
-    bool staged = false;         // rows of y are not whole 16-byte pieces: results pass through shared memory
+    bool staged = false;         // results pass through shared memory: rows of y are not whole 16-byte pieces, or a residual
 };
 
 // How the problem is cut up (tap_choose).
