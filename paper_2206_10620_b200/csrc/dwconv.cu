@@ -8,8 +8,10 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cstdint>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -232,6 +234,23 @@ static const void *kernel_for(xgen_dtype dt, int stride, int v) {
     return dt == XGEN_F32 ? kernel_dt<XGEN_F32>(stride, v) : kernel_dt<XGEN_F16_F32ACC>(stride, v);
 }
 
+// Blocks of the kernel that the device holds at once (asked for once per kernel and device).
+static int resident_blocks(const void *kern, int device) {
+    static std::mutex mu;
+    static std::vector<std::array<intptr_t, 3>> known;
+    std::lock_guard<std::mutex> lock(mu);
+    for (auto &k : known)
+        if (k[0] == (intptr_t)kern && k[1] == device) return (int)k[2];
+    int sms = 148, per_sm = 4;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, 0) != cudaSuccess || per_sm < 1) {
+        cudaGetLastError();
+        per_sm = 4;
+    }
+    known.push_back({(intptr_t)kern, device, sms * per_sm});
+    return sms * per_sm;
+}
+
 static float half_bits_to_float(uint16_t h) {
     const uint32_t sign = (uint32_t)(h >> 15) << 31;
     const int exp = (h >> 10) & 0x1f;
@@ -332,15 +351,22 @@ xgen_status xgen_dwconv_run(const xgen_dwconv_packed *h, const void *x, int32_t 
     P.relu = relu ? 1 : 0;
     P.cvs = h->c / v;
     P.strips = (wo + tx - 1) / tx;
-    // A piece of rows loads one or two rows besides its own, so pieces are as long as leaves kThreads
-    // threads, at least four rows; a small problem is cut to single rows, where the latency counts.
-    constexpr int64_t kThreads = 148 * 2048;
+    const void *const kern = kernel_for(h->dtype, h->stride, v);
+    // Pieces of an image's rows: a piece loads (and at stride 1 adds up) two rows besides its own and costs
+    // about two more to start, so pieces want to be long; but the blocks run in waves of what the GPU holds,
+    // and one that is partly filled costs as much as a full one.
     const int64_t columns = (int64_t)n * P.strips * P.cvs;
-    int rows = (int)std::max<int64_t>(1, columns * ho / kThreads);
-    if (rows < 4) rows = columns * ho / 4 >= kThreads / 4 ? 4 : columns * ho / 2 >= kThreads / 4 ? 2 : 1;
-    rows = std::min(rows, ho);
-    P.segs = (ho + rows - 1) / rows;
-    P.seg_rows = (ho + P.segs - 1) / P.segs;
+    const int at_once = resident_blocks(kern, h->device);
+    double best = 1e30;
+    auto weigh = [&](int rows) {
+        const int segs = (ho + rows - 1) / rows;
+        rows = (ho + segs - 1) / segs;
+        const int64_t waves = ((columns * segs + 127) / 128 + at_once - 1) / at_once;
+        const double t = (double)waves * (rows + 4);
+        if (t < best * 0.999) { best = t; P.segs = segs; P.seg_rows = rows; }
+    };
+    for (int segs = 1; segs <= 12 && segs <= ho; ++segs) weigh((ho + segs - 1) / segs);
+    for (int rows : {8, 6, 4, 3, 2, 1}) if (rows < ho / 12) weigh(rows);
     const int64_t threads = columns * P.segs;
     if (threads > 0x7FFFFFFFLL) return XGEN_ERR_SHAPE;
     P.threads = (unsigned)threads;
@@ -356,7 +382,7 @@ xgen_status xgen_dwconv_run(const xgen_dwconv_packed *h, const void *x, int32_t 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    if (cudaLaunchKernelExC(&cfg, kernel_for(h->dtype, h->stride, v), args) != cudaSuccess) {
+    if (cudaLaunchKernelExC(&cfg, kern, args) != cudaSuccess) {
         cudaGetLastError();
         st = XGEN_ERR_CUDA;
     } else patconv::count_launch();

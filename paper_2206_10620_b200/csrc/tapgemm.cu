@@ -825,9 +825,11 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
     } else if (warp == kEpiWarps + kProdWarps) {
         // ---- matrix instructions: one thread, which also waits.  A wait that gives up is not looked at:
         // nothing per-thread may steer these loops, or every operand is moved to the uniform registers
-        // anew; all later waits then return at once.  Taps are unrolled, a few share a barrier, and the
-        // next barrier is looked at before the instructions of this one are issued: in a rolled loop with
-        // a wait of its own a tap costs 350 cycles, its four instructions of 128 x 128 x 16 take 256. --
+        // anew; all later waits then return at once.  Three taps are unrolled and share a barrier, and
+        // the next barrier is looked at before the instructions of this one are issued: in a rolled loop
+        // with a wait of its own a tap costs 350 cycles, its four instructions of 128 x 128 x 16 take 256.
+        // fp32 has instructions enough in a tap to roll the rest, and less code to fetch at the start of a
+        // short launch. ------------------------------------------------------------------------------
         if (side == 0 && elect_one()) {
             const uint32_t b_rows = (uint32_t)P.nt / (PAIR ? 2 : 1);         // filters whose weights this block holds
             const uint32_t b_tap = PARTS * b_rows;                           // 16-byte units from here on
@@ -851,18 +853,21 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     const uint32_t d = tmem + (uint32_t)buf * (uint32_t)(MT * P.nt);
                     const uint32_t dc = d + 2u * P.nt;      // fp32: the small products (two buffers behind the two of the sums)
                     uint32_t bt = bs;
+#pragma unroll (kF32 ? 1 : 3)
+                    for (int t0 = 0; t0 < TAPS; t0 += 3) {
 #pragma unroll
-                    for (int tap = 0; tap < TAPS; ++tap) {
-                        if ((P.tap_group == 1 || tap % 3 == 0) && !ready)
+                    for (int t1 = 0; t1 < (TAPS == 1 ? 1 : 3); ++t1) {
+                        const int tap = t0 + t1;
+                        if ((P.tap_group == 1 || t1 == 0) && !ready)
                             mbar_wait_long<PAIR>(b_full(b), P.resident ? 0u : phb, &s_abort, P.status, P.wait_us);
-                        const bool last = P.tap_group == 1 || tap % 3 == 2;
+                        const bool last = P.tap_group == 1 || t1 == 2;
                         if (last) {                         // (of its slot: look at the next one)
                             const bool wrap = b + 1 == P.b_slots;
                             ready = mbar_try<PAIR>(b_full(wrap ? 0 : b + 1), P.resident ? 0u : wrap ? phb ^ 1u : phb);
                         }
                         const uint32_t at = as + (uint32_t)P.tap_start[tap] * a_px;
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) {
+                        for (int kk = 0; kk < (kF32 && TAPS == 9 ? 2 : 4); ++kk) {
                             if (kk < kk_n) {
                                 const uint32_t ak = at + kk * a_k, bk = bt + kk * b_k;
                                 const uint32_t first_s = tap > 0 || kk > 0 ? 1u : 0u;       // 0: the first of the stage
@@ -890,6 +895,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                             if (++b == P.b_slots) { b = 0; phb ^= 1u; bs = (uint32_t)b0; }
                             bt = bs;
                         }
+                    }
                     }
                     tc_commit<PAIR>(a_empty(s), both);
                     as += a_step;
@@ -970,14 +976,16 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 } else if (n0 + c >= P.c_out) return;
                 else if (!P.staged) tap_direct<DT, FUSED>(P, s_bias, s_scale, r, pix, out, n0 + c, n0);
                 else {
-#pragma unroll
+#pragma unroll 1
                     for (int h = 0; h < 2; ++h) {
                         __syncwarp();
 #pragma unroll
                         for (int q = 0; q < 4; ++q)
-                            *reinterpret_cast<uint4 *>(st_own + 4 * q) = make_uint4(r[16 * h + 4 * q], r[16 * h + 4 * q + 1], r[16 * h + 4 * q + 2], r[16 * h + 4 * q + 3]);
+                            *reinterpret_cast<uint4 *>(st_own + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
                         __syncwarp();
                         tap_emit<DT, FUSED>(P, st, s_bias, s_scale, n0 + c + 16 * h, n0, lane);
+#pragma unroll
+                        for (int i = 0; i < 16; ++i) r[i] = r[16 + i];
                     }
                     __syncwarp();
                 }
@@ -1013,9 +1021,12 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     }
                     release();
                 }
+#pragma unroll 1
+                for (int q = group; q < chunks && ok; q += kGroups) {
+                    finish(sum[0], 32 * q);
 #pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    if (group + h * kGroups < chunks && ok) finish(sum[h], 32 * (group + h * kGroups));
+                    for (int i = 0; i < 32; ++i) sum[0][i] = sum[1][i];
+                }
             } else {
                 ok = wait(acc_full(buf), ph);
                 tc_fence_after();
@@ -1366,20 +1377,20 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     p.acc_bufs = dt == XGEN_F32 || 2 * mt * p.nt <= 512 ? 2 : 1;
                     const int cols = dt == XGEN_F32 ? 4 * p.nt : p.acc_bufs * mt * p.nt;
                     for (p.tmem_cols = 32; p.tmem_cols < cols;) p.tmem_cols *= 2;
-                    // Cycles of a stage: the matrix instructions (nt / 2 each, 45 to issue one), or what they and
-                    // the copies move through shared memory at 128 bytes a cycle (128 rows of x, the block's
-                    // filters), or what comes from L2.  A slot of weights costs 40 cycles besides, a stage 250.
+                    // Cycles of a stage: the matrix instructions (nt / 2 each; 46 to issue one and 90 for a tap), or
+                    // what they and the copies move through shared memory at 128 bytes a cycle (128 rows of x,
+                    // the block's filters), or what comes from L2.  A pair starts and ends 4000 cycles later.
                     const double kk = (double)tw.planes / p.stages / 2, taps = tw.taps;
                     const double b_stage = taps * kk * 2 * parts * p.nt * 16.0 / ways, b_moved = p.resident && sp == 1 ? b_stage / waves : b_stage;
                     const double x_moved = (double)pixels * kk * 2 * cpp * xb, a_stage = (double)p.a_bytes * (swizzled ? 1 : 2);
-                    const double instr = taps * kk * mt * prod;
-                    const double mma = instr * std::max(p.nt / 2.0, 45.0);
+                    const double per_tap = kk * mt * prod, instr = taps * per_tap;
+                    const double mma = taps * std::max(per_tap * p.nt / 2.0, 90.0 + 46.0 * per_tap);
                     const double shared = (instr * (4096.0 + p.nt * 32.0 / ways) + b_moved + a_stage) / 128.0;
                     const double move = (x_moved + b_moved) / 40.0 + (copied && p.straddle ? 60.0 * p.rows * (s.stride == 1 ? 1 : 4) : 0.0) * 0.5;
                     const double stage = std::max(std::max(mma, shared), move) + 250.0 + 40.0 * taps / p.tap_group;
                     const double out = (double)mt * 128 * p.nt * yb / 24.0;
                     const double item = p.per_split * stage;
-                    double c = 3500.0 + (p.pair ? 2500.0 : 0.0);
+                    double c = 3500.0 + (p.pair ? 4000.0 : 0.0);
                     if (sp == 1) c += waves * std::max(item, p.acc_bufs == 2 ? out : 0.0) + (p.acc_bufs == 2 ? out : waves * out);
                     else c += waves * (item + 3500.0 + 100.0 * sp + mt * 128.0 * p.nt * 4 / 64.0 + out / sp);
                     if (c < best.cycles * 0.999) { best = p; best.cycles = c; }
