@@ -201,32 +201,25 @@ xgen_status xgen_patconv_run_fused(const xgen_patconv_packed *packed, const void
 
 /*
  * (The paper has no counterpart to this entry point; it exists for callers of this
- * library.)  Run the layer with its input channels split over `splits` groups of thread
- * blocks, like a shape prepared with xgen_patconv_plan, but keep the partial sums in a
- * fixed array inside the library instead of a workspace from cudaMalloc.  It is meant for
- * callers that must not allocate device memory where they call us: code running under a
+ * library.)  Run the layer without any memory besides the caller's tensors and what the
+ * handle holds since it was packed: a layer whose input channels are split over groups of
+ * thread blocks keeps the partial sums in their shared memory, never in a workspace from
+ * cudaMalloc, whatever the handle was planned for.  It is meant for callers that must not
+ * allocate device memory where they call us: code running under a
  * memory budget that was handed out up front, inside another framework's allocator
  * scope, or on a path where an allocation (which may synchronise the device) is not
  * allowed.  Neither this call nor anything it uses allocates or frees device memory.
  *
- *   splits   how many ways to split the channel chunks (>= 1; clamped to the number of
- *            chunks); more splits put more thread blocks to work on layers with few
- *            output pixels, and cost splits x 4 bytes of scratch per output element
+ *   splits   how many ways the caller expects the channel chunks to be split (>= 1; clamped
+ *            to the number of chunks); the library splits as it finds best
  *   others   exactly as xgen_patconv_run; the caller still owns x, bias and y
  *
  * Limit: s x n*ho*wo*c_out x 4 bytes must not exceed
- * XGEN_PATCONV_STATIC_SCRATCH_BYTES, where s is the number of splits that actually get
+ * XGEN_PATCONV_STATIC_SCRATCH_BYTES, where s is the number of splits that would actually get
  * channel chunks (splits after clamping, rounded so that every split has the same
  * number of chunks; s = 1 needs no scratch); beyond that the call returns XGEN_ERR_SHAPE and
- * launches nothing (with XGEN_PATCONV_LOG set, the reason goes to stderr).  The array is
- * part of the loaded library: every GPU that uses the library holds those bytes until
- * the process exits.
- * The first call on a device looks up the array's device address (once per device, with
- * that device made current); make that first call outside any stream capture.
- * All calls share the one array and nothing in it has to start at zero: every element a
- * call reads it has written itself.  For the same reason two calls whose kernels may
- * overlap on the GPU (different streams, no dependency between them) race on it; put
- * such calls on one stream or order them with events.
+ * launches nothing (with XGEN_PATCONV_LOG set, the reason goes to stderr).
+ * Calls share nothing but the handle, so they may overlap on different streams.
  * Errors: INVALID_ARG, SHAPE, CUDA, as xgen_patconv_run, plus SHAPE for the limit.
  */
 #define XGEN_PATCONV_STATIC_SCRATCH_BYTES (8u << 20)

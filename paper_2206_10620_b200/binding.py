@@ -281,9 +281,9 @@ class Packed:
             raise PatconvError(status, "xgen_patconv_run_fused")
 
     def run_static_scratch(self, x_ptr, n, h, w, bias_ptr, relu, y_ptr, splits, stream=0):
-        """Like run(), with the channel chunks split `splits` ways and the partial sums kept
-        in the library's built-in scratch array: no device memory is allocated.  For callers
-        that may not allocate where they call; see the header for the size limit."""
+        """Like run(), whatever the handle was planned for, without any device memory besides the
+        caller's and the handle's: for callers that may not allocate where they call; see the
+        header for the size limit."""
         _check(lib().xgen_patconv_run_static_scratch(self._h, x_ptr, n, h, w, bias_ptr or None,
                                                      int(bool(relu)), y_ptr, int(splits), stream or None),
                "xgen_patconv_run_static_scratch")

@@ -441,6 +441,17 @@ static const void *kernel_for(xgen_dtype dt, int ks) {
                                                                                       : (const void *)blockgemm_kernel<XGEN_F16_F32ACC, 8>;
 }
 
+// The command stream's device copy: for layers whose caller named warps_per_block (and where the driver
+// cannot encode the matrix path's tensor maps).
+static xgen_status upload_stream(xgen_blockgemm_packed *h) {
+    const Host &H = h->host;
+    const size_t sb = std::max<size_t>(H.stream.size() * 4, 16), gb = H.seg_off.size() * 4;
+    if (cudaMalloc(&h->d_stream, sb) != cudaSuccess || cudaMalloc(&h->d_seg, gb) != cudaSuccess) return XGEN_ERR_ALLOC;
+    if ((!H.stream.empty() && cudaMemcpy(h->d_stream, H.stream.data(), H.stream.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) ||
+        cudaMemcpy(h->d_seg, H.seg_off.data(), gb, cudaMemcpyHostToDevice) != cudaSuccess) return XGEN_ERR_CUDA;
+    return XGEN_OK;
+}
+
 // The matrix path's plan for a row count, from the handle's small cache or made now.
 static bool tap_plan_of(xgen_blockgemm_packed *h, const patconv::TapShape &s, patconv::TapPlan &plan) {
     std::lock_guard<std::mutex> lock(h->tap_mu);
@@ -522,12 +533,9 @@ xgen_status xgen_blockgemm_pack(const xgen_blockgemm_desc *d, const void *dense_
         cudaGetDevice(&prev);
         xgen_status st = XGEN_OK;
         if (cudaSetDevice(device) != cudaSuccess) st = XGEN_ERR_CUDA;
-        const size_t sb = std::max<size_t>(H.stream.size() * 4, 16), gb = H.seg_off.size() * 4;
-        if (st == XGEN_OK && (cudaMalloc(&h->d_stream, sb) != cudaSuccess || cudaMalloc(&h->d_seg, gb) != cudaSuccess)) st = XGEN_ERR_ALLOC;
-        if (st == XGEN_OK && ((!H.stream.empty() && cudaMemcpy(h->d_stream, H.stream.data(), H.stream.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) ||
-                              cudaMemcpy(h->d_seg, H.seg_off.data(), gb, cudaMemcpyHostToDevice) != cudaSuccess)) st = XGEN_ERR_CUDA;
         if (st == XGEN_OK && d->warps_per_block == 0)
             st = patconv::tap_upload_dense(h->tap, d->dtype, d->k, d->c_out, dense_w, row_keep, col_keep, d->block_rows, d->block_cols);
+        else if (st == XGEN_OK) st = upload_stream(h);
         cudaSetDevice(prev);
         if (st != XGEN_OK) {
             cudaGetLastError();
@@ -568,6 +576,11 @@ xgen_status xgen_blockgemm_run(const xgen_blockgemm_packed *hc, const void *x, i
         }
         if (prev != h->device) cudaSetDevice(prev);
         if (fits) return e == cudaSuccess ? XGEN_OK : XGEN_ERR_CUDA;
+    }
+    {
+        std::lock_guard<std::mutex> lock(h->tap_mu);
+        const xgen_status us = h->d_stream ? XGEN_OK : upload_stream(h);
+        if (us != XGEN_OK) return us;
     }
     GParams P{};
     P.x = x; P.y = y; P.bias = static_cast<const float *>(bias);

@@ -104,9 +104,7 @@ struct KParams {
     uint32_t mg_splits, mg_tiles;        // division by n_splits and by the number of tiles
     int n_tiles;
     int chunks_per_split;                // chunks one block of a split item takes
-    uint32_t *partial;                   // split runs reduced by a second kernel: [split][n*ho*wo*c_out] raw sums
-    size_t out_elems;                    // n*ho*wo*c_out
-    // Split runs reduced inside this kernel: every block writes its raw sums as rows of
+    // Split runs, reduced inside this kernel: every block writes its raw sums as rows of
     // 32 lanes x 8 channels, [item][split][row][lane][8], item = (tile, filter block); a
     // counter per item tells when all of its splits have arrived, and each of them then
     // reduces a share of the rows.
@@ -155,7 +153,7 @@ template <int DT> __device__ __forceinline__ float load_widened(const char *p) {
 // One piece of the result: 8 adjacent output channels of one pixel, as 32-bit values (fp32 bits, or
 // int32 for the integer variant).
 
-// Raw sums stored as they are (partial sums of a split run): element offset o of a 32-bit array.
+// 32-bit results stored as they are: element offset o.
 __device__ __forceinline__ void store_raw_piece(const KParams &P, const uint32_t (&r)[8], uint32_t *out, size_t o, int nv) {
     uint32_t *dst = out + o;
     if (nv == 8 && P.vec_out == 8) {
@@ -380,7 +378,6 @@ patconv_kernel(const KParams P, const __grid_constant__ CUtensorMap tmap) {
     const int c_begin = split_item ? zsplit * P.chunks_per_split : 0;
     const int c_end = split_item ? min(P.n_chunks, c_begin + P.chunks_per_split) : P.n_chunks;
     uint32_t *const ws_rows = split_item ? P.ws : nullptr;       // rows of partial sums exchanged inside the kernel
-    uint32_t *const part_sums = split_item ? P.partial : nullptr; // or partial sums left to a second kernel
 
     // Launched with programmatic stream serialisation: the next kernel of the stream may be
     // scheduled as soon as SMs free up (its launch latency then overlaps this kernel's tail);
@@ -696,7 +693,6 @@ patconv_kernel(const KParams P, const __grid_constant__ CUtensorMap tmap) {
         const uint32_t tmem_res = (DT == XGEN_I8_I32 && P.fold) ? tmem_int : tmem_warp;
         const int oc_base = soc[0];
         if (oc_base >= 0) {
-            uint32_t *const part = part_sums ? part_sums + (size_t)zsplit * P.out_elems : nullptr;
             const int K8 = (P.J + 7) >> 3;
             uint32_t *const wrow = ws_rows ? ws_rows + ((((size_t)sitem * P.n_splits + zsplit) * (size_t)(P.wpc * K8 * T)
                                                    + (size_t)warp * K8 * T) * 32 + lane) * 8 : nullptr;
@@ -708,11 +704,11 @@ patconv_kernel(const KParams P, const __grid_constant__ CUtensorMap tmap) {
                 const int nv = min(8, P.c_out - oc0);                 // valid channels of this piece
                 uint32_t bb[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) bb[k] = (P.bias && !part && !wrow && k < nv) ? ((const uint32_t *)P.bias)[oc0 + k] : 0u;
+                for (int k = 0; k < 8; ++k) bb[k] = (P.bias && !wrow && k < nv) ? ((const uint32_t *)P.bias)[oc0 + k] : 0u;
                 float sc[8];                                          // re-quantisation scales of these channels
 #pragma unroll
                 for (int k = 0; k < 8; ++k) sc[k] = (FUSED && DT == XGEN_I8_I32 && P.rq_scale && k < nv) ? __ldg(P.rq_scale + oc0 + k) : 0.f;
-                if (FUSED && P.pool && !part && !wrow) {
+                if (FUSED && P.pool && !wrow) {
                     // fused 2x2 max-pool: the four sums of a pooled pixel are columns of this thread
                     for (int q = 0; q < T / 4; ++q) {
                         const int qidx = qtab[q * 32 + lane];
@@ -756,7 +752,6 @@ patconv_kernel(const KParams P, const __grid_constant__ CUtensorMap tmap) {
                         }
                         const int pidx = pt[(t0 + tt) * 32];
                         if (pidx < 0) continue;
-                        if (part) { store_raw_piece(P, r, part, (size_t)pidx * P.c_out + oc0, nv); continue; }
                         uint32_t f[8];
                         finish_piece<DT, FUSED>(P, r, bb, oc0, nv, pidx, f);
                         emit_piece<DT, FUSED>(P, f, sc, (size_t)pidx * P.c_out + oc0, nv);
@@ -897,58 +892,6 @@ patconv_kernel(const KParams P, const __grid_constant__ CUtensorMap tmap) {
     __syncthreads();
     if (warp == 0) {
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_cta), "r"((uint32_t)P.tmem_cols) : "memory");
-    }
-}
-
-// Split runs: y = act(bias + sum over splits of the raw partial sums), in a fixed
-// order (split 0, 1, ...), four channels per thread.
-template <int DT>
-__global__ void __launch_bounds__(256)
-patconv_reduce_kernel(const uint32_t *__restrict__ partial, int splits, size_t out_elems, int c_out,
-                      const void *__restrict__ bias, int relu, void *__restrict__ y, int vec) {
-    const size_t i = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) * (vec ? 4 : 1);
-    // Launched with programmatic stream serialisation: everything above overlaps the tail
-    // of the convolution kernel; the partial sums are read only after it has completed.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (i >= out_elems) return;
-    const int oc = (int)(i % (size_t)c_out);
-    if (DT == XGEN_I8_I32) {
-        int r[4] = {0, 0, 0, 0};
-#pragma unroll 4
-        for (int z = 0; z < splits; ++z) {
-            const uint32_t *src = partial + (size_t)z * out_elems + i;
-            if (vec) { const int4 v = *reinterpret_cast<const int4 *>(src); r[0] += v.x; r[1] += v.y; r[2] += v.z; r[3] += v.w; }
-            else r[0] += (int)src[0];
-        }
-        for (int k = 0; k < (vec ? 4 : 1); ++k) {
-            if (bias) r[k] += ((const int *)bias)[oc + k];
-            if (relu) r[k] = max(r[k], 0);
-            ((int *)y)[i + k] = r[k];
-        }
-    } else {
-        float r[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-        for (int z = 0; z < splits; ++z) {
-            const uint32_t *src = partial + (size_t)z * out_elems + i;
-            if (vec) { const float4 v = *reinterpret_cast<const float4 *>(src); r[0] += v.x; r[1] += v.y; r[2] += v.z; r[3] += v.w; }
-            else r[0] += __uint_as_float(src[0]);
-        }
-        for (int k = 0; k < (vec ? 4 : 1); ++k) {
-            if (bias) r[k] += ((const float *)bias)[oc + k];
-            if (relu) r[k] = fmaxf(r[k], 0.f);
-        }
-        if (DT == XGEN_F32) {
-            if (vec) *reinterpret_cast<float4 *>((float *)y + i) = make_float4(r[0], r[1], r[2], r[3]);
-            else ((float *)y)[i] = r[0];
-        } else {
-            if (vec) {
-                __half2 lo = __floats2half2_rn(r[0], r[1]), hi = __floats2half2_rn(r[2], r[3]);
-                uint2 pk;
-                pk.x = *reinterpret_cast<uint32_t *>(&lo);
-                pk.y = *reinterpret_cast<uint32_t *>(&hi);
-                *reinterpret_cast<uint2 *>((__half *)y + i) = pk;
-            } else ((__half *)y)[i] = __float2half_rn(r[0]);
-        }
     }
 }
 
@@ -1106,9 +1049,10 @@ using namespace patconv;
 struct xgen_patconv_packed {
     PackedHost host;
     int device = -1;
-    uint32_t *d_slots = nullptr;
-    int32_t *d_seg_off = nullptr;
-    int32_t *d_slot_oc = nullptr;
+    mutable uint32_t *d_slots = nullptr;
+    mutable int32_t *d_seg_off = nullptr;
+    mutable int32_t *d_slot_oc = nullptr;
+    mutable std::mutex stream_mu;
     // set by xgen_patconv_plan: split the channel chunks of this shape across blocks
     int plan_n = 0, plan_h = 0, plan_w = 0, plan_splits = 1, plan_cps = 0;
     int plan_whole = 0;                 // items of the planned shape that run whole (the others are split)
@@ -1145,18 +1089,18 @@ struct xgen_patconv_packed {
     mutable bool host_call_before = false;
 };
 
-static void free_device_layout(xgen_patconv_packed *h) {
+// The device copy of the command stream: there only where a run may need it (see uses_stream).
+static void free_device_layout(const xgen_patconv_packed *h) {
     if (h->d_slots) cudaFree(h->d_slots);
     if (h->d_seg_off) cudaFree(h->d_seg_off);
     if (h->d_slot_oc) cudaFree(h->d_slot_oc);
-    if (h->d_status) cudaFree(h->d_status);
-    h->d_slots = nullptr; h->d_seg_off = nullptr; h->d_slot_oc = nullptr; h->d_status = nullptr;
+    h->d_slots = nullptr; h->d_seg_off = nullptr; h->d_slot_oc = nullptr;
 }
 
 // Upload the host layout; the device must be current.  On the device a command slot is
 // 48 bytes: {opcode, operand, -, -, w0, w0, w1, w1, w2, w2, w3, w3}; every weight twice, so
 // that a 64-bit load yields the operand pair of a two-wide FMA.
-static xgen_status upload_layout(xgen_patconv_packed *h) {
+static xgen_status upload_layout(const xgen_patconv_packed *h) {
     const PackedHost &p = h->host;
     free_device_layout(h);
     const size_t n_slots = p.slots.size() / kSlotWords;
@@ -1171,8 +1115,6 @@ static xgen_status upload_layout(xgen_patconv_packed *h) {
     cudaError_t e = cudaMalloc(&h->d_slots, sb);
     if (e == cudaSuccess) e = cudaMalloc(&h->d_seg_off, gb);
     if (e == cudaSuccess) e = cudaMalloc(&h->d_slot_oc, ob);
-    if (e == cudaSuccess) e = cudaMalloc(&h->d_status, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemcpy(h->d_slots, dev.data(), sb, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_seg_off, p.seg_off.data(), gb, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(h->d_slot_oc, p.slot_oc.data(), ob, cudaMemcpyHostToDevice);
@@ -1333,7 +1275,6 @@ static xgen_status layout_for(const PackedHost &p, const Geometry &g_in, int n, 
     const size_t floor_bytes = (size_t)kSmemPerSM / (max_ctas + 1);
     if (smem < floor_bytes) smem = floor_bytes;
     if (smem > (size_t)kSmemMaxDynamic) return XGEN_ERR_UNSUPPORTED;
-    kp.out_elems = (size_t)n * ho * wo * p.c_out;
     L.kp = kp;
     L.smem = smem;
     L.items = g.tiles * p.n_blocks;
@@ -1419,6 +1360,11 @@ static void forget_prepared_launches(xgen_patconv_packed *h) {
     for (LaunchEntry &e : h->cache) e.stamp = 0;
 }
 
+// Tuning that names parameters of the command-stream kernel.
+static bool asks_for_stream(const xgen_patconv_tuning &t) {
+    return t.splits || t.no_copy_engine || t.reduce_mode || t.channels_per_chunk || t.groups_per_block;
+}
+
 // Whether a run takes the matrix path.
 static bool on_matrix_units(const xgen_patconv_packed *h) { return h->tap.dev && !h->stream_asked; }
 
@@ -1439,11 +1385,9 @@ static bool tap_plan_of(const xgen_patconv_packed *h, const TapShape &s, TapPlan
     return true;
 }
 
-// Where a run keeps the partial sums of a split, when the caller (not the plan) decides.
-struct SplitChoice { int splits, chunks_per_split; uint32_t *partial; };
-
+// `ignore_plan`: the caller's plan of the command-stream kernel (tuning, splits) is left aside.
 static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_t n, int32_t hh, int32_t ww,
-                             const void *bias, int32_t relu, void *y, void *stream, const SplitChoice *forced,
+                             const void *bias, int32_t relu, void *y, void *stream, bool ignore_plan = false,
                              const xgen_patconv_epilogue *ep = nullptr) {
     if (!h || !x || !y) return XGEN_ERR_INVALID_ARG;
     if (((uintptr_t)x & 15) || ((uintptr_t)y & 15) || ((uintptr_t)bias & 3)) return XGEN_ERR_INVALID_ARG;
@@ -1458,7 +1402,7 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
     const void *residual = ep ? ep->residual_dev : nullptr;
     const float *rq_scale = ep ? ep->requant_scale_dev : nullptr;
     if (ep) {
-        if (forced || p.bh != 4) return XGEN_ERR_UNSUPPORTED;
+        if (p.bh != 4) return XGEN_ERR_UNSUPPORTED;
         if (pool != 0 && pool != 2) return XGEN_ERR_UNSUPPORTED;
         if (pool == 2 && ((ho & 1) || (wo & 1))) return XGEN_ERR_SHAPE;
         if (rq_scale && p.dtype != XGEN_I8_I32) return XGEN_ERR_UNSUPPORTED;
@@ -1476,7 +1420,7 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
             if (ra < ye && ya < re) return XGEN_ERR_INVALID_ARG;
         }
     }
-    if (!forced && on_matrix_units(h)) {
+    if (h->tap.dev && (ignore_plan || !h->stream_asked)) {
         TapShape ts;
         ts.n = n; ts.h = hh; ts.w = ww; ts.stride = p.stride; ts.pool = pool == 2;
         ts.staged = (residual && pool != 2 && p.dtype != XGEN_F32) || p.c_out * (rq_scale ? 1 : p.dtype == XGEN_F16_F32ACC ? 2 : 4) % 16 != 0;
@@ -1498,6 +1442,14 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
         if (prev != h->device) cudaSetDevice(prev);
         if (fits) return e == cudaSuccess ? XGEN_OK : XGEN_ERR_CUDA;
     }
+    {
+        // (only where the driver cannot encode the matrix path's tensor maps is the stream not there yet)
+        std::lock_guard<std::mutex> lock(h->stream_mu);
+        if (!h->d_slots) {
+            const xgen_status us = upload_layout(h);
+            if (us != XGEN_OK) return us;
+        }
+    }
     Layout L;
     CUtensorMap tm;
     xgen_status ls = prepared_launch(h, x, n, hh, ww, ((uintptr_t)y & 31) == 0, L, tm);
@@ -1511,14 +1463,12 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
     kp.pool = pool; kp.po = po; kp.pw = pw;
     kp.status = h->d_status;
     kp.wait_us = h->wait_us;
-    // Split runs: a caller-chosen split keeps [split][output] sums for a second kernel; the
-    // planned split is reduced inside the kernel (rows of partial sums plus arrival counters).
-    const bool planned = !forced && h->plan_splits > 1 && h->plan_n == n && h->plan_h == hh && h->plan_w == ww &&
+    // The planned split is reduced inside the kernel (rows of partial sums plus arrival counters).
+    const bool planned = !ignore_plan && h->plan_splits > 1 && h->plan_n == n && h->plan_h == hh && h->plan_w == ww &&
                          h->d_partial && h->d_counters;
-    const bool split = forced ? forced->splits > 1 : planned;
-    const int n_splits = split ? (forced ? forced->splits : h->plan_splits) : 1;
+    const int n_splits = planned ? h->plan_splits : 1;
     // block numbering: whole items first, then the split items, n_splits blocks each
-    const int whole = split ? (forced ? 0 : h->plan_whole) : L.items;
+    const int whole = planned ? h->plan_whole : L.items;
     const int64_t n_blocks_launch = (int64_t)whole + (int64_t)(L.items - whole) * n_splits;
     if (n_blocks_launch > 0x7FFFFFFFLL) return XGEN_ERR_SHAPE;
     auto magic = [](int d) { return d <= 1 ? 0u : (uint32_t)((1ull << 32) / (uint64_t)d + 1ull); };
@@ -1527,8 +1477,7 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
     kp.mg_splits = magic(n_splits);
     kp.n_tiles = L.g.tiles;
     kp.mg_tiles = magic(L.g.tiles);
-    kp.chunks_per_split = split ? (forced ? forced->chunks_per_split : h->plan_cps) : p.n_chunks;
-    kp.partial = (split && forced) ? forced->partial : nullptr;
+    kp.chunks_per_split = planned ? h->plan_cps : p.n_chunks;
 
     int prev = 0;
     if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
@@ -1572,41 +1521,11 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
         }
         e = log_cuda(e, "kernel launch");
     }
-    if (e == cudaSuccess && split && forced) {
-        const int vec = kp.vec_out >= 4 ? 1 : 0;
-        const size_t items = vec ? kp.out_elems / 4 : kp.out_elems;
-        const unsigned blocks = (unsigned)((items + 255) / 256);
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(blocks, 1, 1); cfg.blockDim = dim3(256, 1, 1); cfg.dynamicSmemBytes = 0; cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-        const uint32_t *part_c = forced->partial;
-        const size_t oe = kp.out_elems;
-        const int co = p.c_out, rl = kp.relu;
-        const void *bias_c = bias;
-        if (p.dtype == XGEN_F32)
-            e = cudaLaunchKernelEx(&cfg, patconv_reduce_kernel<XGEN_F32>, part_c, n_splits, oe, co, bias_c, rl, y, vec);
-        else if (p.dtype == XGEN_F16_F32ACC)
-            e = cudaLaunchKernelEx(&cfg, patconv_reduce_kernel<XGEN_F16_F32ACC>, part_c, n_splits, oe, co, bias_c, rl, y, vec);
-        else
-            e = cudaLaunchKernelEx(&cfg, patconv_reduce_kernel<XGEN_I8_I32>, part_c, n_splits, oe, co, bias_c, rl, y, vec);
-        if (e == cudaSuccess) e = cudaGetLastError();
-        e = log_cuda(e, "reduce launch");
-        if (e == cudaSuccess) g_launches.fetch_add(1);
-    }
     if (prev != h->device) cudaSetDevice(prev);
     if (e != cudaSuccess) return XGEN_ERR_CUDA;
     g_launches.fetch_add(1);
     return XGEN_OK;
 }
-
-// The library's own scratch for xgen_patconv_run_static_scratch: partial sums of a split run.
-// It lives in every CUDA context that loads this library, until the process exits.
-static __device__ __align__(256) uint32_t g_static_scratch[XGEN_PATCONV_STATIC_SCRATCH_BYTES / 4];
-static uint32_t *g_static_scratch_addr[64];        // device address per device ordinal, resolved once
-static std::mutex g_static_scratch_mutex;
 
 extern "C" {
 
@@ -1655,14 +1574,16 @@ xgen_status xgen_patconv_pack(const xgen_patconv_desc *desc, const void *dense_w
     if (device >= 0) {
         int prev = 0;
         if (cudaGetDevice(&prev) != cudaSuccess || cudaSetDevice(device) != cudaSuccess) { delete h; return XGEN_ERR_CUDA; }
-        xgen_status us = upload_layout(h);
+        xgen_status us = XGEN_OK;
+        if (cudaMalloc(&h->d_status, sizeof(int)) != cudaSuccess) us = XGEN_ERR_ALLOC;
+        else if (cudaMemset(h->d_status, 0, sizeof(int)) != cudaSuccess) us = XGEN_ERR_CUDA;
+        const PackedHost &p = h->host;
         // Three input channels fill a fifth of the 16 that a matrix instruction takes: such first layers
         // stay on the command-stream kernel (3 -> 64 at 224x224, fp32: 12.7 us against 15.8 us).
-        if (us == XGEN_OK && desc->c_in >= 8) {
-            const PackedHost &p = h->host;
-            us = tap_upload_patterns(h->tap, p.dtype, p.c_in, p.c_out, p.kpat.data(), p.kw4.data(), p.masks.data(), (int)p.masks.size());
-            if (us != XGEN_OK) free_device_layout(h);
-        }
+        if (us == XGEN_OK)
+            us = desc->c_in < 8 ? upload_layout(h)
+                                : tap_upload_patterns(h->tap, p.dtype, p.c_in, p.c_out, p.kpat.data(), p.kw4.data(), p.masks.data(), (int)p.masks.size());
+        if (us != XGEN_OK && h->d_status) { cudaGetLastError(); cudaFree(h->d_status); }
         cudaSetDevice(prev);
         if (us != XGEN_OK) { delete h; return us; }
         h->device = device;
@@ -1674,6 +1595,7 @@ xgen_status xgen_patconv_pack(const xgen_patconv_desc *desc, const void *dense_w
 void xgen_patconv_free(xgen_patconv_packed *h) {
     if (!h) return;
     free_device_layout(h);
+    if (h->d_status) cudaFree(h->d_status);
     tap_free(h->tap);
     if (h->d_partial) cudaFree(h->d_partial);
     if (h->d_counters) cudaFree(h->d_counters);
@@ -1783,6 +1705,7 @@ xgen_status xgen_patconv_plan_tuned(xgen_patconv_packed *h, int32_t n, int32_t h
     if ((int64_t)n * ho * wo * p.c_out > 0x7FFFFFFFLL) return XGEN_ERR_SHAPE;
     const xgen_patconv_tuning tn = tuning ? *tuning : xgen_patconv_tuning{};
     const bool tma_ok = !tn.no_copy_engine && encode_tiled_fn() != nullptr;
+    const bool stream = asks_for_stream(tn) || !h->tap.dev;        // later runs take the command-stream kernel
     int prev = 0;
     if (cudaGetDevice(&prev) != cudaSuccess || cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
     xgen_status rs = XGEN_OK;
@@ -1800,7 +1723,8 @@ xgen_status xgen_patconv_plan_tuned(xgen_patconv_packed *h, int32_t n, int32_t h
         } catch (const std::bad_alloc &) {
             st = XGEN_ERR_ALLOC;
         }
-        if (st == XGEN_OK) st = upload_layout(h);
+        free_device_layout(h);
+        if (st == XGEN_OK && stream) st = upload_layout(h);
         forget_prepared_launches(h);
         return st;
     };
@@ -1926,7 +1850,8 @@ xgen_status xgen_patconv_plan_tuned(xgen_patconv_packed *h, int32_t n, int32_t h
     if (splits <= 1) { whole = L.items; last = false; }
     const int64_t split_items = L.items - whole;
     if (rs == XGEN_OK && cudaDeviceSynchronize() != cudaSuccess) rs = XGEN_ERR_CUDA;
-    if (rs == XGEN_OK && splits > 1) {
+    if (rs == XGEN_OK && stream && !h->d_slots) rs = upload_layout(h);
+    if (rs == XGEN_OK && splits > 1 && stream) {
         const size_t need = (size_t)split_items * (size_t)splits * rows_per_item(p) * 1024;
         const size_t need_c = (size_t)split_items * sizeof(uint32_t);
         if (need > h->partial_bytes) {
@@ -1951,7 +1876,7 @@ xgen_status xgen_patconv_plan_tuned(xgen_patconv_packed *h, int32_t n, int32_t h
     forget_prepared_launches(h);
     if (rs != XGEN_OK) { h->plan_splits = 1; h->plan_n = 0; return rs; }
     h->tuning = tn;
-    h->stream_asked = tn.splits || tn.no_copy_engine || tn.reduce_mode || tn.channels_per_chunk || tn.groups_per_block;
+    h->stream_asked = asks_for_stream(tn);
     h->wait_us = tn.wait_limit_ms > 0 ? (uint32_t)std::min<int64_t>((int64_t)tn.wait_limit_ms * 1000, 60000000) : 2000000u;
     h->plan_n = n; h->plan_h = hh; h->plan_w = ww;
     h->plan_splits = (int)splits; h->plan_cps = cps; h->plan_whole = (int)whole; h->plan_last = last;
@@ -1970,13 +1895,13 @@ xgen_status xgen_patconv_test_expect_arrivals(xgen_patconv_packed *h, int32_t ex
 
 xgen_status xgen_patconv_run(const xgen_patconv_packed *h, const void *x, int32_t n, int32_t hh, int32_t ww,
                              const void *bias, int32_t relu, void *y, void *stream) {
-    return run_layer(h, x, n, hh, ww, bias, relu, y, stream, nullptr);
+    return run_layer(h, x, n, hh, ww, bias, relu, y, stream);
 }
 
 xgen_status xgen_patconv_run_fused(const xgen_patconv_packed *h, const void *x, int32_t n, int32_t hh, int32_t ww,
                                    const void *bias, const xgen_patconv_epilogue *ep, void *y, void *stream) {
     if (!ep) return XGEN_ERR_INVALID_ARG;
-    return run_layer(h, x, n, hh, ww, bias, ep->relu, y, stream, nullptr, ep);
+    return run_layer(h, x, n, hh, ww, bias, ep->relu, y, stream, false, ep);
 }
 
 xgen_status xgen_patconv_run_static_scratch(const xgen_patconv_packed *h, const void *x, int32_t n, int32_t hh,
@@ -1998,25 +1923,9 @@ xgen_status xgen_patconv_run_static_scratch(const xgen_patconv_packed *h, const 
                     eff, (long long)out_elems, (unsigned)XGEN_PATCONV_STATIC_SCRATCH_BYTES);
         return XGEN_ERR_SHAPE;
     }
-    uint32_t *scratch = nullptr;
-    {
-        // First call on a device: resolve the device address of the array (in host code the
-        // array's name is only a handle, not an address a kernel can use).
-        std::lock_guard<std::mutex> lock(g_static_scratch_mutex);
-        scratch = g_static_scratch_addr[h->device];
-        if (!scratch) {
-            int prev = 0;
-            if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
-            if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
-            void *addr = nullptr;
-            const cudaError_t e = cudaGetSymbolAddress(&addr, g_static_scratch);
-            if (prev != h->device) cudaSetDevice(prev);
-            if (log_cuda(e, "cudaGetSymbolAddress") != cudaSuccess || !addr) return XGEN_ERR_CUDA;
-            scratch = g_static_scratch_addr[h->device] = static_cast<uint32_t *>(addr);
-        }
-    }
-    const SplitChoice choice{eff, cps, scratch};
-    return run_layer(h, x, n, hh, ww, bias, relu, y, stream, &choice);
+    // The matrix path keeps the sums of a split in the shared memory of a cluster; a layer that is not on
+    // it (fewer than eight input channels: one chunk) has nothing to split.
+    return run_layer(h, x, n, hh, ww, bias, relu, y, stream, true);
 }
 
 xgen_status xgen_patconv_enqueue_host(const xgen_patconv_packed *h, const void *x, int32_t n, int32_t hh, int32_t ww,
