@@ -1142,25 +1142,25 @@ __global__ void tap_expand_dense(uint8_t *img, int c_in, int c_out, int rows, co
 static int tap_cpp(xgen_dtype dt) { return dt == XGEN_I8_I32 ? 16 : 8; }
 static int tap_parts(xgen_dtype dt) { return dt == XGEN_F32 ? 3 : 1; }
 
-// The zeroed image, and `extra` bytes of scratch that tap_done gives back.
+// The zeroed image with `extra` bytes of upload scratch behind it, one allocation (a second one that is
+// given back costs a synchronisation and more time than the upload).
 static xgen_status tap_alloc(TapWeights &tw, xgen_dtype dt, int taps, int c_in, int c_out, size_t extra, uint8_t **scratch) {
     tw.dtype = dt; tw.taps = taps; tw.c_in = c_in; tw.c_out = c_out;
     tw.planes = (c_in + 2 * tap_cpp(dt) - 1) / (2 * tap_cpp(dt)) * 2;
     tw.rows = (c_out + 15) / 16 * 16;
     const size_t bytes = (size_t)tw.planes * taps * tap_parts(dt) * tw.rows * 16;
-    cudaError_t e = cudaMalloc(&tw.dev, bytes);
-    if (e == cudaSuccess) e = cudaMalloc(scratch, extra);
+    cudaError_t e = cudaMalloc(&tw.dev, bytes + extra);
     if (e == cudaSuccess) e = cudaMemsetAsync(tw.dev, 0, bytes, 0);
+    *scratch = tw.dev + bytes;
     if (e == cudaSuccess) return XGEN_OK;
     cudaGetLastError();
     tap_free(tw);
     return e == cudaErrorMemoryAllocation ? XGEN_ERR_ALLOC : XGEN_ERR_CUDA;
 }
 
-static xgen_status tap_done(TapWeights &tw, uint8_t *scratch, cudaError_t e) {
+static xgen_status tap_done(TapWeights &tw, cudaError_t e) {
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
-    cudaFree(scratch);
     if (e == cudaSuccess) return XGEN_OK;
     cudaGetLastError();
     tap_free(tw);
@@ -1190,7 +1190,7 @@ xgen_status tap_upload_patterns(TapWeights &tw, xgen_dtype dt, int c_in, int c_o
         else if (dt == XGEN_F16_F32ACC) tap_expand_patterns<XGEN_F16_F32ACC><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, kp, w, mk);
         else tap_expand_patterns<XGEN_I8_I32><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, kp, w, mk);
     }
-    return tap_done(tw, scratch, e);
+    return tap_done(tw, e);
 }
 
 xgen_status tap_upload_dense(TapWeights &tw, xgen_dtype dt, int c_in, int c_out, const void *dense_w, const uint8_t *row_keep,
@@ -1209,7 +1209,7 @@ xgen_status tap_upload_dense(TapWeights &tw, xgen_dtype dt, int c_in, int c_out,
         if (dt == XGEN_F32) tap_expand_dense<XGEN_F32><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, scratch, rk, ck, br, bc);
         else tap_expand_dense<XGEN_F16_F32ACC><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, scratch, rk, ck, br, bc);
     }
-    return tap_done(tw, scratch, e);
+    return tap_done(tw, e);
 }
 
 // ---- plans ---------------------------------------------------------------------

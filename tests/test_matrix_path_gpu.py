@@ -1,0 +1,155 @@
+"""GPU parity of the matrix path where its cuts lie: tiles of 8 x 16 pixels and runs of the raster,
+stages of 64 (fp16), 128 (int8) and 32 (fp32) channels, filter tiles of 32 to 256, pairs of blocks,
+reductions split over a cluster, tensor copies against gathered rows."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2206_10620_b200 import binding, workloads as wl
+from _gpu_util import TOL, check_guards, compare, guarded_output, pack, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def _layer(dtype, n, ci, co, h, w, stride=1, prune=0.5, seed=1, x_dist=None):
+    xd = x_dist or {"f32": "upm1", "f16": "relu_normal", "i8": "u01"}[dtype]
+    spec = wl.LayerSpec("t", n, ci, co, h, w, stride, dtype, prune, 12, "he", xd, 0.05, True, 0)
+    return wl.make_layer(spec, seed=seed)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16", "i8"])
+@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("shape", [
+    (1, 8, 16, 1, 1),         # the fewest channels, one pixel
+    (1, 16, 31, 1, 9),        # one row, one column past an 8-pixel column, ragged filters
+    (3, 17, 33, 16, 8),       # exactly one tile an image; channels of no whole 16 bytes
+    (2, 64, 64, 17, 9),       # one row and one column past a tile; one whole stage (fp16)
+    (5, 80, 40, 7, 7),        # several small images in a tile
+    (2, 144, 129, 15, 29),    # a stage and a piece; one filter past a tile of 128
+    (1, 48, 257, 33, 40),     # one filter past the largest tile
+    (9, 96, 72, 30, 31),      # runs of the raster over all images
+])
+def test_edges_of_tiles(dtype, stride, shape):
+    n, ci, co, h, w = shape
+    d = _layer(dtype, n, ci, co, h, w, stride, seed=sum(shape))
+    pk = pack(d)
+    assert pk.plan_info(n, h, w)["matrix_path"] == 1
+    compare(d, run_gpu(pk, d.x, d.bias, True))
+    compare(d, run_gpu(pk, d.x, None, False), bias=None, relu=False)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16", "i8"])
+@pytest.mark.parametrize("shape", [(1, 512, 96, 14, 14), (1, 320, 512, 7, 7), (2, 256, 40, 9, 12)])
+def test_reduction_split_over_a_cluster(dtype, shape):
+    """Few pixels, many channels: the blocks of a cluster share an item; the result does not depend
+    on when they arrive."""
+    n, ci, co, h, w = shape
+    d = _layer(dtype, n, ci, co, h, w, prune=0.7, seed=ci)
+    pk = pack(d)
+    y = run_gpu(pk, d.x, d.bias, True, plan=True)
+    compare(d, y)
+    for _ in range(3):
+        assert np.array_equal(run_gpu(pk, d.x, d.bias, True), y)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16", "i8"])
+@pytest.mark.parametrize("co", [40, 37])
+@pytest.mark.parametrize("pool", [0, 2])
+def test_fused_operators_behind_tiles_and_splits(dtype, co, pool):
+    import torch
+    for n, ci, h, w in ((3, 24, 14, 22), (1, 256, 12, 10)):
+        d = _layer(dtype, n, ci, co, h, w, seed=co + pool)
+        pk = pack(d)
+        size = n * h * w * co
+        res = (wl.integers(3, "AUX", 1, size, -9999, 9999).astype(np.int32) if dtype == "i8"
+               else (wl.normal(3, "AUX", 1, size) * 0.5).astype(np.float32 if dtype == "f32" else np.float16)).reshape(n, h, w, co)
+        for scale in ([None, (wl.uniform01(4, "AUX", 2, co) * 2e-3 + 1e-4).astype(np.float32)] if dtype == "i8" else [None]):
+            t = torch.uint8 if scale is not None else {"f32": torch.float32, "f16": torch.float16, "i8": torch.int32}[dtype]
+            step = 2 if pool else 1
+            buf, y = guarded_output((n, h // step, w // step, co), t)
+            dev = [torch.from_numpy(np.ascontiguousarray(a)).cuda() if a is not None else None for a in (d.x, d.bias, res, scale)]
+            p = [0 if a is None else a.data_ptr() for a in dev]
+            pk.run_fused(p[0], n, h, w, p[1], y.data_ptr(), relu=True, pool=pool, residual_ptr=p[2], requant_scale_ptr=p[3], zero_point=9)
+            pk.sync()
+            check_guards(buf)
+            ref = oracle.conv_fused(d.x, d.w, d.pid, d.masks, bias=d.bias, relu=True, residual=res, pool=pool, requant_scale=scale, zero_point=9)
+            got = y.cpu().numpy()
+            if dtype == "i8":
+                assert np.array_equal(got.astype(np.int64), ref.astype(np.int64))
+            else:
+                pre, S = oracle.conv(d.x, d.w, d.pid, d.masks, bias=d.bias, relu=False, with_scale=True)
+                bound = TOL[dtype] * np.maximum(np.abs(pre + res), 0.01 * (S + np.abs(res))) + 1e-30
+                if pool:
+                    bound = bound.reshape(n, h // 2, 2, w // 2, 2, co).max(axis=(2, 4))
+                assert (np.abs(got - ref) <= bound).all()
+
+
+def test_fp32_sums_keep_fp32_precision():
+    """Long sums of positive terms, where a truncating accumulator would show: the error stays that of
+    a few roundings, and operands keep all of their bits."""
+    d = _layer("f32", 1, 512, 64, 16, 16, prune=0.0, seed=5, x_dist="u01")
+    d.w = np.abs(d.w)
+    y = run_gpu(pack(d), d.x, None, False)
+    ref = oracle.conv(d.x, d.w, d.pid, d.masks, bias=None, relu=False)
+    assert np.abs(y / ref - 1).max() < 1.5e-6
+    d = _layer("f32", 1, 16, 32, 8, 8, prune=0.0, seed=6)
+    d.x[:] = 0
+    d.x[0, 4, 4, 3] = np.float32(3.4e38)                 # above the largest bf16, below the largest fp32
+    d.w[:] = 0
+    d.w[7, 3] = np.float32(2.0 ** -100)
+    ref = oracle.conv(d.x, d.w, d.pid, d.masks, bias=None, relu=False)
+    np.testing.assert_allclose(run_gpu(pack(d), d.x, None, False), ref, rtol=1e-6, atol=0)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("m", [1, 127, 129, 1000])
+@pytest.mark.parametrize("k,co", [(16, 32), (33, 31), (200, 264)])
+def test_block_pruned_product(dtype, m, k, co):
+    import torch
+    d = wl.make_block_gemm(wl.GemmSpec("t", m, k, co, 16, 16, 0.5, 0.5, dtype), seed=m + k)
+    g = binding.BlockGemm(k, co, 16, 16, dtype, d.w, d.row_keep, d.col_keep)
+    ref, S = oracle.block_gemm(d.x, d.w, d.row_keep, d.col_keep, 16, 16, bias=d.bias, relu=True, with_scale=True)
+    bound = TOL[dtype] * np.maximum(np.abs(ref), 0.01 * S) + 2.0 ** -25
+    t = torch.float32 if dtype == "f32" else torch.float16
+    for shift in (0, 1):                                 # tensors that start on an element, not on 16 bytes
+        x = torch.zeros(m * k + shift, dtype=t, device="cuda")
+        x[shift:] = torch.from_numpy(d.x).cuda().reshape(-1)
+        buf, y = guarded_output((m, co), t)
+        b = torch.from_numpy(d.bias).cuda()
+        g.run(x.data_ptr() + shift * x.element_size(), m, b.data_ptr(), True, y.data_ptr())
+        torch.cuda.synchronize()
+        check_guards(buf)
+        assert (np.abs(y.cpu().numpy().astype(np.float64) - ref) <= bound).all()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("shape", [(1, 6, 1, 1), (2, 2, 13, 5), (1, 20, 40, 33), (40, 64, 17, 30), (3, 7, 2, 9)])
+def test_depthwise_pieces_of_rows(dtype, stride, shape):
+    import torch
+    n, c, h, w = shape
+    d = wl.make_depthwise(wl.DepthwiseSpec("t", n, c, h, w, stride, dtype, 0.2, 12), seed=c)
+    dw = binding.Depthwise(c, stride, dtype, d.masks, d.w, d.pid)
+    t = torch.float32 if dtype == "f32" else torch.float16
+    ho, wo = (h - 1) // stride + 1, (w - 1) // stride + 1
+    buf, y = guarded_output((n, ho, wo, c), t)
+    x, b = torch.from_numpy(d.x).cuda(), torch.from_numpy(d.bias).cuda()
+    dw.run(x.data_ptr(), n, h, w, b.data_ptr(), True, y.data_ptr())
+    torch.cuda.synchronize()
+    check_guards(buf)
+    ref, S = oracle.depthwise(d.x, d.w, d.pid, d.masks, bias=d.bias, relu=True, stride=stride, with_scale=True)
+    err = np.abs(y.cpu().numpy().astype(np.float64) - ref)
+    assert (err <= TOL[dtype] * np.maximum(np.abs(ref), 0.01 * S) + 2.0 ** -25).all()
+
+
+def test_calls_report_errors():
+    pk = pack(_layer("f32", 1, 16, 32, 8, 8))
+    with pytest.raises(binding.PatconvError) as e:
+        pk.run(0, 1, 8, 8, 0, True, 16)
+    assert e.value.status == 1
+    with pytest.raises(TypeError):
+        binding._calls.conv(pk._h.value, 0)
+    pk.close()
+    with pytest.raises(binding.PatconvError) as e:
+        pk.run(16, 1, 8, 8, None, True, 4096)
+    assert e.value.status == 1
