@@ -1423,7 +1423,7 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
     if (h->tap.dev && (ignore_plan || !h->stream_asked)) {
         TapShape ts;
         ts.n = n; ts.h = hh; ts.w = ww; ts.stride = p.stride; ts.pool = pool == 2;
-        ts.staged = (residual && pool != 2 && p.dtype != XGEN_F32) || p.c_out * (rq_scale ? 1 : p.dtype == XGEN_F16_F32ACC ? 2 : 4) % 16 != 0;
+        ts.staged = (residual && pool != 2) || p.c_out * (rq_scale ? 1 : p.dtype == XGEN_F16_F32ACC ? 2 : 4) % 16 != 0;
         int prev = 0;
         if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
         if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;

@@ -329,13 +329,34 @@ __device__ __forceinline__ void tap_emit(const TapParams &P, const uint32_t *st,
     const uint32_t bias = s_bias[c - n0];
     const float scale = FUSED ? s_scale[c - n0] : 0.0f;
     if (!pool) {
-#pragma unroll 4
-        for (int it = 0; it < 16; ++it) {
-            const uint32_t *const row = st + (2 * it + (lane >> 4)) * kStagePitch;
-            const int px = (int)row[16];
-            if (px >= 0) {
-                const size_t off = (size_t)px * P.c_out + c;
-                tap_store1<DT, FUSED>(P, scale, tap_affine1<DT, FUSED>(P, bias, row[lane & 15], off), off);
+        // eight residuals asked for at a time: one by one, 24 images of 32 x 74 x 58 fp32 channels took
+        // 52 us (25 now)
+#pragma unroll 1
+        for (int it = 0; it < 16; it += 8) {
+            const uint32_t *const row0 = st + (2 * it + (lane >> 4)) * kStagePitch;
+            int px[8];
+            uint32_t res[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                px[i] = (int)row0[2 * i * kStagePitch + 16];
+                res[i] = 0u;
+                if (FUSED && P.residual) {
+                    const size_t off = (size_t)max(px[i], 0) * P.c_out + c;
+                    if (DT == XGEN_F16_F32ACC) res[i] = __ldg(static_cast<const unsigned short *>(P.residual) + off);
+                    else res[i] = __ldg(static_cast<const uint32_t *>(P.residual) + off);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                uint32_t v = row0[2 * i * kStagePitch + (lane & 15)];
+                if (DT == XGEN_I8_I32) v += bias + res[i];
+                else {
+                    const float r = DT == XGEN_F16_F32ACC ? __half2float(__ushort_as_half((unsigned short)res[i])) : __uint_as_float(res[i]);
+                    v = __float_as_uint(__uint_as_float(v) + __uint_as_float(bias));
+                    if (FUSED && P.residual) v = __float_as_uint(__uint_as_float(v) + r);
+                }
+                if (P.relu) v = tap_max<DT>(v, 0u);
+                if (px[i] >= 0) tap_store1<DT, FUSED>(P, scale, v, (size_t)px[i] * P.c_out + c);
             }
         }
         return;
