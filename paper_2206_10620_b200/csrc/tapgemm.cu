@@ -1400,7 +1400,9 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     for (p.tmem_cols = 32; p.tmem_cols < cols;) p.tmem_cols *= 2;
                     // Cycles of a stage: the matrix instructions (nt / 2 each; 46 to issue one and 90 for a tap), or
                     // what they and the copies move through shared memory at 128 bytes a cycle (128 rows of x,
-                    // the block's filters), or what comes from L2.  A pair starts and ends 4000 cycles later.
+                    // the block's filters), or what comes from L2.  A pair starts and ends 4000 cycles later, and the
+                    // short stages of a product wait 300 cycles for its other block (1842 filters x 5421 rows,
+                    // fp32: 77 us as pairs, 57 us without).
                     const double kk = (double)tw.planes / p.stages / 2, taps = tw.taps;
                     const double b_stage = taps * kk * 2 * parts * p.nt * 16.0 / ways, b_moved = p.resident && sp == 1 ? b_stage / waves : b_stage;
                     const double x_moved = (double)pixels * kk * 2 * cpp * xb, a_stage = (double)p.a_bytes * (swizzled ? 1 : 2);
@@ -1408,7 +1410,7 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     const double mma = taps * std::max(per_tap * p.nt / 2.0, 90.0 + 46.0 * per_tap);
                     const double shared = (instr * (4096.0 + p.nt * 32.0 / ways) + b_moved + a_stage) / 128.0;
                     const double move = (x_moved + b_moved) / 40.0 + (copied && p.straddle ? 60.0 * p.rows * (s.stride == 1 ? 1 : 4) : 0.0) * 0.5;
-                    const double stage = std::max(std::max(mma, shared), move) + 250.0 + 40.0 * taps / p.tap_group;
+                    const double stage = std::max(std::max(mma, shared), move) + 250.0 + 40.0 * taps / p.tap_group + (p.pair && tw.taps == 1 ? 300.0 : 0.0);
                     const double out = (double)mt * 128 * p.nt * yb / 24.0;
                     const double item = p.per_split * stage;
                     double c = 3500.0 + (p.pair ? 4000.0 : 0.0);
