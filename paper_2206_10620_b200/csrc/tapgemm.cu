@@ -713,35 +713,35 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
         if (!kF32 && P.tma) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
             if (warp == kEpiWarps) {
-                // ---- x by tensor copies, zeros outside the image -------------------------------
-                if (elect_one()) {
-                    int s = 0;
-                    uint32_t ph = 1;
-                    for (int item = item0; item < P.items; item += item_step) {
-                        const TapItem t = tap_item<MT, PAIR>(P, item, side);
-                        s_started = s_started + 1;
-                        for (int ks = k0; ks < k1; ++ks) {
-                            wait(a_empty(s), ph);
-                            const uint32_t bar = lead(a_full(s));
-                            uint32_t dst = sbase + (uint32_t)(s * P.a_bytes) + (P.raster ? (uint32_t)(P.pitch - 1 - t.ox0) * 128u : 0u);
-                            const int c = ks * T::row_ch;
-                            if (side == 0) mbar_expect_tx(a_full(s), (uint32_t)(P.a_tx * (PAIR ? 2 : 1)));
-                            if (TAPS == 1) tensor_load4<PAIR>(dst, &xmap, c, t.v0 * 8, 0, 0, bar);
-                            else {
-                                const int step = (P.row_boxes ? 1 : P.rows) * P.pitch * 128;
-                                for (int region = 0; region < (STRIDE == 1 ? 1 : 4); ++region) {
-                                    const int x0 = STRIDE == 1 ? (P.raster ? 0 : t.ox0) - 1 : 2 * t.ox0 - (region & 1);
-                                    for (int i = 0; i < (P.row_boxes ? P.rows : 1); ++i, dst += step) {
-                                        const TapRow r = tap_row<STRIDE>(P, t, i, region >> 1);
-                                        tensor_load4<PAIR>(dst, &xmap, c, x0, r.y, r.img, bar);
-                                    }
-                                }
+                // ---- x by tensor copies, zeros outside the image; the lanes share the copies of a stage
+                // (rows one by one from one thread cost it 190 cycles each) ---------------------------------
+                int s = 0;
+                uint32_t ph = 1;
+                const int per = TAPS == 1 || !P.row_boxes ? 1 : P.rows, boxes = (TAPS == 1 || STRIDE == 1 ? 1 : 4) * per;
+                const int step = (P.row_boxes ? 1 : P.rows) * P.pitch * 128;
+                for (int item = item0; item < P.items; item += item_step) {
+                    const TapItem t = tap_item<MT, PAIR>(P, item, side);
+                    if (lane == 0) s_started = s_started + 1;
+                    for (int ks = k0; ks < k1; ++ks) {
+                        wait(a_empty(s), ph);
+                        const uint32_t bar = lead(a_full(s));
+                        const uint32_t dst = sbase + (uint32_t)(s * P.a_bytes) + (P.raster ? (uint32_t)(P.pitch - 1 - t.ox0) * 128u : 0u);
+                        const int c = ks * T::row_ch;
+                        if (side == 0 && lane == 0) mbar_expect_tx(a_full(s), (uint32_t)(P.a_tx * (PAIR ? 2 : 1)));
+                        if (TAPS == 1) {
+                            if (lane == 0) tensor_load4<PAIR>(dst, &xmap, c, t.v0 * 8, 0, 0, bar);
+                        } else {
+                            for (int b = lane; b < boxes; b += 32) {
+                                const int region = STRIDE == 1 ? 0 : div_by(b, per, P.row_boxes ? P.mg_rows : 0u), i = b - region * per;
+                                const int x0 = STRIDE == 1 ? (P.raster ? 0 : t.ox0) - 1 : 2 * t.ox0 - (region & 1);
+                                const TapRow r = tap_row<STRIDE>(P, t, i, region >> 1);
+                                tensor_load4<PAIR>(dst + (uint32_t)(b * step), &xmap, c, x0, r.y, r.img, bar);
                             }
-                            if (++s == P.a_stages) { s = 0; ph ^= 1u; }
                         }
+                        __syncwarp();
+                        if (++s == P.a_stages) { s = 0; ph ^= 1u; }
                     }
                 }
-                __syncwarp();
             } else if (FUSED && P.residual && P.splits == 1) {
                 // ---- the residual into L2, an item ahead of its use --------------------------
                 const int pt = tid - (kEpiWarps + 1) * 32;
@@ -1400,7 +1400,9 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     for (p.tmem_cols = 32; p.tmem_cols < cols;) p.tmem_cols *= 2;
                     // Cycles of a stage: the matrix instructions (nt / 2 each; 46 to issue one and 90 for a tap), or
                     // what they and the copies move through shared memory at 128 bytes a cycle (128 rows of x,
-                    // the block's filters), or what comes from L2.  A pair starts and ends 4000 cycles later, and the
+                    // the block's filters), or what comes from L2.  A pair starts and ends later: 4000 cycles where it
+                    // halves much (fp32: three parts of weights; stride 2: single taps in the slots), else 6000
+                    // (256 -> 256 at 14x14, batch 32, fp16: 12.8 us as pairs, 11.7 without); the
                     // short stages of a product wait 300 cycles for its other block (1842 filters x 5421 rows,
                     // fp32: 77 us as pairs, 57 us without).
                     const double kk = (double)tw.planes / p.stages / 2, taps = tw.taps;
@@ -1413,7 +1415,7 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     const double stage = std::max(std::max(mma, shared), move) + 250.0 + 40.0 * taps / p.tap_group + (p.pair && tw.taps == 1 ? 300.0 : 0.0);
                     const double out = (double)mt * 128 * p.nt * yb / 24.0;
                     const double item = p.per_split * stage;
-                    double c = 3500.0 + (p.pair ? 4000.0 : 0.0);
+                    double c = 3500.0 + (p.pair ? dt == XGEN_F32 || s.stride == 2 ? 4000.0 : 6000.0 : 0.0);
                     if (sp == 1) c += waves * std::max(item, p.acc_bufs == 2 ? out : 0.0) + (p.acc_bufs == 2 ? out : waves * out);
                     else c += waves * (item + 3500.0 + 100.0 * sp + mt * 128.0 * p.nt * 4 / 64.0 + out / sp);
                     if (c < best.cycles * 0.999) { best = p; best.cycles = c; }
