@@ -1163,16 +1163,20 @@ __global__ void tap_expand_dense(uint8_t *img, int c_in, int c_out, int rows, co
 static int tap_cpp(xgen_dtype dt) { return dt == XGEN_I8_I32 ? 16 : 8; }
 static int tap_parts(xgen_dtype dt) { return dt == XGEN_F32 ? 3 : 1; }
 
-// The zeroed image with `extra` bytes of upload scratch behind it, one allocation (a second one that is
-// given back costs a synchronisation and more time than the upload).
+// The zeroed image, and `extra` bytes of upload scratch, which stay with the handle: giving them back
+// would cost a synchronisation and more time than the upload.  One allocation, or two where that keeps
+// both within the driver's small blocks of up to 1 MB (128 -> 128 fp32: 0.96 -> 0.57 ms a handle).
 static xgen_status tap_alloc(TapWeights &tw, xgen_dtype dt, int taps, int c_in, int c_out, size_t extra, uint8_t **scratch) {
     tw.dtype = dt; tw.taps = taps; tw.c_in = c_in; tw.c_out = c_out;
     tw.planes = (c_in + 2 * tap_cpp(dt) - 1) / (2 * tap_cpp(dt)) * 2;
     tw.rows = (c_out + 15) / 16 * 16;
     const size_t bytes = (size_t)tw.planes * taps * tap_parts(dt) * tw.rows * 16;
-    cudaError_t e = cudaMalloc(&tw.dev, bytes + extra);
+    constexpr size_t kSmall = 1 << 20;
+    const bool apart = bytes <= kSmall && extra <= kSmall && bytes + extra > kSmall;
+    cudaError_t e = cudaMalloc(&tw.dev, apart ? bytes : bytes + extra);
+    if (e == cudaSuccess && apart) e = cudaMalloc(&tw.scratch, extra);
     if (e == cudaSuccess) e = cudaMemsetAsync(tw.dev, 0, bytes, 0);
-    *scratch = tw.dev + bytes;
+    *scratch = apart ? tw.scratch : tw.dev + bytes;
     if (e == cudaSuccess) return XGEN_OK;
     cudaGetLastError();
     tap_free(tw);
@@ -1190,7 +1194,8 @@ static xgen_status tap_done(TapWeights &tw, cudaError_t e) {
 
 void tap_free(TapWeights &tw) {
     if (tw.dev) cudaFree(tw.dev);
-    tw.dev = nullptr;
+    if (tw.scratch) cudaFree(tw.scratch);
+    tw.dev = tw.scratch = nullptr;
 }
 
 xgen_status tap_upload_patterns(TapWeights &tw, xgen_dtype dt, int c_in, int c_out, const int16_t *kpat, const uint32_t *kw4,

@@ -22,7 +22,7 @@ EncodeTiledFn encode_tiled_fn();
 // input channels (8 fp16 / bf16, 16 int8); a tensor copy takes any range of filters and planes of a
 // tap at once, so neither the filter tile nor the channels per stage is fixed here.
 struct TapWeights {
-    uint8_t *dev = nullptr;
+    uint8_t *dev = nullptr, *scratch = nullptr;      // the image; what it was made from
     xgen_dtype dtype = XGEN_F32;
     int taps = 9, c_in = 0, c_out = 0;
     int planes = 0;              // a multiple of two (a matrix instruction takes two)
