@@ -328,7 +328,19 @@ __device__ __forceinline__ void tap_emit(const TapParams &P, const uint32_t *st,
     if (c >= P.c_out) return;
     const uint32_t bias = s_bias[c - n0];
     const float scale = FUSED ? s_scale[c - n0] : 0.0f;
-    if (!pool) {
+    if (!pool && !(FUSED && P.residual)) {
+#pragma unroll 4
+        for (int it = 0; it < 16; ++it) {
+            const uint32_t *const row = st + (2 * it + (lane >> 4)) * kStagePitch;
+            const int px = (int)row[16];
+            if (px >= 0) {
+                const size_t off = (size_t)px * P.c_out + c;
+                tap_store1<DT, FUSED>(P, scale, tap_affine1<DT, false>(P, bias, row[lane & 15], off), off);
+            }
+        }
+        return;
+    }
+    if constexpr (FUSED) if (!pool) {
         // eight residuals asked for at a time: one by one, 24 images of 32 x 74 x 58 fp32 channels took
         // 52 us (25 now)
 #pragma unroll 1
@@ -339,12 +351,9 @@ __device__ __forceinline__ void tap_emit(const TapParams &P, const uint32_t *st,
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 px[i] = (int)row0[2 * i * kStagePitch + 16];
-                res[i] = 0u;
-                if (FUSED && P.residual) {
-                    const size_t off = (size_t)max(px[i], 0) * P.c_out + c;
-                    if (DT == XGEN_F16_F32ACC) res[i] = __ldg(static_cast<const unsigned short *>(P.residual) + off);
-                    else res[i] = __ldg(static_cast<const uint32_t *>(P.residual) + off);
-                }
+                const size_t off = (size_t)max(px[i], 0) * P.c_out + c;
+                if (DT == XGEN_F16_F32ACC) res[i] = __ldg(static_cast<const unsigned short *>(P.residual) + off);
+                else res[i] = __ldg(static_cast<const uint32_t *>(P.residual) + off);
             }
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -352,8 +361,7 @@ __device__ __forceinline__ void tap_emit(const TapParams &P, const uint32_t *st,
                 if (DT == XGEN_I8_I32) v += bias + res[i];
                 else {
                     const float r = DT == XGEN_F16_F32ACC ? __half2float(__ushort_as_half((unsigned short)res[i])) : __uint_as_float(res[i]);
-                    v = __float_as_uint(__uint_as_float(v) + __uint_as_float(bias));
-                    if (FUSED && P.residual) v = __float_as_uint(__uint_as_float(v) + r);
+                    v = __float_as_uint(__uint_as_float(v) + __uint_as_float(bias) + r);
                 }
                 if (P.relu) v = tap_max<DT>(v, 0u);
                 if (px[i] >= 0) tap_store1<DT, FUSED>(P, scale, v, (size_t)px[i] * P.c_out + c);
@@ -361,20 +369,36 @@ __device__ __forceinline__ void tap_emit(const TapParams &P, const uint32_t *st,
         }
         return;
     }
-    if constexpr (FUSED)
-#pragma unroll 1
-    for (int it = 0; it < 4; ++it) {
-        const int jp = 2 * it + (lane >> 4);
-        const uint32_t *const row = st + ((jp >> 2) * 16 + (jp & 3) * 2) * kStagePitch;
-        if ((int)row[16] < 0) continue;
-        uint32_t best = 0;
+    if constexpr (FUSED) {
+        // pooled: all sixteen residuals of a lane's four windows asked for before the first is used
+        uint32_t res[16];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t *const r = row + ((q & 1) + (q >> 1) * 8) * kStagePitch;
-            const uint32_t v = tap_affine1<DT, FUSED>(P, bias, r[lane & 15], (size_t)(int)r[16] * P.c_out + c);
-            best = q == 0 ? v : tap_max<DT>(best, v);
+        for (int i = 0; i < 16; ++i) {
+            const int jp = 2 * (i >> 2) + (lane >> 4), q = i & 3;
+            const int px = (int)st[((jp >> 2) * 16 + (jp & 3) * 2 + (q & 1) + (q >> 1) * 8) * kStagePitch + 16];
+            res[i] = 0u;
+            if (P.residual) {
+                const size_t off = (size_t)max(px, 0) * P.c_out + c;
+                if (DT == XGEN_F16_F32ACC) res[i] = __float_as_uint(__half2float(__ushort_as_half(__ldg(static_cast<const unsigned short *>(P.residual) + off))));
+                else res[i] = __ldg(static_cast<const uint32_t *>(P.residual) + off);
+            }
         }
-        tap_store1<DT, FUSED>(P, scale, best, (size_t)(int)row[17] * P.c_out + c);
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            const int jp = 2 * it + (lane >> 4);
+            const uint32_t *const row = st + ((jp >> 2) * 16 + (jp & 3) * 2) * kStagePitch;
+            if ((int)row[16] < 0) continue;
+            uint32_t best = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t v = row[((q & 1) + (q >> 1) * 8) * kStagePitch + (lane & 15)];
+                if (DT == XGEN_I8_I32) v += bias + res[4 * it + q];
+                else v = __float_as_uint(__uint_as_float(v) + __uint_as_float(bias) + __uint_as_float(res[4 * it + q]));
+                if (P.relu) v = tap_max<DT>(v, 0u);
+                best = q == 0 ? v : tap_max<DT>(best, v);
+            }
+            tap_store1<DT, FUSED>(P, scale, best, (size_t)(int)row[17] * P.c_out + c);
+        }
     }
 }
 
