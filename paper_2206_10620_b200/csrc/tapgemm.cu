@@ -1527,6 +1527,8 @@ cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p
     auto aligned = [](const void *q, uintptr_t a) { return ((uintptr_t)q & (a - 1)) == 0; };
     P.vec_x = aligned(c.x, 16) && (size_t)tw.c_in * xb % 16 == 0;
     P.tma = dt != XGEN_F32 && P.vec_x && x_map(tw, s, p, c.x, xm);
+    // a plan for tensor copies has no room for the table of pixels that gathering the rows takes
+    if (!P.tma && p.table_bytes == 0) return cudaErrorInvalidValue;
     P.vec_y = aligned(c.y, 16) && (size_t)tw.c_out * yb % 16 == 0;
     P.y32 = aligned(c.y, 32) && (size_t)tw.c_out * yb % 32 == 0;
     P.vec_r = c.residual && aligned(c.residual, 16) && (size_t)tw.c_out * rb % 16 == 0;

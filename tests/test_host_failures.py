@@ -1,0 +1,72 @@
+"""What the host code does when a CUDA call fails, and what a handle holds: the library's own objects
+linked with a stand-in for the CUDA runtime (fake_cuda.cpp), run in a process of its own."""
+import os
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+from paper_2206_10620_b200 import build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    build.build()
+    objs = [os.path.join(build._OBJ_DIR, os.path.splitext(s)[0] + ".o") for s in build._SOURCES]
+    if not all(os.path.exists(o) for o in objs):
+        build.build(force=True)
+    out = str(tmp_path_factory.mktemp("fake") / "libpatconv_fake.so")
+    cuda = os.path.dirname(os.path.dirname(os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")))
+    subprocess.check_call(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", os.path.join(cuda, "include"),
+                           os.path.join(HERE, "fake_cuda.cpp")] + objs + ["-o", out])
+    return out
+
+
+PRELUDE = """
+import ctypes, os
+import numpy as np
+from paper_2206_10620_b200 import binding, workloads as wl
+fake = ctypes.CDLL(os.environ["XGEN_PATCONV_LIB"])
+fake.fake_live_bytes.restype = fake.fake_launch.restype = ctypes.c_longlong
+binding.lib()
+
+def conv(dtype, ci, co, stride=1, prune=0.5, device=0):
+    d = wl.make_layer(wl.LayerSpec("t", 1, ci, co, 4, 4, stride, dtype, prune, 12, "he", "u01", 0.05, True, 0), seed=1)
+    return binding.Packed(ci, co, stride, dtype, d.masks, d.w, d.pid, device=device)
+
+def gemm(dtype, k, co, **kw):
+    d = wl.make_block_gemm(wl.GemmSpec("t", 4, k, co, 16, 16, 0.5, 0.5, dtype), seed=1)
+    return binding.BlockGemm(k, co, 16, 16, dtype, d.w, d.row_keep, d.col_keep, **kw)
+
+def status(call, *a, **kw):
+    try:
+        call(*a, **kw)
+    except binding.PatconvError as e:
+        return e.status
+    return 0
+
+X, Y, B = 1 << 40, 2 << 40, 3 << 40          # addresses of tensors that nothing reads
+"""
+
+
+def _run(fake_lib, code):
+    env = dict(os.environ, XGEN_PATCONV_LIB=fake_lib, PYTHONPATH=os.path.dirname(HERE))
+    r = subprocess.run([sys.executable, "-c", PRELUDE + textwrap.dedent(code)], env=env, capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("dtype,ci", [("f16", 64), ("i8", 128)])
+def test_a_tensor_map_that_cannot_be_made_is_an_error(fake_lib, dtype, ci):
+    """A plan for copied rows holds no table for gathered ones, so the launch must not fall back to them."""
+    _run(fake_lib, """
+        pk = conv(%r, %d, 64)
+        run = lambda: status(pk.run, X, 2, 20, 20, B, True, Y)
+        assert run() == 0 and fake.fake_launches() > 0
+        n = fake.fake_launches()
+        fake.fake_fail_encode(1)             # (the plan, with the map of the weights, is kept: this is x's)
+        assert run() == 6 and fake.fake_launches() == n
+        assert run() == 0 and fake.fake_launches() == n + 1
+    """ % (dtype, ci))
