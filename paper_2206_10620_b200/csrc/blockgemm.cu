@@ -446,10 +446,17 @@ static const void *kernel_for(xgen_dtype dt, int ks) {
 static xgen_status upload_stream(xgen_blockgemm_packed *h) {
     const Host &H = h->host;
     const size_t sb = std::max<size_t>(H.stream.size() * 4, 16), gb = H.seg_off.size() * 4;
-    if (cudaMalloc(&h->d_stream, sb) != cudaSuccess || cudaMalloc(&h->d_seg, gb) != cudaSuccess) return XGEN_ERR_ALLOC;
-    if ((!H.stream.empty() && cudaMemcpy(h->d_stream, H.stream.data(), H.stream.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) ||
-        cudaMemcpy(h->d_seg, H.seg_off.data(), gb, cudaMemcpyHostToDevice) != cudaSuccess) return XGEN_ERR_CUDA;
-    return XGEN_OK;
+    xgen_status st = XGEN_OK;
+    if (cudaMalloc(&h->d_stream, sb) != cudaSuccess || cudaMalloc(&h->d_seg, gb) != cudaSuccess) st = XGEN_ERR_ALLOC;
+    else if ((!H.stream.empty() && cudaMemcpy(h->d_stream, H.stream.data(), H.stream.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess) ||
+             cudaMemcpy(h->d_seg, H.seg_off.data(), gb, cudaMemcpyHostToDevice) != cudaSuccess) st = XGEN_ERR_CUDA;
+    if (st != XGEN_OK) {                 // both are there, or neither: a later run asks by the first
+        cudaGetLastError();
+        if (h->d_stream) cudaFree(h->d_stream);
+        if (h->d_seg) cudaFree(h->d_seg);
+        h->d_stream = nullptr; h->d_seg = nullptr;
+    }
+    return st;
 }
 
 // The matrix path's plan for a row count, from the handle's small cache or made now.

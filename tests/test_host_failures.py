@@ -70,3 +70,19 @@ def test_a_tensor_map_that_cannot_be_made_is_an_error(fake_lib, dtype, ci):
         assert run() == 6 and fake.fake_launches() == n
         assert run() == 0 and fake.fake_launches() == n + 1
     """ % (dtype, ci))
+
+
+def test_an_upload_that_fails_half_way_leaves_nothing(fake_lib):
+    """The block-pruned product's command stream, uploaded by the first run that needs it: a run after a
+    failed one uploads again."""
+    _run(fake_lib, """
+        g = gemm("f32", 64, 48)
+        run = lambda: status(g.run, X, 32, B, True, Y)
+        held, n = fake.fake_live_bytes(), fake.fake_launches()
+        for nth in (1, 2):
+            fake.fake_fail_encode(1)         # the matrix path cannot run, so the stream is asked for
+            fake.fake_fail_alloc(nth)
+            assert run() == 5 and fake.fake_launches() == n and fake.fake_live_bytes() == held
+        fake.fake_fail_encode(1)
+        assert run() == 0 and fake.fake_launches() == n + 1 and fake.fake_live_bytes() > held
+    """)
