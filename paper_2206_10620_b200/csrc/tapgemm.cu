@@ -774,7 +774,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     if (item >= P.items) return;
                     const TapItem t = tap_item<MT, PAIR>(P, item, side);
                     for (int i = pt; i < 128 * MT * lines; i += kProdThreads - 32) {
-                        const int m = i / lines, at = min((i - m * lines) * 128, row - 4);
+                        const int m = i / lines, at = (i - m * lines) * 128;       // (always below `row`: of one filter it may be 2 bytes)
                         const int px = tap_pixel<TAPS>(P, t, m).pix;
                         if (px >= 0)
                             asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const char *>(P.residual) +

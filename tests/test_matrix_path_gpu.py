@@ -84,6 +84,30 @@ def test_fused_operators_behind_tiles_and_splits(dtype, co, pool):
                 assert (np.abs(got - ref) <= bound).all()
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f16", "i8"])
+@pytest.mark.parametrize("co", [1, 2, 65, 129])
+def test_residual_of_a_narrow_last_filter_tile(dtype, co):
+    """The residual is asked for a tile ahead: rows of a few bytes, the tensor's ends included."""
+    import torch
+    n, ci, h, w = 2, 16, 9, 17
+    d = _layer(dtype, n, ci, co, h, w, seed=co)
+    size = n * h * w * co
+    res = (wl.integers(5, "AUX", 1, size, -9999, 9999).astype(np.int32) if dtype == "i8"
+           else (wl.normal(5, "AUX", 1, size) * 0.5).astype(np.float32 if dtype == "f32" else np.float16)).reshape(n, h, w, co)
+    pk = pack(d)
+    x, b, r = (torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (d.x, d.bias, res))
+    buf, y = guarded_output((n, h, w, co), {"f32": torch.float32, "f16": torch.float16, "i8": torch.int32}[dtype])
+    pk.run_fused(x.data_ptr(), n, h, w, b.data_ptr(), y.data_ptr(), relu=False, residual_ptr=r.data_ptr())
+    pk.sync()
+    check_guards(buf)
+    got, ref = y.cpu().numpy(), oracle.conv_fused(d.x, d.w, d.pid, d.masks, bias=d.bias, relu=False, residual=res)
+    if dtype == "i8":
+        assert np.array_equal(got.astype(np.int64), ref.astype(np.int64))
+    else:
+        pre, S = oracle.conv(d.x, d.w, d.pid, d.masks, bias=d.bias, relu=False, with_scale=True)
+        assert (np.abs(got - ref) <= TOL[dtype] * np.maximum(np.abs(pre + res), 0.01 * (S + np.abs(res))) + 1e-30).all()
+
+
 def test_fp32_sums_keep_fp32_precision():
     """Long sums of positive terms, where a truncating accumulator would show: the error stays that of
     a few roundings, and operands keep all of their bits."""
