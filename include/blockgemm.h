@@ -96,6 +96,23 @@ xgen_status xgen_blockgemm_pack(const xgen_blockgemm_desc *desc, const void *den
 xgen_status xgen_blockgemm_run(const xgen_blockgemm_packed *packed, const void *x_dev, int64_t m_rows,
                                const void *bias_dev, int32_t relu, void *y_dev, void *cuda_stream);
 
+/*
+ * Synchronise the stream and report the first CUDA error seen, as a status (XGEN_OK,
+ * XGEN_ERR_CUDA).  The kernels contain no unbounded waits: a wait (for a staged tile, staged
+ * weights or a free stage) that runs out of its bound of 2 s marks the handle, the kernel still
+ * ends, and this call then returns XGEN_ERR_TIMEOUT once (the results are invalid;
+ * xgen_blockgemm_run has returned XGEN_OK long before: it only enqueues).
+ */
+xgen_status xgen_blockgemm_last_status(const xgen_blockgemm_packed *packed, void *cuda_stream);
+
+/*
+ * Testing aid, not for production use (the paper has no counterpart): with extra > 0 the stages of
+ * every later launch wait, 50 ms at most, for `extra` arrivals more than will ever come, so that the
+ * launch ends with XGEN_ERR_TIMEOUT in xgen_blockgemm_last_status; 0 restores normal operation.
+ * A handle packed with warps_per_block has no such waits.  Errors: INVALID_ARG.
+ */
+xgen_status xgen_blockgemm_test_expect_arrivals(xgen_blockgemm_packed *packed, int32_t extra);
+
 /* Fill *stats (see xgen_blockgemm_stats). */
 xgen_status xgen_blockgemm_query(const xgen_blockgemm_packed *packed, xgen_blockgemm_stats *stats);
 

@@ -379,8 +379,9 @@ xgen_status xgen_patconv_plan_info(const xgen_patconv_packed *packed, int32_t n,
 
 /*
  * Testing aid, not for production use (the paper has no counterpart): make every later
- * planned launch of waiting splits of the handle wait for `extra` arrivals more than its own blocks
- * will ever deliver.  With extra > 0 the wait of every block runs out after the handle's
+ * launch of the handle that takes the matrix path, or runs waiting splits, wait for `extra` arrivals
+ * (of staged input; of the blocks of a split) more than will ever
+ * come.  With extra > 0 the wait of every block runs out after the handle's
  * wait limit (xgen_patconv_tuning.wait_limit_ms), the kernel ends normally, and
  * xgen_patconv_last_status returns XGEN_ERR_TIMEOUT once; extra = 0 restores normal
  * operation.  This is how the tests exercise the bounded waits without hanging or

@@ -30,7 +30,7 @@ EXPORTS = ["xgen_patconv_pack", "xgen_patconv_run", "xgen_patconv_run_static_scr
            "xgen_patconv_last_status", "xgen_patconv_free", "xgen_strerror",
            "xgen_patconv_launch_count", "xgen_patconv_probe", "xgen_patconv_run_fused",
            "xgen_blockgemm_pack", "xgen_blockgemm_run", "xgen_blockgemm_query", "xgen_blockgemm_view",
-           "xgen_blockgemm_free",
+           "xgen_blockgemm_free", "xgen_blockgemm_last_status", "xgen_blockgemm_test_expect_arrivals",
            "xgen_dwconv_pack", "xgen_dwconv_run", "xgen_dwconv_query", "xgen_dwconv_free"]
 
 
@@ -166,6 +166,8 @@ def lib():
         L.xgen_blockgemm_run.argtypes = [P, P, ctypes.c_int64, P, I, P, P]
         L.xgen_blockgemm_query.argtypes = [P, ctypes.POINTER(GemmStats)]
         L.xgen_blockgemm_view.argtypes = [P, ctypes.POINTER(GemmHostView)]
+        L.xgen_blockgemm_last_status.argtypes = [P, P]
+        L.xgen_blockgemm_test_expect_arrivals.argtypes = [P, I]
         L.xgen_blockgemm_free.argtypes = [P]
         L.xgen_blockgemm_free.restype = None
         L.xgen_dwconv_pack.argtypes = [ctypes.POINTER(DwDesc), P, P, ctypes.c_int, ctypes.POINTER(P)]
@@ -384,6 +386,12 @@ class BlockGemm:
         status = _calls.gemm(self._h.value, x_ptr, m, bias_ptr, relu, y_ptr, stream)
         if status:
             raise PatconvError(status, "xgen_blockgemm_run")
+
+    def sync(self, stream=0):
+        _check(lib().xgen_blockgemm_last_status(self._h, stream or None), "xgen_blockgemm_last_status")
+
+    def test_expect_arrivals(self, extra):
+        _check(lib().xgen_blockgemm_test_expect_arrivals(self._h, int(extra)), "xgen_blockgemm_test_expect_arrivals")
 
 
 class Depthwise:

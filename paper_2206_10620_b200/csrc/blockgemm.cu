@@ -75,6 +75,7 @@ struct xgen_blockgemm_packed {
     std::mutex tap_mu;
     struct Entry { int64_t m = 0; patconv::TapPlan plan; uint64_t stamp = 0; } tap_cache[4];
     uint64_t tap_stamp = 0;
+    int hook_extra_arrivals = 0;        // testing aid: arrivals that a launch waits for beyond its own
 };
 
 namespace blockgemm {
@@ -577,7 +578,8 @@ xgen_status xgen_blockgemm_run(const xgen_blockgemm_packed *hc, const void *x, i
         const bool fits = tap_plan_of(h, ts, plan);
         cudaError_t e = cudaSuccess;
         if (fits) {
-            const patconv::TapCall call{x, y, bias, nullptr, nullptr, 0, relu, 0, nullptr, 2000000u, true};
+            const patconv::TapCall call{x, y, bias, nullptr, nullptr, 0, relu, 0, h->tap.status, h->hook_extra_arrivals ? 50000u : 2000000u,
+                                         h->hook_extra_arrivals, true};
             e = patconv::tap_launch(h->tap, ts, plan, call, (cudaStream_t)stream);
             if (e != cudaSuccess) cudaGetLastError();
         }
@@ -623,6 +625,29 @@ xgen_status xgen_blockgemm_run(const xgen_blockgemm_packed *hc, const void *x, i
     if (st != XGEN_OK) cudaGetLastError();
     if (prev != h->device) cudaSetDevice(prev);
     return st;
+}
+
+xgen_status xgen_blockgemm_last_status(const xgen_blockgemm_packed *h, void *stream) {
+    if (!h) return XGEN_ERR_INVALID_ARG;
+    if (h->device < 0) return XGEN_ERR_CUDA;
+    int prev = 0;
+    if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
+    if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
+    xgen_status st = XGEN_OK;
+    int flag = 0;
+    if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess || cudaGetLastError() != cudaSuccess) st = XGEN_ERR_CUDA;
+    else if (h->tap.status) {                      // (the command stream's kernel has no waits)
+        if (cudaMemcpy(&flag, h->tap.status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) st = XGEN_ERR_CUDA;
+        else if (flag) st = cudaMemset(h->tap.status, 0, sizeof(int)) == cudaSuccess ? XGEN_ERR_TIMEOUT : XGEN_ERR_CUDA;
+    }
+    if (prev != h->device) cudaSetDevice(prev);
+    return st;
+}
+
+xgen_status xgen_blockgemm_test_expect_arrivals(xgen_blockgemm_packed *h, int32_t extra) {
+    if (!h || extra < 0) return XGEN_ERR_INVALID_ARG;
+    h->hook_extra_arrivals = extra;
+    return XGEN_OK;
 }
 
 xgen_status xgen_blockgemm_query(const xgen_blockgemm_packed *h, xgen_blockgemm_stats *stats) {

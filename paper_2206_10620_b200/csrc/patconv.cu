@@ -1432,7 +1432,7 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
         cudaError_t e = cudaSuccess;
         if (fits) {
             const TapCall call{x, y, bias, residual, rq_scale, ep ? ep->requant_zero_point : 0, relu, pool,
-                               h->d_status, h->wait_us, !h->tuning.no_launch_overlap};
+                               h->d_status, h->wait_us, h->hook_extra_arrivals, !h->tuning.no_launch_overlap};
             if (log_enabled())
                 fprintf(stderr, "libpatconv: matrix path, %d blocks = %d items (form %d, %d row tiles x %d columns x %d filter tiles of %d) x %d splits, %d x 128 pixels%s, %d planes x %d stages, %d + %d x %d taps buffers%s, %zu bytes shared, %.0f cycles expected\n",
                         plan.grid, plan.items, plan.raster ? 2 : plan.straddle, plan.row_tiles, plan.segs, plan.nblk, plan.nt, plan.splits, plan.mt, plan.pair ? " (block pairs)" : "", plan.pl, plan.stages,

@@ -65,25 +65,27 @@ template <bool CLUSTER> __device__ __forceinline__ bool mbar_try(uint32_t mbar, 
 
 // Wait for an mbarrier phase with a bound in time (limit_us microseconds, plus a cap on the
 // polls in case the timer stands still): on expiry the block-wide abort flag and the device
-// status word are set and every later wait returns at once; the warps then leave their
-// loops, so the kernel still runs to its end (releasing tensor memory) with results the
-// host can tell are invalid.  CLUSTER: what other blocks of the cluster wrote before they
-// arrived is seen too.
+// status word are set.  Every later wait of the block is given 100 microseconds at most, more than
+// any copy or matrix instruction takes: roles that go on whatever a wait said stay in step, no more
+// copies are in flight than in an ordinary run, and those that are waited for have landed.  The kernel
+// still runs to its end (releasing tensor memory) with results the host can tell are invalid.
+// CLUSTER: what other blocks of the cluster wrote before they arrived is seen too.
 template <bool CLUSTER>
 __device__ __noinline__ bool mbar_wait_long(uint32_t mbar, uint32_t parity, volatile int *abort_flag, int *status,
                                             uint32_t limit_us) {
     uint64_t t0 = 0;
     for (uint32_t it = 0; it < 40000000u; ++it) {
         if (mbar_try<CLUSTER>(mbar, parity)) return true;
-        if (*abort_flag) return false;
         if ((it & 7u) == 7u) {
             const uint64_t t = global_ns();
             if (t0 == 0) t0 = t;
-            else if (t - t0 > (uint64_t)limit_us * 1000ull) break;
+            else if (t - t0 > (uint64_t)(*abort_flag ? min(limit_us, 100u) : limit_us) * 1000ull) break;
         }
     }
-    *abort_flag = 1;
-    if (status) atomicExch(status, 1);
+    if (!*abort_flag) {
+        *abort_flag = 1;
+        if (status) atomicExch(status, 1);
+    }
     return false;
 }
 template <bool CLUSTER = false>

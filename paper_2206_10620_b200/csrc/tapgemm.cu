@@ -69,6 +69,7 @@ struct TapParams {
     const void *x; void *y; const void *bias; const void *residual; const float *rq_scale;
     int *status;
     uint32_t wait_us;
+    int hold;                                   // testing aid: arrivals that the stages of x wait for beyond their own
     int rq_zero, relu, pool;
     int n, h, w, ho, wo, c_in, c_out;
     int po, pw;                                 // stored extents
@@ -694,7 +695,11 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
     auto acc_full = [&](int s) { return bars + 8u * (2 * kMaxA + 2 * kMaxB + s); };
     auto acc_empty = [&](int s) { return bars + 8u * (2 * kMaxA + 2 * kMaxB + 2 + s); };
     const uint32_t all_done = bars + 8u * (2 * kMaxA + 2 * kMaxB + 4);
-    auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait<PAIR>(bar, parity, &s_abort, P.status, P.wait_us); };
+    // Nothing is steered by what a wait says: lanes of a warp and warps of a role may see it give up at different
+    // places and would part, ahead of a barrier or an instruction that takes them all.  A launch that gave up goes
+    // through all of its work, on whatever the buffers hold, and is reported.
+    auto wait = [&](uint32_t bar, uint32_t parity) { mbar_wait<PAIR>(bar, parity, &s_abort, P.status, P.wait_us); };
+    auto wait_warp = [&](uint32_t bar, uint32_t parity) { wait(bar, parity); __syncwarp(); };
     // Clusters: a pair of blocks (PAIR), or the blocks (pairs) that split an item's reduction.  The even
     // block of a pair holds the barriers that say "operands are there" and "sums have been read".
     const int csize = (PAIR ? 2 : 1) * P.splits;
@@ -710,7 +715,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
     asm volatile("griddepcontrol.launch_dependents;");
     if (tid == 0) {
         s_abort = 0; s_started = 0;
-        for (int i = 0; i < P.a_stages; ++i) { mbar_init(a_full(i), P.tma ? 1 : (PAIR ? 2 : 1) * kProdWarps); mbar_init(a_empty(i), 1); }
+        for (int i = 0; i < P.a_stages; ++i) { mbar_init(a_full(i), (P.tma ? 1 : (PAIR ? 2 : 1) * kProdWarps) + P.hold); mbar_init(a_empty(i), 1); }
         for (int i = 0; i < P.b_slots; ++i) { mbar_init(b_full(i), 1); mbar_init(b_empty(i), 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(acc_full(i), 1); mbar_init(acc_empty(i), (PAIR ? 2 : 1) * kEpiWarps); }
         mbar_init(all_done, 1);
@@ -747,7 +752,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     const TapItem t = tap_item<MT, PAIR>(P, item, side);
                     if (lane == 0) s_started = s_started + 1;
                     for (int ks = k0; ks < k1; ++ks) {
-                        wait(a_empty(s), ph);
+                        wait_warp(a_empty(s), ph);
                         const uint32_t bar = lead(a_full(s));
                         const uint32_t dst = sbase + (uint32_t)(s * P.a_bytes) + (P.raster ? (uint32_t)(P.pitch - 1 - t.ox0) * 128u : 0u);
                         const int c = ks * T::row_ch;
@@ -793,18 +798,17 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             const int pt = tid - kEpiWarps * 32;
             int s = 0;
             uint32_t ph = 1;
-            bool ok = true, par = false;
+            bool par = false;
             const char *const x = static_cast<const char *>(P.x);
             const int total = kF32 ? P.pixels << P.pl_log : P.pixels * 8;
-            for (int item = item0; item < P.items && ok; item += item_step, par = !par) {
+            for (int item = item0; item < P.items; item += item_step, par = !par) {
                 const TapItem t = tap_item<MT, PAIR>(P, item, side);
                 int *const pix = reinterpret_cast<int *>(smem + P.tab_off) + (par ? P.pixels : 0);
                 for (int p = pt; p < P.pixels; p += kProdThreads) pix[p] = tap_source<STRIDE, TAPS>(P, t, p);
                 asm volatile("bar.sync 1, %0;" ::"n"(kProdThreads) : "memory");
                 if (item == item0) asm volatile("griddepcontrol.wait;" ::: "memory");
                 for (int ks = k0; ks < k1; ++ks) {
-                    ok = wait(a_empty(s), ph);
-                    if (!ok) break;
+                    wait_warp(a_empty(s), ph);
                     const uint32_t dst = sbase + (uint32_t)(s * P.a_bytes);
                     const int npl = min(P.pl, planes - ks * P.pl);
                     constexpr int U = kF32 ? 4 : 2;          // pieces of a thread in flight
@@ -975,7 +979,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 }
                 if (P.resident) break;
             }
-            // Nothing may land in shared memory after this block has gone (a wait above may have given up).
+            // Nothing may land in shared memory after this block has gone (the wait for it may have given up).
             for (int q = max(0, issued - P.b_slots); q < issued && side == 0; ++q)
                 for (int it = 0; it < 1000000 && !mbar_ready(b_full(q % P.b_slots), (uint32_t)(q / P.b_slots) & 1u); ++it) {}
         }
@@ -1007,8 +1011,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
         }
         int buf = 0;
         uint32_t ph = 0;
-        bool ok = true;
-        for (int item = item0; item < P.items && ok; item += item_step) {
+        for (int item = item0; item < P.items; item += item_step) {
             const TapItem t = tap_item<MT, PAIR>(P, item, side);
             const TapPixel at = tap_pixel<TAPS>(P, t, sub * 128 + m);
             const int pix = at.pix, out = at.out;
@@ -1045,8 +1048,8 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 uint32_t sum[2][32];                 // chunks `group` and `group` + kGroups
 #pragma unroll
                 for (int i = 0; i < 64; ++i) sum[i / 32][i % 32] = 0u;
-                for (int ks = k0; ks < k1 && ok; ++ks) {
-                    ok = wait(acc_full(buf), ph);
+                for (int ks = k0; ks < k1; ++ks) {
+                    wait_warp(acc_full(buf), ph);
                     tc_fence_after();
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {
@@ -1067,17 +1070,17 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     release();
                 }
 #pragma unroll 1
-                for (int q = group; q < chunks && ok; q += kGroups) {
+                for (int q = group; q < chunks; q += kGroups) {
                     finish(sum[0], 32 * q);
 #pragma unroll
                     for (int i = 0; i < 32; ++i) sum[0][i] = sum[1][i];
                 }
             } else {
-                ok = wait(acc_full(buf), ph);
+                wait_warp(acc_full(buf), ph);
                 tc_fence_after();
                 const uint32_t ta = tmem + lanes + (uint32_t)((buf * MT + sub) * P.nt);
 #pragma unroll 1
-                for (int q = group; q < chunks && ok; q += kGroups) {
+                for (int q = group; q < chunks; q += kGroups) {
                     uint32_t r[32];
                     tmem_ld16(ta + 32 * q, r);
                     tmem_ld16(ta + 32 * q + 16, r + 16);
@@ -1194,13 +1197,14 @@ static xgen_status tap_alloc(TapWeights &tw, xgen_dtype dt, int taps, int c_in, 
     tw.dtype = dt; tw.taps = taps; tw.c_in = c_in; tw.c_out = c_out;
     tw.planes = (c_in + 2 * tap_cpp(dt) - 1) / (2 * tap_cpp(dt)) * 2;
     tw.rows = (c_out + 15) / 16 * 16;
-    const size_t bytes = (size_t)tw.planes * taps * tap_parts(dt) * tw.rows * 16;
+    const size_t image = (size_t)tw.planes * taps * tap_parts(dt) * tw.rows * 16, bytes = image + 16;     // and the status word
     constexpr size_t kSmall = 1 << 20;
     const bool apart = bytes <= kSmall && extra <= kSmall && bytes + extra > kSmall;
     cudaError_t e = cudaMalloc(&tw.dev, apart ? bytes : bytes + extra);
     if (e == cudaSuccess && apart) e = cudaMalloc(&tw.scratch, extra);
     if (e == cudaSuccess) e = cudaMemsetAsync(tw.dev, 0, bytes, 0);
     *scratch = apart ? tw.scratch : tw.dev + bytes;
+    tw.status = reinterpret_cast<int *>(tw.dev + image);
     if (e == cudaSuccess) return XGEN_OK;
     cudaGetLastError();
     tap_free(tw);
@@ -1220,6 +1224,7 @@ void tap_free(TapWeights &tw) {
     if (tw.dev) cudaFree(tw.dev);
     if (tw.scratch) cudaFree(tw.scratch);
     tw.dev = tw.scratch = nullptr;
+    tw.status = nullptr;
 }
 
 xgen_status tap_upload_patterns(TapWeights &tw, xgen_dtype dt, int c_in, int c_out, const int16_t *kpat, const uint32_t *kw4,
@@ -1489,7 +1494,7 @@ cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p
     const int yb = c.rq_scale ? 1 : dt == XGEN_F16_F32ACC ? 2 : 4, rb = dt == XGEN_F16_F32ACC ? 2 : 4;
     TapParams P{};
     P.x = c.x; P.y = c.y; P.bias = c.bias; P.residual = c.residual; P.rq_scale = c.rq_scale;
-    P.status = c.status; P.wait_us = c.wait_us;
+    P.status = c.status; P.wait_us = c.wait_us; P.hold = std::min(c.hold, 1000);       // (a barrier counts to 2^20)
     P.rq_zero = c.rq_zero; P.relu = c.relu ? 1 : 0; P.pool = c.pool;
     P.n = s.n; P.h = s.h; P.w = s.w;
     P.ho = (s.h - 1) / s.stride + 1; P.wo = (s.w - 1) / s.stride + 1;

@@ -23,6 +23,7 @@ EncodeTiledFn encode_tiled_fn();
 // tap at once, so neither the filter tile nor the channels per stage is fixed here.
 struct TapWeights {
     uint8_t *dev = nullptr, *scratch = nullptr;      // the image; what it was made from
+    int *status = nullptr;       // behind the image: set by a kernel whose bounded wait ran out
     xgen_dtype dtype = XGEN_F32;
     int taps = 9, c_in = 0, c_out = 0;
     int planes = 0;              // a multiple of two (a matrix instruction takes two)
@@ -59,6 +60,7 @@ struct TapCall {
     const void *x; void *y; const void *bias; const void *residual; const float *rq_scale;
     int rq_zero, relu, pool;
     int *status; uint32_t wait_us;
+    int hold;                    // testing aid: every stage of x waits for this many arrivals that never come
     bool overlap;                // programmatic stream serialisation
 };
 

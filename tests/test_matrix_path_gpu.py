@@ -146,6 +146,64 @@ def test_block_pruned_product(dtype, m, k, co):
         assert (np.abs(y.cpu().numpy().astype(np.float64) - ref) <= bound).all()
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f16", "i8"])
+@pytest.mark.parametrize("shape", [
+    (1, 16, 32, 8, 8),        # one stage, one item
+    (40, 64, 64, 40, 40),     # several items a block (fp32: pairs of blocks)
+    (32, 256, 256, 28, 28),   # pairs of blocks, several stages
+    (2, 48, 200, 60, 60),     # several filter tiles
+    (1, 512, 96, 14, 14),     # split over a cluster
+])
+def test_a_wait_that_runs_out_is_reported(dtype, shape):
+    """Stages told to wait for an arrival that never comes: every wait ends at its (shortened) limit, the
+    kernel ends by itself and stays inside its tensors, the timeout is reported once, and the next run is
+    as the one before."""
+    import torch
+    n, ci, co, h, w = shape
+    d = _layer(dtype, n, ci, co, h, w, seed=sum(shape))
+    pk = pack(d)
+    pk.plan(n, h, w, wait_limit_ms=20)
+    assert pk.plan_info(n, h, w)["matrix_path"] == 1
+    before = run_gpu(pk, d.x, d.bias, True)
+    pk.test_expect_arrivals(1)
+    x, b = torch.from_numpy(d.x).cuda(), torch.from_numpy(d.bias).cuda()
+    buf, y = guarded_output((n, h, w, co), {"f32": torch.float32, "f16": torch.float16, "i8": torch.int32}[dtype])
+    pk.run(x.data_ptr(), n, h, w, b.data_ptr(), True, y.data_ptr())            # only enqueues: OK
+    with pytest.raises(binding.PatconvError) as e:
+        pk.sync()
+    assert e.value.status == 7
+    check_guards(buf)
+    pk.sync()                                                                  # reported once
+    pk.test_expect_arrivals(0)
+    assert np.array_equal(run_gpu(pk, d.x, d.bias, True), before)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("m,k,co", [(5, 16, 32), (40000, 200, 264), (96, 1000, 500)])
+def test_a_wait_of_the_block_pruned_product_that_runs_out_is_reported(dtype, m, k, co):
+    import torch
+    d = wl.make_block_gemm(wl.GemmSpec("t", m, k, co, 16, 16, 0.5, 0.5, dtype), seed=m + k)
+    g = binding.BlockGemm(k, co, 16, 16, dtype, d.w, d.row_keep, d.col_keep)
+    x, b = torch.from_numpy(d.x).cuda(), torch.from_numpy(d.bias).cuda()
+    buf, y = guarded_output((m, co), torch.float32 if dtype == "f32" else torch.float16)
+    run = lambda: g.run(x.data_ptr(), m, b.data_ptr(), True, y.data_ptr())
+    g.test_expect_arrivals(1)
+    run()
+    with pytest.raises(binding.PatconvError) as e:
+        g.sync()
+    assert e.value.status == 7
+    check_guards(buf)
+    g.sync()
+    g.test_expect_arrivals(0)
+    y.fill_(777.0)
+    run()
+    g.sync()
+    rows = min(m, 512)
+    ref, S = oracle.block_gemm(d.x[-rows:], d.w, d.row_keep, d.col_keep, 16, 16, bias=d.bias, relu=True, with_scale=True)
+    bound = TOL[dtype] * np.maximum(np.abs(ref), 0.01 * S) + 2.0 ** -25
+    assert (np.abs(y.cpu().numpy()[-rows:].astype(np.float64) - ref) <= bound).all()
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f16"])
 @pytest.mark.parametrize("stride", [1, 2])
 @pytest.mark.parametrize("shape", [(1, 6, 1, 1), (2, 2, 13, 5), (1, 20, 40, 33), (40, 64, 17, 30), (3, 7, 2, 9)])
