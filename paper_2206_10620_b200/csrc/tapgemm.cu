@@ -2,8 +2,8 @@
 //
 // What is left of a pruned layer is 4/9 x (1 - prune rate) of a dense one, but the matrix units
 // are 22 times (fp16) to 44 times (int8) the packed-FMA pipe, so the layer is run dense: pruned
-// weights are zeros of the operand.  (0 x infinity is NaN there, as in the definition written out
-// over the masked dense tensor.)
+// weights are zeros of the operand.  0 x infinity is NaN there, so sums that come out infinite or NaN
+// are computed anew from the kept weights alone (tap_anew).
 //
 // The input of a tile with its halo is staged once per group of channels and serves all nine taps:
 // in shared memory a tap is only another start address.  A tile is 128 (256) output pixels, either
@@ -41,6 +41,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -83,6 +84,7 @@ struct TapParams {
     int b_off, tab_off, stage_off, sum_off;     // bytes into dynamic shared memory
     int tmem_cols, acc_bufs, staged;
     int tap_start[9];                           // first staged entry of a tap
+    const uint8_t *wimg; int w_rows;            // the weight image (TapWeights)
     int tma, row_boxes, a_tx;                        // x comes by tensor copies; a copy per staged row
     int vec_x;                                  // 16-byte pieces of x can be copied as they are
     int vec_y, vec_r, y32;                      // 16-byte (32-byte) pieces of y / the residual can be moved whole
@@ -191,6 +193,12 @@ __device__ __forceinline__ uint32_t pack_codes(int a, int b, int c, int d) {
 __device__ __forceinline__ void add2(uint32_t &a0, uint32_t &a1, uint32_t b0, uint32_t b1) {
     asm("{\n .reg .b64 a, b;\n mov.b64 a, {%0, %1};\n mov.b64 b, {%2, %3};\n add.rn.f32x2 a, a, b;\n mov.b64 {%0, %1}, a;\n}"
         : "+r"(a0), "+r"(a1) : "r"(b0), "r"(b1));
+}
+
+// (a0, a1) stays 0 while (v0, v1) is finite, and is NaN for good once it is not.
+__device__ __forceinline__ void nan_of(uint32_t &a0, uint32_t &a1, uint32_t v0, uint32_t v1) {
+    asm("{\n .reg .b64 a, v;\n mov.b64 a, {%0, %1};\n mov.b64 v, {%2, %3};\n fma.rn.f32x2 a, v, %4, a;\n mov.b64 {%0, %1}, a;\n}"
+        : "+r"(a0), "+r"(a1) : "r"(v0), "r"(v1), "l"(0ull));
 }
 
 // Store W results of one pixel, converted; whole 16- or 32-byte pieces where the tensor allows it.
@@ -539,9 +547,82 @@ __device__ __forceinline__ void tap_direct(const TapParams &P, const uint32_t *s
     }
 }
 
+// ---- sums that are not finite -----------------------------------------------------
+// The matrix units multiply pruned weights too, as zeros, so an infinity or NaN of x reaches every
+// filter there, and in fp32 the parts of an infinity do not add up to one.  Every such sum is infinite or
+// NaN (an overflow of finite operands as well), and the layer's own value takes its place: the kept
+// weights of the filter, in fp32, in the order of the image, where kept zeros are -0.  Slow -- a lane reads
+// its filter's weights from end to end -- and bounded: 512 channels take 60 us a sum.
+template <int DT, int STRIDE, int TAPS>
+__device__ __noinline__ uint32_t tap_anew(const TapParams &P, int pix, int oc) {
+    constexpr int cpp = TapTraits<DT>::cpp, parts = TapTraits<DT>::parts;
+    int img = 0, oy = 0, ox = 0;
+    if (TAPS == 9) {
+        const int row = pix / P.wo;
+        ox = pix - row * P.wo;
+        img = row / P.ho;
+        oy = row - img * P.ho;
+    }
+    const size_t part = (size_t)P.w_rows * 16, step = part * parts;
+    const uint8_t *w = P.wimg + (size_t)oc * 16;
+    float sum = 0.0f;
+    for (int c0 = 0; c0 < P.c_in; c0 += cpp)
+        for (int t = 0; t < TAPS; ++t, w += step) {
+            const uint4 a = __ldg(reinterpret_cast<const uint4 *>(w));
+            if ((a.x | a.y | a.z | a.w) == 0u) continue;
+            size_t px = (size_t)pix;
+            bool in = true;
+            if (TAPS == 9) {
+                const int iy = oy * STRIDE + t / 3 - 1, ix = ox * STRIDE + t % 3 - 1;
+                in = (unsigned)iy < (unsigned)P.h && (unsigned)ix < (unsigned)P.w;
+                px = ((size_t)img * P.h + iy) * P.w + ix;
+            }
+            for (int e = 0; e < cpp; ++e) {
+                const unsigned short bits = __ldg(reinterpret_cast<const unsigned short *>(w) + e);
+                if (bits == 0) continue;                                // pruned
+                float wv, xv = 0.0f;
+                const size_t at = px * P.c_in + c0 + e;
+                if (DT == XGEN_F32) {
+                    const float p1 = __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short *>(w + part) + e) << 16);
+                    const float p2 = __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short *>(w + 2 * part) + e) << 16);
+                    wv = __uint_as_float((uint32_t)bits << 16) + (p1 + p2);       // (exact)
+                    if (in) xv = __ldg(static_cast<const float *>(P.x) + at);
+                } else {
+                    wv = __half2float(__ushort_as_half(bits));
+                    if (in) xv = __half2float(__ushort_as_half(__ldg(static_cast<const unsigned short *>(P.x) + at)));
+                }
+                sum = fmaf(wv, xv, sum);
+            }
+            if (sum != sum) return __float_as_uint(sum);
+        }
+    return __float_as_uint(sum);
+}
+// The sums of N channels of a pixel, from channel c on, with those that are not finite computed anew; where all
+// are finite that is N / 2 packed multiply-adds and a branch.
+template <int N> __device__ __forceinline__ bool all_finite(const uint32_t (&v)[N]) {
+    uint32_t a0 = 0u, a1 = 0u, b0 = 0u, b1 = 0u;
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+        nan_of(a0, a1, v[i], v[i + 1]);
+        nan_of(b0, b1, v[i + 2], v[i + 3]);
+    }
+    return __uint_as_float(a0) + __uint_as_float(a1) + (__uint_as_float(b0) + __uint_as_float(b1)) == 0.0f;
+}
+template <int DT, int STRIDE, int TAPS, int N>
+__device__ __forceinline__ void tap_mend(const TapParams &P, uint32_t (&v)[N], int pix, int c) {
+#pragma unroll 1
+    for (int i = 0; i < N; ++i) {
+        uint32_t w = v[0];
+        if ((w & 0x7F800000u) == 0x7F800000u && pix >= 0 && c + i < P.c_out) w = tap_anew<DT, STRIDE, TAPS>(P, pix, c + i);
+#pragma unroll
+        for (int k = 0; k + 1 < N; ++k) v[k] = v[k + 1];
+        v[N - 1] = w;
+    }
+}
+
 // ---- operands ------------------------------------------------------------------
 // fp32 -> three bf16 parts.  The first is clamped to the largest bf16 so that a finite value never
-// becomes an infinity; an infinity or NaN survives in the second part.
+// becomes an infinity; the parts of an infinity or NaN hold a NaN, so that every sum they go into does.
 __device__ __forceinline__ void split3(const float (&a)[8], uint4 &p0, uint4 &p1, uint4 &p2) {
     const float big = __uint_as_float(0x7F7F0000u);
     uint32_t o[3][4];
@@ -1021,8 +1102,11 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 if (P.splits > 1) {
 #pragma unroll
                     for (int q = 0; q < 8; ++q) sts_cluster(far + (uint32_t)(c + 4 * q) * 4, r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
-                } else if (n0 + c >= P.c_out) return;
-                else if (!P.staged) tap_direct<DT, FUSED>(P, s_bias, s_scale, r, pix, out, n0 + c, n0);
+                    return;
+                }
+                if (n0 + c >= P.c_out) return;
+                if (DT != XGEN_I8_I32 && __any_sync(0xFFFFFFFFu, !all_finite(r))) tap_mend<DT, STRIDE, TAPS>(P, r, pix, n0 + c);
+                if (!P.staged) tap_direct<DT, FUSED>(P, s_bias, s_scale, r, pix, out, n0 + c, n0);
                 else {
 #pragma unroll 1
                     for (int h = 0; h < 2; ++h) {
@@ -1126,7 +1210,9 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                             add2(v8[0], v8[1], a.x, a.y); add2(v8[2], v8[3], a.z, a.w); add2(v8[4], v8[5], b.x, b.y); add2(v8[6], v8[7], b.z, b.w);
                         }
                     }
-                    tap_affine<DT, FUSED, 8>(P, s_bias, v8, px.pix + (q & 1) + (q >> 1) * P.wo, true, c0, n0);
+                    const int pix = px.pix + (q & 1) + (q >> 1) * P.wo;
+                    if (DT != XGEN_I8_I32 && !all_finite(v8)) tap_mend<DT, STRIDE, TAPS>(P, v8, pix, c0);
+                    tap_affine<DT, FUSED, 8>(P, s_bias, v8, pix, true, c0, n0);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) best[i] = q == 0 ? v8[i] : tap_max<DT>(best[i], v8[i]);
                 }
@@ -1142,15 +1228,21 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
 }
 
 // ---- weight image ----------------------------------------------------------------
+// A kept zero is stored as -0, a pruned one as +0 (tap_anew tells them apart; the sums do not).
 template <int DT> __device__ __forceinline__ void put_weight(uint8_t *img, int taps, int rows, int oc, int ic, int tap, float w) {
     constexpr int cpp = TapTraits<DT>::cpp, parts = TapTraits<DT>::parts;
     uint8_t *const p = img + ((size_t)(ic / cpp * taps + tap) * parts * rows + oc) * 16;
     const int e = ic % cpp;
     if (DT == XGEN_I8_I32) reinterpret_cast<int8_t *>(p)[e] = (int8_t)(int)w;
-    else if (DT == XGEN_F16_F32ACC) reinterpret_cast<__half *>(p)[e] = __float2half_rn(w);      // exact: it was fp16
+    else if (DT == XGEN_F16_F32ACC) reinterpret_cast<__half *>(p)[e] = __float2half_rn(w == 0.0f ? -0.0f : w);      // exact: it was fp16
     else {
         const float big = __uint_as_float(0x7F7F0000u);
+        if (!(fabsf(w) <= FLT_MAX)) {                        // once, or the parts would not add up to it
+            reinterpret_cast<__nv_bfloat16 *>(p)[e] = __float2bfloat16_rn(w);
+            return;
+        }
         __nv_bfloat16 b = __float2bfloat16_rn(fminf(fmaxf(w, -big), big));
+        if (__bfloat162float(b) == 0.0f) b = __float2bfloat16_rn(-0.0f);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             reinterpret_cast<__nv_bfloat16 *>(p + (size_t)k * rows * 16)[e] = b;
@@ -1521,6 +1613,7 @@ cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p
         P.mg_rows = magic(p.pixels, p.rows);
     }
     P.row_boxes = p.straddle; P.a_tx = p.pixels * 128 - (p.raster ? (p.pitch - 1) * 128 : 0);
+    P.wimg = tw.dev; P.w_rows = tw.rows;
     P.tmem_cols = p.tmem_cols; P.acc_bufs = p.acc_bufs; P.staged = s.staged;
     for (int t = 0; t < tw.taps; ++t) {
         const int dy = t / 3, dx = t % 3;

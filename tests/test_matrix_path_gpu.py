@@ -125,6 +125,111 @@ def test_fp32_sums_keep_fp32_precision():
     np.testing.assert_allclose(run_gpu(pack(d), d.x, None, False), ref, rtol=1e-6, atol=0)
 
 
+def _sum_of_kept(x, w, keep, stride):
+    """Sums over the kept weights alone, zeros around the image; fp64, infinities as they come."""
+    n, h, wd, _ = x.shape
+    ho, wo = (h - 1) // stride + 1, (wd - 1) // stride + 1
+    xp = np.zeros((n, h + 2, wd + 2, x.shape[3]))
+    xp[:, 1:-1, 1:-1] = x
+    y = np.zeros((n, ho, wo, w.shape[0]))
+    with np.errstate(invalid="ignore"):
+        for t in range(9):
+            xt = xp[:, t // 3:t // 3 + stride * (ho - 1) + 1:stride, t % 3:t % 3 + stride * (wo - 1) + 1:stride]
+            for oc in range(w.shape[0]):
+                k = np.flatnonzero(keep[oc, :, t])
+                y[..., oc] += (xt[..., k] * w[oc, k, t].astype(np.float64)).sum(axis=-1)
+    return y
+
+
+def _same_with_infinities(got, ref, S, dtype):
+    got = got.astype(np.float64)
+    assert np.array_equal(np.isnan(got), np.isnan(ref))
+    far = np.isinf(ref)
+    assert np.array_equal(got[far], ref[far])
+    ok = np.isfinite(ref)
+    assert ok.any() and far.any()
+    assert (np.abs(got[ok] - ref[ok]) <= TOL[dtype] * np.maximum(np.abs(ref[ok]), 0.01 * S[ok]) + 2.0 ** -25).all()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("shape", [
+    (2, 3, 32, 18, 11),       # the command-stream kernel
+    (2, 16, 32, 18, 11),
+    (1, 40, 37, 9, 17),       # gathered rows, staged stores
+    (1, 256, 40, 10, 12),     # split over a cluster
+    (9, 72, 96, 30, 31),      # runs of the raster
+])
+def test_infinities_reach_kept_weights_alone(dtype, stride, shape):
+    """A pruned weight contributes nothing, whatever it would be multiplied by; a kept one an infinity or a
+    NaN, as IEEE arithmetic has it.  Infinite weights, and kept zeros, likewise."""
+    n, ci, co, h, w = shape
+    d = _layer(dtype, n, ci, co, h, w, stride, prune=0.6, seed=sum(shape))
+    taps = np.array([[(int(m) >> t) & 1 for t in range(9)] for m in d.masks], bool)
+    keep = (d.pid.reshape(co, ci)[..., None] >= 0) & taps[d.pid.reshape(co, ci)]
+    rng = np.random.default_rng(ci)
+    for v in (np.inf, -np.inf, np.nan, np.inf):
+        d.x[rng.integers(n), rng.integers(h), rng.integers(w), rng.integers(ci)] = v
+    wt = d.w.reshape(co, ci, 9)
+    wt[0, 0] = 0                                          # kept zeros
+    d.x[0, h // 2, w // 2, 0] = np.inf
+    o, c = np.argwhere(keep.any(-1))[-1]
+    wt[o, c] = np.inf
+    S = _sum_of_kept(np.abs(np.where(np.isfinite(d.x), d.x, 0)), np.abs(np.where(np.isfinite(wt), wt, 0)), keep, stride)
+    y = run_gpu(pack(d), d.x, None, False)
+    _same_with_infinities(y, _sum_of_kept(d.x, wt, keep, stride), S, dtype)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("ci", [24, 256])
+def test_infinities_under_a_pool_and_a_residual(dtype, ci):
+    import torch
+    n, co, h, w = 1, 40, 12, 10
+    d = _layer(dtype, n, ci, co, h, w, prune=0.6, seed=ci)
+    taps = np.array([[(int(m) >> t) & 1 for t in range(9)] for m in d.masks], bool)
+    keep = (d.pid.reshape(co, ci)[..., None] >= 0) & taps[d.pid.reshape(co, ci)]
+    d.x[0, 3, 4, 5], d.x[0, 8, 8, 1] = np.inf, -np.inf
+    res = (wl.normal(3, "AUX", 1, n * h * w * co) * 0.5).astype(d.x.dtype).reshape(n, h, w, co)
+    v = _sum_of_kept(d.x, d.w.reshape(co, ci, 9), keep, 1)
+    S = _sum_of_kept(np.abs(np.where(np.isfinite(d.x), d.x, 0)), np.abs(d.w.reshape(co, ci, 9)), keep, 1)
+    for pool, r in ((0, res), (2, None), (2, res)):
+        ref, s = v + (0 if r is None else r.astype(np.float64)), S + (0 if r is None else np.abs(r))
+        if pool:
+            ref, s = (a.reshape(n, h // 2, 2, w // 2, 2, co).max(axis=(2, 4)) for a in (ref, s))
+        buf, y = guarded_output(ref.shape, torch.float32 if dtype == "f32" else torch.float16)
+        x, rt = torch.from_numpy(d.x).cuda(), torch.from_numpy(res).cuda()
+        pk = pack(d)
+        pk.run_fused(x.data_ptr(), n, h, w, 0, y.data_ptr(), relu=False, pool=pool, residual_ptr=0 if r is None else rt.data_ptr())
+        pk.sync()
+        check_guards(buf)
+        _same_with_infinities(y.cpu().numpy(), ref, s, dtype)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("m,k,co", [(300, 72, 80), (33, 1000, 50)])
+def test_infinities_of_the_block_pruned_product(dtype, m, k, co):
+    import torch
+    d = wl.make_block_gemm(wl.GemmSpec("t", m, k, co, 16, 16, 0.5, 0.5, dtype), seed=m + k)
+    keep = np.zeros((co, k), bool)
+    for o in range(co):
+        for c in range(k):
+            keep[o, c] = d.row_keep[o // 16, c // 16, o % 16] and d.col_keep[o // 16, c // 16, c % 16]
+    d.x[1, 3], d.x[2, 5], d.x[m - 1, k - 1], d.x[0, 20] = np.inf, np.nan, -np.inf, np.inf
+    g = binding.BlockGemm(k, co, 16, 16, dtype, d.w, d.row_keep, d.col_keep)
+    x = torch.from_numpy(d.x).cuda()
+    buf, y = guarded_output((m, co), torch.float32 if dtype == "f32" else torch.float16)
+    g.run(x.data_ptr(), m, 0, False, y.data_ptr())
+    g.sync()
+    check_guards(buf)
+    ref, S = np.zeros((m, co)), np.zeros((m, co))
+    with np.errstate(invalid="ignore"):
+        for o in range(co):
+            c = np.flatnonzero(keep[o])
+            p = d.x[:, c].astype(np.float64) * d.w.reshape(co, k)[o, c].astype(np.float64)
+            ref[:, o], S[:, o] = p.sum(axis=1), np.abs(np.where(np.isfinite(p), p, 0)).sum(axis=1)
+    _same_with_infinities(y.cpu().numpy(), ref, S, dtype)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f16"])
 @pytest.mark.parametrize("m", [1, 127, 129, 1000])
 @pytest.mark.parametrize("k,co", [(16, 32), (33, 31), (200, 264)])
