@@ -1252,13 +1252,14 @@ template <int DT> __device__ __forceinline__ void put_weight(uint8_t *img, int t
     }
 }
 
+// Kernels k0 to k0 + count - 1 of [c_out][c_in].
 template <int DT>
-__global__ void tap_expand_patterns(uint8_t *img, int c_in, int c_out, int rows, const int16_t *kpat, const uint4 *kw4,
+__global__ void tap_expand_patterns(uint8_t *img, int c_in, int rows, int k0, int count, const int16_t *kpat, const uint4 *kw4,
                                     const uint16_t *masks) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= c_in * c_out || kpat[k] < 0) return;
-    const uint4 w = kw4[k];
-    const unsigned mask = masks[kpat[k]];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, k = k0 + i;
+    if (i >= count || kpat[i] < 0) return;
+    const uint4 w = kw4[i];
+    const unsigned mask = masks[kpat[i]];
     int n = 0;
     for (int t = 0; t < 9; ++t)
         if ((mask >> t) & 1) {
@@ -1268,34 +1269,30 @@ __global__ void tap_expand_patterns(uint8_t *img, int c_in, int c_out, int rows,
 }
 
 template <int DT>
-__global__ void tap_expand_dense(uint8_t *img, int c_in, int c_out, int rows, const void *dense, const uint8_t *row_keep,
+__global__ void tap_expand_dense(uint8_t *img, int c_in, int rows, int k0, int count, const void *dense, const uint8_t *row_keep,
                                  const uint8_t *col_keep, int br, int bc) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= c_in * c_out) return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, k = k0 + i;
+    if (i >= count) return;
     const int oc = k / c_in, ic = k % c_in;
     const size_t blk = (size_t)(oc / br) * ((c_in + bc - 1) / bc) + ic / bc;
     if (!row_keep[blk * br + oc % br] || !col_keep[blk * bc + ic % bc]) return;
-    const float w = DT == XGEN_F32 ? static_cast<const float *>(dense)[k] : __half2float(static_cast<const __half *>(dense)[k]);
+    const float w = DT == XGEN_F32 ? static_cast<const float *>(dense)[i] : __half2float(static_cast<const __half *>(dense)[i]);
     put_weight<DT>(img, 1, rows, oc, ic, 0, w);
 }
 
 static int tap_cpp(xgen_dtype dt) { return dt == XGEN_I8_I32 ? 16 : 8; }
 static int tap_parts(xgen_dtype dt) { return dt == XGEN_F32 ? 3 : 1; }
 
-// The zeroed image, and `extra` bytes of upload scratch, which stay with the handle: giving them back
-// would cost a synchronisation and more time than the upload.  One allocation, or two where that keeps
-// both within the driver's small blocks of up to 1 MB (128 -> 128 fp32: 0.96 -> 0.57 ms a handle).
+// The zeroed image, and `extra` bytes of upload scratch, which tap_done gives back.
 static xgen_status tap_alloc(TapWeights &tw, xgen_dtype dt, int taps, int c_in, int c_out, size_t extra, uint8_t **scratch) {
     tw.dtype = dt; tw.taps = taps; tw.c_in = c_in; tw.c_out = c_out;
     tw.planes = (c_in + 2 * tap_cpp(dt) - 1) / (2 * tap_cpp(dt)) * 2;
     tw.rows = (c_out + 15) / 16 * 16;
     const size_t image = (size_t)tw.planes * taps * tap_parts(dt) * tw.rows * 16, bytes = image + 16;     // and the status word
-    constexpr size_t kSmall = 1 << 20;
-    const bool apart = bytes <= kSmall && extra <= kSmall && bytes + extra > kSmall;
-    cudaError_t e = cudaMalloc(&tw.dev, apart ? bytes : bytes + extra);
-    if (e == cudaSuccess && apart) e = cudaMalloc(&tw.scratch, extra);
+    cudaError_t e = cudaMalloc(&tw.dev, bytes);
+    if (e == cudaSuccess) e = cudaMalloc(&tw.scratch, extra);
     if (e == cudaSuccess) e = cudaMemsetAsync(tw.dev, 0, bytes, 0);
-    *scratch = apart ? tw.scratch : tw.dev + bytes;
+    *scratch = tw.scratch;
     tw.status = reinterpret_cast<int *>(tw.dev + image);
     if (e == cudaSuccess) return XGEN_OK;
     cudaGetLastError();
@@ -1306,6 +1303,8 @@ static xgen_status tap_alloc(TapWeights &tw, xgen_dtype dt, int taps, int c_in, 
 static xgen_status tap_done(TapWeights &tw, cudaError_t e) {
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+    if (tw.scratch) cudaFree(tw.scratch);
+    tw.scratch = nullptr;
     if (e == cudaSuccess) return XGEN_OK;
     cudaGetLastError();
     tap_free(tw);
@@ -1319,42 +1318,53 @@ void tap_free(TapWeights &tw) {
     tw.status = nullptr;
 }
 
+// Weights go up in pieces that keep the scratch within the driver's small blocks (1 MB): an allocation
+// beyond them takes longer than the upload, and kept for the handle's life (as one allocation with the image)
+// it held a third of an fp32 image again.
+constexpr size_t kPiece = 1 << 20;
+
 xgen_status tap_upload_patterns(TapWeights &tw, xgen_dtype dt, int c_in, int c_out, const int16_t *kpat, const uint32_t *kw4,
                                 const uint16_t *masks, int n_masks) {
-    const size_t nk = (size_t)c_in * c_out, wb = nk * 16, pb = nk * 2;
+    const size_t nk = (size_t)c_in * c_out, mb = ((size_t)n_masks * 2 + 15) / 16 * 16;
+    const size_t piece = std::min(nk, (kPiece - mb) / 18 / 8 * 8);             // 16 bytes of weights and two of pattern each
     uint8_t *scratch = nullptr;
-    const xgen_status st = tap_alloc(tw, dt, 9, c_in, c_out, wb + pb + (size_t)n_masks * 2, &scratch);
+    const xgen_status st = tap_alloc(tw, dt, 9, c_in, c_out, mb + piece * 18, &scratch);
     if (st != XGEN_OK) return st;
-    cudaError_t e = cudaMemcpyAsync(scratch, kw4, wb, cudaMemcpyHostToDevice, 0);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(scratch + wb, kpat, pb, cudaMemcpyHostToDevice, 0);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(scratch + wb + pb, masks, (size_t)n_masks * 2, cudaMemcpyHostToDevice, 0);
-    const unsigned blocks = (unsigned)((nk + 255) / 256);
-    const uint4 *w = reinterpret_cast<const uint4 *>(scratch);
-    const int16_t *kp = reinterpret_cast<const int16_t *>(scratch + wb);
-    const uint16_t *mk = reinterpret_cast<const uint16_t *>(scratch + wb + pb);
-    if (e == cudaSuccess) {
-        if (dt == XGEN_F32) tap_expand_patterns<XGEN_F32><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, kp, w, mk);
-        else if (dt == XGEN_F16_F32ACC) tap_expand_patterns<XGEN_F16_F32ACC><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, kp, w, mk);
-        else tap_expand_patterns<XGEN_I8_I32><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, kp, w, mk);
+    const uint16_t *mk = reinterpret_cast<const uint16_t *>(scratch);
+    const uint4 *w = reinterpret_cast<const uint4 *>(scratch + mb);
+    const int16_t *kp = reinterpret_cast<const int16_t *>(scratch + mb + piece * 16);
+    cudaError_t e = cudaMemcpyAsync(scratch, masks, (size_t)n_masks * 2, cudaMemcpyHostToDevice, 0);
+    for (size_t k0 = 0; k0 < nk && e == cudaSuccess; k0 += piece) {
+        const size_t n = std::min(piece, nk - k0);
+        e = cudaMemcpyAsync(scratch + mb, kw4 + k0 * 4, n * 16, cudaMemcpyHostToDevice, 0);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(scratch + mb + piece * 16, kpat + k0, n * 2, cudaMemcpyHostToDevice, 0);
+        if (e != cudaSuccess) break;
+        const unsigned blocks = (unsigned)((n + 255) / 256);
+        if (dt == XGEN_F32) tap_expand_patterns<XGEN_F32><<<blocks, 256>>>(tw.dev, c_in, tw.rows, (int)k0, (int)n, kp, w, mk);
+        else if (dt == XGEN_F16_F32ACC) tap_expand_patterns<XGEN_F16_F32ACC><<<blocks, 256>>>(tw.dev, c_in, tw.rows, (int)k0, (int)n, kp, w, mk);
+        else tap_expand_patterns<XGEN_I8_I32><<<blocks, 256>>>(tw.dev, c_in, tw.rows, (int)k0, (int)n, kp, w, mk);
     }
     return tap_done(tw, e);
 }
 
 xgen_status tap_upload_dense(TapWeights &tw, xgen_dtype dt, int c_in, int c_out, const void *dense_w, const uint8_t *row_keep,
                              const uint8_t *col_keep, int br, int bc) {
-    const size_t n = (size_t)c_in * c_out, wb = (n * (dt == XGEN_F32 ? 4 : 2) + 15) / 16 * 16;
+    const size_t nk = (size_t)c_in * c_out, wb = dt == XGEN_F32 ? 4 : 2;
     const size_t blocks_of = (size_t)((c_out + br - 1) / br) * ((c_in + bc - 1) / bc);
+    const size_t rb = blocks_of * br, cb = blocks_of * bc, fb = (rb + cb + 15) / 16 * 16;     // the keep flags, whole
+    const size_t piece = std::min(nk, (std::max(kPiece, fb + kPiece / 4) - fb) / wb / 8 * 8);
     uint8_t *scratch = nullptr;
-    const xgen_status st = tap_alloc(tw, dt, 1, c_in, c_out, wb + blocks_of * ((size_t)br + bc), &scratch);
+    const xgen_status st = tap_alloc(tw, dt, 1, c_in, c_out, fb + piece * wb, &scratch);
     if (st != XGEN_OK) return st;
-    uint8_t *rk = scratch + wb, *ck = rk + blocks_of * br;
-    cudaError_t e = cudaMemcpyAsync(scratch, dense_w, n * (dt == XGEN_F32 ? 4 : 2), cudaMemcpyHostToDevice, 0);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(rk, row_keep, blocks_of * br, cudaMemcpyHostToDevice, 0);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(ck, col_keep, blocks_of * bc, cudaMemcpyHostToDevice, 0);
-    const unsigned blocks = (unsigned)((n + 255) / 256);
-    if (e == cudaSuccess) {
-        if (dt == XGEN_F32) tap_expand_dense<XGEN_F32><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, scratch, rk, ck, br, bc);
-        else tap_expand_dense<XGEN_F16_F32ACC><<<blocks, 256>>>(tw.dev, c_in, c_out, tw.rows, scratch, rk, ck, br, bc);
+    cudaError_t e = cudaMemcpyAsync(scratch, row_keep, rb, cudaMemcpyHostToDevice, 0);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(scratch + rb, col_keep, cb, cudaMemcpyHostToDevice, 0);
+    for (size_t k0 = 0; k0 < nk && e == cudaSuccess; k0 += piece) {
+        const size_t n = std::min(piece, nk - k0);
+        e = cudaMemcpyAsync(scratch + fb, static_cast<const char *>(dense_w) + k0 * wb, n * wb, cudaMemcpyHostToDevice, 0);
+        if (e != cudaSuccess) break;
+        const unsigned blocks = (unsigned)((n + 255) / 256);
+        if (dt == XGEN_F32) tap_expand_dense<XGEN_F32><<<blocks, 256>>>(tw.dev, c_in, tw.rows, (int)k0, (int)n, scratch + fb, scratch, scratch + rb, br, bc);
+        else tap_expand_dense<XGEN_F16_F32ACC><<<blocks, 256>>>(tw.dev, c_in, tw.rows, (int)k0, (int)n, scratch + fb, scratch, scratch + rb, br, bc);
     }
     return tap_done(tw, e);
 }

@@ -22,7 +22,8 @@ EncodeTiledFn encode_tiled_fn();
 // input channels (8 fp16 / bf16, 16 int8); a tensor copy takes any range of filters and planes of a
 // tap at once, so neither the filter tile nor the channels per stage is fixed here.
 struct TapWeights {
-    uint8_t *dev = nullptr, *scratch = nullptr;      // the image; what it was made from
+    uint8_t *dev = nullptr;      // the image
+    uint8_t *scratch = nullptr;  // what it is made from, while it is made
     int *status = nullptr;       // behind the image: set by a kernel whose bounded wait ran out
     xgen_dtype dtype = XGEN_F32;
     int taps = 9, c_in = 0, c_out = 0;

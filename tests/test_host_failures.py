@@ -86,3 +86,27 @@ def test_an_upload_that_fails_half_way_leaves_nothing(fake_lib):
         fake.fake_fail_encode(1)
         assert run() == 0 and fake.fake_launches() == n + 1 and fake.fake_live_bytes() > held
     """)
+
+
+def test_a_handle_holds_its_weight_image_and_no_more(fake_lib):
+    """The scratch of the upload is given back; a failed upload leaves nothing."""
+    _run(fake_lib, """
+        round16 = lambda n: -(-n // 16) * 16
+        for dtype, ci, co in (("f32", 16, 32), ("f32", 300, 260), ("f16", 300, 260), ("i8", 300, 260)):
+            per, parts = {"f32": (8, 3), "f16": (8, 1), "i8": (16, 1)}[dtype]
+            image = -(-ci // (2 * per)) * 2 * 9 * parts * round16(co) * 16
+            held = fake.fake_live_bytes()
+            pk = conv(dtype, ci, co)
+            assert image < fake.fake_live_bytes() - held <= image + 64, (dtype, fake.fake_live_bytes() - held - image)
+            pk.close()
+            assert fake.fake_live_bytes() == held
+        for dtype, k, co in (("f32", 700, 500), ("f16", 33, 31)):
+            image = -(-k // 16) * 2 * {"f32": 3, "f16": 1}[dtype] * round16(co) * 16
+            held = fake.fake_live_bytes()
+            g = gemm(dtype, k, co)
+            assert image < fake.fake_live_bytes() - held <= image + 64
+            g.close()
+            for nth in (1, 2):
+                fake.fake_fail_alloc(nth)
+                assert status(gemm, dtype, k, co) == 5 and fake.fake_live_bytes() == held
+    """)

@@ -329,6 +329,22 @@ def test_depthwise_pieces_of_rows(dtype, stride, shape):
     assert (err <= TOL[dtype] * np.maximum(np.abs(ref), 0.01 * S) + 2.0 ** -25).all()
 
 
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("k,co,block", [(520, 1100, 1), (600, 1000, 32)])     # keep flags beyond 1 MB; several pieces of weights
+def test_weights_uploaded_in_pieces(dtype, k, co, block):
+    import torch
+    d = wl.make_block_gemm(wl.GemmSpec("t", 9, k, co, block, block, 0.5, 0.5, dtype), seed=block)
+    g = binding.BlockGemm(k, co, block, block, dtype, d.w, d.row_keep, d.col_keep)
+    x, b = torch.from_numpy(d.x).cuda(), torch.from_numpy(d.bias).cuda()
+    buf, y = guarded_output((9, co), torch.float32 if dtype == "f32" else torch.float16)
+    g.run(x.data_ptr(), 9, b.data_ptr(), True, y.data_ptr())
+    g.sync()
+    check_guards(buf)
+    ref, S = oracle.block_gemm(d.x, d.w, d.row_keep, d.col_keep, block, block, bias=d.bias, relu=True, with_scale=True)
+    bound = TOL[dtype] * np.maximum(np.abs(ref), 0.01 * S) + 2.0 ** -25
+    assert (np.abs(y.cpu().numpy().astype(np.float64) - ref) <= bound).all()
+
+
 def test_calls_report_errors():
     pk = pack(_layer("f32", 1, 16, 32, 8, 8))
     with pytest.raises(binding.PatconvError) as e:
