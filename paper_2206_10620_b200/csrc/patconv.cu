@@ -1578,10 +1578,18 @@ xgen_status xgen_patconv_pack(const xgen_patconv_desc *desc, const void *dense_w
         if (cudaMalloc(&h->d_status, sizeof(int)) != cudaSuccess) us = XGEN_ERR_ALLOC;
         else if (cudaMemset(h->d_status, 0, sizeof(int)) != cudaSuccess) us = XGEN_ERR_CUDA;
         const PackedHost &p = h->host;
-        // Three input channels fill a fifth of the 16 that a matrix instruction takes: such first layers
-        // stay on the command-stream kernel (3 -> 64 at 224x224, fp32: 12.7 us against 15.8 us).
+        // A few input channels fill little of the 16 (32) that a matrix instruction takes, and rows of fp16 or
+        // int8 that are not whole 16-byte pieces are gathered: such first layers stay on the command-stream
+        // kernel.  -> 64 filters at 224x224, unpruned, command stream against matrix path, us, by input channels:
+        //   fp32     1: 10.4, 12.9   2: 11.5, 12.9   3: 12.6, 12.9   4: 13.3, 12.9   5: 14.8, 13.0   7: 17.2, 13.0
+        //   fp32 with 60 % pruned    3: 10.7, 12.9   4: 11.0, 12.9   5: 12.2, 12.9   6: 13.0, 12.9
+        //   fp16     1: 8.9, 15.6    3: 11.0, 16.9   5: 13.9, 17.1   7: 15.8, 16.8   8: 16.4, 10.1
+        //   int8     1: 12.0, 15.7   3: 13.8, 16.7   5: 16.5, 16.8   7: 18.6, 17.2 (60 % pruned 14.8, 17.2)
+        // and 32 images of 112x112 at stride 2, 32 filters: fp32 3: 23.2, 27.4   4: 36.5, 27.4   5: 31.0, 29.3; fp16 7: 31.2, 56.7.
+        // (Small images run faster on the matrix units at every count -- 3 -> 32 at 32x32, fp32: 9.4, 5.9 -- but a
+        // handle does not know its images, and few of these layers see such.)
         if (us == XGEN_OK)
-            us = desc->c_in < 8 ? upload_layout(h)
+            us = desc->c_in < (desc->dtype == XGEN_F32 ? 5 : 8) ? upload_layout(h)
                                 : tap_upload_patterns(h->tap, p.dtype, p.c_in, p.c_out, p.kpat.data(), p.kw4.data(), p.masks.data(), (int)p.masks.size());
         if (us != XGEN_OK && h->d_status) { cudaGetLastError(); cudaFree(h->d_status); }
         cudaSetDevice(prev);
@@ -1924,7 +1932,7 @@ xgen_status xgen_patconv_run_static_scratch(const xgen_patconv_packed *h, const 
         return XGEN_ERR_SHAPE;
     }
     // The matrix path keeps the sums of a split in the shared memory of a cluster; a layer that is not on
-    // it (fewer than eight input channels: one chunk) has nothing to split.
+    // it (a few input channels: one chunk) has nothing to split.
     return run_layer(h, x, n, hh, ww, bias, relu, y, stream, true);
 }
 

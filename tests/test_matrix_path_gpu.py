@@ -20,7 +20,7 @@ def _layer(dtype, n, ci, co, h, w, stride=1, prune=0.5, seed=1, x_dist=None):
 @pytest.mark.parametrize("dtype", ["f32", "f16", "i8"])
 @pytest.mark.parametrize("stride", [1, 2])
 @pytest.mark.parametrize("shape", [
-    (1, 8, 16, 1, 1),         # the fewest channels, one pixel
+    (1, 8, 16, 1, 1),         # one pixel
     (1, 16, 31, 1, 9),        # one row, one column past an 8-pixel column, ragged filters
     (3, 17, 33, 16, 8),       # exactly one tile an image; channels of no whole 16 bytes
     (2, 64, 64, 17, 9),       # one row and one column past a tile; one whole stage (fp16)
@@ -36,6 +36,19 @@ def test_edges_of_tiles(dtype, stride, shape):
     assert pk.plan_info(n, h, w)["matrix_path"] == 1
     compare(d, run_gpu(pk, d.x, d.bias, True))
     compare(d, run_gpu(pk, d.x, None, False), bias=None, relu=False)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16", "i8"])
+@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("ci", [1, 3, 4, 5, 7, 8])
+def test_either_side_of_the_fewest_channels(dtype, stride, ci):
+    """fp32 layers of five channels and fp16 / int8 layers of eight are the first on the matrix units."""
+    n, co, h, w = 2, 40, 19, 26
+    d = _layer(dtype, n, ci, co, h, w, stride, prune=0.2, seed=ci)
+    pk = pack(d)
+    assert pk.plan_info(n, h, w)["matrix_path"] == int(ci >= (5 if dtype == "f32" else 8))
+    compare(d, run_gpu(pk, d.x, d.bias, True))
+    compare(d, run_gpu(pk, d.x, None, False, plan=True), bias=None, relu=False)
 
 
 @pytest.mark.parametrize("dtype", ["f32", "f16", "i8"])
@@ -155,6 +168,7 @@ def _same_with_infinities(got, ref, S, dtype):
 @pytest.mark.parametrize("stride", [1, 2])
 @pytest.mark.parametrize("shape", [
     (2, 3, 32, 18, 11),       # the command-stream kernel
+    (2, 5, 32, 18, 11),       # (fp32: the fewest channels of the matrix path)
     (2, 16, 32, 18, 11),
     (1, 40, 37, 9, 17),       # gathered rows, staged stores
     (1, 256, 40, 10, 12),     # split over a cluster
