@@ -12,7 +12,12 @@
  *   y[m][oc] = act( bias[oc] + sum_{c: W[oc][c] survives} W[oc][c] * x[m][c] )
  *
  * with x [m_rows][k] row-major (one row per pixel of an NHWC activation tensor,
- * m_rows = n*h*w, or one row per token) and act = ReLU or identity.
+ * m_rows = n*h*w, or one row per token) and act = ReLU or identity.  Pruned entries
+ * contribute nothing, also where they meet an infinity or a NaN.
+ *
+ * The product runs dense on the tensor cores, with zeros for the pruned entries, as the matrix path
+ * of patconv.h does (the same precision); a handle packed with warps_per_block executes the
+ * packed stream instead.
  *
  * Same conventions as patconv.h: plain C ABI, every function returns a status,
  * *_host is host memory, *_dev memory of the device the handle was packed for.
@@ -47,8 +52,9 @@ typedef struct {
     int64_t weights_kept;       /* entries whose row and column are kept in their block = useful
                                    multiply-adds per row of x                                     */
     int64_t weight_bytes;       /* bytes of the kept weights at the layer's storage precision    */
-    int64_t stream_bytes;       /* bytes of the packed stream on the device (every kept weight
-                                   widened to fp32; headers, padding and the offset table included) */
+    int64_t stream_bytes;       /* bytes of the packed stream (every kept weight widened to fp32;
+                                   headers, padding and the offset table included); on the device
+                                   only for a handle packed with warps_per_block (see device_bytes) */
     int64_t padded_slots;       /* weight slots of the stream that hold padding zeros (a column
                                    group is filled up to eight columns)                          */
     int64_t column_groups;      /* activation loads in the stream: one per group of up to eight
@@ -60,6 +66,10 @@ typedef struct {
     int32_t stage_cols;         /* input columns staged per pipeline step                        */
     int32_t n_stages;
     int32_t max_stage_bytes;    /* largest per-(thread block, stage) piece of the stream         */
+    int64_t device_bytes;       /* device memory that the handle holds as it stands: the matrix path's
+                                   weight image (all of W, pruned entries as zeros: 2 bytes in fp16, 6
+                                   in fp32, as three bf16 parts; rows and columns rounded up to 16),
+                                   or the packed stream                                          */
 } xgen_blockgemm_stats;
 
 /*
@@ -82,9 +92,9 @@ xgen_status xgen_blockgemm_pack(const xgen_blockgemm_desc *desc, const void *den
 /*
  * Run the layer (paper Sec. 2.1: only the kept rows and columns of every block are computed;
  * Sec. 2.2: bias and ReLU fused).
- *   x_dev    [m_rows][k] row-major, the dtype's activation type, element-aligned (fp16: an
- *            even k and 4-byte alignment let the rows be staged by asynchronous copies;
- *            otherwise they are staged with plain loads)
+ *   x_dev    [m_rows][k] row-major, the dtype's activation type, element-aligned (fp16: a
+ *            k that is a multiple of 8 and 16-byte alignment let the copy engine fetch the rows;
+ *            otherwise they are gathered)
  *   bias_dev [c_out] fp32, 4-byte aligned, or NULL
  *   y_dev    [m_rows][c_out] row-major, element-aligned, must not overlap x_dev (16-byte
  *            alignment and a row of a multiple of 16 bytes give 16-byte stores)

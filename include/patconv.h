@@ -11,7 +11,14 @@
  *                          W[oc][ic][t] * x[n][oy*s + dy(t) - 1][ox*s + dx(t) - 1][ic] )
  *
  * with t = 3*dy + dx, zero padding of 1, stride s in {1,2}, cross-correlation
- * (no kernel flip), act = ReLU or identity.
+ * (no kernel flip), act = ReLU or identity.  Pruned weights contribute nothing, also
+ * where they meet an infinity or a NaN; ReLU keeps a NaN on the matrix path.
+ *
+ * Two kernels compute it.  The matrix path runs the layer dense on the tensor cores, with zeros for
+ * the pruned weights, and is what a call takes by default.  The command-stream kernel
+ * executes the kept kernels one by one; layers of a few input channels (fp32: up to four,
+ * else up to seven) take it, and handles whose caller names one of its tuning parameters
+ * (xgen_patconv_plan_tuned).  Both accumulate in fp32 (int32).
  *
  * Plain C ABI: pointers and sizes only.  Every function returns a status code;
  * nothing throws, aborts or traps.  Unless stated otherwise a pointer named
@@ -63,16 +70,17 @@ typedef struct {
     int64_t kernels_surviving;    /* kernels with a pattern (not removed)                     */
     int64_t macs_per_pixel;       /* 4 * kernels_surviving: useful multiply-adds per output pixel */
     int64_t weight_bytes;         /* bytes of kept weights at the layer's storage precision   */
-    int64_t index_bytes;          /* bytes the device copy stores beyond weight_bytes: the
-                                     command stream (48-byte slots: 16 bytes of opcode and
-                                     operand, every kept weight widened to fp32 and stored
-                                     twice) plus the offset and slot tables, less weight_bytes */
+    int64_t index_bytes;          /* bytes of the command stream as the device stores it (48-byte
+                                     slots: 16 bytes of opcode and operand, every kept weight
+                                     widened to fp32 and stored twice) plus the offset and slot
+                                     tables, less weight_bytes.  Most handles keep no such copy
+                                     there (see device_bytes)                                   */
     int64_t compact_index_bytes;  /* the information in those bytes: one opcode byte and one
                                      operand byte per command, plus the offset and slot tables
                                      (what a byte-packed encoding of this layout would take)   */
     int64_t csr_index_bytes;      /* index bytes CSR would need for the same non-zeros
                                      (one 4-byte column per weight + one row pointer per filter) */
-    int64_t stream_bytes;         /* bytes of the command stream as stored on the device
+    int64_t stream_bytes;         /* bytes of the command stream alone, as the device stores it
                                      (48-byte slots: every kept weight is stored twice there) */
     int32_t filters_per_group;    /* J: filters one warp accumulates together                 */
     int32_t groups_per_block;     /* filter groups (warps) per thread block                   */
@@ -85,6 +93,14 @@ typedef struct {
                                      input channel that group is connected to)                */
     double  group_imbalance;      /* worst thread block: max / mean of surviving kernels over
                                      the block's groups (its warps share the staged tiles)    */
+    int64_t image_bytes;          /* bytes of the matrix path's weight image, 0 for a handle without
+                                     one: all of the dense layer's weights, pruned ones as zeros, 9
+                                     taps of 2 (fp16), 1 (int8) or 6 bytes (fp32, as three bf16
+                                     parts), channels and filters rounded up to 16 (int8: channels
+                                     to 32)                                                     */
+    int64_t device_bytes;         /* device memory that the handle holds as it stands: the image
+                                     or the command stream with its tables, or both, the workspace
+                                     of a planned split and the staging buffers of host calls  */
 } xgen_patconv_stats;
 
 /* Read-only view of the packed layout on the host, for inspection and tests.
@@ -146,10 +162,10 @@ xgen_status xgen_patconv_pack(const xgen_patconv_desc *desc, const void *dense_w
  *   cuda_stream  a cudaStream_t passed as void* (NULL = default stream)
  * Only enqueues work on the stream: no synchronisation, no device allocation.
  * The caller keeps x, bias and y alive until the stream reaches that work.
- * Concurrent calls on different streams are allowed for unplanned shapes (the
- * handle only remembers, under a lock, the launch geometry and tensor map of the
- * last few (shape, x address) pairs, so repeated calls skip that work).  For a
- * shape prepared with xgen_patconv_plan see the rules there.
+ * Concurrent calls on different streams are allowed on the matrix path, and on the command-stream
+ * kernel for unplanned shapes (the handle only remembers, under a lock, the launch geometry of
+ * the last few shapes, and there tensor maps by x address, so repeated calls skip that work).  For a
+ * shape prepared with xgen_patconv_plan on the command-stream kernel see the rules there.
  * Errors: INVALID_ARG (null or misaligned pointer, y overlapping x), SHAPE
  * (n,h,w < 1 or a tensor beyond 2^31-1 elements), UNSUPPORTED (a tile of this
  * shape does not fit shared or tensor memory), CUDA (launch failure or
@@ -191,8 +207,9 @@ typedef struct {
  * are honoured as in xgen_patconv_run.
  * Errors as xgen_patconv_run, plus INVALID_ARG (NULL epilogue, misaligned residual or scale),
  * SHAPE (pooling an odd extent), UNSUPPORTED (pool other than 0 or 2; re-quantisation of a
- * floating-point layer; a handle whose last xgen_patconv_plan chose 4x2-pixel blocks -- plan
- * it again with xgen_patconv_tuning.no_small_blocks).
+ * floating-point layer; a handle whose last xgen_patconv_plan chose 4x2-pixel blocks for the
+ * command-stream kernel, whichever kernel it runs -- plan it again with
+ * xgen_patconv_tuning.no_small_blocks).
  */
 xgen_status xgen_patconv_run_fused(const xgen_patconv_packed *packed, const void *x_dev, int32_t n,
                                    int32_t h, int32_t w, const void *bias_dev,
@@ -263,7 +280,12 @@ xgen_status xgen_patconv_enqueue_host(const xgen_patconv_packed *packed, const v
                                       void *y_host, void *cuda_stream);
 
 /*
- * Optional: prepare the handle for one input shape.  Layers with few output
+ * Optional: prepare the handle for one input shape.  On the matrix path every shape is planned by the
+ * first call that meets it; there this call only checks the shape, and nothing of what
+ * follows applies: blocks that share a reduction are one cluster, need no workspace and wait for nobody
+ * outside it.  The rest is about handles that run the command-stream kernel
+ * (xgen_patconv_plan_stats.matrix_path = 0; the fields of its plan are reported for every handle).
+ *   Layers with few output
  * pixels do not fill the GPU with (pixel tile x filter block) work items; for
  * such a shape this call lets later xgen_patconv_run calls split the input
  * channels across thread blocks (the paper does not discuss this; it is the
@@ -294,8 +316,8 @@ xgen_status xgen_patconv_enqueue_host(const xgen_patconv_packed *packed, const v
  *   Either way two planned split launches of ONE handle must not run at the same
  * time (they share the workspace and the counters): one stream, or events.
  * The call allocates the workspace and the counters, owned by the handle, so it
- * synchronises the device and must not be called while the handle is in use.
- * Without this call every shape runs unsplit.
+ * synchronises the device and must not be called while the handle is in use
+ * (whichever kernel it runs).  Without this call every shape runs unsplit.
  * Errors: INVALID_ARG, SHAPE, UNSUPPORTED, ALLOC, CUDA.
  */
 xgen_status xgen_patconv_plan(xgen_patconv_packed *packed, int32_t n, int32_t h, int32_t w);
@@ -305,7 +327,11 @@ xgen_status xgen_patconv_plan(xgen_patconv_packed *packed, int32_t n, int32_t h,
  * Representation carries "tuning-decided parameters" next to the pattern
  * information).  xgen_patconv_plan chooses them itself; a caller that has
  * measured better ones passes them here.  Zero in every field = the library's
- * own choice.
+ * own choice.  splits, no_copy_engine, reduce_mode, channels_per_chunk and groups_per_block are
+ * parameters of the command-stream kernel: naming one has every later run take it, until the
+ * handle is planned without.  Of the shapes timed it is the faster one for fp32
+ * layers with 87 % and more of their kernels pruned and many channels on few pixels (512->512 at 28x28:
+ * 2 % at 87.5 %, 10 % at 90 %, 14 % at 95 %; 64->64 at 224x224: 4 % at 90 %).
  *   splits             channel splits of the planned shape (clamped to what is
  *                      resident at once and to the number of channel chunks)
  *   no_copy_engine     stage input tiles with plain loads instead of the tensor
@@ -313,7 +339,7 @@ xgen_status xgen_patconv_plan(xgen_patconv_packed *packed, int32_t n, int32_t h,
  *   no_launch_overlap  launch without programmatic stream serialisation, i.e. a
  *                      run starts only when its predecessor in the stream has
  *                      ended (every later run of the handle)
- *   wait_limit_ms      bound of the device-side waits, milliseconds (default
+ *   wait_limit_ms      bound of the device-side waits of both kernels, milliseconds (default
  *                      2000, at most 60000)
  *   no_small_blocks    keep 4x4 output pixels per thread even for shapes that the
  *                      planner would run with 4x2 pixels per thread (a single small
@@ -370,7 +396,16 @@ typedef struct {
                                    waits) rather than by all of their blocks after a wait         */
     int32_t matrix_path;        /* 1: a run takes the matrix units instead (dense taps, pruned weights as
                                    zeros), because the caller's tuning names no parameter of the
-                                   command-stream kernel; the fields above describe that kernel's plan */
+                                   command-stream kernel; the fields above describe that kernel's plan,
+                                   the fields below the launch of an xgen_patconv_run (0 otherwise)   */
+    int32_t matrix_items;       /* (tile or pair of tiles, range of filters) to be worked through      */
+    int32_t matrix_splits;      /* thread blocks (pairs) of a cluster that share an item's channels    */
+    int32_t matrix_blocks;      /* thread blocks of the launch                                         */
+    int32_t matrix_cluster;     /* thread blocks of a cluster                                          */
+    int32_t matrix_threads;     /* threads of a block                                                  */
+    int32_t matrix_filters;     /* filters of an item                                                  */
+    int32_t matrix_stages;      /* pieces that the input channels are staged in                        */
+    int64_t matrix_shared_bytes; /* dynamic shared memory of a block                                   */
 } xgen_patconv_plan_stats;
 
 /* Fill *stats for the shape.  No CUDA work is enqueued.  Errors: INVALID_ARG, SHAPE, UNSUPPORTED. */

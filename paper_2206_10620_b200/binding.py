@@ -50,7 +50,8 @@ class Stats(ctypes.Structure):
                 ("n_blocks", ctypes.c_int32), ("channels_per_chunk", ctypes.c_int32),
                 ("n_chunks", ctypes.c_int32), ("patterns_compiled", ctypes.c_int32),
                 ("max_segment_slots", ctypes.c_int32),
-                ("load_commands", ctypes.c_int64), ("group_imbalance", ctypes.c_double)]
+                ("load_commands", ctypes.c_int64), ("group_imbalance", ctypes.c_double),
+                ("image_bytes", ctypes.c_int64), ("device_bytes", ctypes.c_int64)]
 
 
 class Tuning(ctypes.Structure):
@@ -69,7 +70,11 @@ class PlanStats(ctypes.Structure):
                 ("lanes_n", ctypes.c_int32), ("pixels_per_lane", ctypes.c_int32), ("stages", ctypes.c_int32),
                 ("uses_copy_engine", ctypes.c_int32), ("shared_bytes", ctypes.c_int64),
                 ("workspace_bytes", ctypes.c_int64), ("covered", ctypes.c_double),
-                ("last_arriver", ctypes.c_int32), ("matrix_path", ctypes.c_int32)]
+                ("last_arriver", ctypes.c_int32), ("matrix_path", ctypes.c_int32),
+                ("matrix_items", ctypes.c_int32), ("matrix_splits", ctypes.c_int32),
+                ("matrix_blocks", ctypes.c_int32), ("matrix_cluster", ctypes.c_int32),
+                ("matrix_threads", ctypes.c_int32), ("matrix_filters", ctypes.c_int32),
+                ("matrix_stages", ctypes.c_int32), ("matrix_shared_bytes", ctypes.c_int64)]
 
 
 class ProbeResult(ctypes.Structure):
@@ -95,7 +100,7 @@ class GemmStats(ctypes.Structure):
                 ("row_commands", ctypes.c_int64), ("rows_per_warp", ctypes.c_int32),
                 ("warps_per_block", ctypes.c_int32), ("row_blocks", ctypes.c_int32),
                 ("stage_cols", ctypes.c_int32), ("n_stages", ctypes.c_int32),
-                ("max_stage_bytes", ctypes.c_int32)]
+                ("max_stage_bytes", ctypes.c_int32), ("device_bytes", ctypes.c_int64)]
 
 
 class DwDesc(ctypes.Structure):

@@ -653,6 +653,7 @@ xgen_status xgen_blockgemm_test_expect_arrivals(xgen_blockgemm_packed *h, int32_
 xgen_status xgen_blockgemm_query(const xgen_blockgemm_packed *h, xgen_blockgemm_stats *stats) {
     if (!h || !stats) return XGEN_ERR_INVALID_ARG;
     *stats = h->host.stats;
+    stats->device_bytes = (int64_t)h->tap.bytes + (h->d_stream ? stats->stream_bytes : 0);
     return XGEN_OK;
 }
 

@@ -1368,6 +1368,14 @@ static bool asks_for_stream(const xgen_patconv_tuning &t) {
 // Whether a run takes the matrix path.
 static bool on_matrix_units(const xgen_patconv_packed *h) { return h->tap.dev && !h->stream_asked; }
 
+// What the matrix path's plan of a call depends on.
+static TapShape tap_shape(const PackedHost &p, int n, int hh, int ww, int pool, bool residual, bool requant) {
+    TapShape ts;
+    ts.n = n; ts.h = hh; ts.w = ww; ts.stride = p.stride; ts.pool = pool == 2;
+    ts.staged = (residual && pool != 2) || p.c_out * (requant ? 1 : p.dtype == XGEN_F16_F32ACC ? 2 : 4) % 16 != 0;
+    return ts;
+}
+
 // The matrix path's plan of a shape, from the handle's small cache or made now.
 static bool tap_plan_of(const xgen_patconv_packed *h, const TapShape &s, TapPlan &plan) {
     std::lock_guard<std::mutex> lock(h->tap_mu);
@@ -1421,9 +1429,7 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
         }
     }
     if (h->tap.dev && (ignore_plan || !h->stream_asked)) {
-        TapShape ts;
-        ts.n = n; ts.h = hh; ts.w = ww; ts.stride = p.stride; ts.pool = pool == 2;
-        ts.staged = (residual && pool != 2) || p.c_out * (rq_scale ? 1 : p.dtype == XGEN_F16_F32ACC ? 2 : 4) % 16 != 0;
+        const TapShape ts = tap_shape(p, n, hh, ww, pool, residual != nullptr, rq_scale != nullptr);
         int prev = 0;
         if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
         if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
@@ -1629,6 +1635,10 @@ xgen_status xgen_patconv_out_shape(const xgen_patconv_packed *h, int32_t hh, int
 xgen_status xgen_patconv_query(const xgen_patconv_packed *h, xgen_patconv_stats *s) {
     if (!h || !s) return XGEN_ERR_INVALID_ARG;
     *s = h->host.stats;
+    s->image_bytes = h->tap.dev ? (int64_t)(h->tap.bytes - 16) : 0;
+    const int64_t stream = h->d_slots ? s->index_bytes + s->weight_bytes + 2 * kDevSlotBytes : 0;
+    s->device_bytes = (int64_t)h->tap.bytes + stream + (int64_t)(h->d_status ? sizeof(int) : 0) + (int64_t)h->partial_bytes +
+                      (int64_t)h->counter_bytes + (int64_t)h->hx_bytes + (int64_t)h->hy_bytes + (h->d_hb ? (int64_t)h->host.c_out * 4 : 0);
     return XGEN_OK;
 }
 
@@ -1693,7 +1703,21 @@ xgen_status xgen_patconv_plan_info(const xgen_patconv_packed *h, int32_t n, int3
     out->uses_copy_engine = L.kp.use_tma;
     out->shared_bytes = (int64_t)L.smem;
     out->last_arriver = planned && h->plan_last ? 1 : 0;
-    out->matrix_path = on_matrix_units(h) ? 1 : 0;
+    if (on_matrix_units(h)) {
+        int prev = 0;
+        if (cudaGetDevice(&prev) != cudaSuccess || cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
+        TapPlan tp;
+        const bool fits = tap_plan_of(h, tap_shape(p, n, hh, ww, 0, false, false), tp);
+        cudaSetDevice(prev);
+        if (fits) {
+            out->matrix_path = 1;
+            out->matrix_items = tp.items; out->matrix_splits = tp.splits; out->matrix_blocks = tp.grid;
+            out->matrix_cluster = (tp.pair ? 2 : 1) * tp.splits;
+            out->matrix_threads = tap_block_threads(p.dtype);
+            out->matrix_filters = tp.nt; out->matrix_stages = tp.stages;
+            out->matrix_shared_bytes = (int64_t)tp.smem;
+        }
+    }
     out->workspace_bytes = planned ? (int64_t)((size_t)(L.items - h->plan_whole) * (size_t)h->plan_splits * rows_per_item(p) * 1024) : 0;
     return XGEN_OK;
 }

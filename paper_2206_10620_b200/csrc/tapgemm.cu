@@ -1289,6 +1289,7 @@ static xgen_status tap_alloc(TapWeights &tw, xgen_dtype dt, int taps, int c_in, 
     tw.planes = (c_in + 2 * tap_cpp(dt) - 1) / (2 * tap_cpp(dt)) * 2;
     tw.rows = (c_out + 15) / 16 * 16;
     const size_t image = (size_t)tw.planes * taps * tap_parts(dt) * tw.rows * 16, bytes = image + 16;     // and the status word
+    tw.bytes = bytes;
     cudaError_t e = cudaMalloc(&tw.dev, bytes);
     if (e == cudaSuccess) e = cudaMalloc(&tw.scratch, extra);
     if (e == cudaSuccess) e = cudaMemsetAsync(tw.dev, 0, bytes, 0);
@@ -1316,6 +1317,7 @@ void tap_free(TapWeights &tw) {
     if (tw.scratch) cudaFree(tw.scratch);
     tw.dev = tw.scratch = nullptr;
     tw.status = nullptr;
+    tw.bytes = 0;
 }
 
 // Weights go up in pieces that keep the scratch within the driver's small blocks (1 MB): an allocation
@@ -1416,6 +1418,8 @@ static int tap_clusters(int size, int device, int sms) {
     k = n > 0 ? n : -1;
     return k;
 }
+
+int tap_block_threads(xgen_dtype dt) { return tap_threads(dt); }
 
 bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &best) {
     static int sm_count[64];

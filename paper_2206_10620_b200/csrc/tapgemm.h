@@ -24,6 +24,7 @@ EncodeTiledFn encode_tiled_fn();
 struct TapWeights {
     uint8_t *dev = nullptr;      // the image
     uint8_t *scratch = nullptr;  // what it is made from, while it is made
+    size_t bytes = 0;            // device memory: the image and the status word
     int *status = nullptr;       // behind the image: set by a kernel whose bounded wait ran out
     xgen_dtype dtype = XGEN_F32;
     int taps = 9, c_in = 0, c_out = 0;
@@ -74,6 +75,8 @@ xgen_status tap_upload_patterns(TapWeights &tw, xgen_dtype dt, int c_in, int c_o
                                 const uint32_t *kw4, const uint16_t *masks, int n_masks);
 void tap_free(TapWeights &tw);
 
+// Threads of a block.
+int tap_block_threads(xgen_dtype dt);
 // Pick a plan for the shape; false: this shape cannot run here.
 bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &plan);
 cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &plan, const TapCall &c, cudaStream_t st);

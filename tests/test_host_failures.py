@@ -110,3 +110,34 @@ def test_a_handle_holds_its_weight_image_and_no_more(fake_lib):
                 fake.fake_fail_alloc(nth)
                 assert status(gemm, dtype, k, co) == 5 and fake.fake_live_bytes() == held
     """)
+
+
+def test_queries_tell_of_what_runs_and_what_is_held(fake_lib):
+    """xgen_patconv_plan_info's matrix_* fields are the launch of a run, device_bytes is what was allocated."""
+    _run(fake_lib, """
+        for dtype in ("f32", "f16", "i8"):
+            for n, ci, co, h, w in ((1, 16, 32, 8, 8), (40, 64, 64, 40, 40), (32, 256, 256, 28, 28), (1, 512, 96, 14, 14), (3, 67, 93, 45, 77)):
+                held = fake.fake_live_bytes()
+                pk = conv(dtype, ci, co)
+                pk.plan(n, h, w)
+                info, st = pk.plan_info(n, h, w), pk.stats()
+                assert info["matrix_path"] == 1 and st["image_bytes"] > 0
+                assert st["device_bytes"] == fake.fake_live_bytes() - held
+                pk.run(X, n, h, w, B, True, Y)
+                got = [info["matrix_" + k] for k in ("blocks", "threads", "shared_bytes", "cluster")]
+                assert got == [fake.fake_launch(i) for i in range(4)], (got, dtype, n, ci, co, h, w)
+                pk.plan(n, h, w, splits=2)
+                info = pk.plan_info(n, h, w)
+                pk.run(X, n, h, w, B, True, Y)
+                assert info["matrix_path"] == 0 == info["matrix_blocks"]
+                assert [info["blocks"], info["threads_per_block"], info["shared_bytes"]] == [fake.fake_launch(i) for i in range(3)]
+                assert pk.stats()["device_bytes"] == fake.fake_live_bytes() - held
+                pk.close()
+        pk = conv("f32", 16, 32, device=-1)
+        assert pk.stats()["device_bytes"] == 0 and pk.plan_info(1, 8, 8)["matrix_path"] == 0
+        for kw in ({}, {"warps_per_block": 4}):
+            held = fake.fake_live_bytes()
+            g = gemm("f16", 200, 70, **kw)
+            assert g.stats()["device_bytes"] == fake.fake_live_bytes() - held
+            g.close()
+    """)
