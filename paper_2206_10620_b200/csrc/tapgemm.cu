@@ -28,7 +28,10 @@
 // The matrix unit truncates when it adds to its accumulator (measured: a chain of 288 steps ends
 // 1.5e-5 low, one of 9 steps 1.6e-7), so the leading product is accumulated for one stage only
 // (at most 18 steps) and then added, rounded, to sums in registers; the five small products have
-// an accumulator of their own, where truncation is 2^-8 of that, and are added the same way.
+// an accumulator of their own, where truncation is 2^-8 of that, and are added the same way.  fp16 chains of
+// more than 288 steps are cut every 144 (288) and added, rounded, to sums in tensor memory, by instances of
+// their own (CUT): 4096 channels of positive terms came out 7.3e-5 low in one chain, 4.2e-6 now; 512 do 8.5e-6.
+// (Time of uncut and cut, 32 images of 14x14 x 1024 -> 1024: 90.8, 97.6 us; 4096 rows x 8192 -> 1024: 57.2, 57.3.)
 //
 // Roles: 8 or 16 epilogue warps (tensor memory -> registers -> y), 6 producer warps (x), one
 // warp that issues the matrix instructions, one that fetches weights with tensor copies.  Blocks are
@@ -78,7 +81,7 @@ struct TapParams {
     int vh, straddle;                           // virtual rows per image; tiles may cross images
     uint32_t mg_vh, mg_pitch, mg_rows;          // division by these as a multiplication (div_by)
     int raster, pitch, rows, pixels, sub_px;    // staged tile: entries of a row, rows (of a parity), entries; of the second sub-tile
-    int segs, nblk, nt, items, splits, per_split, stages;
+    int segs, nblk, nt, items, splits, per_split, stages, cut;
     int pl, pl_log, plane_pitch;
     int a_stages, a_bytes, b_slots, resident, b_bytes, tap_group;
     int b_off, tab_off, stage_off, sum_off;     // bytes into dynamic shared memory
@@ -752,7 +755,7 @@ template <int TAPS> __device__ __forceinline__ TapPixel tap_pixel(const TapParam
     return TapPixel{pix, P.pool ? (img * P.po + oy / 2) * P.pw + ox / 2 : pix};
 }
 
-template <int DT, int STRIDE, int TAPS, int MT, bool PAIR>
+template <int DT, int STRIDE, int TAPS, int MT, bool PAIR, bool CUT>
 __global__ void __launch_bounds__(tap_threads(DT), 1)
 tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap) {
     using T = TapTraits<DT>;
@@ -971,12 +974,12 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             const uint32_t a_k = kF32 ? (uint32_t)P.plane_pitch * 2 / 16 : 2u, b_k = b_plane * 2, a_p = a_part / 16, b_p = b_rows;
             constexpr uint32_t a_px = kF32 ? 1 : 8;
             const uint32_t a_sub = (uint32_t)P.sub_px * a_px, a_step = (uint32_t)P.a_bytes / 16, b_step = (uint32_t)P.b_bytes / 16;
-            int s = 0, b = 0, buf = 0;
+            int s = 0, b = 0, buf = 0, run = 0;                             // run: stages since the accumulator was empty (CUT)
             uint32_t pha = 0, phb = 0, phc = 1, as = (uint32_t)a0, bs = (uint32_t)b0;
             bool ready = mbar_try<PAIR>(b_full(0), 0);
             for (int item = item0; item < P.items; item += item_step) {
                 for (int ks = k0; ks < k1; ++ks) {
-                    if (kF32 || ks == k0) wait(acc_empty(buf), phc);
+                    if (kF32 || (CUT ? run == 0 : ks == k0)) wait(acc_empty(buf), phc);
                     wait(a_full(s), pha);
                     tc_fence_after();
                     const int kk_n = min(P.pl, planes - ks * P.pl) / 2;
@@ -1001,7 +1004,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                             if (kk < kk_n) {
                                 const uint32_t ak = at + kk * a_k, bk = bt + kk * b_k;
                                 const uint32_t first_s = tap > 0 || kk > 0 ? 1u : 0u;       // 0: the first of the stage
-                                const uint32_t first_i = first_s | (ks > k0 ? 1u : 0u);     // 0: the first of the item
+                                const uint32_t first_i = first_s | ((CUT ? run > 0 : ks > k0) ? 1u : 0u);     // 0: the first of the item (CUT: of its part)
                                 if (kF32) {
                                     mma_f16<PAIR>(d, ak, a_hi, bk, b_hi, idesc, first_s);
                                     mma_f16<PAIR>(dc, ak, a_hi, bk + b_p, b_hi, idesc, first_s);
@@ -1030,7 +1033,9 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     tc_commit<PAIR>(a_empty(s), both);
                     as += a_step;
                     if (++s == P.a_stages) { s = 0; pha ^= 1u; as = (uint32_t)a0; }
-                    if (kF32 || ks + 1 == k1) {
+                    ++run;
+                    if (kF32 || ks + 1 == k1 || (CUT && run == P.cut)) {
+                        run = 0;
                         tc_commit<PAIR>(acc_full(buf), both);
                         if (++buf == P.acc_bufs) { buf = 0; phc ^= 1u; }
                     }
@@ -1158,6 +1163,38 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     finish(sum[0], 32 * q);
 #pragma unroll
                     for (int i = 0; i < 32; ++i) sum[0][i] = sum[1][i];
+                }
+            } else if (CUT) {
+                // the accumulator's sums go onto the item's, in columns behind the accumulators
+                for (int ks = k0; ks < k1; ks += P.cut) {
+                    wait_warp(acc_full(buf), ph);
+                    tc_fence_after();
+                    const uint32_t ta = tmem + lanes + (uint32_t)((buf * MT + sub) * P.nt), tt = tmem + lanes + (uint32_t)((P.acc_bufs * MT + sub) * P.nt);
+                    const bool first = ks == k0, last = ks + P.cut >= k1;
+#pragma unroll 1
+                    for (int q = group; q < chunks; q += kGroups) {
+                        uint32_t r[32];
+                        tmem_ld16(ta + 32 * q, r);
+                        tmem_ld16(ta + 32 * q + 16, r + 16);
+                        tmem_wait_ld();
+                        if (!first) {
+#pragma unroll
+                            for (int h = 0; h < 32; h += 16) {
+                                uint32_t t16[16];
+                                tmem_ld16(tt + 32 * q + h, t16);
+                                tmem_wait_ld();
+#pragma unroll
+                                for (int i = 0; i < 16; i += 2) add2(r[h + i], r[h + i + 1], t16[i], t16[i + 1]);
+                            }
+                        }
+                        if (last) finish(r, 32 * q);
+                        else {
+                            tmem_st16(tt + 32 * q, r);
+                            tmem_st16(tt + 32 * q + 16, r + 16);
+                            tmem_wait_st();
+                        }
+                    }
+                    release();
                 }
             } else {
                 wait_warp(acc_full(buf), ph);
@@ -1372,17 +1409,24 @@ xgen_status tap_upload_dense(TapWeights &tw, xgen_dtype dt, int c_in, int c_out,
 }
 
 // ---- plans ---------------------------------------------------------------------
-template <int DT, int TAPS> static const void *tap_kernel_dt(int stride, int mt, bool pair) {
-#define TAP_PICK(S, M) (pair ? (const void *)tap_kernel<DT, S, TAPS, M, true> : (const void *)tap_kernel<DT, S, TAPS, M, false>)
+template <int DT, int TAPS> static const void *tap_kernel_dt(int stride, int mt, bool pair, bool cut) {
+#define TAP_PICK_CUT(S, M, C) (pair ? (const void *)tap_kernel<DT, S, TAPS, M, true, C> : (const void *)tap_kernel<DT, S, TAPS, M, false, C>)
+#define TAP_PICK(S, M) TAP_PICK_CUT(S, M, false)
     constexpr int M2 = DT == XGEN_F32 ? 1 : 2, S2 = TAPS == 1 ? 1 : 2;      // (what there is no instance of is never asked for)
+    constexpr bool C = DT == XGEN_F16_F32ACC;
+    if (cut) {
+        if (stride == 1) return mt == 2 ? TAP_PICK_CUT(1, M2, C) : TAP_PICK_CUT(1, 1, C);
+        return mt == 2 ? TAP_PICK_CUT(S2, M2, C) : TAP_PICK_CUT(S2, 1, C);
+    }
     if (stride == 1) return mt == 2 ? TAP_PICK(1, M2) : TAP_PICK(1, 1);
     return mt == 2 ? TAP_PICK(S2, M2) : TAP_PICK(S2, 1);
 #undef TAP_PICK
+#undef TAP_PICK_CUT
 }
-static const void *tap_kernel_of(xgen_dtype dt, int stride, int taps, int mt, bool pair) {
-    if (taps == 1) return dt == XGEN_F32 ? tap_kernel_dt<XGEN_F32, 1>(1, mt, pair) : tap_kernel_dt<XGEN_F16_F32ACC, 1>(1, mt, pair);
-    if (dt == XGEN_F32) return tap_kernel_dt<XGEN_F32, 9>(stride, mt, pair);
-    return dt == XGEN_F16_F32ACC ? tap_kernel_dt<XGEN_F16_F32ACC, 9>(stride, mt, pair) : tap_kernel_dt<XGEN_I8_I32, 9>(stride, mt, pair);
+static const void *tap_kernel_of(xgen_dtype dt, int stride, int taps, int mt, bool pair, bool cut) {
+    if (taps == 1) return dt == XGEN_F32 ? tap_kernel_dt<XGEN_F32, 1>(1, mt, pair, cut) : tap_kernel_dt<XGEN_F16_F32ACC, 1>(1, mt, pair, cut);
+    if (dt == XGEN_F32) return tap_kernel_dt<XGEN_F32, 9>(stride, mt, pair, cut);
+    return dt == XGEN_F16_F32ACC ? tap_kernel_dt<XGEN_F16_F32ACC, 9>(stride, mt, pair, cut) : tap_kernel_dt<XGEN_I8_I32, 9>(stride, mt, pair, cut);
 }
 
 // Once per kernel and device: large shared memory, clusters of 16.
@@ -1406,7 +1450,7 @@ static int tap_clusters(int size, int device, int sms) {
     std::lock_guard<std::mutex> lock(mu);
     int &k = known[device][size];
     if (k) return k;
-    const void *kern = tap_kernel_of(XGEN_F16_F32ACC, 1, 9, 1, false);
+    const void *kern = tap_kernel_of(XGEN_F16_F32ACC, 1, 9, 1, false, false);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)size); cfg.blockDim = dim3(tap_threads(XGEN_F16_F32ACC)); cfg.dynamicSmemBytes = kTapSmemMax;
     cudaLaunchAttribute at[1];
@@ -1499,6 +1543,13 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     p.per_split = (p.stages + sp - 1) / sp;
                     p.splits = (p.stages + p.per_split - 1) / p.per_split;
                     if (p.splits != sp) continue;
+                    // fp16: 4 steps of 16 channels a tap and stage; a chain of more than 288 (512 channels in nine taps)
+                    // is cut: every 144 steps where its sums and two accumulators fit tensor memory, every 288 with one
+                    p.cut = 0;
+                    if (dt == XGEN_F16_F32ACC && p.per_split * tw.taps * 4 > 288) {
+                        if (2 * mt * p.nt > 512) continue;
+                        p.cut = (3 * mt * p.nt <= 512 ? 144 : 288) / (tw.taps * 4);
+                    }
                     int64_t waves;
                     if (sp == 1) {
                         const int units = p.pair ? std::max(0, tap_clusters(2, device, sms)) : sms;
@@ -1535,8 +1586,8 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     if (!fits) continue;
                     p.smem = (size_t)p.a_stages * p.a_bytes + (size_t)p.b_slots * p.b_bytes + tables;
                     if (p.smem > (size_t)kTapSmemMax) continue;
-                    p.acc_bufs = dt == XGEN_F32 || 2 * mt * p.nt <= 512 ? 2 : 1;
-                    const int cols = dt == XGEN_F32 ? 4 * p.nt : p.acc_bufs * mt * p.nt;
+                    p.acc_bufs = dt == XGEN_F32 || (p.cut ? 3 : 2) * mt * p.nt <= 512 ? 2 : 1;
+                    const int cols = dt == XGEN_F32 ? 4 * p.nt : (p.acc_bufs + (p.cut ? 1 : 0)) * mt * p.nt;
                     for (p.tmem_cols = 32; p.tmem_cols < cols;) p.tmem_cols *= 2;
                     // Cycles of a stage: the matrix instructions (nt / 2 each; 46 to issue one and 90 for a tap), or
                     // what they and the copies move through shared memory at 128 bytes a cycle (128 rows of x,
@@ -1554,7 +1605,8 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     const double move = (x_moved + b_moved) / 40.0 + (copied && p.straddle ? 60.0 * p.rows * (s.stride == 1 ? 1 : 4) : 0.0) * 0.5;
                     const double stage = std::max(std::max(mma, shared), move) + 250.0 + 40.0 * taps / p.tap_group + (p.pair && tw.taps == 1 ? 300.0 : 0.0);
                     const double out = (double)mt * 128 * p.nt * yb / 24.0;
-                    const double item = p.per_split * stage;
+                    // (one accumulator that is cut waits for its sums to be added)
+                    const double item = p.per_split * stage + (p.cut && p.acc_bufs == 1 ? (p.per_split - 1) / p.cut * 1500.0 : 0.0);
                     double c = 3500.0 + (p.pair ? dt == XGEN_F32 || s.stride == 2 ? 4000.0 : 6000.0 : 0.0);
                     if (sp == 1) c += waves * std::max(item, p.acc_bufs == 2 ? out : 0.0) + (p.acc_bufs == 2 ? out : waves * out);
                     else c += waves * (item + 3500.0 + 100.0 * sp + mt * 128.0 * p.nt * 4 / 64.0 + out / sp);
@@ -1608,7 +1660,7 @@ cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p
     P.npix = s.rows;
     P.c_in = tw.c_in; P.c_out = tw.c_out;
     P.vh = p.vh; P.straddle = p.straddle;
-    P.segs = p.segs; P.nblk = p.nblk; P.nt = p.nt; P.items = p.items; P.splits = p.splits; P.per_split = p.per_split; P.stages = p.stages;
+    P.segs = p.segs; P.nblk = p.nblk; P.nt = p.nt; P.items = p.items; P.splits = p.splits; P.per_split = p.per_split; P.stages = p.stages; P.cut = p.cut;
     P.pl = p.pl; P.pl_log = p.pl == 2 ? 1 : p.pl == 4 ? 2 : 3; P.plane_pitch = p.plane_pitch;
     P.a_stages = p.a_stages; P.b_slots = p.b_slots; P.resident = p.resident;
     P.b_bytes = p.b_bytes; P.tap_group = p.tap_group;
@@ -1647,7 +1699,7 @@ cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p
     // D fp32 (int32), A fp16 / bf16 / u8, B fp16 / bf16 / s8, both K-major, 128 rows (256 of a pair)
     P.idesc = ((uint32_t)(p.nt >> 3) << 17) | ((p.pair ? 16u : 8u) << 24) |
               (dt == XGEN_I8_I32 ? (2u << 4) | (1u << 10) : (1u << 4) | (dt == XGEN_F32 ? (1u << 7) | (1u << 10) : 0u));
-    const void *kern = tap_kernel_of(dt, s.stride, tw.taps, p.mt, p.pair);
+    const void *kern = tap_kernel_of(dt, s.stride, tw.taps, p.mt, p.pair, p.cut != 0);
     int device = 0;
     cudaError_t e = cudaGetDevice(&device);
     if (e == cudaSuccess) e = tap_allow(kern, device);

@@ -48,6 +48,7 @@ struct TapPlan {
     int nt = 0, nblk = 0;        // filters of a tile, tiles of filters
     int pl = 0, stages = 0;      // planes per stage, stages of the whole reduction
     int splits = 1, per_split = 0;   // blocks that share an item's reduction (one cluster), stages of each
+    int cut = 0;                 // fp16: stages after which sums leave the matrix unit's accumulator (0: all of them)
     int vh = 0, straddle = 0, segs = 0, row_tiles = 0, items = 0, grid = 0;
     int raster = 0, pitch = 0, rows = 0, pixels = 0;     // staged tile: entries of a row, rows (of a parity), entries
     int a_stages = 0, a_bytes = 0, b_slots = 0, b_bytes = 0, tap_group = 1, resident = 0;

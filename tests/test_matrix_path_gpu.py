@@ -138,6 +138,55 @@ def test_fp32_sums_keep_fp32_precision():
     np.testing.assert_allclose(run_gpu(pack(d), d.x, None, False), ref, rtol=1e-6, atol=0)
 
 
+@pytest.mark.parametrize("ci", [512, 1024, 4096])
+def test_fp16_sums_of_many_channels(ci):
+    """Matrix instructions truncate when they add: a step loses less than a unit of the accumulator's last
+    place, 2^-23 of the sum so far; half of one on the average, and of a sum that on the average is half there, so
+    2^-25 a step of the whole where all terms are positive.  No chain is longer than 288 steps."""
+    d = _layer("f16", 2, ci, 64, 16, 16, prune=0.0, seed=ci)
+    d.w = np.abs(d.w)
+    pk = pack(d)
+    assert pk.plan_info(74, 16, 16)["matrix_splits"] == 1
+    y = run_gpu(pk, np.tile(d.x, (37, 1, 1, 1)), None, False)
+    assert np.array_equal(y[:2], y[-2:])
+    ref = oracle.conv(d.x, d.w, d.pid, d.masks, bias=None, relu=False)
+    steps = min(9 * (ci // 16), 288)
+    assert (np.abs(y[:2] - ref) <= (2.0 ** -11 + steps * 2.0 ** -23) * ref + 2.0 ** -25).all()
+    # (the mean of 2^15 roundings to fp16 is within 2^-11 / 2^7 of none)
+    assert -steps * 2.0 ** -25 - 2.0 ** -18 <= (y[:2] / ref - 1).mean() <= 2.0 ** -18
+
+
+@pytest.mark.parametrize("n,ci,co,hw,stride", [
+    (74, 600, 64, 16, 1),         # two accumulators, cut every 4 stages, a short last part
+    (74, 600, 64, 32, 2),
+    (74, 640, 256, 16, 1),        # one accumulator, cut every 8 stages, pairs of blocks
+    (40, 640, 256, 20, 1),        # two tiles a block
+    (10, 4096, 64, 16, 1),        # split over a cluster and cut
+])
+def test_fp16_chains_that_are_cut(n, ci, co, hw, stride):
+    d = _layer("f16", 1, ci, co, hw, hw, stride, prune=0.4, seed=ci + co)
+    x = np.tile(d.x, (n, 1, 1, 1))
+    y = run_gpu(pack(d), x, d.bias, True)
+    assert (y == y[:1]).all()
+    compare(d, y[:1])
+
+
+@pytest.mark.parametrize("m,k,co", [(20000, 4700, 256), (20000, 4616, 40), (300, 6000, 100)])
+def test_fp16_products_whose_chains_are_cut(m, k, co):
+    import torch
+    d = wl.make_block_gemm(wl.GemmSpec("t", 100, k, co, 16, 16, 0.7, 0.7, "f16"), seed=k)
+    g = binding.BlockGemm(k, co, 16, 16, "f16", d.w, d.row_keep, d.col_keep)
+    x, b = torch.from_numpy(d.x).cuda().repeat(m // 100, 1), torch.from_numpy(d.bias).cuda()
+    buf, y = guarded_output((m, co), torch.float16)
+    g.run(x.data_ptr(), m, b.data_ptr(), True, y.data_ptr())
+    g.sync()
+    check_guards(buf)
+    got = y.cpu().numpy().reshape(-1, 100, co)
+    assert (got == got[:1]).all()
+    ref, S = oracle.block_gemm(d.x, d.w, d.row_keep, d.col_keep, 16, 16, bias=d.bias, relu=True, with_scale=True)
+    assert (np.abs(got[0].astype(np.float64) - ref) <= TOL["f16"] * np.maximum(np.abs(ref), 0.01 * S) + 2.0 ** -25).all()
+
+
 def _sum_of_kept(x, w, keep, stride):
     """Sums over the kept weights alone, zeros around the image; fp64, infinities as they come."""
     n, h, wd, _ = x.shape
