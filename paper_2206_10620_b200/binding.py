@@ -129,7 +129,7 @@ _calls = None           # the extension, its calls bound to the loaded library
 
 
 def _bind_calls(L):
-    path = _build.CALLS_PATH if os.path.exists(_build.CALLS_PATH) else _build.build_calls()
+    path = _build.build_calls()             # (one made from other sources would marshal other arguments)
     spec = importlib.util.spec_from_file_location("_calls", path)
     m = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(m)
@@ -139,7 +139,7 @@ def _bind_calls(L):
 
 
 def lib():
-    """Load libpatconv.so (building it first if it is missing or stale)."""
+    """Load libpatconv.so (building it first if it is missing)."""
     global _lib, _calls
     if _lib is None:
         path = os.environ.get("XGEN_PATCONV_LIB") or _build.LIB_PATH    # another build of the library, if named

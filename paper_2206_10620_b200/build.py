@@ -1,6 +1,7 @@
 """Build libpatconv.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
 from __future__ import annotations
 
+import hashlib
 import os
 import subprocess
 import sys
@@ -34,13 +35,21 @@ def _mtime(name: str) -> float:
 
 
 def build_calls(force: bool = False) -> str:
-    """Compile the CPython extension that marshals the enqueueing calls (host code only)."""
+    """Compile the CPython extension that marshals the enqueueing calls (host code only), unless the one
+    that is there was made from these sources."""
     src = os.path.join(_CSRC, "calls.cpp")
-    newest = max(os.path.getmtime(f) for f in [src] + [os.path.join(_INC, h) for h in ("patconv.h", "blockgemm.h", "dwconv.h")])
-    if force or not os.path.exists(CALLS_PATH) or os.path.getmtime(CALLS_PATH) < newest:
+    digest = hashlib.sha256()
+    for f in [src] + [os.path.join(_INC, h) for h in ("patconv.h", "blockgemm.h", "dwconv.h")]:
+        with open(f, "rb") as fh:
+            digest.update(fh.read())
+    tag = "sources " + digest.hexdigest()          # stands in the file: a copy of the tree need not keep its times
+    if not force and os.path.exists(CALLS_PATH):
+        with open(CALLS_PATH, "rb") as fh:
+            force = tag.encode() not in fh.read()
+    if force or not os.path.exists(CALLS_PATH):
         tmp = CALLS_PATH + ".tmp%d" % os.getpid()
         subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-I", _INC,
-                               "-I", sysconfig.get_paths()["include"], src, "-o", tmp])
+                               "-I", sysconfig.get_paths()["include"], '-DXGEN_CALLS_TAG="%s"' % tag, src, "-o", tmp])
         os.replace(tmp, CALLS_PATH)
     return CALLS_PATH
 

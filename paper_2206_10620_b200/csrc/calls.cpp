@@ -85,6 +85,8 @@ static PyMethodDef methods[] = {
     {"bind", fast(bind), METH_FASTCALL, nullptr},   {"conv", fast(run<false>), METH_FASTCALL, nullptr},
     {"fused", fast(fused), METH_FASTCALL, nullptr}, {"gemm", fast(gemm), METH_FASTCALL, nullptr},
     {"dw", fast(run<true>), METH_FASTCALL, nullptr}, {nullptr, nullptr, 0, nullptr}};
+// What the extension was made from: build.py looks for it in the file.
+extern "C" __attribute__((used, visibility("default"))) const char xgen_calls_tag[] = XGEN_CALLS_TAG;
 static PyModuleDef module = {PyModuleDef_HEAD_INIT, "_calls", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 PyMODINIT_FUNC PyInit__calls(void) { return PyModule_Create(&module); }

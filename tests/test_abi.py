@@ -30,6 +30,17 @@ def test_header_symbols_are_exported():
     assert sorted(binding.EXPORTS) == names
 
 
+def test_a_stale_extension_is_made_anew(tmp_path, monkeypatch):
+    """The marshalling extension is tied to the sources it was made from, not to their times."""
+    path = str(tmp_path / "_calls.abi3.so")
+    monkeypatch.setattr(build, "CALLS_PATH", path)
+    with open(path, "wb") as f:                    # newer than every source, and not an extension
+        f.write(b"sources of something else")
+    assert hasattr(binding._bind_calls(binding.lib()), "conv")
+    made = os.stat(path).st_mtime_ns
+    assert build.build_calls() == path and os.stat(path).st_mtime_ns == made
+
+
 def test_strerror_and_launch_count():
     assert binding.strerror(0) == "ok"
     assert "pattern" in binding.strerror(2)
