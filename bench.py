@@ -9,10 +9,11 @@ output pixels / time, i.e. structural non-zeros only.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 
-Before the timed region the library's own microbenchmarks measure the rates of
-the fp32 FMA pipe (scalar and packed) and of the integer dot-product pipe, and
-the launch floor of a kernel shaped like the convolution kernels; the roofline
-figures are taken against those measured rates.  After the headline workload
+Roofline figures are taken against measured rates: layers on the matrix path
+(`tap_kernel`, all of a layer's weights, pruned ones as zeros) against a dense
+bf16 matrix product, fp32 counting its six bf16 products; layers on the
+command-stream kernel against the fp32 FMA pipe, whose rate, and the launch
+floor, the library's own microbenchmarks measure before the timed region.  After the headline workload
 the other named workloads (single layer, ResNet-50 and ResNet-18 3x3 stacks,
 the large-batch points of the single-layer sweep) are timed the same way and
 reported under "configs".
@@ -44,11 +45,11 @@ from paper_2206_10620_b200 import workloads as wl  # noqa: E402
 
 METRIC = "pattern-pruned conv3x3 useful GFLOP/s (VGG-16 3x3 stack, non-zero MACs only)"
 UNIT = "GFLOP/s"
-# FP32 pipe peak from unit counts and the maximum SM clock:
-# 148 SMs x 128 FMA lanes x 2 flop x 1.965 GHz.
-FP32_DERIVED_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
-KERNEL_SOURCES = ["paper_2206_10620_b200/csrc/patconv.cu", "paper_2206_10620_b200/csrc/gen_core.py",
-                  "paper_2206_10620_b200/csrc/pack.cpp"]
+# Matrix-unit products that a multiply-add of the dense layer takes, in bf16 products: fp32 operands are
+# three bf16 parts of which six products are taken; int8 runs at twice the rate.
+MATRIX_PRODUCTS = {"f32": 6.0, "f16": 1.0, "i8": 0.5}
+KERNEL_SOURCES = ["paper_2206_10620_b200/csrc/" + f for f in
+                  ("tapgemm.cu", "tapgemm.h", "ptx.cuh", "patconv.cu", "gen_core.py", "pack.cpp")]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic_vgg16_step.txt")
 
 
@@ -60,7 +61,7 @@ def kernel_source_digest() -> str:
 
 
 def recorded_traffic():
-    """DRAM bytes per launch of the convolution kernel from the committed ncu capture, or None
+    """DRAM bytes per launch of the convolution kernels from the committed ncu capture, or None
     when the kernel sources have changed since that capture was taken."""
     try:
         txt = open(TRAFFIC_FILE).read()
@@ -95,11 +96,13 @@ def workload(name="vgg16"):
     return wl.CONFIGS[name]()
 
 
-def measured_hbm_gbs():
+def measured_peaks():
+    """(copy rate in GB/s, bf16 matrix rate in TFLOP/s, where from)."""
     try:
-        return json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"], "measured"
+        m = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
+        return m["hbm_gbs"], m["bf16_tflops"], "measured"
     except Exception:
-        return 6650.0, "fallback"
+        return 6650.0, 1590.0, "fallback"
 
 
 class ClockSampler:
@@ -251,19 +254,18 @@ def stats(ms_list):
     return {"mean": float(a.mean()), "median": float(np.median(a)), "min": float(a.min()), "max": float(a.max())}
 
 
-def layer_bounds(s, fp32_tflops, dp4a_tmacs, hbm_gbs):
-    """Ideal times of one layer in seconds: on the fp32 FMA pipe (what every variant runs on), on
-    the integer dot-product pipe (the int8 variant's other yardstick) and on HBM."""
-    t_fp32 = 2.0 * s.useful_macs() / (fp32_tflops * 1e12)
-    t_dp4a = s.useful_macs() / (dp4a_tmacs * 1e12) if s.dtype == "i8" else None
-    t_hbm = s.compulsory_bytes() / (hbm_gbs * 1e9)
-    return t_fp32, t_dp4a, t_hbm
+def layer_bounds(s, matrix, fp32_tflops, bf16_tflops, hbm_gbs):
+    """Ideal times of one layer in seconds: on the pipe that its kernel runs on (the matrix units with the
+    whole dense layer, or the fp32 FMA pipe with the kept weights) and on HBM."""
+    t_pipe = (2.0 * s.dense_macs() * MATRIX_PRODUCTS[s.dtype] / (bf16_tflops * 1e12) if matrix
+              else 2.0 * s.useful_macs() / (fp32_tflops * 1e12))
+    return t_pipe, s.compulsory_bytes() / (hbm_gbs * 1e9)
 
 
-def time_block_gemm(torch, binding, dev, stream, flush, fp32_tflops, hbm_gbs, oracle_check=True, only="", reps=5):
+def time_block_gemm(torch, binding, dev, stream, flush, bf16_tflops, hbm_gbs, oracle_check=True, only="", reps=5):
     """Times xgen_blockgemm_run on the 1x1 layers of ResNet-50 in matrix form.  Per layer: median
-    microseconds, useful TFLOP/s (kept weights only), the fraction of the fp32 FMA pipe and of the
-    binding roofline (the slower of kept multiply-adds on that pipe and compulsory bytes at HBM rate)."""
+    microseconds, useful TFLOP/s (kept weights only), and the fraction of the binding roofline (the slower
+    of the dense product on the matrix units and compulsory bytes at HBM rate)."""
     out = {"layers": [], "recipe": "ResNet-50 1x1 convolutions as [batch*pixels, c_in] x [c_out, c_in]^T, batch 32, fp16 storage, "
                                    "32x32 pruning blocks, 40 % of rows and 40 % of columns kept per block"}
     t_all = ideal_all = flops_all = 0.0
@@ -289,12 +291,12 @@ def time_block_gemm(torch, binding, dev, stream, flush, fp32_tflops, hbm_gbs, or
             ts.append(e0.elapsed_time(e1))
         us = float(np.median(ts)) * 1e3
         macs = d.useful_macs()
-        t_alu = 2.0 * macs / (fp32_tflops * 1e12)
+        t_mma = 2.0 * d.dense_macs() * MATRIX_PRODUCTS[spec.dtype] / (bf16_tflops * 1e12)
         t_hbm = d.compulsory_bytes() / (hbm_gbs * 1e9)
         rec = {"layer": spec.name, "rows": spec.m, "us": round(us, 2), "useful_tflops": round(2.0 * macs / us * 1e-6, 2),
                "dense_equiv_tflops": round(2.0 * d.dense_macs() / us * 1e-6, 2),
-               "frac_of_fp32_pipe": round(t_alu * 1e6 / us, 4), "bound": "alu" if t_alu >= t_hbm else "hbm",
-               "ideal_us": round(max(t_alu, t_hbm) * 1e6, 2), "frac_of_binding_roofline": round(max(t_alu, t_hbm) * 1e6 / us, 4)}
+               "bound": "tensor" if t_mma >= t_hbm else "hbm",
+               "ideal_us": round(max(t_mma, t_hbm) * 1e6, 2), "frac_of_binding_roofline": round(max(t_mma, t_hbm) * 1e6 / us, 4)}
         if oracle_check and spec.m <= 8192:
             import oracle
             got = y[:256].cpu().numpy().astype(np.float64)
@@ -302,14 +304,13 @@ def time_block_gemm(torch, binding, dev, stream, flush, fp32_tflops, hbm_gbs, or
             rec["parity_ok"] = bool((np.abs(got - ref) <= 2e-3 * np.maximum(np.abs(ref), 0.01 * S) + 1e-30).all())
         out["layers"].append(rec)
         t_all += us
-        ideal_all += max(t_alu, t_hbm) * 1e6
+        ideal_all += max(t_mma, t_hbm) * 1e6
         flops_all += 2.0 * macs
         del pk, x, b, y
     torch.cuda.empty_cache()
     if t_all > 0:
         out["total_us"] = round(t_all, 1)
         out["useful_tflops"] = round(flops_all / t_all * 1e-6, 2)
-        out["frac_of_fp32_pipe"] = round(flops_all / t_all * 1e-6 / fp32_tflops, 4)
         out["frac_of_binding_roofline"] = round(ideal_all / t_all, 4)
     return out
 
@@ -385,12 +386,11 @@ def run_gpu(args):
     # --- pipe rates and launch floor, measured in this process before anything is timed
     probe = binding.probe(local)
     fp32_peak = max(probe["ffma_tflops"], probe["ffma2_tflops"])
-    dp4a_peak = probe["dp4a_tmacs"]
-    hbm, hbm_src = measured_hbm_gbs()
+    hbm, bf16_peak, peaks_src = measured_peaks()
 
     if args.block_gemm_only:                        # profiling aid: one layer of the matrix products, nothing else
         flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)
-        rec = time_block_gemm(torch, binding, dev, torch.cuda.current_stream().cuda_stream, flush, fp32_peak, hbm,
+        rec = time_block_gemm(torch, binding, dev, torch.cuda.current_stream().cuda_stream, flush, bf16_peak, hbm,
                               oracle_check=False, only=args.block_gemm_only, reps=3)
         print(json.dumps({"block_gemm": rec, "measured_peaks": probe}), flush=True)
         return
@@ -449,42 +449,39 @@ def run_gpu(args):
             torch.cuda.synchronize()
             ts.append(e0.elapsed_time(e1))
         t_ms = float(np.median(ts))
-        t_fp32, t_dp4a, t_hbm = layer_bounds(s, fp32_peak, dp4a_peak, hbm)
         info = pk.plan_info(s.n, s.h, s.w)
+        matrix = info["matrix_path"] == 1
+        t_pipe, t_hbm = layer_bounds(s, matrix, fp32_peak, bf16_peak, hbm)
         rec = {"layer": s.name, "us": round(t_ms * 1e3, 2), "us_min": round(min(ts) * 1e3, 2),
-               "ideal_us": round(max(t_fp32, t_hbm) * 1e6, 2), "launch_floor_us": round(probe["launch_floor_us"], 2),
+               "ideal_us": round(max(t_pipe, t_hbm) * 1e6, 2), "launch_floor_us": round(probe["launch_floor_us"], 2),
                "useful_gflops": round(2.0 * s.useful_macs() / t_ms / 1e6, 1),
                "dense_equiv_gflops": round(2.0 * s.dense_macs() / t_ms / 1e6, 1),
-               "bound": "alu" if t_fp32 >= t_hbm else "hbm",
-               "roofline_frac": round(max(t_fp32, t_hbm) / (t_ms * 1e-3), 4),
-               "grid": "%d tiles x %d filter blocks x %d splits" % (info["tiles"], info["filter_blocks"], info["splits"])}
-        if t_dp4a is not None:
-            rec["roofline_frac_dp4a"] = round(max(t_dp4a, t_hbm) / (t_ms * 1e-3), 4)
+               "kernel": "tap_kernel" if matrix else "patconv_kernel",
+               "bound": ("tensor" if matrix else "alu") if t_pipe >= t_hbm else "hbm",
+               "roofline_frac": round(max(t_pipe, t_hbm) / (t_ms * 1e-3), 4),
+               "grid": "%d blocks (clusters of %d), %d items x %d splits" % (
+                   info["matrix_blocks"], info["matrix_cluster"], info["matrix_items"], info["matrix_splits"]) if matrix
+               else "%d tiles x %d filter blocks x %d splits" % (info["tiles"], info["filter_blocks"], info["splits"])}
         per_layer.append(rec)
     layer_ms = sum(p["us"] for p in per_layer) * 1e-3
 
-    # The dominant kernel is the only kernel of the step: its achieved rate is the step's useful
-    # flops over the timed region (this rank's K steps, events on the launching stream).
+    # The dominant kernel is tap_kernel: its achieved rate is the matrix-unit products of its layers over the
+    # whole timed region (this rank's K steps, events on the launching stream; other layers' time included).
     own_ms = st_flushed["mean"]
-    achieved = 2.0 * useful / (own_ms * 1e-3) / 1e12
-    binding_ms = sum(max(layer_bounds(s, fp32_peak, dp4a_peak, hbm)[0], layer_bounds(s, fp32_peak, dp4a_peak, hbm)[2])
-                     for s in specs) * 1e3
-    med_mhz = clocks.get("sm_mhz") or 0.0
-    roofline = {"bound": "alu", "achieved": achieved, "peak": fp32_peak, "unit": "TFLOP/s",
-                "frac": achieved / fp32_peak,
+    on_matrix = [t[2].plan_info(t[0].n, t[0].h, t[0].w)["matrix_path"] == 1 for t in stack.layers]
+    issued = sum(2.0 * s.dense_macs() * MATRIX_PRODUCTS[s.dtype] for s, m in zip(specs, on_matrix) if m)
+    achieved = issued / (own_ms * 1e-3) / 1e12
+    binding_ms = sum(max(layer_bounds(s, m, fp32_peak, bf16_peak, hbm)) for s, m in zip(specs, on_matrix)) * 1e3
+    roofline = {"bound": "tensor", "achieved": achieved, "peak": bf16_peak, "unit": "TFLOP/s",
+                "frac": achieved / bf16_peak,
                 "traffic": recorded_traffic() if args.workload == "vgg16" and not args.only else None,
-                "kernel": "patconv_kernel (all %d layers of the step)" % len(specs),
-                "peak_source": "measured in this run: register-only fp32 FMA microbenchmarks at full occupancy "
-                               "(scalar %.1f, packed %.1f TFLOP/s); derived 148 SMs x 128 lanes x 2 x 1.965 GHz = %.2f"
-                               % (probe["ffma_tflops"], probe["ffma2_tflops"], FP32_DERIVED_TFLOPS),
-                "peak_derived": FP32_DERIVED_TFLOPS, "frac_of_derived_peak": achieved / FP32_DERIVED_TFLOPS,
-                "hbm_peak_gbs": hbm, "hbm_peak_source": hbm_src,
+                "kernel": "tap_kernel (%d of the %d layers of the step; the others patconv_kernel)" % (sum(on_matrix), len(specs)),
+                "achieved_is": "bf16 products of the dense layers, six per fp32 multiply-add",
+                "peak_source": "%s: dense bf16 matrix product of the library, burst" % peaks_src,
+                "hbm_peak_gbs": hbm, "hbm_peak_source": peaks_src,
                 "binding_roofline_ms": binding_ms, "frac_of_binding_roofline": binding_ms / own_ms,
                 "isolated_layers_ms": layer_ms,
-                "frac_isolated_layers": 2.0 * useful / (layer_ms * 1e-3) / 1e12 / fp32_peak,
-                "ms_x_median_sm_mhz": own_ms * med_mhz,
-                "frac_at_sampled_clock": (achieved / (fp32_peak * med_mhz / probe["sm_clock_mhz"])
-                                          if med_mhz and probe["sm_clock_mhz"] else None)}
+                "ms_x_median_sm_mhz": own_ms * (clocks.get("sm_mhz") or 0.0)}
 
     # --- parity of what was timed: the three smallest layers against the CPU oracle (outside the timing)
     parity_checked = []
@@ -561,18 +558,13 @@ def run_gpu(args):
             torch.cuda.synchronize()
             st_c = stats(stk.timed_steps(stream, args.config_steps, flush))
             t = st_c["median"] * 1e-3
-            bind = sum(max(layer_bounds(s, fp32_peak, dp4a_peak, hbm)[0], layer_bounds(s, fp32_peak, dp4a_peak, hbm)[2])
-                       for s in sp)
+            matrix = [l[2].plan_info(l[0].n, l[0].h, l[0].w)["matrix_path"] == 1 for l in stk.layers]
+            bind = sum(max(layer_bounds(s, m, fp32_peak, bf16_peak, hbm)) for s, m in zip(sp, matrix))
             rec = {"ms_per_step": st_c, "steps": args.config_steps, "layers": len(sp), "dtype": sp[0].dtype,
                    "batch": sp[0].n, "useful_tflops": 2.0 * stk.useful / t / 1e12,
                    "dense_equiv_tflops": 2.0 * stk.dense / t / 1e12,
-                   "frac_of_fp32_pipe": 2.0 * stk.useful / t / 1e12 / fp32_peak,
+                   "matrix_layers": sum(matrix),
                    "binding_roofline_ms": bind * 1e3, "frac_of_binding_roofline": bind / t}
-            if sp[0].dtype == "i8":
-                bind_d = sum(max(layer_bounds(s, fp32_peak, dp4a_peak, hbm)[1], layer_bounds(s, fp32_peak, dp4a_peak, hbm)[2])
-                             for s in sp)
-                rec["frac_of_dp4a_pipe"] = stk.useful / t / 1e12 / dp4a_peak
-                rec["frac_of_binding_roofline_dp4a"] = bind_d / t
             configs[name] = rec
             del stk
             torch.cuda.empty_cache()
@@ -631,7 +623,7 @@ def run_gpu(args):
     # weights), each layer alone after an L2 flush
     block_gemm = {}
     if rank == 0 and world == 1 and not args.no_configs and args.workload == "vgg16" and not args.only:
-        block_gemm = time_block_gemm(torch, binding, dev, stream, flush, fp32_peak, hbm, oracle_check=not args.no_parity)
+        block_gemm = time_block_gemm(torch, binding, dev, stream, flush, bf16_peak, hbm, oracle_check=not args.no_parity)
 
     depthwise = {}
     if rank == 0 and world == 1 and not args.no_configs and args.workload == "vgg16" and not args.only:
