@@ -10,6 +10,7 @@
  *   y = act( bias[c] + sum_{t in pattern(c)} W[c][t] * x[n][oy*s + dy(t) - 1][ox*s + dx(t) - 1][c] )
  *
  * with t = 3*dy + dx, zero padding of 1, stride s in {1,2}, act = ReLU or identity.
+ * (Pruned taps are multiplied as zeros: an infinity or NaN of x under one gives a NaN.)
  * Same conventions as patconv.h.
  */
 #ifndef XGEN_DWCONV_H

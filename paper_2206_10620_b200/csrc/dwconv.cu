@@ -106,9 +106,9 @@ template <int V> __device__ __forceinline__ void fma_v(float (&acc)[V], const fl
 // strip of TX output pixels and walks down a piece of the image's rows: an input row is loaded once
 // (the next row while this one is used), widened once, and added to the three output rows that it
 // belongs to (stride 2: an odd row is kept for the next output row).  All nine taps run with masked
-// weights, two channels an instruction: skipping a tap would save no traffic.  256 images' rows of
-// 56x56x128 fp16, batch 32: 24.2 us with a thread per output strip (each input row loaded and widened
-// three times, 825 instructions for 16 results).
+// weights, two channels an instruction: skipping a tap would save no traffic.  32 images of
+// 56x56x128 fp16: 24.2 us with a thread per output strip (each input row loaded and widened
+// three times, 825 instructions for 16 results), 16.4 us now.
 // S = stride, V = channels per thread (4, 2 or 1), TX = output pixels per thread along x.
 template <int DT, int S, int V, int TX>
 __global__ void __launch_bounds__(128) dwconv_kernel(const __grid_constant__ DParams P) {

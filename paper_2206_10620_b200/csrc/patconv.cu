@@ -1089,7 +1089,7 @@ struct xgen_patconv_packed {
     mutable bool host_call_before = false;
 };
 
-// The device copy of the command stream: there only where a run may need it (see uses_stream).
+// The device copy of the command stream: there only where a run may need it (asks_for_stream, or few input channels).
 static void free_device_layout(const xgen_patconv_packed *h) {
     if (h->d_slots) cudaFree(h->d_slots);
     if (h->d_seg_off) cudaFree(h->d_seg_off);

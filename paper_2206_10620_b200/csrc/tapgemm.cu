@@ -1,7 +1,9 @@
 // The pattern-pruned convolution and the block-pruned matrix product on the matrix units.
 //
 // What is left of a pruned layer is 4/9 x (1 - prune rate) of a dense one, but the matrix units
-// are 22 times (fp16) to 44 times (int8) the packed-FMA pipe, so the layer is run dense: pruned
+// are 22 times (fp16) to 44 times (int8) the packed-FMA pipe, 4 times in fp32 (six bf16 products), and the
+// command stream reaches 20 to 45 % of that, so the layer is run dense (fp32 layers of 512 channels on few
+// pixels are faster on the command stream from 88 % of the kernels pruned on, by 10 % at 90): pruned
 // weights are zeros of the operand.  0 x infinity is NaN there, so sums that come out infinite or NaN
 // are computed anew from the kept weights alone (tap_anew).
 //
