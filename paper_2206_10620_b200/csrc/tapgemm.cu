@@ -5,7 +5,7 @@
 // command stream reaches 20 to 45 % of that, so the layer is run dense (fp32 layers of 512 channels on few
 // pixels are faster on the command stream from 88 % of the kernels pruned on, by 10 % at 90): pruned
 // weights are zeros of the operand.  0 x infinity is NaN there, so sums that come out infinite or NaN
-// are computed anew from the kept weights alone (tap_anew).
+// are computed anew from the kept weights alone (tap_repair).
 //
 // The input of a tile with its halo is staged once per group of channels and serves all nine taps:
 // in shared memory a tap is only another start address.  A tile is 128 (256) output pixels, either
@@ -552,79 +552,6 @@ __device__ __forceinline__ void tap_direct(const TapParams &P, const uint32_t *s
     }
 }
 
-// ---- sums that are not finite -----------------------------------------------------
-// The matrix units multiply pruned weights too, as zeros, so an infinity or NaN of x reaches every
-// filter there, and in fp32 the parts of an infinity do not add up to one.  Every such sum is infinite or
-// NaN (an overflow of finite operands as well), and the layer's own value takes its place: the kept
-// weights of the filter, in fp32, in the order of the image, where kept zeros are -0.  Slow -- a lane reads
-// its filter's weights from end to end -- and bounded: 512 channels take 60 us a sum.
-template <int DT, int STRIDE, int TAPS>
-__device__ __noinline__ uint32_t tap_anew(const TapParams &P, int pix, int oc) {
-    constexpr int cpp = TapTraits<DT>::cpp, parts = TapTraits<DT>::parts;
-    int img = 0, oy = 0, ox = 0;
-    if (TAPS == 9) {
-        const int row = pix / P.wo;
-        ox = pix - row * P.wo;
-        img = row / P.ho;
-        oy = row - img * P.ho;
-    }
-    const size_t part = (size_t)P.w_rows * 16, step = part * parts;
-    const uint8_t *w = P.wimg + (size_t)oc * 16;
-    float sum = 0.0f;
-    for (int c0 = 0; c0 < P.c_in; c0 += cpp)
-        for (int t = 0; t < TAPS; ++t, w += step) {
-            const uint4 a = __ldg(reinterpret_cast<const uint4 *>(w));
-            if ((a.x | a.y | a.z | a.w) == 0u) continue;
-            size_t px = (size_t)pix;
-            bool in = true;
-            if (TAPS == 9) {
-                const int iy = oy * STRIDE + t / 3 - 1, ix = ox * STRIDE + t % 3 - 1;
-                in = (unsigned)iy < (unsigned)P.h && (unsigned)ix < (unsigned)P.w;
-                px = ((size_t)img * P.h + iy) * P.w + ix;
-            }
-            for (int e = 0; e < cpp; ++e) {
-                const unsigned short bits = __ldg(reinterpret_cast<const unsigned short *>(w) + e);
-                if (bits == 0) continue;                                // pruned
-                float wv, xv = 0.0f;
-                const size_t at = px * P.c_in + c0 + e;
-                if (DT == XGEN_F32) {
-                    const float p1 = __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short *>(w + part) + e) << 16);
-                    const float p2 = __uint_as_float((uint32_t)__ldg(reinterpret_cast<const unsigned short *>(w + 2 * part) + e) << 16);
-                    wv = __uint_as_float((uint32_t)bits << 16) + (p1 + p2);       // (exact)
-                    if (in) xv = __ldg(static_cast<const float *>(P.x) + at);
-                } else {
-                    wv = __half2float(__ushort_as_half(bits));
-                    if (in) xv = __half2float(__ushort_as_half(__ldg(static_cast<const unsigned short *>(P.x) + at)));
-                }
-                sum = fmaf(wv, xv, sum);
-            }
-            if (sum != sum) return __float_as_uint(sum);
-        }
-    return __float_as_uint(sum);
-}
-// The sums of N channels of a pixel, from channel c on, with those that are not finite computed anew; where all
-// are finite that is N / 2 packed multiply-adds and a branch.
-template <int N> __device__ __forceinline__ bool all_finite(const uint32_t (&v)[N]) {
-    uint32_t a0 = 0u, a1 = 0u, b0 = 0u, b1 = 0u;
-#pragma unroll
-    for (int i = 0; i < N; i += 4) {
-        nan_of(a0, a1, v[i], v[i + 1]);
-        nan_of(b0, b1, v[i + 2], v[i + 3]);
-    }
-    return __uint_as_float(a0) + __uint_as_float(a1) + (__uint_as_float(b0) + __uint_as_float(b1)) == 0.0f;
-}
-template <int DT, int STRIDE, int TAPS, int N>
-__device__ __forceinline__ void tap_mend(const TapParams &P, uint32_t (&v)[N], int pix, int c) {
-#pragma unroll 1
-    for (int i = 0; i < N; ++i) {
-        uint32_t w = v[0];
-        if ((w & 0x7F800000u) == 0x7F800000u && pix >= 0 && c + i < P.c_out) w = tap_anew<DT, STRIDE, TAPS>(P, pix, c + i);
-#pragma unroll
-        for (int k = 0; k + 1 < N; ++k) v[k] = v[k + 1];
-        v[N - 1] = w;
-    }
-}
-
 // ---- operands ------------------------------------------------------------------
 // fp32 -> three bf16 parts.  The first is clamped to the largest bf16 so that a finite value never
 // becomes an infinity; the parts of an infinity or NaN hold a NaN, so that every sum they go into does.
@@ -757,6 +684,134 @@ template <int TAPS> __device__ __forceinline__ TapPixel tap_pixel(const TapParam
     return TapPixel{pix, P.pool ? (img * P.po + oy / 2) * P.pw + ox / 2 : pix};
 }
 
+// ---- sums that are not finite -----------------------------------------------------
+// The matrix units multiply pruned weights too, as zeros, so an infinity or NaN of x reaches every
+// filter there, and in fp32 the parts of an infinity do not add up to one.  Every such sum is infinite or
+// NaN (an overflow of finite operands as well), and the layer's own value takes its place: the kept
+// weights of the filter, in fp32, in the order of the image, where kept zeros are -0.  A lane goes through the
+// weights of four adjacent filters from end to end, lanes side by side over their pixels.
+__device__ __forceinline__ uint32_t half_of(const uint4 &a, int e) {
+    const uint32_t w = e / 2 == 0 ? a.x : e / 2 == 1 ? a.y : e / 2 == 2 ? a.z : a.w;
+    return w >> (16 * (e % 2)) & 0xFFFFu;
+}
+template <int DT, int STRIDE, int TAPS>
+__device__ __noinline__ uint4 tap_anew(const TapParams &P, int pix, int oc) {
+    constexpr int cpp = TapTraits<DT>::cpp, parts = TapTraits<DT>::parts;
+    int img = 0, oy = 0, ox = 0;
+    if (TAPS == 9) {
+        const int row = pix / P.wo;
+        ox = pix - row * P.wo;
+        img = row / P.ho;
+        oy = row - img * P.ho;
+    }
+    const size_t part = (size_t)P.w_rows * 16, step = part * parts;
+    const uint8_t *w = P.wimg + (size_t)oc * 16;
+    float sum[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll 1
+    for (int c = 0; c < P.c_in; c += cpp) {
+#pragma unroll (DT == XGEN_F32 || TAPS == 1 ? 1 : 3)
+        for (int t = 0; t < TAPS; ++t, w += step) {
+            const uint4 z = make_uint4(0, 0, 0, 0);
+            const int iy = TAPS == 9 ? oy * STRIDE + t / 3 - 1 : 0, ix = TAPS == 9 ? ox * STRIDE + t % 3 - 1 : 0;
+            const bool in = TAPS == 1 || ((unsigned)iy < (unsigned)P.h && (unsigned)ix < (unsigned)P.w);
+            const size_t at = (TAPS == 9 ? ((size_t)img * P.h + iy) * P.w + ix : (size_t)pix) * P.c_in + c;
+            uint4 a[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) a[j] = __ldg(reinterpret_cast<const uint4 *>(w) + j);
+            float x8[8];                          // zeros outside the image
+            if (DT == XGEN_F32) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) x8[e] = in && c + e < P.c_in ? __ldg(static_cast<const float *>(P.x) + at + e) : 0.0f;
+            } else {
+                const unsigned short *const x = static_cast<const unsigned short *>(P.x) + at;
+                if (P.vec_x) {
+                    const uint4 q = in ? __ldg(reinterpret_cast<const uint4 *>(x)) : z;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) x8[e] = __half2float(__ushort_as_half((unsigned short)half_of(q, e)));
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) x8[e] = in && c + e < P.c_in ? __half2float(__ushort_as_half(__ldg(x + e))) : 0.0f;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                uint4 b1 = z, b2 = z;
+                if (DT == XGEN_F32) {
+                    b1 = __ldg(reinterpret_cast<const uint4 *>(w + part) + j);
+                    b2 = __ldg(reinterpret_cast<const uint4 *>(w + 2 * part) + j);
+                }
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const uint32_t bits = half_of(a[j], e);
+                    const float wv = DT == XGEN_F32 ? __uint_as_float(bits << 16) + (__uint_as_float(half_of(b1, e) << 16) + __uint_as_float(half_of(b2, e) << 16))
+                                                    : __half2float(__ushort_as_half((unsigned short)bits));      // (exact)
+                    if (bits) sum[j] = fmaf(wv, x8[e], sum[j]);                 // (0: pruned)
+                }
+            }
+        }
+        const float all = sum[0] * sum[1] * sum[2] * sum[3];
+        if (all != all && sum[0] != sum[0] && sum[1] != sum[1] && sum[2] != sum[2] && sum[3] != sum[3]) break;
+    }
+    return make_uint4(__float_as_uint(sum[0]), __float_as_uint(sum[1]), __float_as_uint(sum[2]), __float_as_uint(sum[3]));
+}
+template <int N> __device__ __forceinline__ bool all_finite(const uint32_t (&v)[N]) {
+    uint32_t a0 = 0u, a1 = 0u, b0 = 0u, b1 = 0u;
+#pragma unroll
+    for (int i = 0; i < N; i += 4) {
+        nan_of(a0, a1, v[i], v[i + 1]);
+        nan_of(b0, b1, v[i + 2], v[i + 3]);
+    }
+    return __uint_as_float(a0) + __uint_as_float(a1) + (__uint_as_float(b0) + __uint_as_float(b1)) == 0.0f;
+}
+// All threads of a block, for what the block has stored: threads side by side over four filters each.
+template <int DT, int STRIDE, int TAPS, int MT, bool PAIR>
+__device__ __noinline__ void tap_repair(const TapParams &P) {
+    // (the block's place anew: nothing need be kept for this until the end)
+    const unsigned csize = (PAIR ? 2 : 1) * P.splits, crank = blockIdx.x % csize;
+    const int side = PAIR ? (int)crank & 1 : 0, rank = (int)crank / (PAIR ? 2 : 1);
+    const int item0 = (int)(blockIdx.x / csize), item_step = P.splits > 1 ? P.items : (int)(gridDim.x / csize);
+    const int groups = P.nt / 4;
+    const bool pool = TAPS == 9 && P.pool;
+#pragma unroll 1
+    for (int item = item0; item < P.items; item += item_step) {
+        const TapItem t = tap_item<MT, PAIR>(P, item, side);
+#pragma unroll 1
+        for (int i = threadIdx.x; i < 128 * MT * groups; i += tap_threads(DT)) {
+            const int m = i / groups, c = t.n0 + (i - m * groups) * 4;
+            const TapPixel at = tap_pixel<TAPS>(P, t, m);
+            if (at.pix < 0 || c >= P.c_out || (P.splits > 1 && m / 16 % P.splits != rank)) continue;
+            if (pool && ((at.pix / P.wo % P.ho | at.pix % P.wo) & 1)) continue;              // (a window is its first pixel's)
+            const size_t off = (size_t)at.out * P.c_out + c;
+            bool odd[4], any = false;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                odd[j] = c + j < P.c_out &&
+                         (DT == XGEN_F32 ? (static_cast<const volatile uint32_t *>(P.y)[off + j] & 0x7F800000u) == 0x7F800000u
+                                         : (static_cast<const volatile unsigned short *>(P.y)[off + j] & 0x7C00u) == 0x7C00u);
+                any |= odd[j];
+            }
+            if (!any) continue;
+            uint32_t best[4] = {0u, 0u, 0u, 0u};
+#pragma unroll 1
+            for (int q = 0; q < (pool ? 4 : 1); ++q) {
+                const int pix = at.pix + (q & 1) + (q >> 1) * P.wo;
+                const uint4 s4 = tap_anew<DT, STRIDE, TAPS>(P, pix, c);
+                const uint32_t s[4] = {s4.x, s4.y, s4.z, s4.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (!odd[j]) continue;
+                    const uint32_t v = tap_affine1<DT, TAPS == 9>(P, P.bias ? static_cast<const uint32_t *>(P.bias)[c + j] : 0u, s[j],
+                                                                  (size_t)pix * P.c_out + c + j);
+                    best[j] = q == 0 ? v : tap_max<DT>(best[j], v);
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (odd[j]) tap_store1<DT, TAPS == 9>(P, 0.0f, best[j], off + j);
+        }
+    }
+}
+
 template <int DT, int STRIDE, int TAPS, int MT, bool PAIR, bool CUT>
 __global__ void __launch_bounds__(tap_threads(DT), 1)
 tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap) {
@@ -767,6 +822,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ uint32_t s_tmem;
     __shared__ int s_abort;
+    __shared__ int s_odd;                        // a sum has come out infinite or NaN
     __shared__ volatile int s_started;           // items whose x is being fetched
     __shared__ __align__(8) uint64_t s_bars[2 * kMaxA + 2 * kMaxB + 5];
     __shared__ __align__(16) uint32_t s_bias[kMaxFilterTile];
@@ -800,7 +856,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
 
     asm volatile("griddepcontrol.launch_dependents;");
     if (tid == 0) {
-        s_abort = 0; s_started = 0;
+        s_abort = 0; s_started = 0; s_odd = 0;
         for (int i = 0; i < P.a_stages; ++i) { mbar_init(a_full(i), (P.tma ? 1 : (PAIR ? 2 : 1) * kProdWarps) + P.hold); mbar_init(a_empty(i), 1); }
         for (int i = 0; i < P.b_slots; ++i) { mbar_init(b_full(i), 1); mbar_init(b_empty(i), 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(acc_full(i), 1); mbar_init(acc_empty(i), (PAIR ? 2 : 1) * kEpiWarps); }
@@ -1112,7 +1168,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     return;
                 }
                 if (n0 + c >= P.c_out) return;
-                if (DT != XGEN_I8_I32 && __any_sync(0xFFFFFFFFu, !all_finite(r))) tap_mend<DT, STRIDE, TAPS>(P, r, pix, n0 + c);
+                if (DT != XGEN_I8_I32 && !all_finite(r)) s_odd = 1;
                 if (!P.staged) tap_direct<DT, FUSED>(P, s_bias, s_scale, r, pix, out, n0 + c, n0);
                 else {
 #pragma unroll 1
@@ -1250,7 +1306,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                         }
                     }
                     const int pix = px.pix + (q & 1) + (q >> 1) * P.wo;
-                    if (DT != XGEN_I8_I32 && !all_finite(v8)) tap_mend<DT, STRIDE, TAPS>(P, v8, pix, c0);
+                    if (DT != XGEN_I8_I32 && !all_finite(v8)) s_odd = 1;
                     tap_affine<DT, FUSED, 8>(P, s_bias, v8, pix, true, c0, n0);
 #pragma unroll
                     for (int i = 0; i < 8; ++i) best[i] = q == 0 ? v8[i] : tap_max<DT>(best[i], v8[i]);
@@ -1264,6 +1320,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
     tc_fence_before();
     __syncthreads();
     if (warp == kEpiWarps + kProdWarps) tmem_free<PAIR>(tmem, (uint32_t)P.tmem_cols);
+    if (DT != XGEN_I8_I32 && s_odd) tap_repair<DT, STRIDE, TAPS, MT, PAIR>(P);
 }
 
 // ---- weight image ----------------------------------------------------------------
