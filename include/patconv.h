@@ -103,7 +103,8 @@ typedef struct {
                                      to 32)                                                     */
     int64_t device_bytes;         /* device memory that the handle holds as it stands: the image
                                      or the command stream with its tables, or both, the workspace
-                                     of a planned split and the staging buffers of host calls  */
+                                     of a planned split and the staging buffers of host calls.  (All
+                                     handles of a device share 1 MB for the upload of weights, beside) */
 } xgen_patconv_stats;
 
 /* Read-only view of the packed layout on the host, for inspection and tests.

@@ -1379,55 +1379,81 @@ __global__ void tap_expand_dense(uint8_t *img, int c_in, int rows, int k0, int c
 static int tap_cpp(xgen_dtype dt) { return dt == XGEN_I8_I32 ? 16 : 8; }
 static int tap_parts(xgen_dtype dt) { return dt == XGEN_F32 ? 3 : 1; }
 
-// The zeroed image, and `extra` bytes of upload scratch, which tap_done gives back.
-static xgen_status tap_alloc(TapWeights &tw, xgen_dtype dt, int taps, int c_in, int c_out, size_t extra, uint8_t **scratch) {
-    tw.dtype = dt; tw.taps = taps; tw.c_in = c_in; tw.c_out = c_out;
-    tw.planes = (c_in + 2 * tap_cpp(dt) - 1) / (2 * tap_cpp(dt)) * 2;
-    tw.rows = (c_out + 15) / 16 * 16;
-    const size_t image = (size_t)tw.planes * taps * tap_parts(dt) * tw.rows * 16, bytes = image + 16;     // and the status word
-    tw.bytes = bytes;
-    cudaError_t e = cudaMalloc(&tw.dev, bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&tw.scratch, extra);
-    if (e == cudaSuccess) e = cudaMemsetAsync(tw.dev, 0, bytes, 0);
-    *scratch = tw.scratch;
-    tw.status = reinterpret_cast<int *>(tw.dev + image);
-    if (e == cudaSuccess) return XGEN_OK;
-    cudaGetLastError();
-    tap_free(tw);
-    return e == cudaErrorMemoryAllocation ? XGEN_ERR_ALLOC : XGEN_ERR_CUDA;
+// Upload scratch: kPiece bytes a device, shared by all handles of the process, there while any handle is.  (Allocated
+// and freed by every handle it cost 0.6 ms of the 2.2 that a 1000 x 1000 fp32 handle takes; kept by every handle
+// it held a third of an fp32 image again.)  An upload holds `mu` until it has been waited for.
+constexpr size_t kPiece = 1 << 20;
+struct TapScratch {
+    std::mutex mu;
+    uint8_t *dev = nullptr;
+    int users = 0;               // weight images there are
+};
+static TapScratch &tap_scratch(int device) {
+    static TapScratch all[64];
+    return all[device & 63];
 }
 
-static xgen_status tap_done(TapWeights &tw, cudaError_t e) {
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(0);
-    if (tw.scratch) cudaFree(tw.scratch);
-    tw.scratch = nullptr;
-    if (e == cudaSuccess) return XGEN_OK;
-    cudaGetLastError();
-    tap_free(tw);
-    return XGEN_ERR_CUDA;
-}
+// One upload into a new zeroed image.  Ends with `done`, or leaves nothing.
+struct TapUpload {
+    TapWeights &tw;
+    TapScratch &sc;
+    std::unique_lock<std::mutex> lock;
+    uint8_t *scratch = nullptr, *own = nullptr;      // `own`: more than kPiece was asked for
+    explicit TapUpload(TapWeights &w, int device) : tw(w), sc(tap_scratch(device)), lock(sc.mu) { tw.device = device; }
+    ~TapUpload() {
+        if (own) cudaFree(own);
+        if (sc.users == 0 && sc.dev) { cudaFree(sc.dev); sc.dev = nullptr; }
+    }
+    xgen_status begin(xgen_dtype dt, int taps, int c_in, int c_out, size_t extra) {
+        tw.dtype = dt; tw.taps = taps; tw.c_in = c_in; tw.c_out = c_out;
+        tw.planes = (c_in + 2 * tap_cpp(dt) - 1) / (2 * tap_cpp(dt)) * 2;
+        tw.rows = (c_out + 15) / 16 * 16;
+        const size_t image = (size_t)tw.planes * taps * tap_parts(dt) * tw.rows * 16;
+        tw.bytes = image + 16;                       // and the status word
+        cudaError_t e = cudaMalloc(&tw.dev, tw.bytes);
+        if (e == cudaSuccess && extra > kPiece) e = cudaMalloc(&own, extra);
+        else if (e == cudaSuccess && !sc.dev) e = cudaMalloc(&sc.dev, kPiece);
+        if (e == cudaSuccess) e = cudaMemsetAsync(tw.dev, 0, tw.bytes, 0);
+        scratch = own ? own : sc.dev;
+        if (e != cudaSuccess) return fail(e);
+        tw.status = reinterpret_cast<int *>(tw.dev + image);
+        return XGEN_OK;
+    }
+    xgen_status done(cudaError_t e) {
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+        if (e != cudaSuccess) return fail(e);
+        ++sc.users;
+        return XGEN_OK;
+    }
+    xgen_status fail(cudaError_t e) {
+        cudaGetLastError();
+        if (tw.dev) cudaFree(tw.dev);
+        tw = TapWeights();
+        return e == cudaErrorMemoryAllocation ? XGEN_ERR_ALLOC : XGEN_ERR_CUDA;
+    }
+};
 
 void tap_free(TapWeights &tw) {
-    if (tw.dev) cudaFree(tw.dev);
-    if (tw.scratch) cudaFree(tw.scratch);
-    tw.dev = tw.scratch = nullptr;
-    tw.status = nullptr;
-    tw.bytes = 0;
+    if (!tw.dev) return;
+    TapScratch &sc = tap_scratch(tw.device);
+    std::lock_guard<std::mutex> lock(sc.mu);
+    cudaFree(tw.dev);
+    if (--sc.users == 0 && sc.dev) { cudaFree(sc.dev); sc.dev = nullptr; }
+    tw = TapWeights();
 }
 
-// Weights go up in pieces that keep the scratch within the driver's small blocks (1 MB): an allocation
-// beyond them takes longer than the upload, and kept for the handle's life (as one allocation with the image)
-// it held a third of an fp32 image again.
-constexpr size_t kPiece = 1 << 20;
-
+// Weights go up in pieces of the scratch.
 xgen_status tap_upload_patterns(TapWeights &tw, xgen_dtype dt, int c_in, int c_out, const int16_t *kpat, const uint32_t *kw4,
                                 const uint16_t *masks, int n_masks) {
     const size_t nk = (size_t)c_in * c_out, mb = ((size_t)n_masks * 2 + 15) / 16 * 16;
     const size_t piece = std::min(nk, (kPiece - mb) / 18 / 8 * 8);             // 16 bytes of weights and two of pattern each
-    uint8_t *scratch = nullptr;
-    const xgen_status st = tap_alloc(tw, dt, 9, c_in, c_out, mb + piece * 18, &scratch);
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess) return XGEN_ERR_CUDA;
+    TapUpload up(tw, device);
+    const xgen_status st = up.begin(dt, 9, c_in, c_out, mb + piece * 18);
     if (st != XGEN_OK) return st;
+    uint8_t *const scratch = up.scratch;
     const uint16_t *mk = reinterpret_cast<const uint16_t *>(scratch);
     const uint4 *w = reinterpret_cast<const uint4 *>(scratch + mb);
     const int16_t *kp = reinterpret_cast<const int16_t *>(scratch + mb + piece * 16);
@@ -1442,7 +1468,7 @@ xgen_status tap_upload_patterns(TapWeights &tw, xgen_dtype dt, int c_in, int c_o
         else if (dt == XGEN_F16_F32ACC) tap_expand_patterns<XGEN_F16_F32ACC><<<blocks, 256>>>(tw.dev, c_in, tw.rows, (int)k0, (int)n, kp, w, mk);
         else tap_expand_patterns<XGEN_I8_I32><<<blocks, 256>>>(tw.dev, c_in, tw.rows, (int)k0, (int)n, kp, w, mk);
     }
-    return tap_done(tw, e);
+    return up.done(e);
 }
 
 xgen_status tap_upload_dense(TapWeights &tw, xgen_dtype dt, int c_in, int c_out, const void *dense_w, const uint8_t *row_keep,
@@ -1451,9 +1477,12 @@ xgen_status tap_upload_dense(TapWeights &tw, xgen_dtype dt, int c_in, int c_out,
     const size_t blocks_of = (size_t)((c_out + br - 1) / br) * ((c_in + bc - 1) / bc);
     const size_t rb = blocks_of * br, cb = blocks_of * bc, fb = (rb + cb + 15) / 16 * 16;     // the keep flags, whole
     const size_t piece = std::min(nk, (std::max(kPiece, fb + kPiece / 4) - fb) / wb / 8 * 8);
-    uint8_t *scratch = nullptr;
-    const xgen_status st = tap_alloc(tw, dt, 1, c_in, c_out, fb + piece * wb, &scratch);
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess) return XGEN_ERR_CUDA;
+    TapUpload up(tw, device);
+    const xgen_status st = up.begin(dt, 1, c_in, c_out, fb + piece * wb);
     if (st != XGEN_OK) return st;
+    uint8_t *const scratch = up.scratch;
     cudaError_t e = cudaMemcpyAsync(scratch, row_keep, rb, cudaMemcpyHostToDevice, 0);
     if (e == cudaSuccess) e = cudaMemcpyAsync(scratch + rb, col_keep, cb, cudaMemcpyHostToDevice, 0);
     for (size_t k0 = 0; k0 < nk && e == cudaSuccess; k0 += piece) {
@@ -1464,7 +1493,7 @@ xgen_status tap_upload_dense(TapWeights &tw, xgen_dtype dt, int c_in, int c_out,
         if (dt == XGEN_F32) tap_expand_dense<XGEN_F32><<<blocks, 256>>>(tw.dev, c_in, tw.rows, (int)k0, (int)n, scratch + fb, scratch, scratch + rb, br, bc);
         else tap_expand_dense<XGEN_F16_F32ACC><<<blocks, 256>>>(tw.dev, c_in, tw.rows, (int)k0, (int)n, scratch + fb, scratch, scratch + rb, br, bc);
     }
-    return tap_done(tw, e);
+    return up.done(e);
 }
 
 // ---- plans ---------------------------------------------------------------------

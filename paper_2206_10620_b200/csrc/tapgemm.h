@@ -23,7 +23,7 @@ EncodeTiledFn encode_tiled_fn();
 // tap at once, so neither the filter tile nor the channels per stage is fixed here.
 struct TapWeights {
     uint8_t *dev = nullptr;      // the image
-    uint8_t *scratch = nullptr;  // what it is made from, while it is made
+    int device = -1;
     size_t bytes = 0;            // device memory: the image and the status word
     int *status = nullptr;       // behind the image: set by a kernel whose bounded wait ran out
     xgen_dtype dtype = XGEN_F32;

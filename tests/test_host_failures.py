@@ -89,8 +89,14 @@ def test_an_upload_that_fails_half_way_leaves_nothing(fake_lib):
 
 
 def test_a_handle_holds_its_weight_image_and_no_more(fake_lib):
-    """The scratch of the upload is given back; a failed upload leaves nothing."""
+    """The scratch of the upload is shared, 1 MB while there is any handle; a failed upload leaves nothing."""
     _run(fake_lib, """
+        assert fake.fake_live_bytes() == 0
+        for nth in (1, 2, 3):
+            fake.fake_fail_alloc(nth)
+            assert status(conv, "f32", 16, 32) == 5 and fake.fake_live_bytes() == 0
+        first = gemm("f16", 32, 32)
+        assert fake.fake_live_bytes() <= (1 << 20) + 2 * 32 * 32 + 64
         round16 = lambda n: -(-n // 16) * 16
         for dtype, ci, co in (("f32", 16, 32), ("f32", 300, 260), ("f16", 300, 260), ("i8", 300, 260)):
             per, parts = {"f32": (8, 3), "f16": (8, 1), "i8": (16, 1)}[dtype]
@@ -106,15 +112,17 @@ def test_a_handle_holds_its_weight_image_and_no_more(fake_lib):
             g = gemm(dtype, k, co)
             assert image < fake.fake_live_bytes() - held <= image + 64
             g.close()
-            for nth in (1, 2):
-                fake.fake_fail_alloc(nth)
-                assert status(gemm, dtype, k, co) == 5 and fake.fake_live_bytes() == held
+            fake.fake_fail_alloc(1)
+            assert status(gemm, dtype, k, co) == 5 and fake.fake_live_bytes() == held
+        first.close()
+        assert fake.fake_live_bytes() == 0
     """)
 
 
 def test_queries_tell_of_what_runs_and_what_is_held(fake_lib):
     """xgen_patconv_plan_info's matrix_* fields are the launch of a run, device_bytes is what was allocated."""
     _run(fake_lib, """
+        keep = gemm("f16", 32, 32)                # (the shared scratch is there)
         for dtype in ("f32", "f16", "i8"):
             for n, ci, co, h, w in ((1, 16, 32, 8, 8), (40, 64, 64, 40, 40), (32, 256, 256, 28, 28), (1, 512, 96, 14, 14), (3, 67, 93, 45, 77)):
                 held = fake.fake_live_bytes()
