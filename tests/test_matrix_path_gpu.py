@@ -243,6 +243,26 @@ def test_infinities_reach_kept_weights_alone(dtype, stride, shape):
     _same_with_infinities(y, _sum_of_kept(d.x, wt, keep, stride), S, dtype)
 
 
+@pytest.mark.parametrize("dtype,n,ci,co,hw", [
+    ("f16", 16, 128, 256, 28),    # two tiles a block
+    ("f16", 48, 256, 256, 28),    # pairs of blocks, several items each
+    ("f32", 48, 128, 256, 28),    # pairs, several items
+    ("f16", 74, 600, 64, 16),     # chains that are cut
+    ("f16", 10, 4096, 64, 16),    # split and cut
+])
+def test_infinities_in_every_item_of_a_block(dtype, n, ci, co, hw):
+    """The same image over and over: what is computed anew does not depend on the place."""
+    d = _layer(dtype, 1, ci, co, hw, hw, prune=0.6, seed=ci)
+    taps = np.array([[(int(m) >> t) & 1 for t in range(9)] for m in d.masks], bool)
+    keep = (d.pid.reshape(co, ci)[..., None] >= 0) & taps[d.pid.reshape(co, ci)]
+    d.x[0, 3, 4, 5], d.x[0, hw - 1, hw - 1, ci - 1], d.x[0, 9, 0, 1] = np.inf, -np.inf, np.nan
+    y = run_gpu(pack(d), np.tile(d.x, (n, 1, 1, 1)), None, False)
+    assert np.array_equal(y, np.broadcast_to(y[:1], y.shape), equal_nan=True)
+    w = d.w.reshape(co, ci, 9)
+    S = _sum_of_kept(np.abs(np.where(np.isfinite(d.x), d.x, 0)), np.abs(w), keep, 1)
+    _same_with_infinities(y[:1], _sum_of_kept(d.x, w, keep, 1), S, dtype)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f16"])
 @pytest.mark.parametrize("ci", [24, 256])
 def test_infinities_under_a_pool_and_a_residual(dtype, ci):
