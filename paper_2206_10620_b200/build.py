@@ -12,16 +12,17 @@ _CSRC = os.path.join(_HERE, "csrc")
 _INC = os.path.join(os.path.dirname(_HERE), "include")
 LIB_PATH = os.path.join(_HERE, "libpatconv.so")
 CALLS_PATH = os.path.join(_HERE, "_calls.abi3.so")     # the enqueueing calls for Python
-_SOURCES = ["patconv.cu", "tapgemm.cu", "blockgemm.cu", "dwconv.cu", "probe.cu", "pack.cpp"]
-_DEPS = _SOURCES + ["patconv_internal.h", "ptx.cuh", "tapgemm.h", "gen_core.py", "gen_blockgemm.py", os.path.join(_INC, "patconv.h"),
+_SOURCES = ["patconv.cu", "tapgemm.cu", "fewconv.cu", "blockgemm.cu", "dwconv.cu", "probe.cu", "pack.cpp"]
+_DEPS = _SOURCES + ["patconv_internal.h", "ptx.cuh", "tapgemm.h", "fewconv.h", "gen_core.py", "gen_blockgemm.py", os.path.join(_INC, "patconv.h"),
                     os.path.join(_INC, "blockgemm.h"), os.path.join(_INC, "dwconv.h")]
 
 
 _OBJ_DIR = os.path.join(_HERE, "_build")
 # what each source includes besides itself
 _INCLUDES = {
-    "patconv.cu": ["patconv_internal.h", "ptx.cuh", "tapgemm.h", "gen_core.py", os.path.join(_INC, "patconv.h")],
+    "patconv.cu": ["patconv_internal.h", "ptx.cuh", "tapgemm.h", "fewconv.h", "gen_core.py", os.path.join(_INC, "patconv.h")],
     "tapgemm.cu": ["patconv_internal.h", "ptx.cuh", "tapgemm.h", os.path.join(_INC, "patconv.h")],
+    "fewconv.cu": ["patconv_internal.h", "fewconv.h", os.path.join(_INC, "patconv.h")],
     "blockgemm.cu": ["patconv_internal.h", "tapgemm.h", "gen_blockgemm.py", os.path.join(_INC, "patconv.h"),
                      os.path.join(_INC, "blockgemm.h")],
     "dwconv.cu": ["patconv_internal.h", os.path.join(_INC, "patconv.h"), os.path.join(_INC, "dwconv.h")],

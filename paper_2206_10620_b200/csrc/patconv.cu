@@ -41,6 +41,7 @@
 #include "core_gen.inc"
 #include "patconv_internal.h"
 #include "ptx.cuh"
+#include "fewconv.h"
 #include "tapgemm.h"
 
 namespace patconv {
@@ -1071,6 +1072,7 @@ struct xgen_patconv_packed {
     // the layer as dense taps on the matrix units (tapgemm.cu): what a run takes unless the caller
     // has asked for parameters of the command-stream kernel
     TapWeights tap;
+    FewWeights few;                     // ... or a layer of a few input channels on the FP32 pipe (fewconv.cu)
     bool stream_asked = false;
     mutable std::mutex tap_mu;
     mutable TapEntry tap_cache[kLaunchCache];
@@ -1368,6 +1370,17 @@ static bool asks_for_stream(const xgen_patconv_tuning &t) {
 // Whether a run takes the matrix path.
 static bool on_matrix_units(const xgen_patconv_packed *h) { return h->tap.dev && !h->stream_asked; }
 
+// A layer of a few input channels: whether the command stream, whose work is the kept kernels alone, beats the dense kernel.
+// An image of 224x224 of a large batch takes the dense kernel 1.9 us a channel (64 filters), the stream 5 (fp32), 5.5 (fp16) or
+// 7 us (int8) and about one for every kept kernel of a filter: 9 images, 60 % pruned, dense against stream, us: fp32 4 channels
+// 70.5, 62.8; fp16 7: 121, 83.9; int8 7: 115, 97.4 (unpruned, one image: 9.8, 12.9; 15.5, 15.7; 14.3, 18.4).  Small images, stride 2 and
+// filters that do not fill its warps leave the stream's threads idle (32 x 112x112, 3 -> 32, stride 2: 8.6, 19.9).
+static bool stream_is_faster(const PackedHost &p, int64_t pixels) {
+    if (p.stride != 1 || p.c_out % 64 != 0 || pixels < 40000) return false;
+    const double fixed = p.dtype == XGEN_F32 ? 5.0 : p.dtype == XGEN_F16_F32ACC ? 5.5 : 7.0;
+    return fixed + (double)p.stats.kernels_surviving / p.c_out < 1.9 * p.c_in;
+}
+
 // What the matrix path's plan of a call depends on.
 static TapShape tap_shape(const PackedHost &p, int n, int hh, int ww, int pool, bool residual, bool requant) {
     TapShape ts;
@@ -1447,6 +1460,14 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
         }
         if (prev != h->device) cudaSetDevice(prev);
         if (fits) return e == cudaSuccess ? XGEN_OK : XGEN_ERR_CUDA;
+    }
+    if (h->few.dev && !ep && (ignore_plan || (!h->stream_asked && !stream_is_faster(p, (int64_t)n * ho * wo)))) {
+        int prev = 0;
+        if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
+        if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
+        const cudaError_t e = log_cuda(few_launch(h->few, x, n, hh, ww, p.stride, bias, relu != 0, y, !h->tuning.no_launch_overlap, (cudaStream_t)stream), "few-channel kernel launch");
+        if (prev != h->device) cudaSetDevice(prev);
+        return e == cudaSuccess ? XGEN_OK : XGEN_ERR_CUDA;
     }
     {
         // (only where the driver cannot encode the matrix path's tensor maps is the stream not there yet)
@@ -1585,18 +1606,16 @@ xgen_status xgen_patconv_pack(const xgen_patconv_desc *desc, const void *dense_w
         else if (cudaMemset(h->d_status, 0, sizeof(int)) != cudaSuccess) us = XGEN_ERR_CUDA;
         const PackedHost &p = h->host;
         // A few input channels fill little of the 16 (32) that a matrix instruction takes, and rows of fp16 or
-        // int8 that are not whole 16-byte pieces are gathered: such first layers stay on the command-stream
-        // kernel.  -> 64 filters at 224x224, unpruned, command stream against matrix path, us, by input channels:
-        //   fp32     1: 10.4, 12.9   2: 11.5, 12.9   3: 12.6, 12.9   4: 13.3, 12.9   5: 14.8, 13.0   7: 17.2, 13.0
-        //   fp32 with 60 % pruned    3: 10.7, 12.9   4: 11.0, 12.9   5: 12.2, 12.9   6: 13.0, 12.9
-        //   fp16     1: 8.9, 15.6    3: 11.0, 16.9   5: 13.9, 17.1   7: 15.8, 16.8   8: 16.4, 10.1
-        //   int8     1: 12.0, 15.7   3: 13.8, 16.7   5: 16.5, 16.8   7: 18.6, 17.2 (60 % pruned 14.8, 17.2)
-        // and 32 images of 112x112 at stride 2, 32 filters: fp32 3: 23.2, 27.4   4: 36.5, 27.4   5: 31.0, 29.3; fp16 7: 31.2, 56.7.
-        // (Small images run faster on the matrix units at every count -- 3 -> 32 at 32x32, fp32: 9.4, 5.9 -- but a
-        // handle does not know its images, and few of these layers see such.)
-        if (us == XGEN_OK)
-            us = desc->c_in < (desc->dtype == XGEN_F32 ? 5 : 8) ? upload_layout(h)
-                                : tap_upload_patterns(h->tap, p.dtype, p.c_in, p.c_out, p.kpat.data(), p.kw4.data(), p.masks.data(), (int)p.masks.size());
+        // int8 that are not whole 16-byte pieces go through the producer warps: such layers run on the FP32 pipe (fewconv.cu),
+        // with operators fused behind them, the caller's tuning or few kernels left (stream_is_faster) on the command stream.
+        // The line between (few_channels), 224x224 -> 64 filters, us, on either side of it: fp32 4: 10.1, 5: 12.8; fp16 7: 15.5, 8: 8.8
+        // (rows of whole 16-byte pieces, by tensor copies; 7 gathered: 16.8); int8 7: 14.3 (gathered 17.2).
+        if (us == XGEN_OK && few_channels(desc->dtype, desc->c_in)) {
+            us = upload_layout(h);
+            if (us == XGEN_OK) us = few_upload(h->few, p.dtype, p.c_in, p.c_out, p.kpat.data(), p.kw4.data(), p.masks.data());
+            if (us != XGEN_OK) free_device_layout(h);
+        } else if (us == XGEN_OK)
+            us = tap_upload_patterns(h->tap, p.dtype, p.c_in, p.c_out, p.kpat.data(), p.kw4.data(), p.masks.data(), (int)p.masks.size());
         if (us != XGEN_OK && h->d_status) { cudaGetLastError(); cudaFree(h->d_status); }
         cudaSetDevice(prev);
         if (us != XGEN_OK) { delete h; return us; }
@@ -1611,6 +1630,7 @@ void xgen_patconv_free(xgen_patconv_packed *h) {
     free_device_layout(h);
     if (h->d_status) cudaFree(h->d_status);
     tap_free(h->tap);
+    few_free(h->few);
     if (h->d_partial) cudaFree(h->d_partial);
     if (h->d_counters) cudaFree(h->d_counters);
     if (h->d_hx) cudaFree(h->d_hx);
@@ -1637,7 +1657,7 @@ xgen_status xgen_patconv_query(const xgen_patconv_packed *h, xgen_patconv_stats 
     *s = h->host.stats;
     s->image_bytes = h->tap.dev ? (int64_t)(h->tap.bytes - 16) : 0;
     const int64_t stream = h->d_slots ? s->index_bytes + s->weight_bytes + 2 * kDevSlotBytes : 0;
-    s->device_bytes = (int64_t)h->tap.bytes + stream + (int64_t)(h->d_status ? sizeof(int) : 0) + (int64_t)h->partial_bytes +
+    s->device_bytes = (int64_t)h->tap.bytes + stream + (h->few.dev ? (int64_t)9 * h->few.c_in * h->few.rows * 4 : 0) + (int64_t)(h->d_status ? sizeof(int) : 0) + (int64_t)h->partial_bytes +
                       (int64_t)h->counter_bytes + (int64_t)h->hx_bytes + (int64_t)h->hy_bytes + (h->d_hb ? (int64_t)h->host.c_out * 4 : 0);
     return XGEN_OK;
 }
