@@ -12,8 +12,8 @@ _CSRC = os.path.join(_HERE, "csrc")
 _INC = os.path.join(os.path.dirname(_HERE), "include")
 LIB_PATH = os.path.join(_HERE, "libpatconv.so")
 CALLS_PATH = os.path.join(_HERE, "_calls.abi3.so")     # the enqueueing calls for Python
-_SOURCES = ["patconv.cu", "tapgemm.cu", "fewconv.cu", "blockgemm.cu", "dwconv.cu", "probe.cu", "pack.cpp"]
-_DEPS = _SOURCES + ["patconv_internal.h", "ptx.cuh", "tapgemm.h", "fewconv.h", "gen_core.py", "gen_blockgemm.py", os.path.join(_INC, "patconv.h"),
+_SOURCES = ["patconv.cu", "tapgemm.cu", "tapgemm_f32.cu", "tapgemm_f16.cu", "tapgemm_f16_cut.cu", "tapgemm_i8.cu", "fewconv.cu", "blockgemm.cu", "dwconv.cu", "probe.cu", "pack.cpp"]
+_DEPS = _SOURCES + ["patconv_internal.h", "ptx.cuh", "tapgemm.h", "tapgemm_kernel.cuh", "fewconv.h", "gen_core.py", "gen_blockgemm.py", os.path.join(_INC, "patconv.h"),
                     os.path.join(_INC, "blockgemm.h"), os.path.join(_INC, "dwconv.h")]
 
 
@@ -21,7 +21,8 @@ _OBJ_DIR = os.path.join(_HERE, "_build")
 # what each source includes besides itself
 _INCLUDES = {
     "patconv.cu": ["patconv_internal.h", "ptx.cuh", "tapgemm.h", "fewconv.h", "gen_core.py", os.path.join(_INC, "patconv.h")],
-    "tapgemm.cu": ["patconv_internal.h", "ptx.cuh", "tapgemm.h", os.path.join(_INC, "patconv.h")],
+    **{"tapgemm%s.cu" % part: ["patconv_internal.h", "ptx.cuh", "tapgemm.h", "tapgemm_kernel.cuh", os.path.join(_INC, "patconv.h")]
+       for part in ("", "_f32", "_f16", "_f16_cut", "_i8")},
     "fewconv.cu": ["patconv_internal.h", "fewconv.h", os.path.join(_INC, "patconv.h")],
     "blockgemm.cu": ["patconv_internal.h", "tapgemm.h", "gen_blockgemm.py", os.path.join(_INC, "patconv.h"),
                      os.path.join(_INC, "blockgemm.h")],

@@ -73,7 +73,7 @@ struct xgen_blockgemm_packed {
     // warps_per_block, a parameter of the kernel below
     patconv::TapWeights tap;
     std::mutex tap_mu;
-    struct Entry { int64_t m = 0; patconv::TapPlan plan; uint64_t stamp = 0; } tap_cache[4];
+    struct Entry { int64_t m = 0; bool gather = false; patconv::TapPlan plan; uint64_t stamp = 0; } tap_cache[4];
     uint64_t tap_stamp = 0;
     int hook_extra_arrivals = 0;        // testing aid: arrivals that a launch waits for beyond its own
 };
@@ -465,7 +465,7 @@ static bool tap_plan_of(xgen_blockgemm_packed *h, const patconv::TapShape &s, pa
     std::lock_guard<std::mutex> lock(h->tap_mu);
     auto *victim = &h->tap_cache[0];
     for (auto &e : h->tap_cache) {
-        if (e.stamp && e.m == s.rows) {
+        if (e.stamp && e.m == s.rows && e.gather == s.gather) {
             e.stamp = ++h->tap_stamp;
             plan = e.plan;
             return true;
@@ -473,7 +473,7 @@ static bool tap_plan_of(xgen_blockgemm_packed *h, const patconv::TapShape &s, pa
         if (e.stamp < victim->stamp) victim = &e;
     }
     if (!patconv::tap_choose(h->tap, s, h->device, plan)) return false;
-    victim->m = s.rows; victim->plan = plan; victim->stamp = ++h->tap_stamp;
+    victim->m = s.rows; victim->gather = s.gather; victim->plan = plan; victim->stamp = ++h->tap_stamp;
     return true;
 }
 
@@ -571,16 +571,22 @@ xgen_status xgen_blockgemm_run(const xgen_blockgemm_packed *hc, const void *x, i
     if (h->tap.dev) {
         patconv::TapShape ts;
         ts.n = 1; ts.w = 8; ts.h = (int)((m + 7) / 8); ts.rows = m; ts.staged = H.c_out * (int)eb % 16 != 0;
+        ts.gather = (uintptr_t)x % 16 != 0;
         int prev = 0;
         cudaGetDevice(&prev);
         if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
         patconv::TapPlan plan;
-        const bool fits = tap_plan_of(h, ts, plan);
+        bool fits = tap_plan_of(h, ts, plan);
         cudaError_t e = cudaSuccess;
         if (fits) {
             const patconv::TapCall call{x, y, bias, nullptr, nullptr, 0, relu, 0, h->tap.status, h->hook_extra_arrivals ? 50000u : 2000000u,
                                          h->hook_extra_arrivals, true};
             e = patconv::tap_launch(h->tap, ts, plan, call, (cudaStream_t)stream);
+            if (e == cudaErrorNotSupported && !ts.gather) {       // no tensor map of x: its rows are gathered
+                ts.gather = true;
+                fits = tap_plan_of(h, ts, plan);
+                if (fits) e = patconv::tap_launch(h->tap, ts, plan, call, (cudaStream_t)stream);
+            }
             if (e != cudaSuccess) cudaGetLastError();
         }
         if (prev != h->device) cudaSetDevice(prev);

@@ -38,7 +38,8 @@ struct TapShape {
     int stride = 1;
     int64_t rows = 0;            // product: rows of x (0 for a convolution)
     bool pool = false;
-    bool staged = false;         // results pass through shared memory: rows of y are not whole 16-byte pieces, or a residual
+    bool gather = false;         // rows of x are not whole aligned 16-byte pieces although their length is (its address is not)
+    bool staged = false;         // results pass through shared memory: rows of y are not whole 16-byte pieces
 };
 
 // How the problem is cut up (tap_choose).
@@ -51,8 +52,9 @@ struct TapPlan {
     int cut = 0;                 // fp16: stages after which sums leave the matrix unit's accumulator (0: all of them)
     int vh = 0, straddle = 0, segs = 0, row_tiles = 0, items = 0, grid = 0;
     int raster = 0, pitch = 0, rows = 0, pixels = 0;     // staged tile: entries of a row, rows (of a parity), entries
-    int a_stages = 0, a_bytes = 0, b_slots = 0, b_bytes = 0, tap_group = 1, resident = 0;
+    int a_stages = 0, a_bytes = 0, b_slots = 0, b_bytes = 0, tap_group = 1, resident = 0, operands = 0;   // (bytes of all of them)
     int plane_pitch = 0, table_bytes = 0;
+    int raw_slots = 0, raw_bytes = 0, raw_pitch = 0;     // rows of x that the producer warps shift into place (none: tensor copies, or fp32)
     size_t smem = 0;
     int tmem_cols = 0, acc_bufs = 0;
     double cycles = 0;           // what the cost model expects

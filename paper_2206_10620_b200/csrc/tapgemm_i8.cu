@@ -1,0 +1,10 @@
+// The matrix path's kernels for int8 (tapgemm_kernel.cuh), compiled on their own.
+#include "tapgemm_kernel.cuh"
+
+namespace patconv {
+
+const void *tap_kernel_i8(int stride, int taps, int mt, bool pair, bool fused, bool gather) {
+    return tap_pick_layer<XGEN_I8_I32, false>(stride, taps, mt, pair, fused, gather);
+}
+
+}  // namespace patconv
