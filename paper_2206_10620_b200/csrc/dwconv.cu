@@ -109,22 +109,21 @@ template <int BYTES> __device__ __forceinline__ void copy_v(uint32_t dst, const 
 
 // Memory binds the layer (4 useful multiply-adds per two activations moved), so the kernel is built to
 // keep loads in flight and to spend few instructions on an element.  A thread owns V channels of a
-// strip of TX output pixels and walks down a piece of the image's rows: an input row is loaded once, widened once, and
-// added to the three output rows that it belongs to (stride 2: an odd row is kept for the next output row).  All nine
-// taps run with masked weights, two channels an instruction: skipping a tap would save no traffic.
-// Rows come kAhead ahead of their use by asynchronous copies into shared memory that is the thread's own (so no thread waits
-// for another, and rows on their way hold no registers).
-// 32 images of 56x56x128 fp16: 24.2 us with a thread per output strip (each input row loaded and widened three times, 825
-// instructions for 16 results), 16.2 us with rows walked and one row ahead in registers, 14.7 us
-// now (10x39x39x960 fp16 17.8 -> 15.8; 11x49x39x112 5.5 -> 6.0).
+// strip of TX output pixels and walks down a piece of the image's rows: an input row is loaded once
+// (the next row while this one is used), widened once, and added to the three output rows that it
+// belongs to (stride 2: an odd row is kept for the next output row).  All nine taps run with masked
+// weights, two channels an instruction: skipping a tap would save no traffic.  32 images of
+// 56x56x128 fp16: 24.2 us with a thread per output strip (each input row loaded and widened
+// three times, 825 instructions for 16 results), 16.2 us with rows walked.
+// AHEAD (stride 1): rows come kAhead ahead of their use, by asynchronous copies into shared memory that is the thread's
+// own, so no thread waits for another and rows on their way hold no registers: 14.7 us (see where it is chosen).
 // S = stride, V = channels per thread (4, 2 or 1), TX = output pixels per thread along x.
 constexpr int kAhead = 3, kSlots = kAhead + 1;
-template <int DT, int S, int V, int TX>
+template <int DT, int S, int V, int TX, bool AHEAD>
 __global__ void __launch_bounds__(128) dwconv_kernel(const __grid_constant__ DParams P) {
     constexpr int NC = (TX - 1) * S + 3;            // input columns a strip needs
     constexpr int kBytes = V * (DT == XGEN_F32 ? 4 : 2);
-    constexpr bool kAsync = kBytes >= 4;            // (a copy takes 4 bytes at least: single fp16 channels go through registers)
-    __shared__ __align__(16) unsigned char ring[kAsync ? kSlots * NC * 128 * kBytes : 16];
+    __shared__ __align__(16) unsigned char ring[AHEAD ? kSlots * NC * 128 * kBytes : 16];
     asm volatile("griddepcontrol.launch_dependents;");
     const unsigned id = blockIdx.x * 128u + threadIdx.x;
     if (id >= P.threads) return;
@@ -153,51 +152,11 @@ __global__ void __launch_bounds__(128) dwconv_kernel(const __grid_constant__ DPa
     bool col_ok[NC];
 #pragma unroll
     for (int j = 0; j < NC; ++j) col_ok[j] = (unsigned)(ox0 * S + j - 1) < (unsigned)P.w;
-    // Rows of the piece one after the other, `next` the one that is asked for next.
-    const int last = S == 1 ? oy1 : 2 * oy1 - 1;
-    int next = S * oy0 - 1;
-    constexpr int kRegs = kAsync ? 1 : S;           // rows ahead in registers
-    Raw<DT, V> raw[kRegs][NC];
-    unsigned put = 0, got = 0;
-    const uint32_t mine = (uint32_t)__cvta_generic_to_shared(ring) + threadIdx.x * kBytes;
-    auto ask = [&](int which) {
-        const bool row_ok = next <= last && (unsigned)next < (unsigned)P.h;
-        const unsigned at = x0 + (unsigned)next * row_elems + (unsigned)(ox0 * S - 1) * (unsigned)P.c;
-        if constexpr (kAsync) {
-            const uint32_t dst = mine + put * (NC * 128 * kBytes);
+    auto fetch = [&](Raw<DT, V> (&raw)[NC], int iy) {
+        const bool row_ok = (unsigned)iy < (unsigned)P.h;
+        const unsigned at = x0 + (unsigned)iy * row_elems + (unsigned)(ox0 * S - 1) * (unsigned)P.c;
 #pragma unroll
-            for (int j = 0; j < NC; ++j) {
-                const bool ok = row_ok && col_ok[j];
-                copy_v<kBytes>(dst + j * (128 * kBytes), static_cast<const char *>(P.x) + (ok ? (size_t)(at + (unsigned)j * (unsigned)P.c) * (DT == XGEN_F32 ? 4 : 2) : 0), ok);
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");
-            put = put + 1 == kSlots ? 0 : put + 1;
-        } else {
-#pragma unroll
-            for (int j = 0; j < NC; ++j) raw[which][j] = load_raw<DT, V>(P.x, at + (unsigned)j * (unsigned)P.c, row_ok && col_ok[j]);
-        }
-        ++next;
-    };
-    // The next row, widened; `which`: of the rows in registers.
-    auto take = [&](float (&col)[NC][V], int which) {
-        if constexpr (kAsync) {
-            ask(0);
-            asm volatile("cp.async.wait_group %0;" ::"n"(kAhead) : "memory");
-            const unsigned char *const src = ring + got * (NC * 128 * kBytes) + threadIdx.x * kBytes;
-#pragma unroll
-            for (int j = 0; j < NC; ++j) {
-                Raw<DT, V> t;
-                if constexpr (kBytes == 16) { const uint4 u = *reinterpret_cast<const uint4 *>(src + j * (128 * kBytes)); t.r[0] = u.x; t.r[1] = u.y; t.r[2] = u.z; t.r[3] = u.w; }
-                else if constexpr (kBytes == 8) { const uint2 u = *reinterpret_cast<const uint2 *>(src + j * (128 * kBytes)); t.r[0] = u.x; t.r[1] = u.y; }
-                else t.r[0] = *reinterpret_cast<const uint32_t *>(src + j * (128 * kBytes));
-                widen<DT, V>(t, col[j]);
-            }
-            got = got + 1 == kSlots ? 0 : got + 1;
-        } else {
-#pragma unroll
-            for (int j = 0; j < NC; ++j) widen<DT, V>(raw[which][j], col[j]);
-            ask(which);
-        }
+        for (int j = 0; j < NC; ++j) raw[j] = load_raw<DT, V>(P.x, at + (unsigned)j * (unsigned)P.c, row_ok && col_ok[j]);
     };
     auto emit = [&](const float (&acc)[TX][V], int oy) {
         const unsigned at = ((n * (unsigned)P.ho + (unsigned)oy) * (unsigned)P.wo + (unsigned)ox0) * (unsigned)P.c + ch;
@@ -225,21 +184,61 @@ __global__ void __launch_bounds__(128) dwconv_kernel(const __grid_constant__ DPa
 #pragma unroll
             for (int dx = 0; dx < 3; ++dx) fma_v<V>(acc[t], wt[3 * dy + dx], col[t * S + dx]);
     };
+    auto widen_row = [&](const Raw<DT, V> (&raw)[NC], float (&col)[NC][V]) {
 #pragma unroll
-    for (int i = 0; i < (kAsync ? kAhead : S); ++i) ask(i);
+        for (int j = 0; j < NC; ++j) widen<DT, V>(raw[j], col[j]);
+    };
+
     if constexpr (S == 1) {
         float acc[3][TX][V];
         start(acc[1]);
         start(acc[2]);
+        Raw<DT, V> raw[NC];
+        int next = oy0 - 1;                         // AHEAD: the row that is asked for next
+        unsigned put = 0, got = 0;
+        const uint32_t mine = (uint32_t)__cvta_generic_to_shared(ring) + threadIdx.x * kBytes;
+        auto ask = [&]() {
+            const bool row_ok = next <= oy1 && (unsigned)next < (unsigned)P.h;
+            const unsigned at = x0 + (unsigned)next * row_elems + (unsigned)(ox0 - 1) * (unsigned)P.c;
+            const uint32_t dst = mine + put * (NC * 128 * kBytes);
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                const bool ok = row_ok && col_ok[j];
+                copy_v<AHEAD ? kBytes : 16>(dst + j * (128 * kBytes), static_cast<const char *>(P.x) + (ok ? (size_t)(at + (unsigned)j * (unsigned)P.c) * (DT == XGEN_F32 ? 4 : 2) : 0), ok);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            put = put + 1 == kSlots ? 0 : put + 1;
+            ++next;
+        };
+        auto take = [&](float (&col)[NC][V]) {
+            ask();
+            asm volatile("cp.async.wait_group %0;" ::"n"(kAhead) : "memory");
+            const unsigned char *const src = ring + got * (NC * 128 * kBytes) + threadIdx.x * kBytes;
+#pragma unroll
+            for (int j = 0; j < NC; ++j) {
+                Raw<DT, V> t;
+                if constexpr (kBytes == 16) { const uint4 u = *reinterpret_cast<const uint4 *>(src + j * (128 * kBytes)); t.r[0] = u.x; t.r[1] = u.y; t.r[2] = u.z; t.r[3] = u.w; }
+                else if constexpr (kBytes == 8) { const uint2 u = *reinterpret_cast<const uint2 *>(src + j * (128 * kBytes)); t.r[0] = u.x; t.r[1] = u.y; }
+                widen<DT, V>(t, col[j]);
+            }
+            got = got + 1 == kSlots ? 0 : got + 1;
+        };
+        if constexpr (AHEAD) {
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) ask();
+        } else fetch(raw, oy0 - 1);
         // input row r goes to output rows r + 1 (starting it), r, and r - 1 (finishing it); the three
         // accumulators change places, so three steps are written out
-#pragma unroll 1
         for (int r = oy0 - 1; r <= oy1; r += 3) {
 #pragma unroll
             for (int u = 0; u < 3; ++u) {
                 if (r + u > oy1) break;
                 float col[NC][V];
-                take(col, 0);
+                if constexpr (AHEAD) take(col);
+                else {
+                    widen_row(raw, col);
+                    if (r + u < oy1) fetch(raw, r + u + 1);
+                }
                 start(acc[u]);
                 add_row(acc[u], col, 0);
                 add_row(acc[(u + 2) % 3], col, 1);
@@ -248,15 +247,20 @@ __global__ void __launch_bounds__(128) dwconv_kernel(const __grid_constant__ DPa
             }
         }
     } else {
+        Raw<DT, V> even[NC], odd[NC];
         float above[NC][V], col[NC][V], acc[TX][V];
-        take(above, 0);
-#pragma unroll 1
+        fetch(odd, 2 * oy0 - 1);
+        fetch(even, 2 * oy0);
+        widen_row(odd, above);
+        fetch(odd, 2 * oy0 + 1);
         for (int oy = oy0; oy < oy1; ++oy) {
             start(acc);
             add_row(acc, above, 0);
-            take(col, 1 % kRegs);
+            widen_row(even, col);
+            if (oy + 1 < oy1) fetch(even, 2 * oy + 2);
             add_row(acc, col, 1);
-            take(above, 0);
+            widen_row(odd, above);
+            if (oy + 1 < oy1) fetch(odd, 2 * oy + 3);
             add_row(acc, above, 2);
             emit(acc, oy);
         }
@@ -265,15 +269,18 @@ __global__ void __launch_bounds__(128) dwconv_kernel(const __grid_constant__ DPa
 
 constexpr int kStrip1 = 4, kStrip2 = 2;     // output pixels per thread at stride 1 / 2
 
-template <int DT> static const void *kernel_dt(int stride, int v) {
-    if (stride == 1)
-        return v == 4 ? (const void *)dwconv_kernel<DT, 1, 4, kStrip1> : v == 2 ? (const void *)dwconv_kernel<DT, 1, 2, kStrip1>
-                                                                                 : (const void *)dwconv_kernel<DT, 1, 1, kStrip1>;
-    return v == 4 ? (const void *)dwconv_kernel<DT, 2, 4, kStrip2> : v == 2 ? (const void *)dwconv_kernel<DT, 2, 2, kStrip2>
-                                                                             : (const void *)dwconv_kernel<DT, 2, 1, kStrip2>;
+template <int DT> static const void *kernel_dt(int stride, int v, bool ahead) {
+    if (stride == 1) {
+        if (ahead && v == 4) return (const void *)dwconv_kernel<DT, 1, 4, kStrip1, true>;
+        if constexpr (DT == XGEN_F32) if (ahead && v == 2) return (const void *)dwconv_kernel<DT, 1, 2, kStrip1, true>;
+        return v == 4 ? (const void *)dwconv_kernel<DT, 1, 4, kStrip1, false> : v == 2 ? (const void *)dwconv_kernel<DT, 1, 2, kStrip1, false>
+                                                                                        : (const void *)dwconv_kernel<DT, 1, 1, kStrip1, false>;
+    }
+    return v == 4 ? (const void *)dwconv_kernel<DT, 2, 4, kStrip2, false> : v == 2 ? (const void *)dwconv_kernel<DT, 2, 2, kStrip2, false>
+                                                                                    : (const void *)dwconv_kernel<DT, 2, 1, kStrip2, false>;
 }
-static const void *kernel_for(xgen_dtype dt, int stride, int v) {
-    return dt == XGEN_F32 ? kernel_dt<XGEN_F32>(stride, v) : kernel_dt<XGEN_F16_F32ACC>(stride, v);
+static const void *kernel_for(xgen_dtype dt, int stride, int v, bool ahead) {
+    return dt == XGEN_F32 ? kernel_dt<XGEN_F32>(stride, v, ahead) : kernel_dt<XGEN_F16_F32ACC>(stride, v, ahead);
 }
 
 // Blocks of the kernel that the device holds at once (asked for once per kernel and device).
@@ -393,7 +400,12 @@ xgen_status xgen_dwconv_run(const xgen_dwconv_packed *h, const void *x, int32_t 
     P.relu = relu ? 1 : 0;
     P.cvs = h->c / v;
     P.strips = (wo + tx - 1) / tx;
-    const void *const kern = kernel_for(h->dtype, h->stride, v);
+    // Rows ahead, where a call is long enough for bandwidth to count and accesses are 8 bytes or more (a copy of 4 bytes
+    // costs as much), us without and with: fp16 32x56x56x128 (51 MB) 16.2, 14.7; 123x188x336 (31 MB) 11.6, 11.0;
+    // fp32 16x56x56x128 12.8, 10.0; but 11x49x39x112 (9 MB) 5.5, 6.0; 20x14x14x512 4.5, 5.0; single fp32 channels 8x42x42x881 25.0, 27.0;
+    // pairs of fp16 8x42x42x882 17.5, 21.5; stride 2, two rows ahead in registers, 8x112x112x64 3.7, 5.0.
+    const bool ahead = h->stride == 1 && v * (int)eb >= 8 && (xe + ye) * (int64_t)eb >= 24000000;
+    const void *const kern = kernel_for(h->dtype, h->stride, v, ahead);
     // Pieces of an image's rows: a piece loads (and at stride 1 adds up) two rows besides its own and costs
     // about two more to start, so pieces want to be long; but the blocks run in waves of what the GPU holds,
     // and one that is partly filled costs as much as a full one.
