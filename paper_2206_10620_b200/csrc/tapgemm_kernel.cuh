@@ -472,7 +472,7 @@ __device__ __forceinline__ void tap_direct(const TapParams &P, const uint32_t *s
 // through shared memory.  Pixels px[2 h + r]: row 16 h + 8 r + lane / 4 of the warp's 32; sum v[8 h + 4 i + 2 r + e]:
 // channel c + 8 i + 2 (lane % 4) + e.  The residual is asked for before the sums are waited for.
 // (32 lanes a pixel each touched 32 lines an access; by way of shared memory 256 x 64 int32 residuals took 7000 cycles:
-// 64 images of 28x28x128 int8 @QUAD@.)
+// 64 images of 28x28x128 int8 20.5 us, 16.0 now.)
 template <int DT> struct QuadRes { uint32_t v[DT == XGEN_F16_F32ACC ? 8 : 16]; };
 template <int DT> __device__ __forceinline__ void quad_residual(const TapParams &P, QuadRes<DT> &res, const int (&px)[4], int c) {
     c += 2 * (threadIdx.x & 3);
@@ -794,6 +794,11 @@ __device__ __noinline__ void tap_repair(const TapParams &P) {
     }
 }
 
+static __device__ __noinline__ void tap_pause() {
+    const uint64_t t = global_ns();
+    for (int it = 0; it < 1000000 && global_ns() - t < 50000u; ++it) {}
+}
+
 template <int DT, int STRIDE, int TAPS, int MT, bool PAIR, bool CUT, bool FUSED, bool GATHER>
 __global__ void __launch_bounds__(tap_threads(DT), 1)
 tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap) {
@@ -824,12 +829,10 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
     // through all of its work, on whatever the buffers hold, and is reported.
     auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait<PAIR>(bar, parity, &s_abort, P.status, P.wait_us); };
     auto wait_warp = [&](uint32_t bar, uint32_t parity) { wait(bar, parity); __syncwarp(); };
-    // A role whose wait has given up is out of step, and its next waits may return too early.  A buffer's barrier must not be
-    // armed again while a copy into it is on its way, so such a role issues its copies 50 us apart.
-    auto pace = [&]() {
-        const uint64_t t = global_ns();
-        for (int it = 0; it < 1000000 && global_ns() - t < 50000u; ++it) {}
-    };
+    // A role whose wait has given up is out of step: its next waits may return before what they stand for has come (their
+    // barriers are a phase behind), and it hands buffers on before they are filled.  A barrier must not be armed again while a copy
+    // that it counts is on its way, so from then on the role pauses 50 us at every buffer that it fills or hands on (`late`, the
+    // role's own: in a register, where a look at the block's flag for every buffer cost 128->128@56^2/2 14.3 -> 16.1 us).
     // Clusters: a pair of blocks (PAIR), or the blocks (pairs) that split an item's reduction.  The even
     // block of a pair holds the barriers that say "operands are there" and "sums have been read".
     const int csize = (PAIR ? 2 : 1) * P.splits;
@@ -886,7 +889,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     if (lane == 0) s_started = s_started + 1;
                     for (int ks = k0; ks < k1; ++ks) {
                         if (!wait(a_empty(s), ph)) late = true;
-                        if (late) pace();
+                        if (late) tap_pause();
                         __syncwarp();
                         const uint32_t bar = lead(a_full(s));
                         const uint32_t dst = sbase + (uint32_t)(s * P.a_bytes) + (P.raster ? (uint32_t)(P.pitch - 1 - t.ox0) * 128u : 0u);
@@ -1137,14 +1140,15 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             const uint32_t a_sub = (uint32_t)P.sub_px * a_px, a_step = (uint32_t)P.a_bytes / 16, b_step = (uint32_t)P.b_bytes / 16;
             int s = 0, b = 0, buf = 0, run = 0;                             // run: stages since the accumulator was empty (CUT)
             uint32_t pha = 0, phb = 0, phc = 1, as = (uint32_t)a0, bs = (uint32_t)b0;
-            bool ready = mbar_test<PAIR>(b_full(0), 0), look = true;           // look: weights may still be on their way
+            bool ready = mbar_test<PAIR>(b_full(0), 0), look = true, late = false;           // look: weights may still be on their way
             // a tap's first entry is that of its row and that of its column of taps
             const uint32_t row0 = (uint32_t)P.tap_start[0] * a_px, row1 = TAPS == 1 ? 0u : (uint32_t)P.tap_start[3] * a_px, row2 = TAPS == 1 ? 0u : (uint32_t)P.tap_start[6] * a_px;
             const uint32_t col0 = 0u, col1 = TAPS == 1 ? 0u : (uint32_t)(P.tap_start[1] - P.tap_start[0]) * a_px, col2 = TAPS == 1 ? 0u : (uint32_t)(P.tap_start[2] - P.tap_start[0]) * a_px;
             for (int item = item0; item < P.items; item += item_step) {
                 for (int ks = k0; ks < k1; ++ks) {
-                    if (kF32 || (CUT ? run == 0 : ks == k0)) wait(acc_empty(buf), phc);
-                    wait(a_full(s), pha);
+                    if ((kF32 || (CUT ? run == 0 : ks == k0)) && !wait(acc_empty(buf), phc)) late = true;
+                    if (!wait(a_full(s), pha)) late = true;
+                    if (late) tap_pause();
                     tc_fence_after();
                     const int kk_n = min(P.pl, planes - ks * P.pl) / 2;
                     const uint32_t d = tmem + (uint32_t)buf * (uint32_t)(MT * P.nt);
@@ -1158,8 +1162,10 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                         const int tap = t0 + t1;
                         const bool last = P.tap_group == 1 || t1 == 2;
                         if (look) {
-                            if ((P.tap_group == 1 || t1 == 0) && !ready)
-                                mbar_wait_long<PAIR>(b_full(b), P.resident ? 0u : phb, &s_abort, P.status, P.wait_us);
+                            if ((P.tap_group == 1 || t1 == 0) && !ready) {
+                                if (!mbar_wait_long<PAIR>(b_full(b), P.resident ? 0u : phb, &s_abort, P.status, P.wait_us)) late = true;
+                            }
+                            if (late) tap_pause();
                             if (last) {                     // (of its slot: look at the next one)
                                 const bool wrap = b + 1 == P.b_slots;
                                 ready = mbar_test<PAIR>(b_full(wrap ? 0 : b + 1), P.resident ? 0u : wrap ? phb ^ 1u : phb);
@@ -1234,7 +1240,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 for (int ks = k0; ks < k1; ++ks) {
                     for (int tap = 0; tap < TAPS; tap += P.tap_group) {
                         if (issued >= P.b_slots && !wait(b_empty(b), ph)) late = true;
-                        if (late) pace();
+                        if (late) tap_pause();
                         // one copy for a slot: pieces of 2 KB with a copy of their own cost 50 cycles
                         // of issue apiece and held the whole kernel to 5.5 TB/s of weights
                         if (side == 0) mbar_expect_tx(b_full(b), (uint32_t)P.b_bytes * (PAIR ? 2 : 1));
@@ -1288,7 +1294,11 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
         auto advance = [&]() {
             if (++buf == P.acc_bufs) { buf = 0; ph ^= 1u; }
         };
-        for (int item = item0; item < P.items; item += item_step, next -= CUT ? 0 : chunks) {        // (CUT: chunks stay with their group, whose sums wait in tensor memory)
+        // A group that leaves out items must not miss a whole turn of the accumulators, or it takes the end of one turn for that
+        // of the next: with a buffer an item (fp16, int8) the items that a group leaves out are always the same buffers'; fp32, with a
+        // buffer a stage, where an item has two at most.  (CUT: the chunks' sums wait in tensor memory for their group.)
+        const bool turn = !CUT && (!kF32 || k1 - k0 <= 2);
+        for (int item = item0; item < P.items; item += item_step, next = turn ? next - chunks : group) {
             if (next >= chunks) {
                 for (int ks = kF32 || CUT ? k0 : k1 - 1; ks < k1; ks += CUT ? P.cut : 1) advance();
                 continue;

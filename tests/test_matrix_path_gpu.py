@@ -439,3 +439,61 @@ def test_calls_report_errors():
     with pytest.raises(binding.PatconvError) as e:
         pk.run(16, 1, 8, 8, None, True, 4096)
     assert e.value.status == 1
+
+
+@pytest.mark.parametrize("co", [17, 32, 40, 96])
+@pytest.mark.parametrize("ci,stride", [(24, 1), (50, 1), (160, 1), (160, 2)])
+def test_fp32_tiles_of_few_filters(co, ci, stride):
+    """Items of one to many stages, several to a block, in chunks that go round the epilogue's warps or stay."""
+    n, h = (90, 23) if stride == 1 else (40, 61)
+    d = _layer("f32", 1, ci, co, h, h, stride, prune=0.4, seed=co + ci)
+    y = run_gpu(pack(d), np.tile(d.x, (n, 1, 1, 1)), d.bias, True)
+    assert (y == y[:1]).all()
+    compare(d, y[:1])
+
+
+@pytest.mark.parametrize("m,k,co", [(60000, 40, 32), (60000, 200, 20), (40000, 352, 96)])
+def test_fp32_products_of_few_filters(m, k, co):
+    d = wl.make_block_gemm(wl.GemmSpec("t", 600, k, co, 16, 16, 0.5, 0.5, "f32"), seed=k)
+    import torch
+    g = binding.BlockGemm(k, co, 16, 16, "f32", d.w, d.row_keep, d.col_keep)
+    x, b = torch.from_numpy(np.tile(d.x, (m // 600 + 1, 1))[:m]).cuda(), torch.from_numpy(d.bias).cuda()
+    y = torch.empty((m, co), device="cuda")
+    g.run(x.data_ptr(), m, b.data_ptr(), True, y.data_ptr())
+    g.sync()
+    y = y.cpu().numpy()
+    assert all((y[i:i + 600] == y[:len(y[i:i + 600])]).all() for i in range(600, m, 600))
+    ref, S = oracle.block_gemm(d.x, d.w, d.row_keep, d.col_keep, 16, 16, bias=d.bias, relu=True, with_scale=True)
+    assert (np.abs(y[:600] - ref) <= TOL["f32"] * np.maximum(np.abs(ref), 0.01 * S) + 1e-30).all()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16", "i8"])
+@pytest.mark.parametrize("ci", [1, 2, 3, 4, 5, 7])
+@pytest.mark.parametrize("n,h,w,co,stride", [
+    (1, 5, 3, 16, 1),             # one pixel a thread, one group of filters
+    (2, 40, 61, 33, 1),           # two; three groups, filters that are not whole pieces
+    (3, 90, 131, 70, 2),          # more than 64 filters
+    (4, 111, 113, 64, 1),         # four
+])
+def test_few_channels(dtype, ci, n, h, w, co, stride):
+    if dtype == "f32" and ci > 4:
+        pytest.skip("on the matrix units")
+    # (no zeros in x: where all of a window is zero the result is the bias, and half a spacing of fp16's subnormals,
+    # 2^-25, is more than 2e-3 of a bias below 1.5e-5)
+    d = _layer(dtype, n, ci, co, h, w, stride, prune=0.3, seed=ci + co, x_dist="u01" if dtype == "i8" else "upm1")
+    compare(d, run_gpu(pack(d), d.x, d.bias, True))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+def test_few_channels_infinities_under_pruned_weights(dtype):
+    """As on the command stream, which goes through the kept weights alone."""
+    d = _layer(dtype, 1, 3, 32, 20, 30, prune=0.6, seed=3)
+    d.x[0, 7, 11, 1] = np.inf
+    d.x[0, 15, 20, 0] = np.nan
+    stream = pack(d)
+    stream.plan(1, 20, 30, splits=1)
+    y, ref = run_gpu(pack(d), d.x, d.bias, False).astype(np.float64), run_gpu(stream, d.x, d.bias, False).astype(np.float64)
+    fine = np.isfinite(ref)
+    assert np.array_equal(np.isfinite(y), fine) and 0 < (~fine).sum() < 2 * 9 * 32
+    assert np.array_equal(y[~fine], ref[~fine], equal_nan=True)
+    assert (np.abs(y[fine] - ref[fine]) <= 2 * TOL[dtype] * np.maximum(np.abs(ref[fine]), 0.01)).all()
