@@ -14,11 +14,12 @@
  * (no kernel flip), act = ReLU or identity.  Pruned weights contribute nothing, also
  * where they meet an infinity or a NaN; ReLU keeps a NaN on the matrix path.
  *
- * Two kernels compute it.  The matrix path runs the layer dense on the tensor cores, with zeros for
- * the pruned weights, and is what a call takes by default.  The command-stream kernel
- * executes the kept kernels one by one; layers of a few input channels (fp32: up to four,
- * else up to seven) take it, and handles whose caller names one of its tuning parameters
- * (xgen_patconv_plan_tuned).  Both accumulate in fp32 (int32).  The matrix
+ * Three kernels compute it.  The matrix path runs the layer dense on the tensor cores, with zeros for
+ * the pruned weights, and is what a call takes by default.  Layers of a few input channels (fp32: up to
+ * four, else up to seven) run dense on the FP32 pipe, by a kernel that has no plan.  The command-stream kernel
+ * executes the kept kernels one by one; layers of a few input channels take it with operators fused behind
+ * them, or where few of a large image's kernels are left, and handles whose caller names one of its tuning parameters
+ * (xgen_patconv_plan_tuned).  All accumulate in fp32 (int32).  The matrix
  * units truncate when they add, so their chains of additions are cut short and the parts added rounded: fp16
  * sums of positive terms come out low by up to 9e-6 of themselves (a fiftieth of an fp16 unit), fp32
  * sums by 2e-7.
