@@ -1382,10 +1382,10 @@ static bool stream_is_faster(const PackedHost &p, int64_t pixels) {
 }
 
 // What the matrix path's plan of a call depends on.
-static TapShape tap_shape(const PackedHost &p, int n, int hh, int ww, int pool, bool requant) {
+static TapShape tap_shape(const PackedHost &p, int n, int hh, int ww, int pool, bool residual, bool requant) {
     TapShape ts;
     ts.n = n; ts.h = hh; ts.w = ww; ts.stride = p.stride; ts.pool = pool == 2;
-    ts.staged = p.c_out * (requant ? 1 : p.dtype == XGEN_F16_F32ACC ? 2 : 4) % 16 != 0;
+    ts.staged = (residual && pool != 2 && p.dtype == XGEN_F32) || p.c_out * (requant ? 1 : p.dtype == XGEN_F16_F32ACC ? 2 : 4) % 16 != 0;
     return ts;
 }
 
@@ -1442,7 +1442,7 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
         }
     }
     if (h->tap.dev && (ignore_plan || !h->stream_asked)) {
-        const TapShape ts = tap_shape(p, n, hh, ww, pool, rq_scale != nullptr);
+        const TapShape ts = tap_shape(p, n, hh, ww, pool, residual != nullptr, rq_scale != nullptr);
         int prev = 0;
         if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
         if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
@@ -1727,7 +1727,7 @@ xgen_status xgen_patconv_plan_info(const xgen_patconv_packed *h, int32_t n, int3
         int prev = 0;
         if (cudaGetDevice(&prev) != cudaSuccess || cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
         TapPlan tp;
-        const bool fits = tap_plan_of(h, tap_shape(p, n, hh, ww, 0, false), tp);
+        const bool fits = tap_plan_of(h, tap_shape(p, n, hh, ww, 0, false, false), tp);
         cudaSetDevice(prev);
         if (fits) {
             out->matrix_path = 1;

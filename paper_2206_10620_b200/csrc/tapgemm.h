@@ -39,7 +39,7 @@ struct TapShape {
     int64_t rows = 0;            // product: rows of x (0 for a convolution)
     bool pool = false;
     bool gather = false;         // rows of x are not whole aligned 16-byte pieces although their length is (its address is not)
-    bool staged = false;         // results pass through shared memory: rows of y are not whole 16-byte pieces
+    bool staged = false;         // results pass through shared memory: rows of y are not whole 16-byte pieces, or fp32 with a residual
 };
 
 // How the problem is cut up (tap_choose).

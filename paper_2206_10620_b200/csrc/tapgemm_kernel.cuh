@@ -282,11 +282,42 @@ __device__ __forceinline__ void tap_store1(const TapParams &P, float scale, uint
 
 // A warp's 32 pixels x 16 channels, staged as rows of kStagePitch words: 16 sums, the pixel of the
 // unpooled result (-1: none), where it is stored (pooled: the window whose first pixel it is).  Finish
-// and store them so that neighbouring lanes hold neighbouring elements: where rows of y are not whole 16-byte pieces.
+// and store them so that neighbouring lanes hold neighbouring elements: where rows of y are not whole 16-byte pieces, and fp32
+// with a residual (its sums are in registers, a pixel a lane; held in quads, as tap_quad has them, they cost every stage a choice of
+// loads: 81 x 9x9, 91 -> 192 with residual 18.7 -> 19.2 us).
 template <int DT, bool FUSED>
 __device__ __forceinline__ void tap_emit(const TapParams &P, const uint32_t *st, const uint32_t *s_bias, const float *s_scale,
                                          int c_base, int n0, int lane) {
     const bool pool = FUSED && P.pool;
+    if constexpr (FUSED && DT == XGEN_F32) if (P.vec_y && P.vec_r && !pool) {
+        const int c = c_base + (lane & 3) * 4;
+        if (c >= P.c_out) return;
+        const uint4 b = *reinterpret_cast<const uint4 *>(s_bias + (c - n0));
+        const uint32_t *const row0 = st + (lane >> 2) * kStagePitch;
+        uint4 res[4];
+        int px[4];
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            px[it] = (int)row0[it * 8 * kStagePitch + 16];
+            const size_t off = (size_t)max(px[it], 0) * P.c_out + c;
+            res[it] = __ldg(reinterpret_cast<const uint4 *>(static_cast<const uint32_t *>(P.residual) + off));
+        }
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {
+            const uint4 a = *reinterpret_cast<const uint4 *>(row0 + it * 8 * kStagePitch + (lane & 3) * 4);
+            uint32_t v[4] = {a.x, a.y, a.z, a.w};
+            add2(v[0], v[1], b.x, b.y); add2(v[2], v[3], b.z, b.w);
+            add2(v[0], v[1], res[it].x, res[it].y); add2(v[2], v[3], res[it].z, res[it].w);
+            if (P.relu) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] = tap_max<DT>(v[i], 0u);
+            }
+            if (px[it] < 0) continue;
+            const size_t off = (size_t)px[it] * P.c_out + c;
+            *reinterpret_cast<uint4 *>(static_cast<uint32_t *>(P.y) + off) = make_uint4(v[0], v[1], v[2], v[3]);
+        }
+        return;
+    }
     const int c = c_base + (lane & 15);          // a lane keeps its channel, half-warps take a pixel each
     if (c >= P.c_out) return;
     const uint32_t bias = s_bias[c - n0];
@@ -467,7 +498,7 @@ __device__ __forceinline__ void tap_direct(const TapParams &P, const uint32_t *s
     }
 }
 
-// Sums with a residual, in the layout of tmem_ld_quad: a lane holds two adjacent channels (of each of two blocks of
+// fp16 and int8 sums with a residual, in the layout of tmem_ld_quad: a lane holds two adjacent channels (of each of two blocks of
 // eight) of four pixels, so that the four lanes of a quad hold 32 adjacent bytes of the residual and of y and nothing need pass
 // through shared memory.  Pixels px[2 h + r]: row 16 h + 8 r + lane / 4 of the warp's 32; sum v[8 h + 4 i + 2 r + e]:
 // channel c + 8 i + 2 (lane % 4) + e.  The residual is asked for before the sums are waited for.
@@ -1307,9 +1338,9 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             const TapPixel at = tap_pixel<TAPS>(P, t, sub * 128 + m);
             const int pix = at.pix, out = at.out;
             if (P.staged && P.splits == 1) { st_own[16] = (uint32_t)pix; st_own[17] = (uint32_t)out; }
-            const bool quad = FUSED && P.residual && !P.pool && !P.staged && P.splits == 1;
+            const bool quad = FUSED && !kF32 && P.residual && !P.pool && !P.staged && P.splits == 1;
             int px4[4];
-            if (FUSED) {
+            if (FUSED && !kF32) {
 #pragma unroll
                 for (int k = 0; k < 4; ++k) px4[k] = __shfl_sync(0xFFFFFFFFu, pix, 16 * (k / 2) + 8 * (k % 2) + lane / 4);
             }
@@ -1363,8 +1394,8 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                         if (q < chunks) {
                             const uint32_t ta = tmem + lanes + (uint32_t)(buf * P.nt + 32 * q + h % 2 * 16);
                             uint32_t a[16], b[16];
-                            if (quad) { tmem_ld_quad(ta, a); tmem_ld_quad(ta + P.acc_bufs * P.nt, b); }
-                            else { tmem_ld16(ta, a); tmem_ld16(ta + P.acc_bufs * P.nt, b); }
+                            tmem_ld16(ta, a);
+                            tmem_ld16(ta + P.acc_bufs * P.nt, b);
                             tmem_wait_ld();
 #pragma unroll
                             for (int i = 0; i < 16; i += 2) {
@@ -1378,15 +1409,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 }
 #pragma unroll 1
                 for (; next < chunks; next += kGroups) {
-                    if (quad) {
-                        if (!all_finite(sum[0])) s_odd = 1;
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const int c = n0 + 32 * next + 16 * h;
-                            QuadRes<DT> res;
-                            if (c < P.c_out) { quad_residual<DT>(P, res, px4, c); tap_quad<DT>(P, s_bias, s_scale, sum[0] + 16 * h, res, px4, c, n0); }
-                        }
-                    } else finish(sum[0], 32 * next);
+                    finish(sum[0], 32 * next);
 #pragma unroll
                     for (int i = 0; i < 32; ++i) sum[0][i] = sum[1][i];
                 }
