@@ -1453,9 +1453,9 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
             const TapCall call{x, y, bias, residual, rq_scale, ep ? ep->requant_zero_point : 0, relu, pool,
                                h->d_status, h->wait_us, h->hook_extra_arrivals, !h->tuning.no_launch_overlap};
             if (log_enabled())
-                fprintf(stderr, "libpatconv: matrix path, %d blocks = %d items (form %d, %d row tiles x %d columns x %d filter tiles of %d) x %d splits, %d x 128 pixels%s, %d planes x %d stages (cut every %d), %d + %d x %d taps buffers%s, %zu bytes shared, %.0f cycles expected\n",
+                fprintf(stderr, "libpatconv: matrix path, %d blocks = %d items (form %d, %d row tiles x %d columns x %d filter tiles of %d) x %d splits, %d x 128 pixels%s, %d planes x %d stages (cut every %d), %d + %d x %d taps buffers%s, %d x %d pixels of rows, %zu bytes shared, %.0f cycles expected\n",
                         plan.grid, plan.items, plan.raster ? 2 : plan.straddle, plan.row_tiles, plan.segs, plan.nblk, plan.nt, plan.splits, plan.mt, plan.pair ? " (block pairs)" : "", plan.pl, plan.stages, plan.cut,
-                        plan.a_stages, plan.b_slots, plan.tap_group, plan.resident ? " (resident weights)" : "", plan.smem, plan.cycles);
+                        plan.a_stages, plan.b_slots, plan.tap_group, plan.resident ? " (resident weights)" : "", plan.raw_slots, plan.raw_px, plan.smem, plan.cycles);
             e = log_cuda(tap_launch(h->tap, ts, plan, call, (cudaStream_t)stream), "matrix kernel launch");
         }
         if (prev != h->device) cudaSetDevice(prev);

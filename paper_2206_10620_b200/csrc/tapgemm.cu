@@ -72,6 +72,8 @@ __global__ void tap_expand_dense(uint8_t *img, int c_in, int rows, int k0, int c
 
 static int tap_cpp(xgen_dtype dt) { return dt == XGEN_I8_I32 ? 16 : 8; }
 static int tap_parts(xgen_dtype dt) { return dt == XGEN_F32 ? 3 : 1; }
+// A pixel's planes of a stage, as a power of two.
+static int row_log(int pl) { return pl <= 2 ? 1 : pl <= 4 ? 2 : 3; }
 
 // Upload scratch: kPiece bytes a device, shared by all handles of the process, there while any handle is.  (Allocated
 // and freed by every handle it cost 0.6 ms of the 2.2 that a 1000 x 1000 fp32 handle takes; kept by every handle
@@ -334,62 +336,95 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     const size_t sums = sp > 1 ? (size_t)sp * ((8 * mt + sp - 1) / sp) * 64 * p.nt : s.staged ? (size_t)epi_warps(dt) * kStageBytes : 0;
                     const int64_t uses = (sp == 1 ? waves : 1) * p.per_split;      // stages one block goes through
                     // Shared memory: two tiles of x (more for a plain product, whose stages are short), the rest
-                    // weights, by three taps if at least three such slots fit.
-                    // fp16 and int8 rows that the producer warps shift into place: up to two stages of them on their way (three of a product).
-                    bool fits = false;
+                    // weights, by three taps if at least three such slots fit.  fp16 and int8 rows that the producer warps
+                    // shift into place: up to two stages of them on their way (three of a product).  The tiles of stride 2 (612
+                    // pixels) leave no room for those: quarters or eighths of a stage, or one tile of x, whatever
+                    // is weighed best, so that there is a plan whatever else takes room.  (Without one 32 images of 56x56x67 -> 93
+                    // fp16 took 176 us on the command stream, 42.6 now; 28x28x503 -> 256 1230, 59; int8 168, 21 and 1092, 33.)
                     size_t tables = sums;
                     const int raw_top = copied || dt == XGEN_F32 ? 0 : (int)std::min<int64_t>(uses, tw.taps == 1 ? 4 : 3);
-                    for (p.raw_slots = raw_top; p.raw_slots >= std::min(raw_top, 1) && !fits; --p.raw_slots) {
-                    p.raw_pitch = p.pl * 16 + 16;
-                    p.raw_bytes = pixels * p.raw_pitch;
-                    p.table_bytes = tw.taps == 1 || copied ? 0 : ((dt == XGEN_F32 ? 2 : p.raw_slots) * pixels * 4 + 127) / 128 * 128;
-                    tables = sums + p.table_bytes + (size_t)p.raw_slots * p.raw_bytes;
-                    for (p.tap_group = tw.taps == 1 ? 1 : 3; p.tap_group >= 1 && !fits; p.tap_group -= 2) {
-                        p.b_bytes = p.tap_group * p.pl * parts * p.nt * 16 / ways;
-                        const int all_b = p.per_split * tw.taps / p.tap_group;
-                        for (p.a_stages = (int)std::min<int64_t>(uses, tw.taps == 1 ? kMaxA : 2); p.a_stages >= 1; --p.a_stages) {
-                            const size_t left_a = (size_t)p.a_stages * p.a_bytes + tables;
-                            if (left_a >= (size_t)kTapSmemMax) continue;
-                            const int room = (int)std::min<size_t>(kMaxB, ((size_t)kTapSmemMax - left_a) / p.b_bytes);
-                            p.resident = all_b <= room;
-                            p.b_slots = std::min(room, all_b);
-                            if (p.b_slots >= std::min(all_b, 3) && p.a_stages >= std::min<int64_t>(2, uses)) { fits = true; break; }
+                    const int two = (int)std::min<int64_t>(2, uses);
+                    auto place = [&](int least_a) {
+                        p.raw_pitch = p.pl * 16 + 16;
+                        p.raw_bytes = p.raw_px * p.raw_pitch;
+                        p.table_bytes = tw.taps == 1 || copied ? 0 : ((dt == XGEN_F32 ? 2 : p.raw_slots) * pixels * 4 + 127) / 128 * 128;
+                        tables = sums + p.table_bytes + (size_t)p.raw_slots * p.raw_bytes;
+                        for (p.tap_group = tw.taps == 1 ? 1 : 3; p.tap_group >= 1; p.tap_group -= 2) {
+                            p.b_bytes = p.tap_group * p.pl * parts * p.nt * 16 / ways;
+                            const int all_b = p.per_split * tw.taps / p.tap_group;
+                            for (p.a_stages = (int)std::min<int64_t>(uses, tw.taps == 1 ? kMaxA : 2); p.a_stages >= least_a; --p.a_stages) {
+                                const size_t left_a = (size_t)p.a_stages * p.a_bytes + tables;
+                                if (left_a >= (size_t)kTapSmemMax) continue;
+                                const int room = (int)std::min<size_t>(kMaxB, ((size_t)kTapSmemMax - left_a) / p.b_bytes);
+                                p.resident = all_b <= room;
+                                p.b_slots = std::min(room, all_b);
+                                if (p.b_slots >= std::min(all_b, 3)) return true;
+                            }
                         }
-                        if (fits) break;
+                        return false;
+                    };
+                    // What that makes of the time: the cost model, in cycles.
+                    auto weigh = [&](bool large) {
+                        // (the operands' buffers hold a block's own sums before they leave)
+                        p.operands = std::max(p.a_stages * p.a_bytes + p.b_slots * p.b_bytes, sp > 1 ? 512 * mt * p.nt : 0);
+                        p.smem = (size_t)p.operands + tables;
+                        if (p.smem > (size_t)kTapSmemMax) return;
+                        p.acc_bufs = p.cut ? (3 * mt * p.nt <= 512 ? 2 : 1) : (dt == XGEN_F32 ? 2 : 1) * 4 * mt * p.nt <= 512 ? 4 : dt == XGEN_F32 || 2 * mt * p.nt <= 512 ? 2 : 1;
+                        const int cols = (dt == XGEN_F32 ? 2 * p.acc_bufs : p.acc_bufs + (p.cut ? 1 : 0)) * mt * p.nt;
+                        for (p.tmem_cols = 32; p.tmem_cols < cols;) p.tmem_cols *= 2;
+                        // Cycles of a stage: the matrix instructions (nt / 2 each; 46 to issue one and 90 for a tap), or
+                        // what they and the copies move through shared memory at 128 bytes a cycle (128 rows of x,
+                        // the block's filters), or what comes from L2.  A pair starts and ends later: 4000 cycles where it
+                        // halves much (fp32: three parts of weights; stride 2: single taps in the slots), else 6000
+                        // (256 -> 256 at 14x14, batch 32, fp16: 12.8 us as pairs, 11.7 without); the
+                        // short stages of a product wait 300 cycles for its other block (1842 filters x 5421 rows,
+                        // fp32: 77 us as pairs, 57 us without).
+                        const double kk = (double)tw.planes / p.stages / 2, taps = tw.taps;
+                        const double b_stage = taps * kk * 2 * parts * p.nt * 16.0 / ways, b_moved = p.resident && sp == 1 ? b_stage / waves : b_stage;
+                        const double x_moved = (double)pixels * kk * 2 * cpp * xb, a_stage = (double)p.a_bytes * (swizzled ? 1 : 2);
+                        const double per_tap = kk * mt * prod, instr = taps * per_tap;
+                        const double mma = taps * std::max(per_tap * p.nt / 2.0, 90.0 + 46.0 * per_tap);
+                        const double shared = (instr * (4096.0 + p.nt * 32.0 / ways) + b_moved + a_stage) / 128.0;
+                        const double move = (x_moved + b_moved) / 40.0 + (copied && p.straddle ? 60.0 * p.rows * (s.stride == 1 ? 1 : 4) : 0.0) * 0.5;
+                        // cycles of the producer warps for a piece; no stage of x ahead
+                        const double make = copied ? 0.0 : (double)pixels * kk * 2 * (swizzled ? 2.0 : 3.0) + (swizzled && p.raw_slots == 1 ? 1200.0 : 0.0);
+                        const double ends = 250.0 + 40.0 * taps / p.tap_group + (p.pair && tw.taps == 1 ? 300.0 : 0.0);
+                        const double out = (double)mt * 128 * p.nt * yb / 24.0;
+                        // (one accumulator that is cut waits for its sums to be added)
+                        const double cuts = p.cut && p.acc_bufs == 1 ? (p.per_split - 1) / p.cut * 1500.0 : 0.0;
+                        const double item = p.per_split * (std::max(std::max(mma, shared), std::max(move, make)) + ends) + cuts;
+                        double run = waves * std::max(item, sp == 1 && p.acc_bufs >= 2 ? out : 0.0), c = 3500.0 + (p.pair ? dt == XGEN_F32 || s.stride == 2 ? 4000.0 : 6000.0 : 0.0);
+                        if (large) {                                   // (rows shifted into place at stride 2)
+                            // The first stage is made before anything else happens; a piece takes the producer warps 2.2 cycles, one
+                            // outside the image 0.8; x takes 1500 cycles to come, of which the parts ahead hide a share, and so
+                            // does a slot of weights; one tile of x is only copied while the instructions read it; the blocks
+                            // of a split begin anew in every wave.
+                            const double full = std::min(1.0, 1.15 * s.n * s.h * s.w / ((double)tiles_all * pixels)), n_parts = (pixels + p.raw_px - 1) / p.raw_px;
+                            const double pieces = (double)((int64_t)pixels << row_log(p.pl)) * (0.8 + 1.4 * full);
+                            const double make = pieces + (n_parts > 1.0 ? n_parts * (300.0 + std::max(0.0, 1500.0 - (p.raw_slots - 1) * 0.6 * pieces / n_parts)) : p.raw_slots == 1 ? 1200.0 : 0.0);
+                            const double slots = p.b_slots * p.tap_group;
+                            const double busy = std::max(std::max(mma, p.resident ? 0.0 : (taps - slots) * 1500.0 / slots), std::max(shared, move));
+                            auto block = [&](double n) { return p.a_stages >= two ? make + (n - 1) * std::max(busy, make) + busy : n * (make + std::max(0.0, busy - 0.3 * pieces)); };
+                            run = sp == 1 ? std::max(block((double)uses), p.acc_bufs >= 2 ? waves * out : 0.0) + waves * (p.per_split * ends + cuts)
+                                          : waves * (block(p.per_split) + p.per_split * ends + cuts) + (waves - 1) * 3500.0;
+                        }
+                        if (sp == 1) c += run + (p.acc_bufs >= 2 ? out : waves * out);
+                        else c += run + waves * (2500.0 + 100.0 * sp + mt * 128.0 * p.nt * 4 / 64.0 + out / sp);
+                        if (c < best.cycles * 0.999) { best = p; best.cycles = c; }
+                    };
+                    p.raw_px = pixels;
+                    if (raw_top == 0 || s.stride == 1) {
+                        bool fits = false;
+                        for (p.raw_slots = raw_top; p.raw_slots >= std::min(raw_top, 1) && !(fits = place(two));) --p.raw_slots;
+                        if (fits) weigh(false);
+                    } else {
+                        const int q_step = kProdThreads >> row_log(p.pl);             // pixels that the producer warps take at a time
+                        for (int of : {1, 4, 8})
+                            for (p.raw_slots = of == 1 ? raw_top : 4; p.raw_slots >= (of == 1 ? 1 : 2); --p.raw_slots) {
+                                p.raw_px = of == 1 ? pixels : ((pixels + of - 1) / of + q_step - 1) / q_step * q_step;
+                                if (place(two) || place(1)) weigh(true);
+                            }
                     }
-                    if (fits) break;
-                    }
-                    if (!fits) continue;
-                    // (the operands' buffers hold a block's own sums before they leave)
-                    p.operands = std::max(p.a_stages * p.a_bytes + p.b_slots * p.b_bytes, sp > 1 ? 512 * mt * p.nt : 0);
-                    p.smem = (size_t)p.operands + tables;
-                    if (p.smem > (size_t)kTapSmemMax) continue;
-                    p.acc_bufs = p.cut ? (3 * mt * p.nt <= 512 ? 2 : 1) : (dt == XGEN_F32 ? 2 : 1) * 4 * mt * p.nt <= 512 ? 4 : dt == XGEN_F32 || 2 * mt * p.nt <= 512 ? 2 : 1;
-                    const int cols = (dt == XGEN_F32 ? 2 * p.acc_bufs : p.acc_bufs + (p.cut ? 1 : 0)) * mt * p.nt;
-                    for (p.tmem_cols = 32; p.tmem_cols < cols;) p.tmem_cols *= 2;
-                    // Cycles of a stage: the matrix instructions (nt / 2 each; 46 to issue one and 90 for a tap), or
-                    // what they and the copies move through shared memory at 128 bytes a cycle (128 rows of x,
-                    // the block's filters), or what comes from L2.  A pair starts and ends later: 4000 cycles where it
-                    // halves much (fp32: three parts of weights; stride 2: single taps in the slots), else 6000
-                    // (256 -> 256 at 14x14, batch 32, fp16: 12.8 us as pairs, 11.7 without); the
-                    // short stages of a product wait 300 cycles for its other block (1842 filters x 5421 rows,
-                    // fp32: 77 us as pairs, 57 us without).
-                    const double kk = (double)tw.planes / p.stages / 2, taps = tw.taps;
-                    const double b_stage = taps * kk * 2 * parts * p.nt * 16.0 / ways, b_moved = p.resident && sp == 1 ? b_stage / waves : b_stage;
-                    const double x_moved = (double)pixels * kk * 2 * cpp * xb, a_stage = (double)p.a_bytes * (swizzled ? 1 : 2);
-                    const double per_tap = kk * mt * prod, instr = taps * per_tap;
-                    const double mma = taps * std::max(per_tap * p.nt / 2.0, 90.0 + 46.0 * per_tap);
-                    const double shared = (instr * (4096.0 + p.nt * 32.0 / ways) + b_moved + a_stage) / 128.0;
-                    const double move = (x_moved + b_moved) / 40.0 + (copied && p.straddle ? 60.0 * p.rows * (s.stride == 1 ? 1 : 4) : 0.0) * 0.5;
-                    const double make = copied ? 0.0 : (double)pixels * kk * 2 * (swizzled ? 2.0 : 3.0) + (swizzled && p.raw_slots == 1 ? 1200.0 : 0.0);      // cycles of the producer warps for a piece; no stage of x ahead
-                    const double stage = std::max(std::max(mma, shared), std::max(move, make)) + 250.0 + 40.0 * taps / p.tap_group + (p.pair && tw.taps == 1 ? 300.0 : 0.0);
-                    const double out = (double)mt * 128 * p.nt * yb / 24.0;
-                    // (one accumulator that is cut waits for its sums to be added)
-                    const double item = p.per_split * stage + (p.cut && p.acc_bufs == 1 ? (p.per_split - 1) / p.cut * 1500.0 : 0.0);
-                    double c = 3500.0 + (p.pair ? dt == XGEN_F32 || s.stride == 2 ? 4000.0 : 6000.0 : 0.0);
-                    if (sp == 1) c += waves * std::max(item, p.acc_bufs >= 2 ? out : 0.0) + (p.acc_bufs >= 2 ? out : waves * out);
-                    else c += waves * (item + 2500.0 + 100.0 * sp + mt * 128.0 * p.nt * 4 / 64.0 + out / sp);
-                    if (c < best.cycles * 0.999) { best = p; best.cycles = c; }
                 }
             }
         }
@@ -447,8 +482,8 @@ cudaError_t tap_launch(const TapWeights &tw, const TapShape &s, const TapPlan &p
     P.b_off = p.a_stages * p.a_bytes;
     P.tab_off = p.operands;
     P.raw_off = P.tab_off + p.table_bytes;
-    P.raw_slots = p.raw_slots; P.raw_bytes = p.raw_bytes; P.raw_pitch = p.raw_pitch;
-    P.row_log = p.pl <= 2 ? 1 : p.pl <= 4 ? 2 : 3;
+    P.raw_slots = p.raw_slots; P.raw_px = p.raw_px; P.raw_bytes = p.raw_bytes; P.raw_pitch = p.raw_pitch;
+    P.row_log = row_log(p.pl);
     P.stage_off = P.sum_off = P.raw_off + p.raw_slots * p.raw_bytes;       // (the one or the other)
     P.raster = p.raster; P.pitch = p.pitch; P.rows = p.rows; P.pixels = p.pixels; P.sub_px = p.raster ? 128 : 16 * p.pitch;
     {

@@ -54,7 +54,7 @@ struct TapPlan {
     int raster = 0, pitch = 0, rows = 0, pixels = 0;     // staged tile: entries of a row, rows (of a parity), entries
     int a_stages = 0, a_bytes = 0, b_slots = 0, b_bytes = 0, tap_group = 1, resident = 0, operands = 0;   // (bytes of all of them)
     int plane_pitch = 0, table_bytes = 0;
-    int raw_slots = 0, raw_bytes = 0, raw_pitch = 0;     // rows of x that the producer warps shift into place (none: tensor copies, or fp32)
+    int raw_slots = 0, raw_px = 0, raw_bytes = 0, raw_pitch = 0;     // rows of x that the producer warps shift into place (none: tensor copies, or fp32)
     size_t smem = 0;
     int tmem_cols = 0, acc_bufs = 0;
     double cycles = 0;           // what the cost model expects

@@ -79,7 +79,7 @@ struct TapParams {
     int segs, nblk, nt, items, splits, per_split, stages, cut;
     int pl, plane_pitch;
     int a_stages, a_bytes, b_slots, resident, b_bytes, tap_group;
-    int raw_slots, raw_bytes, raw_pitch, row_log;    // x as it lies in memory: buffers, bytes of one and of a pixel; pieces of a pixel (log2)
+    int raw_slots, raw_px, raw_bytes, raw_pitch, row_log;    // x as it lies in memory: buffers, pixels and bytes of one, bytes of a pixel; pieces of a pixel (log2)
     int b_off, tab_off, raw_off, stage_off, sum_off;     // bytes into dynamic shared memory
     int tmem_cols, acc_bufs, staged;
     int tap_start[9];                           // first staged entry of a tap
@@ -988,7 +988,8 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     for (int i = lane;; i += 32) {
                         const int p = (i >> g_log) * q_step + (own << g_log) + (i & ((1 << g_log) - 1));
                         if (p >= P.pixels) break;
-                        pix[p] = tap_source<STRIDE, TAPS>(P, t, p);
+                        const int at = tap_source<STRIDE, TAPS>(P, t, p);
+                        pix[p] = kF32 || at < 0 ? at : (int)((uint32_t)at * (uint32_t)row_bytes);      // fp16, int8: bytes from x on
                     }
                     __syncwarp();
                 }
@@ -1061,36 +1062,65 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 make(v1);
             }
             } else {
-            // fp16, int8: a stage's rows are copied as they lie in memory (the aligned 16-byte pieces that hold a wanted byte,
-            // zeros outside the image) into one of raw_slots buffers, raw_slots - 1 stages ahead of their use, and shifted
+            // fp16, int8: a stage's rows (or a part of them: raw_px, a multiple of q_step, where a stage's do not fit) are
+            // copied as they lie in memory (the aligned 16-byte pieces that hold a wanted byte, zeros outside the image)
+            // into one of raw_slots buffers, raw_slots - 1 of them ahead of their use, and shifted
             // into place from there.  A warp copies and shifts the same pixels, so warps need not meet.
+            // Pieces are taken U at a time.  (The large tiles of stride 2 four: with two a stage waited for the latency of its
+            // shared memory, 32 images of 28x28x503 -> 256 fp16 60.4 us, 55.5 now; four that all lie outside the image, as most do
+            // of a tile over small images, are neither copied nor shifted.)
+            constexpr int U = STRIDE == 2 ? 4 : 2;
+            constexpr uint32_t kNone = 0xFFFFFFFFu;      // (bytes from x on: it has fewer than 2^31 elements)
+            auto sources = [&](uint32_t (&px)[U], const int *pix, int first, int q, int end) {
+                uint32_t all = kNone;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int qu = STRIDE == 2 ? q + u * q_step : min(q + u * q_step, end - 1);
+                    if (STRIDE == 2 && qu >= end) px[u] = kNone;       // (its table entry may be another warp's, and not there yet)
+                    else px[u] = TAPS == 9 ? (uint32_t)pix[qu] : (int64_t)first + qu < P.npix ? (uint32_t)(first + qu) * (uint32_t)row_bytes : kNone;
+                    all &= px[u];
+                }
+                return STRIDE == 2 && all == kNone;
+            };
             int slot_f = 0, slot = 0, tab = 0, row = 0;
+            int part_f = 0, part = 0;                    // first pixel of the part
             const int ahead = P.raw_slots - 1;
 #pragma unroll 1
             for (int turn = -ahead; item < P.items; ++turn) {
                 if (item_f < P.items) {
-                    if (ks_f == k0) begin();
+                    if (ks_f == k0 && part_f == 0) begin();
                     const int *const pix = table(tab_f);
+                    const int end = min(part_f + P.raw_px, P.pixels);
                     const int npl = min(P.pl, planes - ks_f * P.pl), want = min(npl * T::cpp, P.c_in - ks_f * P.pl * T::cpp) * T::xb;
                     uint32_t d = sbase + (uint32_t)(P.raw_off + slot_f * P.raw_bytes + q0 * P.raw_pitch + pl * kPiece);
                     const char *const at = x + (size_t)(ks_f * P.pl * T::cpp) * T::xb;
                     if (pl < npl) {
-#pragma unroll 2
-                        for (int q = q0; q < P.pixels; q += q_step, d += (uint32_t)(q_step * P.raw_pitch)) {
-                            const int px = TAPS == 9 ? pix[q] : (int64_t)row_f + q < P.npix ? row_f + q : -1;
-                            const char *const src = at + (size_t)max(px, 0) * row_bytes;
-                            const int lead = P.vec_x ? 0 : (int)(reinterpret_cast<uintptr_t>(src) & 15);
-                            const int left = px < 0 ? 0 : lead + want - pl * kPiece;          // wanted bytes from this piece on
-                            const char *const from = src - lead;
-                            copy16(d, from + (left > 0 ? pl * kPiece : 0), left > 0 ? 16u : 0u);
-                            if (!P.vec_x && pl == npl - 1) copy16(d + kPiece, from + (left > kPiece ? (pl + 1) * kPiece : 0), left > kPiece ? 16u : 0u);
+#pragma unroll 1
+                        for (int q = part_f + q0; q < end; q += U * q_step, d += (uint32_t)(U * q_step * P.raw_pitch)) {
+                            uint32_t px[U];
+                            if (sources(px, pix, row_f, q, end)) continue;
+#pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                if (q + u * q_step >= end) break;
+                                const char *const src = at + (px[u] == kNone ? 0u : px[u]);
+                                const int lead = P.vec_x ? 0 : (int)(reinterpret_cast<uintptr_t>(src) & 15);
+                                const int left = px[u] == kNone ? 0 : lead + want - pl * kPiece;          // wanted bytes from this piece on
+                                const char *const from = src - lead;
+                                const uint32_t to = d + (uint32_t)(u * q_step * P.raw_pitch);
+                                copy16(to, from + (left > 0 ? pl * kPiece : 0), left > 0 ? 16u : 0u);
+                                if (!P.vec_x && pl == npl - 1) copy16(to + kPiece, from + (left > kPiece ? (pl + 1) * kPiece : 0), left > kPiece ? 16u : 0u);
+                            }
                         }
                     }
                     if (++slot_f == P.raw_slots) slot_f = 0;
-                    if (++ks_f == k1) {
-                        ks_f = k0;
-                        item_f += item_step;
-                        if (++tab_f == P.raw_slots) tab_f = 0;
+                    part_f = end;
+                    if (part_f == P.pixels) {
+                        part_f = 0;
+                        if (++ks_f == k1) {
+                            ks_f = k0;
+                            item_f += item_step;
+                            if (++tab_f == P.raw_slots) tab_f = 0;
+                        }
                     }
                 }
                 copy_commit();
@@ -1099,33 +1129,39 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 else if (ahead == 1) copy_wait<1>();
                 else if (ahead == 2) copy_wait<2>();
                 else copy_wait<3>();
-                wait_warp(a_empty(s), ph);
+                if (part == 0) wait(a_empty(s), ph);
+                __syncwarp();
+                const int end = min(part + P.raw_px, P.pixels);
                 const unsigned char *const raw = smem + P.raw_off + slot * P.raw_bytes + pl * kPiece;
                 const uint32_t dst = sbase + (uint32_t)(s * P.a_bytes);
                 const int npl = min(P.pl, planes - ks * P.pl), left = P.c_in - (ks * P.pl + pl) * T::cpp;      // channels there are from this piece on
                 if (TAPS == 1 && ks == k0) row = tap_item<MT, PAIR>(P, item, side).v0 * 8;
                 if (pl < npl) {
                     const int *const pix = table(tab);
-                    constexpr int U = 2, W = 4;          // pieces at a time: their loads side by side
+                    const uint32_t at15 = (uint32_t)reinterpret_cast<uintptr_t>(x) + (uint32_t)(ks * P.pl * T::cpp * T::xb);
 #pragma unroll 1
-                    for (int q = q0; q < P.pixels; q += U * q_step) {
-                        uint32_t v[U][W];
+                    for (int q = part + q0; q < end; q += U * q_step) {
+                        uint32_t px[U], v[U][4];
+                        if (sources(px, pix, row, q, end)) {
+#pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                const int qu = q + u * q_step;
+                                if (qu < end) sts128(dst + (uint32_t)(qu * 128 + ((pl ^ (qu & 7)) << 4)), make_uint4(0u, 0u, 0u, 0u));
+                            }
+                            continue;
+                        }
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
-                            const int qu = min(q + u * q_step, P.pixels - 1);
-                            const uint4 *const in = reinterpret_cast<const uint4 *>(raw + qu * P.raw_pitch);
+                            const uint4 *const in = reinterpret_cast<const uint4 *>(raw + (min(q + u * q_step, end - 1) - (STRIDE == 2 ? part : 0)) * P.raw_pitch);
                             const uint4 a = in[0];
                             v[u][0] = a.x; v[u][1] = a.y; v[u][2] = a.z; v[u][3] = a.w;
-                            if (P.vec_x) continue;
-                            const int px = TAPS == 9 ? max(pix[qu], 0) : (int)min((int64_t)row + qu, P.npix - 1);
-                            const int lead = (int)(reinterpret_cast<uintptr_t>(x + (size_t)(ks * P.pl * T::cpp) * T::xb + (size_t)px * row_bytes) & 15);
-                            shift16(v[u], in[1], lead);
+                            if (!P.vec_x) shift16(v[u], in[1], (int)(at15 + px[u]) & 15);
                         }
                         if (!P.vec_x && left < T::cpp) {       // (0 or less: a plane that fills a pair up)
 #pragma unroll
                             for (int u = 0; u < U; ++u)
 #pragma unroll
-                                for (int e = 0; e < W; ++e) {
+                                for (int e = 0; e < 4; ++e) {
                                     const int bytes = left * T::xb - 4 * e;
                                     if (bytes < 4) v[u][e] = bytes <= 0 ? 0u : v[u][e] & ((1u << (8 * bytes)) - 1u);
                                 }
@@ -1133,14 +1169,20 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
                             const int qu = q + u * q_step;
-                            if (qu < P.pixels) sts128(dst + (uint32_t)(qu * 128 + ((pl ^ (qu & 7)) << 4)), make_uint4(v[u][0], v[u][1], v[u][2], v[u][3]));
+                            if (qu < end) sts128(dst + (uint32_t)(qu * 128 + ((pl ^ (qu & 7)) << 4)), make_uint4(v[u][0], v[u][1], v[u][2], v[u][3]));
                         }
                     }
                 }
+                if (++slot == P.raw_slots) slot = 0;
+                part = end;
+                if (part < P.pixels) {
+                    __syncwarp();                        // (the buffer is filled anew)
+                    continue;
+                }
+                part = 0;
                 fence_async_proxy();
                 __syncwarp();
                 if (lane == 0) arrive_lead(a_full(s));
-                if (++slot == P.raw_slots) slot = 0;
                 if (++s == P.a_stages) { s = 0; ph ^= 1u; }
                 if (++ks == k1) {
                     ks = k0;

@@ -149,3 +149,33 @@ def test_queries_tell_of_what_runs_and_what_is_held(fake_lib):
             assert g.stats()["device_bytes"] == fake.fake_live_bytes() - held
             g.close()
     """)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16", "i8"])
+@pytest.mark.parametrize("stride", [1, 2])
+def test_every_layer_of_the_matrix_path_has_a_plan(fake_lib, dtype, stride):
+    """No shape falls back to the command stream: whatever its rows, tiles, batch and fused operators are, a run launches the
+    matrix kernel and allocates nothing."""
+    _run(fake_lib, """
+        dtype, stride = %r, %d
+        threads = {"f32": 16, "f16": 24, "i8": 24}[dtype] * 32
+        for ci in (8, 17, 33, 67, 128, 131, 503):
+            for co in (16, 37, 93, 256, 400):
+                pk = conv(dtype, ci, co, stride)
+                for n, h, w in ((1, 1, 1), (1, 14, 14), (1, 57, 57), (4, 224, 224), (32, 56, 56), (8, 112, 112), (64, 28, 28), (200, 7, 7), (2, 200, 111), (3, 5, 700)):
+                    if n * h * w * max(ci, co) >= 2 ** 31:
+                        continue
+                    held, launches = fake.fake_live_bytes(), fake.fake_launches()
+                    ho, wo = pk.out_shape(h, w)
+                    pool = 2 if ho %% 2 == 0 and wo %% 2 == 0 else 0
+                    assert pk.plan_info(n, h, w)["matrix_path"] == 1, (ci, co, n, h, w)
+                    calls = [lambda: pk.run(X, n, h, w, B, True, Y), lambda: pk.run_fused(X, n, h, w, B, Y, residual_ptr=3 << 41),
+                             lambda: pk.run_fused(X, n, h, w, B, Y, pool=pool, residual_ptr=3 << 41)]
+                    if dtype == "i8":
+                        calls.append(lambda: pk.run_fused(X, n, h, w, B, Y, residual_ptr=3 << 41, requant_scale_ptr=B))
+                    for call in calls:
+                        call()
+                        assert fake.fake_launch(1) == threads, (ci, co, n, h, w)
+                    assert fake.fake_live_bytes() == held and fake.fake_launches() == launches + len(calls)
+                pk.close()
+    """ % (dtype, stride))

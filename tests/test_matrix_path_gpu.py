@@ -51,6 +51,29 @@ def test_either_side_of_the_fewest_channels(dtype, stride, ci):
     compare(d, run_gpu(pk, d.x, None, False, plan=True), bias=None, relu=False)
 
 
+@pytest.mark.parametrize("dtype", ["f16", "i8"])
+@pytest.mark.parametrize("stride,shape", [
+    (2, (24, 67, 93, 56, 56)),     # several items of a block, two stages each (int8: one); elements stored one by one
+    (2, (24, 131, 40, 41, 57)),    # ... of three stages (two); whole pieces of y
+    (2, (30, 17, 37, 64, 50)),     # one short stage
+    (2, (6, 503, 256, 28, 28)),    # eight stages (four): fp16 chains that are cut
+    (2, (1, 67, 300, 13, 17)),     # one item a block: whole stages
+    (1, (3, 67, 93, 45, 77)),      # a raster of 467 entries
+    (1, (5, 33, 31, 20, 140)),
+    (1, (72, 103, 285, 66, 5)),    # several items of a block, columns of zeros in the raster
+])
+def test_rows_shifted_in_parts_of_a_stage(dtype, stride, shape):
+    """Rows of x that are not whole 16-byte pieces, in tiles too large for the shared memory of whole stages."""
+    n, ci, co, h, w = shape
+    d = _layer(dtype, n, ci, co, h, w, stride, seed=ci)
+    pk = pack(d)
+    assert pk.plan_info(n, h, w)["matrix_path"] == 1
+    y = run_gpu(pk, d.x, d.bias, True)
+    compare(d, y)
+    for _ in range(2):
+        assert np.array_equal(run_gpu(pk, d.x, d.bias, True), y)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "f16", "i8"])
 @pytest.mark.parametrize("shape", [(1, 512, 96, 14, 14), (1, 320, 512, 7, 7), (2, 256, 40, 9, 12)])
 def test_reduction_split_over_a_cluster(dtype, shape):
