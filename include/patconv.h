@@ -165,7 +165,10 @@ xgen_status xgen_patconv_pack(const xgen_patconv_desc *desc, const void *dense_w
  *   y_dev    [n][ho][wo][c_out] NHWC, 16-byte aligned, must not overlap x_dev;
  *            ho, wo as xgen_patconv_out_shape reports
  *   cuda_stream  a cudaStream_t passed as void* (NULL = default stream)
- * Only enqueues work on the stream: no synchronisation, no device allocation.
+ * Only enqueues work on the stream: no synchronisation, no device allocation.  (The exception: where
+ * the driver cannot describe tensors to the copy engine, a layer of the matrix path falls back to the command
+ * stream, which xgen_patconv_plan uploads, or else the first run; inside a stream capture that run is
+ * UNSUPPORTED.)
  * The caller keeps x, bias and y alive until the stream reaches that work.
  * Concurrent calls on different streams are allowed on the matrix path, and on the command-stream
  * kernel for unplanned shapes (the handle only remembers, under a lock, the launch geometry of
@@ -242,7 +245,8 @@ xgen_status xgen_patconv_run_fused(const xgen_patconv_packed *packed, const void
  * number of chunks; s = 1 needs no scratch); beyond that the call returns XGEN_ERR_SHAPE and
  * launches nothing (with XGEN_PATCONV_LOG set, the reason goes to stderr).
  * Calls share nothing but the handle, so they may overlap on different streams.
- * Errors: INVALID_ARG, SHAPE, CUDA, as xgen_patconv_run, plus SHAPE for the limit.
+ * Errors: INVALID_ARG, SHAPE, CUDA, as xgen_patconv_run, plus SHAPE for the limit, and UNSUPPORTED where
+ * xgen_patconv_run would upload the command stream first.
  */
 #define XGEN_PATCONV_STATIC_SCRATCH_BYTES (8u << 20)
 xgen_status xgen_patconv_run_static_scratch(const xgen_patconv_packed *packed, const void *x_dev,

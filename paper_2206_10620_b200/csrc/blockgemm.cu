@@ -594,8 +594,15 @@ xgen_status xgen_blockgemm_run(const xgen_blockgemm_packed *hc, const void *x, i
     }
     {
         std::lock_guard<std::mutex> lock(h->tap_mu);
-        const xgen_status us = h->d_stream ? XGEN_OK : upload_stream(h);
-        if (us != XGEN_OK) return us;
+        if (!h->d_stream) {
+            if (patconv::being_captured((cudaStream_t)stream)) return XGEN_ERR_UNSUPPORTED;
+            int prev = 0;
+            if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
+            if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
+            const xgen_status us = upload_stream(h);
+            if (prev != h->device) cudaSetDevice(prev);
+            if (us != XGEN_OK) return us;
+        }
     }
     GParams P{};
     P.x = x; P.y = y; P.bias = static_cast<const float *>(bias);

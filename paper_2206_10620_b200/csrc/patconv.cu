@@ -1152,6 +1152,10 @@ EncodeTiledFn encode_tiled_fn() {
     });
     return fn;
 }
+bool being_captured(cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+}
 }  // namespace patconv
 
 template <int DT, int STRIDE, bool FUSED, int BH>
@@ -1470,10 +1474,16 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
         return e == cudaSuccess ? XGEN_OK : XGEN_ERR_CUDA;
     }
     {
-        // (only where the driver cannot encode the matrix path's tensor maps is the stream not there yet)
+        // The stream is not there yet where neither packing nor a plan has seen that it is needed: the driver cannot encode the
+        // matrix path's tensor maps.  It is uploaded by the first run that may allocate.
         std::lock_guard<std::mutex> lock(h->stream_mu);
         if (!h->d_slots) {
+            if (ignore_plan || being_captured((cudaStream_t)stream)) return XGEN_ERR_UNSUPPORTED;
+            int prev = 0;
+            if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
+            if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
             const xgen_status us = upload_layout(h);
+            if (prev != h->device) cudaSetDevice(prev);
             if (us != XGEN_OK) return us;
         }
     }
@@ -1757,7 +1767,7 @@ xgen_status xgen_patconv_plan_tuned(xgen_patconv_packed *h, int32_t n, int32_t h
     if ((int64_t)n * ho * wo * p.c_out > 0x7FFFFFFFLL) return XGEN_ERR_SHAPE;
     const xgen_patconv_tuning tn = tuning ? *tuning : xgen_patconv_tuning{};
     const bool tma_ok = !tn.no_copy_engine && encode_tiled_fn() != nullptr;
-    const bool stream = asks_for_stream(tn) || !h->tap.dev;        // later runs take the command-stream kernel
+    const bool stream = asks_for_stream(tn) || !h->tap.dev || !encode_tiled_fn();        // later runs take the command-stream kernel
     int prev = 0;
     if (cudaGetDevice(&prev) != cudaSuccess || cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;
     xgen_status rs = XGEN_OK;

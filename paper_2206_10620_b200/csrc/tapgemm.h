@@ -16,6 +16,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn encode_tiled_fn();
+// Whether a stream records a graph, in which nothing may be allocated (patconv.cu).
+bool being_captured(cudaStream_t st);
 
 // The layer's weights as the kernel reads them: pruned entries are zeros, fp32 weights are three
 // bf16 parts whose sum is the weight.  Bytes [plane][tap][part][filter][16]: a plane is 16 bytes of

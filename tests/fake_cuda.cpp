@@ -15,6 +15,8 @@ static cudaError_t last = cudaSuccess;
 static cudaError_t is(cudaError_t e) { if (e != cudaSuccess) last = e; return e; }
 // grid, block, dynamic shared memory, cluster of the last launch
 static long long launch[4];
+// the current device, that of the last allocation; whether streams are being captured, and the driver has no tensor maps
+static int device = 0, alloc_device = -1, capturing = 0, no_encode = 0;
 
 extern "C" {
 // The n-th allocation (encoding of a tensor map) from now on fails; 0: none does.
@@ -23,9 +25,14 @@ void fake_fail_encode(int n) { fail_encode = n; }
 long long fake_live_bytes() { return live_bytes; }
 int fake_launches() { return launches; }
 long long fake_launch(int what) { return launch[what]; }
+int fake_alloc_device() { return alloc_device; }
+int fake_device() { return device; }
+void fake_capture(int on) { capturing = on; }
+void fake_no_encode(int on) { no_encode = on; }
 
 cudaError_t cudaMalloc(void **p, size_t n) {
     if (fail_alloc && --fail_alloc == 0) return is(cudaErrorMemoryAllocation);
+    alloc_device = device;
     *p = aligned_alloc(256, (n + 255) / 256 * 256);
     live[*p] = n;
     live_bytes += (long long)n;
@@ -66,8 +73,12 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int *n, const void *, 
 }
 cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int) { return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int *v, cudaDeviceAttr, int) { *v = sms; return cudaSuccess; }
-cudaError_t cudaGetDevice(int *d) { *d = 0; return cudaSuccess; }
-cudaError_t cudaSetDevice(int) { return cudaSuccess; }
+cudaError_t cudaGetDevice(int *d) { *d = device; return cudaSuccess; }
+cudaError_t cudaSetDevice(int d) { device = d; return cudaSuccess; }
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s) {
+    *s = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+    return cudaSuccess;
+}
 cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
 cudaError_t cudaGetLastError() { const cudaError_t e = last; last = cudaSuccess; return e; }
 const char *cudaGetErrorString(cudaError_t) { return "fake"; }
@@ -90,8 +101,8 @@ static CUresult encode(CUtensorMap *m, CUtensorMapDataType, cuuint32_t, void *, 
     return CUDA_SUCCESS;
 }
 cudaError_t cudaGetDriverEntryPoint(const char *, void **p, unsigned long long, cudaDriverEntryPointQueryResult *q) {
-    *p = (void *)encode;
-    if (q) *q = cudaDriverEntryPointSuccess;
+    *p = no_encode ? nullptr : (void *)encode;
+    if (q) *q = no_encode ? cudaDriverEntryPointSymbolNotFound : cudaDriverEntryPointSuccess;
     return cudaSuccess;
 }
 

@@ -179,3 +179,39 @@ def test_every_layer_of_the_matrix_path_has_a_plan(fake_lib, dtype, stride):
                     assert fake.fake_live_bytes() == held and fake.fake_launches() == launches + len(calls)
                 pk.close()
     """ % (dtype, stride))
+
+
+def test_the_stream_of_a_layer_without_a_plan_is_uploaded_where_it_may_be(fake_lib):
+    """The command stream that a run falls back to goes to the handle's device, whichever is current, and never
+    from inside a capture or a call that promises not to allocate."""
+    _run(fake_lib, """
+        for pk, run in ((conv("f16", 33, 48, 2, device=1), lambda p: status(p.run, X, 2, 20, 20, B, True, Y)),
+                        (gemm("f32", 64, 48, device=1), lambda p: status(p.run, X, 32, B, True, Y))):
+            held, n = fake.fake_live_bytes(), fake.fake_launches()
+            fake.fake_capture(1)
+            fake.fake_fail_encode(1)             # the matrix path has no plan
+            assert run(pk) == 4 and fake.fake_launches() == n and fake.fake_live_bytes() == held
+            fake.fake_capture(0)
+            if hasattr(pk, "run_static_scratch"):
+                fake.fake_fail_encode(1)
+                assert status(pk.run_static_scratch, X, 2, 20, 20, B, True, Y, 1) == 4
+                assert fake.fake_launches() == n and fake.fake_live_bytes() == held
+            fake.fake_fail_encode(1)
+            assert fake.fake_device() == 0 and run(pk) == 0 and fake.fake_device() == 0
+            assert fake.fake_alloc_device() == 1 and fake.fake_launches() == n + 1 and fake.fake_live_bytes() > held
+            pk.close()
+    """)
+
+
+def test_a_plan_uploads_the_stream_where_there_are_no_tensor_maps(fake_lib):
+    _run(fake_lib, """
+        fake.fake_no_encode(1)
+        pk = conv("f16", 64, 48, device=1)
+        pk.plan(2, 20, 20)
+        assert fake.fake_alloc_device() == 1
+        held, n = fake.fake_live_bytes(), fake.fake_launches()
+        fake.fake_capture(1)
+        assert status(pk.run, X, 2, 20, 20, B, True, Y) == 0
+        assert status(pk.run_static_scratch, X, 2, 20, 20, B, True, Y, 1) == 0
+        assert fake.fake_launches() == n + 2 and fake.fake_live_bytes() == held
+    """)
