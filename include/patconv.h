@@ -12,7 +12,8 @@
  *
  * with t = 3*dy + dx, zero padding of 1, stride s in {1,2}, cross-correlation
  * (no kernel flip), act = ReLU or identity.  Pruned weights contribute nothing, also
- * where they meet an infinity or a NaN; ReLU keeps a NaN on the matrix path.
+ * where they meet an infinity or a NaN; ReLU keeps a NaN on the matrix path, and makes it 0 on the
+ * other two.
  *
  * Three kernels compute it.  The matrix path runs the layer dense on the tensor cores, with zeros for
  * the pruned weights, and is what a call takes by default.  Layers of a few input channels (fp32: up to

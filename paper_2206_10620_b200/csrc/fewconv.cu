@@ -53,14 +53,15 @@ template <int DT, int CIN> __device__ __forceinline__ void few_pixel(const FewPa
     for (int e = 0; e < CIN; ++e) v[e] = few_value<DT>(P.x, i + e);
 }
 
-// Store one result.
+// Store one result.  (ReLU of a NaN is 0, as on the command stream, which the same handle's fused runs and its runs of large images
+// with few kernels left take.)
 template <int DT> __device__ __forceinline__ void few_store1(const FewParams &P, size_t i, float sum, const void *bias, int c) {
     if constexpr (DT == XGEN_I8_I32) {
         const int v = (int)sum + (bias ? static_cast<const int *>(bias)[c] : 0);          // (exact: at most 7 x 4 products below 2^15)
         static_cast<int *>(P.y)[i] = P.relu ? max(v, 0) : v;
     } else {
         float v = sum + (bias ? static_cast<const float *>(bias)[c] : 0.0f);
-        if (P.relu) asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(v) : "f"(v));
+        if (P.relu) v = fmaxf(v, 0.0f);
         if constexpr (DT == XGEN_F32) static_cast<float *>(P.y)[i] = v;
         else static_cast<__half *>(P.y)[i] = __float2half_rn(v);
     }
@@ -184,7 +185,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_kernel(const __grid_consta
                     o[4 * q + e] = (uint32_t)(P.relu ? max(v, 0) : v);
                 } else {
                     float v = acc[p][4 * q + e] + __uint_as_float(bb[e]);
-                    if (P.relu) asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(v) : "f"(v));
+                    if (P.relu) v = fmaxf(v, 0.0f);
                     o[4 * q + e] = __float_as_uint(v);
                 }
             }

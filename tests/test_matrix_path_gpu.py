@@ -520,3 +520,21 @@ def test_few_channels_infinities_under_pruned_weights(dtype):
     assert np.array_equal(np.isfinite(y), fine) and 0 < (~fine).sum() < 2 * 9 * 32
     assert np.array_equal(y[~fine], ref[~fine], equal_nan=True)
     assert (np.abs(y[fine] - ref[fine]) <= 2 * TOL[dtype] * np.maximum(np.abs(ref[fine]), 0.01)).all()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16"])
+@pytest.mark.parametrize("co", [32, 37])          # whole pieces of y; elements one by one
+def test_few_channels_relu_of_a_nan(dtype, co):
+    """The same, with and without other operators behind it, as on the command stream: 0."""
+    d = _layer(dtype, 1, 3, co, 20, 30, prune=0.6, seed=4)
+    d.x[0, 7, 11, 1] = np.inf                     # (infinite sums of both signs)
+    d.x[0, 7, 12, 1] = -np.inf                    # (and sums of both: NaN)
+    d.x[0, 15, 20, 0] = np.nan
+    few, stream = pack(d), pack(d)
+    stream.plan(1, 20, 30, splits=1)
+    raw, ref = run_gpu(stream, d.x, d.bias, False), run_gpu(stream, d.x, d.bias, True).astype(np.float64)
+    y = run_gpu(few, d.x, d.bias, True).astype(np.float64)
+    assert np.isnan(raw).sum() > 20 and not np.isnan(ref).any() and (y[np.isnan(raw)] == 0).all()
+    assert np.array_equal(np.isinf(y), np.isinf(ref)) and np.isinf(y).any()
+    fine = np.isfinite(ref)
+    assert (np.abs(y[fine] - ref[fine]) <= 2 * TOL[dtype] * np.maximum(np.abs(ref[fine]), 0.01)).all()
