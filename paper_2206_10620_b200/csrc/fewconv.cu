@@ -57,7 +57,8 @@ template <int DT, int CIN> __device__ __forceinline__ void few_pixel(const FewPa
 // with few kernels left take.)
 template <int DT> __device__ __forceinline__ void few_store1(const FewParams &P, size_t i, float sum, const void *bias, int c) {
     if constexpr (DT == XGEN_I8_I32) {
-        const int v = (int)sum + (bias ? static_cast<const int *>(bias)[c] : 0);          // (exact: at most 7 x 4 products below 2^15)
+        // (the sum is exact, at most 7 x 4 products below 2^15; a bias that takes it past 2^31 wraps, as on the matrix path)
+        const int v = (int)((uint32_t)(int)sum + (bias ? static_cast<const uint32_t *>(bias)[c] : 0u));
         static_cast<int *>(P.y)[i] = P.relu ? max(v, 0) : v;
     } else {
         float v = sum + (bias ? static_cast<const float *>(bias)[c] : 0.0f);
@@ -181,7 +182,7 @@ __global__ void __launch_bounds__(kFewThreads, 3) few_kernel(const __grid_consta
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 if constexpr (DT == XGEN_I8_I32) {
-                    const int v = (int)acc[p][4 * q + e] + (int)bb[e];
+                    const int v = (int)((uint32_t)(int)acc[p][4 * q + e] + bb[e]);
                     o[4 * q + e] = (uint32_t)(P.relu ? max(v, 0) : v);
                 } else {
                     float v = acc[p][4 * q + e] + __uint_as_float(bb[e]);

@@ -538,3 +538,14 @@ def test_few_channels_relu_of_a_nan(dtype, co):
     assert np.array_equal(np.isinf(y), np.isinf(ref)) and np.isinf(y).any()
     fine = np.isfinite(ref)
     assert (np.abs(y[fine] - ref[fine]) <= 2 * TOL[dtype] * np.maximum(np.abs(ref[fine]), 0.01)).all()
+
+
+@pytest.mark.parametrize("ci,co", [(3, 32), (3, 37), (64, 32)])       # dense on the FP32 pipe, whole pieces and not; matrix units
+def test_int32_results_wrap(ci, co):
+    d = _layer("i8", 1, ci, co, 9, 11, prune=0.3, seed=ci)
+    bias = np.where(np.arange(co) % 2, 2 ** 31 - 1, -2 ** 31).astype(np.int32)
+    ref = oracle.conv(d.x, d.w, d.pid, d.masks, bias=None, relu=False).astype(np.int64) + bias
+    wrapped = (ref + 2 ** 31) % 2 ** 32 - 2 ** 31
+    assert (wrapped != ref).any()
+    assert np.array_equal(run_gpu(pack(d), d.x, bias, False).astype(np.int64), wrapped)
+    assert np.array_equal(run_gpu(pack(d), d.x, bias, True).astype(np.int64), np.maximum(wrapped, 0))
