@@ -1042,6 +1042,8 @@ constexpr int kLaunchCache = 4;
 
 // A plan of the matrix path for one shape.
 struct TapEntry { TapShape shape; TapPlan plan; uint64_t stamp = 0; };
+// Which kernel a layer of a few input channels runs on, by shape.
+struct FewEntry { int n = 0, ho = 0, wo = 0, bh = 0; bool stream = false; uint64_t stamp = 0; };
 
 }  // namespace patconv
 
@@ -1076,6 +1078,7 @@ struct xgen_patconv_packed {
     bool stream_asked = false;
     mutable std::mutex tap_mu;
     mutable TapEntry tap_cache[kLaunchCache];
+    mutable FewEntry few_cache[kLaunchCache];
     mutable uint64_t tap_stamp = 0;
     // prepared launches (shape, input address)
     mutable std::mutex cache_mu;
@@ -1374,15 +1377,48 @@ static bool asks_for_stream(const xgen_patconv_tuning &t) {
 // Whether a run takes the matrix path.
 static bool on_matrix_units(const xgen_patconv_packed *h) { return h->tap.dev && !h->stream_asked; }
 
-// A layer of a few input channels: whether the command stream, whose work is the kept kernels alone, beats the dense kernel.
-// An image of 224x224 of a large batch takes the dense kernel 1.9 us a channel (64 filters), the stream 5 (fp32), 5.5 (fp16) or
-// 7 us (int8) and about one for every kept kernel of a filter: 9 images, 60 % pruned, dense against stream, us: fp32 4 channels
-// 70.5, 62.8; fp16 7: 121, 83.9; int8 7: 115, 97.4 (unpruned, one image: 9.8, 12.9; 15.5, 15.7; 14.3, 18.4).  Small images, stride 2 and
-// filters that do not fill its warps leave the stream's threads idle (32 x 112x112, 3 -> 32, stride 2: 8.6, 19.9).
-static bool stream_is_faster(const PackedHost &p, int64_t pixels) {
-    if (p.stride != 1 || p.c_out % 64 != 0 || pixels < 40000) return false;
-    const double fixed = p.dtype == XGEN_F32 ? 5.0 : p.dtype == XGEN_F16_F32ACC ? 5.5 : 7.0;
-    return fixed + (double)p.stats.kernels_surviving / p.c_out < 1.9 * p.c_in;
+// A layer of a few input channels: whether the command stream, whose work is the kept kernels alone, beats the dense kernel
+// (by 5 %).  Both are modelled, in us: the dense kernel by pixels x filters (its lanes come in groups of one, two or four times 16, so 80
+// filters cost 128) and channels, the stream by the waves of its blocks (registers hold two of ten warps or fewer on an SM, one
+// of more) and what the warps of a wave keep.  Fitted to 601 calls of stride 1 (12000 pixels and more, 16 to 500
+// filters, 0 to 90 % pruned): the faster of the two is missed by 0.9 % on average; the dense kernel always, 7.9 %.
+// us, dense and stream, fp32 4 channels of 9 x 224x224: -> 48 unpruned 73.2, 43.8; -> 64, 90 % pruned 69.7, 55.6; -> 96 unpruned 131, 91.8;
+// one image -> 64 unpruned 10.4, 13.0, 90 % pruned 10.3, 9.5; fp16 7 -> 80, 90 % pruned, 29.2, 11.7.  Stride 2 and small images leave the
+// stream's threads idle (32 x 112x112, 3 -> 32, stride 2: 8.6, 19.9).
+static bool stream_is_faster(const PackedHost &p, int n, int ho, int wo) {
+    const int64_t pixels = (int64_t)n * ho * wo;
+    if (p.stride != 1 || pixels < 12000) return false;
+    // a call; a pixel and filter; times its channels; more at seven channels; where rows of y are not whole 16-byte pieces
+    constexpr double kDense[3][5] = {{2.591, 9.981e-6, 6.763e-6, 0.0, 3.543e-6}, {2.143, 11.254e-6, 6.574e-6, 8.914e-6, 4.186e-6}, {3.062, 9.542e-6, 7.231e-6, 2.284e-6, 3.321e-6}};
+    // a call; a wave; a warp in it; times its kept kernels; a block and channel; a warp, where rows are not whole pieces
+    constexpr double kStream[3][6] = {{0.681, 8.944, 0.176, 0.134, 0.0, 2.261}, {1.682, 7.053, 0.228, 0.143, 0.247, 3.097}, {2.321, 8.489, 0.270, 0.145, 0.112, 2.467}};
+    const double *const d = kDense[p.dtype], *const s = kStream[p.dtype];
+    const bool ragged = (size_t)p.c_out * (p.dtype == XGEN_F16_F32ACC ? 2 : 4) % 16 != 0;
+    const int sixteens = (p.c_out + 15) / 16, lanes = sixteens > 2 ? 4 : sixteens;
+    const double units = (double)pixels * ((sixteens + lanes - 1) / lanes * lanes);
+    const double dense = d[0] + units * (d[1] + d[2] * p.c_in + (p.c_in >= 7 ? d[3] : 0.0)) + (ragged ? d[4] * (double)pixels * p.c_out : 0.0);
+    Geometry g = grid_geometry(n, ho, wo, 1, p.bh), rows;
+    if (row_geometry(n, ho, wo, 1, p.bh, rows) && rows.covered > 1.08 * g.covered) g = rows;
+    const double per_sm = std::max(1, 65536 / ((p.wpc + kProducerWarps) * 32 * 96)), items = (double)g.tiles * p.n_blocks;
+    const double waves = std::ceil(items / (148 * per_sm)), blocks = waves > 1.0 ? per_sm : std::min(per_sm, items / 148);
+    const double warps = blocks * std::min<double>(p.wpc, (double)((p.c_out + 7) / 8) / p.n_blocks);
+    const double kept = (double)p.stats.kernels_surviving / p.c_out;
+    const double stream = s[0] + waves * (s[1] + warps * (s[2] + s[3] * kept + (ragged ? s[5] : 0.0)) + s[4] * blocks * p.c_in);
+    return stream * 1.05 < dense;
+}
+// The same, from the handle's small cache or weighed now.
+static bool takes_stream(const xgen_patconv_packed *h, int n, int ho, int wo) {
+    std::lock_guard<std::mutex> lock(h->tap_mu);
+    FewEntry *victim = &h->few_cache[0];
+    for (FewEntry &e : h->few_cache) {
+        if (e.stamp && e.n == n && e.ho == ho && e.wo == wo && e.bh == h->host.bh) {
+            e.stamp = ++h->tap_stamp;
+            return e.stream;
+        }
+        if (e.stamp < victim->stamp) victim = &e;
+    }
+    *victim = FewEntry{n, ho, wo, h->host.bh, stream_is_faster(h->host, n, ho, wo), ++h->tap_stamp};
+    return victim->stream;
 }
 
 // What the matrix path's plan of a call depends on.
@@ -1465,7 +1501,7 @@ static xgen_status run_layer(const xgen_patconv_packed *h, const void *x, int32_
         if (prev != h->device) cudaSetDevice(prev);
         if (fits) return e == cudaSuccess ? XGEN_OK : XGEN_ERR_CUDA;
     }
-    if (h->few.dev && !ep && (ignore_plan || (!h->stream_asked && !stream_is_faster(p, (int64_t)n * ho * wo)))) {
+    if (h->few.dev && !ep && (ignore_plan || (!h->stream_asked && !takes_stream(h, n, ho, wo)))) {
         int prev = 0;
         if (cudaGetDevice(&prev) != cudaSuccess) return XGEN_ERR_CUDA;
         if (prev != h->device && cudaSetDevice(h->device) != cudaSuccess) return XGEN_ERR_CUDA;

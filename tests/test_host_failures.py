@@ -215,3 +215,23 @@ def test_a_plan_uploads_the_stream_where_there_are_no_tensor_maps(fake_lib):
         assert status(pk.run_static_scratch, X, 2, 20, 20, B, True, Y, 1) == 0
         assert fake.fake_launches() == n + 2 and fake.fake_live_bytes() == held
     """)
+
+
+def test_layers_of_a_few_channels_take_the_faster_kernel(fake_lib):
+    """Large images of which little is left, and filters that do not fill the dense kernel's warps: the command stream; small
+    images, stride 2 and whole layers: the dense kernel, and always where nothing may be allocated."""
+    _run(fake_lib, """
+        for dtype, ci, co, n, hw, prune, stride, stream in (
+                ("f32", 4, 48, 9, 224, 0.0, 1, True), ("f32", 4, 96, 9, 224, 0.0, 1, True), ("f32", 4, 80, 1, 224, 0.9, 1, True),
+                ("f32", 4, 64, 9, 224, 0.9, 1, True), ("f16", 7, 80, 1, 224, 0.9, 1, True), ("i8", 7, 48, 9, 224, 0.9, 1, True),
+                ("f32", 3, 64, 1, 224, 0.0, 1, False), ("f32", 3, 64, 9, 224, 0.0, 1, False), ("f16", 3, 32, 9, 224, 0.0, 1, False),
+                ("f32", 4, 48, 1, 60, 0.9, 1, False), ("i8", 3, 64, 4, 224, 0.5, 1, False), ("f16", 7, 80, 4, 224, 0.9, 2, False)):
+            pk = conv(dtype, ci, co, stride, prune)
+            n0 = fake.fake_launches()
+            for _ in range(2):                       # weighed, and from the cache
+                pk.run(X, n, hw, hw, B, True, Y)
+                assert (fake.fake_launch(1) != 128) == stream, (dtype, ci, co, n, hw, prune, stride)
+            pk.run_static_scratch(X, n, hw, hw, B, True, Y, 1)
+            assert fake.fake_launch(1) == 128 and fake.fake_launches() == n0 + 3
+            pk.close()
+    """)
