@@ -294,7 +294,9 @@ xgen_status xgen_patconv_enqueue_host(const xgen_patconv_packed *packed, const v
  * first call that meets it; there this call only checks the shape, and nothing of what
  * follows applies: blocks that share a reduction are one cluster, need no workspace and wait for nobody
  * outside it.  The rest is about handles that run the command-stream kernel
- * (xgen_patconv_plan_stats.matrix_path = 0; the fields of its plan are reported for every handle).
+ * (xgen_patconv_plan_stats.matrix_path = 0; the fields of its plan are reported for every handle).  A layer of a few
+ * input channels is prepared for it too, since its fused runs take it, whichever kernel the plain ones take
+ * (few_channel_path).
  *   Layers with few output
  * pixels do not fill the GPU with (pixel tile x filter block) work items; for
  * such a shape this call lets later xgen_patconv_run calls split the input
@@ -407,7 +409,7 @@ typedef struct {
     int32_t matrix_path;        /* 1: a run takes the matrix units instead (dense taps, pruned weights as
                                    zeros), because the caller's tuning names no parameter of the
                                    command-stream kernel; the fields above describe that kernel's plan,
-                                   the fields below the launch of an xgen_patconv_run (0 otherwise)   */
+                                   the matrix_ fields the launch of an xgen_patconv_run (0 otherwise)  */
     int32_t matrix_items;       /* (tile or pair of tiles, range of filters) to be worked through      */
     int32_t matrix_splits;      /* thread blocks (pairs) of a cluster that share an item's channels    */
     int32_t matrix_blocks;      /* thread blocks of the launch                                         */
@@ -415,6 +417,9 @@ typedef struct {
     int32_t matrix_threads;     /* threads of a block                                                  */
     int32_t matrix_filters;     /* filters of an item                                                  */
     int32_t matrix_stages;      /* pieces that the input channels are staged in                        */
+    int32_t few_channel_path;   /* 1: an xgen_patconv_run takes the dense kernel for a few input channels,
+                                   which has no plan; the fields above describe the command stream, which
+                                   runs with fused operators take                                     */
     int64_t matrix_shared_bytes; /* dynamic shared memory of a block                                   */
 } xgen_patconv_plan_stats;
 

@@ -74,7 +74,8 @@ class PlanStats(ctypes.Structure):
                 ("matrix_items", ctypes.c_int32), ("matrix_splits", ctypes.c_int32),
                 ("matrix_blocks", ctypes.c_int32), ("matrix_cluster", ctypes.c_int32),
                 ("matrix_threads", ctypes.c_int32), ("matrix_filters", ctypes.c_int32),
-                ("matrix_stages", ctypes.c_int32), ("matrix_shared_bytes", ctypes.c_int64)]
+                ("matrix_stages", ctypes.c_int32), ("few_channel_path", ctypes.c_int32),
+                ("matrix_shared_bytes", ctypes.c_int64)]
 
 
 class ProbeResult(ctypes.Structure):

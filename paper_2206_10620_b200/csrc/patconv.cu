@@ -1784,6 +1784,7 @@ xgen_status xgen_patconv_plan_info(const xgen_patconv_packed *h, int32_t n, int3
             out->matrix_shared_bytes = (int64_t)tp.smem;
         }
     }
+    out->few_channel_path = h->few.dev && !h->stream_asked && !takes_stream(h, n, (hh - 1) / p.stride + 1, (ww - 1) / p.stride + 1) ? 1 : 0;
     out->workspace_bytes = planned ? (int64_t)((size_t)(L.items - h->plan_whole) * (size_t)h->plan_splits * rows_per_item(p) * 1024) : 0;
     return XGEN_OK;
 }

@@ -229,9 +229,15 @@ def test_layers_of_a_few_channels_take_the_faster_kernel(fake_lib):
             pk = conv(dtype, ci, co, stride, prune)
             n0 = fake.fake_launches()
             for _ in range(2):                       # weighed, and from the cache
+                assert pk.plan_info(n, hw, hw)["few_channel_path"] == int(not stream)
                 pk.run(X, n, hw, hw, B, True, Y)
                 assert (fake.fake_launch(1) != 128) == stream, (dtype, ci, co, n, hw, prune, stride)
             pk.run_static_scratch(X, n, hw, hw, B, True, Y, 1)
             assert fake.fake_launch(1) == 128 and fake.fake_launches() == n0 + 3
+            pk.plan(n, hw, hw, splits=1)             # the caller asks for the stream
+            pk.run(X, n, hw, hw, B, True, Y)
+            assert fake.fake_launch(1) != 128 and pk.plan_info(n, hw, hw)["few_channel_path"] == 0
             pk.close()
+        for handle in (conv("f32", 16, 32), conv("f32", 3, 32, device=-1)):
+            assert handle.plan_info(1, 224, 224)["few_channel_path"] == 0
     """)

@@ -549,3 +549,27 @@ def test_int32_results_wrap(ci, co):
     assert (wrapped != ref).any()
     assert np.array_equal(run_gpu(pack(d), d.x, bias, False).astype(np.int64), wrapped)
     assert np.array_equal(run_gpu(pack(d), d.x, bias, True).astype(np.int64), np.maximum(wrapped, 0))
+
+
+@pytest.mark.parametrize("dtype,ci", [("f32", 4), ("f16", 7), ("i8", 7)])
+@pytest.mark.parametrize("co,prune,few", [(48, 0.9, 0), (33, 0.9, None), (64, 0.0, None)])
+def test_few_channels_on_either_kernel(dtype, ci, co, prune, few):
+    """A large image of which little is left runs on the command stream, with the results of the dense kernel."""
+    n, h, w = 1, 224, 210
+    d = _layer(dtype, n, ci, co, h, w, prune=prune, seed=co, x_dist="u01" if dtype == "i8" else "upm1")
+    pk = pack(d)
+    assert few is None or pk.plan_info(n, h, w)["few_channel_path"] == few
+    compare(d, run_gpu(pk, d.x, d.bias, True))
+    dense = pack(d)
+    compare(d, _run_static(dense, d))
+
+
+def _run_static(pk, d):
+    import torch
+    s = d.spec
+    x, b = torch.from_numpy(d.x).cuda(), torch.from_numpy(d.bias).cuda()
+    buf, y = guarded_output((s.n, s.h, s.w, s.c_out), {"f32": torch.float32, "f16": torch.float16, "i8": torch.int32}[s.dtype])
+    pk.run_static_scratch(x.data_ptr(), s.n, s.h, s.w, b.data_ptr(), True, y.data_ptr(), 1)
+    pk.sync()
+    check_guards(buf)
+    return y.cpu().numpy()
