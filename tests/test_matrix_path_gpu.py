@@ -552,7 +552,7 @@ def test_int32_results_wrap(ci, co):
 
 
 @pytest.mark.parametrize("dtype,ci", [("f32", 4), ("f16", 7), ("i8", 7)])
-@pytest.mark.parametrize("co,prune,few", [(48, 0.9, 0), (33, 0.9, None), (64, 0.0, None)])
+@pytest.mark.parametrize("co,prune,few", [(96, 0.9, 0), (33, 0.9, None), (64, 0.0, None)])
 def test_few_channels_on_either_kernel(dtype, ci, co, prune, few):
     """A large image of which little is left runs on the command stream, with the results of the dense kernel."""
     n, h, w = 1, 224, 210
