@@ -11,8 +11,8 @@ output pixels / time, i.e. structural non-zeros only.
 
 Roofline figures are taken against measured rates: layers on the matrix path
 (`tap_kernel`, all of a layer's weights, pruned ones as zeros) against a dense
-bf16 matrix product, fp32 counting its six bf16 products; layers on the
-command-stream kernel against the fp32 FMA pipe, whose rate, and the launch
+bf16 matrix product, fp32 counting its six bf16 products; layers of a few input
+channels (`few_kernel`, dense too) and on the command-stream kernel against the fp32 FMA pipe, whose rate, and the launch
 floor, the library's own microbenchmarks measure before the timed region.  After the headline workload
 the other named workloads (single layer, ResNet-50 and ResNet-18 3x3 stacks,
 the large-batch points of the single-layer sweep) are timed the same way and
@@ -49,7 +49,8 @@ UNIT = "GFLOP/s"
 # three bf16 parts of which six products are taken; int8 runs at twice the rate.
 MATRIX_PRODUCTS = {"f32": 6.0, "f16": 1.0, "i8": 0.5}
 KERNEL_SOURCES = ["paper_2206_10620_b200/csrc/" + f for f in
-                  ("tapgemm.cu", "tapgemm.h", "ptx.cuh", "patconv.cu", "gen_core.py", "pack.cpp")]
+                  ("tapgemm_kernel.cuh", "tapgemm_f32.cu", "tapgemm_f16.cu", "tapgemm_f16_cut.cu", "tapgemm_i8.cu", "tapgemm.cu",
+                   "tapgemm.h", "ptx.cuh", "fewconv.cu", "fewconv.h", "patconv.cu", "gen_core.py", "pack.cpp")]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "dram_traffic_vgg16_step.txt")
 
 
@@ -254,11 +255,17 @@ def stats(ms_list):
     return {"mean": float(a.mean()), "median": float(np.median(a)), "min": float(a.min()), "max": float(a.max())}
 
 
-def layer_bounds(s, matrix, fp32_tflops, bf16_tflops, hbm_gbs):
+def kernel_of(s, pk):
+    """The kernel that a plain run of a layer launches."""
+    info = pk.plan_info(s.n, s.h, s.w)
+    return "tap_kernel" if info["matrix_path"] else "few_kernel" if info["few_channel_path"] else "patconv_kernel"
+
+
+def layer_bounds(s, kernel, fp32_tflops, bf16_tflops, hbm_gbs):
     """Ideal times of one layer in seconds: on the pipe that its kernel runs on (the matrix units with the
-    whole dense layer, or the fp32 FMA pipe with the kept weights) and on HBM."""
-    t_pipe = (2.0 * s.dense_macs() * MATRIX_PRODUCTS[s.dtype] / (bf16_tflops * 1e12) if matrix
-              else 2.0 * s.useful_macs() / (fp32_tflops * 1e12))
+    whole dense layer, the fp32 FMA pipe with it, or with the kept weights) and on HBM."""
+    t_pipe = (2.0 * s.dense_macs() * MATRIX_PRODUCTS[s.dtype] / (bf16_tflops * 1e12) if kernel == "tap_kernel"
+              else 2.0 * (s.dense_macs() if kernel == "few_kernel" else s.useful_macs()) / (fp32_tflops * 1e12))
     return t_pipe, s.compulsory_bytes() / (hbm_gbs * 1e9)
 
 
@@ -450,32 +457,34 @@ def run_gpu(args):
             ts.append(e0.elapsed_time(e1))
         t_ms = float(np.median(ts))
         info = pk.plan_info(s.n, s.h, s.w)
-        matrix = info["matrix_path"] == 1
-        t_pipe, t_hbm = layer_bounds(s, matrix, fp32_peak, bf16_peak, hbm)
+        kernel = kernel_of(s, pk)
+        matrix = kernel == "tap_kernel"
+        t_pipe, t_hbm = layer_bounds(s, kernel, fp32_peak, bf16_peak, hbm)
         rec = {"layer": s.name, "us": round(t_ms * 1e3, 2), "us_min": round(min(ts) * 1e3, 2),
                "ideal_us": round(max(t_pipe, t_hbm) * 1e6, 2), "launch_floor_us": round(probe["launch_floor_us"], 2),
                "useful_gflops": round(2.0 * s.useful_macs() / t_ms / 1e6, 1),
                "dense_equiv_gflops": round(2.0 * s.dense_macs() / t_ms / 1e6, 1),
-               "kernel": "tap_kernel" if matrix else "patconv_kernel",
+               "kernel": kernel,
                "bound": ("tensor" if matrix else "alu") if t_pipe >= t_hbm else "hbm",
                "roofline_frac": round(max(t_pipe, t_hbm) / (t_ms * 1e-3), 4),
                "grid": "%d blocks (clusters of %d), %d items x %d splits" % (
                    info["matrix_blocks"], info["matrix_cluster"], info["matrix_items"], info["matrix_splits"]) if matrix
-               else "%d tiles x %d filter blocks x %d splits" % (info["tiles"], info["filter_blocks"], info["splits"])}
+               else "-" if kernel == "few_kernel" else "%d tiles x %d filter blocks x %d splits" % (info["tiles"], info["filter_blocks"], info["splits"])}
         per_layer.append(rec)
     layer_ms = sum(p["us"] for p in per_layer) * 1e-3
 
     # The dominant kernel is tap_kernel: its achieved rate is the matrix-unit products of its layers over the
     # whole timed region (this rank's K steps, events on the launching stream; other layers' time included).
     own_ms = st_flushed["mean"]
-    on_matrix = [t[2].plan_info(t[0].n, t[0].h, t[0].w)["matrix_path"] == 1 for t in stack.layers]
-    issued = sum(2.0 * s.dense_macs() * MATRIX_PRODUCTS[s.dtype] for s, m in zip(specs, on_matrix) if m)
+    kernels = [kernel_of(t[0], t[2]) for t in stack.layers]
+    issued = sum(2.0 * s.dense_macs() * MATRIX_PRODUCTS[s.dtype] for s, k in zip(specs, kernels) if k == "tap_kernel")
     achieved = issued / (own_ms * 1e-3) / 1e12
-    binding_ms = sum(max(layer_bounds(s, m, fp32_peak, bf16_peak, hbm)) for s, m in zip(specs, on_matrix)) * 1e3
+    binding_ms = sum(max(layer_bounds(s, k, fp32_peak, bf16_peak, hbm)) for s, k in zip(specs, kernels)) * 1e3
     roofline = {"bound": "tensor", "achieved": achieved, "peak": bf16_peak, "unit": "TFLOP/s",
                 "frac": achieved / bf16_peak,
                 "traffic": recorded_traffic() if args.workload == "vgg16" and not args.only else None,
-                "kernel": "tap_kernel (%d of the %d layers of the step; the others patconv_kernel)" % (sum(on_matrix), len(specs)),
+                "kernel": "tap_kernel (%d of the %d layers of the step%s)" % (
+                    kernels.count("tap_kernel"), len(specs), "".join("; %s %d" % (k, kernels.count(k)) for k in sorted(set(kernels) - {"tap_kernel"}))),
                 "achieved_is": "bf16 products of the dense layers, six per fp32 multiply-add",
                 "peak_source": "%s: dense bf16 matrix product of the library, burst" % peaks_src,
                 "hbm_peak_gbs": hbm, "hbm_peak_source": peaks_src,
@@ -558,12 +567,12 @@ def run_gpu(args):
             torch.cuda.synchronize()
             st_c = stats(stk.timed_steps(stream, args.config_steps, flush))
             t = st_c["median"] * 1e-3
-            matrix = [l[2].plan_info(l[0].n, l[0].h, l[0].w)["matrix_path"] == 1 for l in stk.layers]
-            bind = sum(max(layer_bounds(s, m, fp32_peak, bf16_peak, hbm)) for s, m in zip(sp, matrix))
+            ran = [kernel_of(l[0], l[2]) for l in stk.layers]
+            bind = sum(max(layer_bounds(s, k, fp32_peak, bf16_peak, hbm)) for s, k in zip(sp, ran))
             rec = {"ms_per_step": st_c, "steps": args.config_steps, "layers": len(sp), "dtype": sp[0].dtype,
                    "batch": sp[0].n, "useful_tflops": 2.0 * stk.useful / t / 1e12,
                    "dense_equiv_tflops": 2.0 * stk.dense / t / 1e12,
-                   "matrix_layers": sum(matrix),
+                   "matrix_layers": ran.count("tap_kernel"),
                    "binding_roofline_ms": bind * 1e3, "frac_of_binding_roofline": bind / t}
             configs[name] = rec
             del stk
