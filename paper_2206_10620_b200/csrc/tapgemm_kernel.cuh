@@ -825,11 +825,6 @@ __device__ __noinline__ void tap_repair(const TapParams &P) {
     }
 }
 
-static __device__ __noinline__ void tap_pause() {
-    const uint64_t t = global_ns();
-    for (int it = 0; it < 1000000 && global_ns() - t < 50000u; ++it) {}
-}
-
 template <int DT, int STRIDE, int TAPS, int MT, bool PAIR, bool CUT, bool FUSED, bool GATHER>
 __global__ void __launch_bounds__(tap_threads(DT), 1)
 tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensorMap wmap, const __grid_constant__ CUtensorMap xmap) {
@@ -855,21 +850,27 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
     auto acc_full = [&](int s) { return bars + 8u * (2 * kMaxA + 2 * kMaxB + s); };
     auto acc_empty = [&](int s) { return bars + 8u * (2 * kMaxA + 2 * kMaxB + kMaxAcc + s); };
     const uint32_t all_done = bars + 8u * (2 * kMaxA + 2 * kMaxB + 2 * kMaxAcc), sums_there = all_done + 8u;
-    // Nothing is steered by what a wait says: lanes of a warp and warps of a role may see it give up at different
-    // places and would part, ahead of a barrier or an instruction that takes them all.  A launch that gave up goes
-    // through all of its work, on whatever the buffers hold, and is reported.
+    // A role that fills buffers or issues ends where a wait of its gives up: it arms no barrier, copies nothing and hands no buffer
+    // on any more.  So a barrier is armed again only when what it counted has come (an arrival where none is missing is a
+    // fault), whatever the others are at; they wait for what this role owes them until their own waits give up, and end too.  The
+    // lanes of a warp decide together: they may see a wait give up at different places.  What has been copied is waited for
+    // before the block goes.  The epilogue, which arms nothing, goes through its work on whatever there is (its residual and sums
+    // leave no registers for a way out: 64 images of 28x28x128 int8 with residual 17.0 us, 18.9 with one), and the launch is reported.
     auto wait = [&](uint32_t bar, uint32_t parity) { return mbar_wait<PAIR>(bar, parity, &s_abort, P.status, P.wait_us); };
     auto wait_warp = [&](uint32_t bar, uint32_t parity) { wait(bar, parity); __syncwarp(); };
-    // A role whose wait has given up is out of step: its next waits may return before what they stand for has come (their
-    // barriers are a phase behind), and it hands buffers on before they are filled.  A barrier must not be armed again while a copy
-    // that it counts is on its way, so from then on the role pauses 50 us at every buffer that it fills or hands on (`late`, the
-    // role's own: in a register, where a look at the block's flag for every buffer cost 128->128@56^2/2 14.3 -> 16.1 us).
+    auto agreed = [&](uint32_t bar, uint32_t parity) { return __all_sync(0xFFFFFFFFu, wait(bar, parity)) != 0; };
     // Clusters: a pair of blocks (PAIR), or the blocks (pairs) that split an item's reduction.  The even
     // block of a pair holds the barriers that say "operands are there" and "sums have been read".
     const int csize = (PAIR ? 2 : 1) * P.splits;
     const int crank = csize > 1 ? (int)(blockIdx.x % (unsigned)csize) : 0;
     const int side = PAIR ? crank & 1 : 0, rank = PAIR ? crank >> 1 : crank;
     const uint16_t both = (uint16_t)(3u << (crank & ~1));
+    // Copies that barriers first, first + 1, ... of `slots` in turn count, the last of `armed`, have come.  (Bounded, for what will not
+    // come; the second block's copies are counted by the first's barriers: it waits for as long as one poll lasts.)
+    auto drain = [&](uint32_t first, int slots, int armed) {
+        for (int q = side == 0 ? max(0, armed - slots) : armed - 1; q < armed; ++q)
+            for (int it = 0; it < 100000 && !mbar_ready(first + 8u * (uint32_t)(q % slots), (uint32_t)(q / slots) & 1u); ++it) {}
+    };
     auto lead = [&](uint32_t bar) { return PAIR ? cluster_addr(bar, (uint32_t)(crank & ~1)) : bar; };
     auto arrive_lead = [&](uint32_t bar) {
         if (PAIR) mbar_arrive_cluster(lead(bar));
@@ -910,18 +911,18 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             if (warp == kEpiWarps) {
                 // ---- x by tensor copies, zeros outside the image; the lanes share the copies of a stage
                 // (rows one by one from one thread cost it 190 cycles each) ---------------------------------
-                int s = 0;
+                int s = 0, armed = 0;
                 uint32_t ph = 1;
-                bool late = false;
+                bool alive = true;
                 const int per = TAPS == 1 || !P.row_boxes ? 1 : P.rows, boxes = (TAPS == 1 || STRIDE == 1 ? 1 : 4) * per;
                 const int step = (P.row_boxes ? 1 : P.rows) * P.pitch * 128;
-                for (int item = item0; item < P.items; item += item_step) {
+                for (int item = item0; item < P.items && alive; item += item_step) {
                     const TapItem t = tap_item<MT, PAIR>(P, item, side);
                     if (lane == 0) s_started = s_started + 1;
                     for (int ks = k0; ks < k1; ++ks) {
-                        if (!wait(a_empty(s), ph)) late = true;
-                        if (late) tap_pause();
-                        __syncwarp();
+                        alive = agreed(a_empty(s), ph);
+                        if (!alive) break;
+                        ++armed;
                         const uint32_t bar = lead(a_full(s));
                         const uint32_t dst = sbase + (uint32_t)(s * P.a_bytes) + (P.raster ? (uint32_t)(P.pitch - 1 - t.ox0) * 128u : 0u);
                         const int c = ks * T::row_ch;
@@ -940,6 +941,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                         if (++s == P.a_stages) { s = 0; ph ^= 1u; }
                     }
                 }
+                if (!alive) drain(a_full(0), P.a_stages, armed);
             } else if (FUSED && P.residual && P.splits == 1) {
                 // ---- the residual into L2, an item ahead of its use --------------------------
                 const int pt = tid - (kEpiWarps + 1) * 32;
@@ -959,6 +961,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 int done = 0;
                 for (int item = item0; item < P.items; item += item_step, ++done) {
                     for (int it = 0; it < 100000 && s_started <= done; ++it) __nanosleep(100);     // (a pace, nothing depends on it)
+                    if (s_started <= done) break;
                     fetch(item + item_step);
                 }
             }
@@ -1028,7 +1031,10 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 }
             };
             auto make = [&](const uint32_t (&v)[U][8]) {
-                if (q == 0) wait_warp(a_empty(s), ph);
+                if (q == 0 && !agreed(a_empty(s), ph)) {
+                    item = P.items;
+                    return;
+                }
                 const uint32_t dst = sbase + (uint32_t)(s * P.a_bytes + pl * P.plane_pitch);
                 const bool some = pl < min(P.pl, planes - ks * P.pl);
 #pragma unroll
@@ -1129,8 +1135,8 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 else if (ahead == 1) copy_wait<1>();
                 else if (ahead == 2) copy_wait<2>();
                 else copy_wait<3>();
-                if (part == 0) wait(a_empty(s), ph);
-                __syncwarp();
+                if (part != 0) __syncwarp();
+                else if (!agreed(a_empty(s), ph)) break;
                 const int end = min(part + P.raw_px, P.pixels);
                 const unsigned char *const raw = smem + P.raw_off + slot * P.raw_bytes + pl * kPiece;
                 const uint32_t dst = sbase + (uint32_t)(s * P.a_bytes);
@@ -1190,12 +1196,11 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     if (++tab == P.raw_slots) tab = 0;
                 }
             }
+            copy_wait<0>();
             }
         }
     } else if (warp == kEpiWarps + kProdWarps) {
-        // ---- matrix instructions: one thread, which also waits.  A wait that gives up is not looked at:
-        // nothing per-thread may steer these loops, or every operand is moved to the uniform registers
-        // anew; all later waits then return at once.  Three taps are unrolled and share a barrier, and
+        // ---- matrix instructions: one thread, which also waits (and leaves where a wait gives up).  Three taps are unrolled and share a barrier, and
         // the next barrier is looked at before the instructions of this one are issued: in a rolled loop
         // with a wait of its own a tap costs 350 cycles, its four instructions of 128 x 128 x 16 take 256.
         // fp32 has instructions enough in a tap to roll the rest, and less code to fetch at the start of a
@@ -1213,15 +1218,14 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             const uint32_t a_sub = (uint32_t)P.sub_px * a_px, a_step = (uint32_t)P.a_bytes / 16, b_step = (uint32_t)P.b_bytes / 16;
             int s = 0, b = 0, buf = 0, run = 0;                             // run: stages since the accumulator was empty (CUT)
             uint32_t pha = 0, phb = 0, phc = 1, as = (uint32_t)a0, bs = (uint32_t)b0;
-            bool ready = mbar_test<PAIR>(b_full(0), 0), look = true, late = false;           // look: weights may still be on their way
+            bool ready = mbar_test<PAIR>(b_full(0), 0), look = true;           // look: weights may still be on their way
             // a tap's first entry is that of its row and that of its column of taps
             const uint32_t row0 = (uint32_t)P.tap_start[0] * a_px, row1 = TAPS == 1 ? 0u : (uint32_t)P.tap_start[3] * a_px, row2 = TAPS == 1 ? 0u : (uint32_t)P.tap_start[6] * a_px;
             const uint32_t col0 = 0u, col1 = TAPS == 1 ? 0u : (uint32_t)(P.tap_start[1] - P.tap_start[0]) * a_px, col2 = TAPS == 1 ? 0u : (uint32_t)(P.tap_start[2] - P.tap_start[0]) * a_px;
             for (int item = item0; item < P.items; item += item_step) {
                 for (int ks = k0; ks < k1; ++ks) {
-                    if ((kF32 || (CUT ? run == 0 : ks == k0)) && !wait(acc_empty(buf), phc)) late = true;
-                    if (!wait(a_full(s), pha)) late = true;
-                    if (late) tap_pause();
+                    if ((kF32 || (CUT ? run == 0 : ks == k0)) && !wait(acc_empty(buf), phc)) goto gone;
+                    if (!wait(a_full(s), pha)) goto gone;
                     tc_fence_after();
                     const int kk_n = min(P.pl, planes - ks * P.pl) / 2;
                     const uint32_t d = tmem + (uint32_t)buf * (uint32_t)(MT * P.nt);
@@ -1236,9 +1240,8 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                         const bool last = P.tap_group == 1 || t1 == 2;
                         if (look) {
                             if ((P.tap_group == 1 || t1 == 0) && !ready) {
-                                if (!mbar_wait_long<PAIR>(b_full(b), P.resident ? 0u : phb, &s_abort, P.status, P.wait_us)) late = true;
+                                if (!mbar_wait_long<PAIR>(b_full(b), P.resident ? 0u : phb, &s_abort, P.status, P.wait_us)) goto gone;
                             }
-                            if (late) tap_pause();
                             if (last) {                     // (of its slot: look at the next one)
                                 const bool wrap = b + 1 == P.b_slots;
                                 ready = mbar_test<PAIR>(b_full(wrap ? 0 : b + 1), P.resident ? 0u : wrap ? phb ^ 1u : phb);
@@ -1299,6 +1302,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 }
                 if (P.resident) look = false;
             }
+        gone:
             tc_commit<PAIR>(all_done, both);
         }
         __syncwarp();
@@ -1308,12 +1312,10 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
         if (elect_one()) {
             int b = 0, issued = 0;
             uint32_t ph = 1;
-            bool late = false;
             for (int item = item0; item < P.items; item += item_step) {
                 for (int ks = k0; ks < k1; ++ks) {
                     for (int tap = 0; tap < TAPS; tap += P.tap_group) {
-                        if (issued >= P.b_slots && !wait(b_empty(b), ph)) late = true;
-                        if (late) tap_pause();
+                        if (issued >= P.b_slots && !wait(b_empty(b), ph)) goto last;
                         // one copy for a slot: pieces of 2 KB with a copy of their own cost 50 cycles
                         // of issue apiece and held the whole kernel to 5.5 TB/s of weights
                         if (side == 0) mbar_expect_tx(b_full(b), (uint32_t)P.b_bytes * (PAIR ? 2 : 1));
@@ -1325,9 +1327,9 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 }
                 if (P.resident) break;
             }
+        last:
             // Nothing may land in shared memory after this block has gone (the wait for it may have given up).
-            for (int q = max(0, issued - P.b_slots); q < issued && side == 0; ++q)
-                for (int it = 0; it < 1000000 && !mbar_ready(b_full(q % P.b_slots), (uint32_t)(q / P.b_slots) & 1u); ++it) {}
+            if (side == 0 || *(volatile int *)&s_abort) drain(b_full(0), P.b_slots, issued);
         }
         __syncwarp();
     } else {
@@ -1416,8 +1418,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                     __syncwarp();
                 }
             };
-            // A chunk (fp32: all of the warp's) is in registers.  (Arrivals count for one: after a wait that gave up the roles are
-            // out of step, a phase may lack one arrival only, and one for two, or two lanes' at once, is then a fault.)
+            // A chunk (fp32: all of the warp's) is in registers.
             auto release = [&]() {
                 tc_fence_before();
                 __syncwarp();

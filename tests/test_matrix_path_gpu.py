@@ -573,3 +573,32 @@ def _run_static(pk, d):
     pk.sync()
     check_guards(buf)
     return y.cpu().numpy()
+
+
+@pytest.mark.parametrize("dtype,stride,shape", [
+    ("f16", 2, (24, 67, 93, 56, 56)),      # rows shifted into place, several stages a block
+    ("i8", 2, (24, 67, 93, 56, 56)),
+    ("f32", 1, (16, 264, 200, 28, 28)),    # pairs of blocks whose weights stream
+    ("f16", 1, (32, 1024, 256, 14, 14)),   # chains that are cut
+])
+def test_roles_end_where_a_wait_gives_up(dtype, stride, shape):
+    """However many stages are left, a launch that gave up ends soon: nobody goes on filling buffers for the others."""
+    import time
+    import torch
+    n, ci, co, h, w = shape
+    d = _layer(dtype, n, ci, co, h, w, stride, seed=ci)
+    pk = pack(d)
+    pk.plan(n, h, w, wait_limit_ms=20)
+    before = run_gpu(pk, d.x, d.bias, True)
+    pk.test_expect_arrivals(1)
+    x, b = torch.from_numpy(d.x).cuda(), torch.from_numpy(d.bias).cuda()
+    buf, y = guarded_output(before.shape, {"f32": torch.float32, "f16": torch.float16, "i8": torch.int32}[dtype])
+    torch.cuda.synchronize()
+    t0 = time.monotonic()
+    pk.run(x.data_ptr(), n, h, w, b.data_ptr(), True, y.data_ptr())
+    with pytest.raises(binding.PatconvError) as e:
+        pk.sync()
+    assert e.value.status == 7 and time.monotonic() - t0 < 1.0
+    check_guards(buf)
+    pk.test_expect_arrivals(0)
+    assert np.array_equal(run_gpu(pk, d.x, d.bias, True), before)
