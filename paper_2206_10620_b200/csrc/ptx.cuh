@@ -91,24 +91,20 @@ template <bool CLUSTER> __device__ __forceinline__ bool mbar_try(uint32_t mbar, 
     return ok != 0;
 }
 
-// Wait for an mbarrier phase with a bound in time (limit_us microseconds, plus a cap on the
-// polls in case the timer stands still): on expiry the block-wide abort flag and the device
-// status word are set.  Every later wait of the block is given 100 microseconds at most, more than
-// any copy or matrix instruction takes: roles that go on whatever a wait said stay in step, no more
-// copies are in flight than in an ordinary run, and those that are waited for have landed.  The kernel
+// Wait for an mbarrier phase with a bound in time (limit_us microseconds and three tries of kSleepNs; in case
+// the timer stands still, a cap on the tries: 80 seconds at most): on expiry the block-wide abort flag and the device
+// status word are set.  Every later wait of the block is given 100 microseconds and those tries, more than
+// any copy or matrix instruction takes, so that a launch that gave up ends soon (nothing else rests on it).  The kernel
 // still runs to its end (releasing tensor memory) with results the host can tell are invalid.
 // CLUSTER: what other blocks of the cluster wrote before they arrived is seen too.
 template <bool CLUSTER>
 __device__ __noinline__ bool mbar_wait_long(uint32_t mbar, uint32_t parity, volatile int *abort_flag, int *status,
                                             uint32_t limit_us) {
-    uint64_t t0 = 0;
-    for (uint32_t it = 0; it < 40000000u; ++it) {
+    if (mbar_try<CLUSTER>(mbar, parity)) return true;
+    const uint64_t t0 = global_ns();
+    for (uint32_t it = 0; it < 4000000u; ++it) {
         if (mbar_try<CLUSTER>(mbar, parity)) return true;
-        if ((it & 7u) == 7u) {
-            const uint64_t t = global_ns();
-            if (t0 == 0) t0 = t;
-            else if (t - t0 > (uint64_t)(*abort_flag ? min(limit_us, 100u) : limit_us) * 1000ull) break;
-        }
+        if (global_ns() - t0 > (uint64_t)(*abort_flag ? min(limit_us, 100u) : limit_us) * 1000ull) break;
     }
     if (!*abort_flag) {
         *abort_flag = 1;
