@@ -401,10 +401,12 @@ xgen_status xgen_dwconv_run(const xgen_dwconv_packed *h, const void *x, int32_t 
     P.cvs = h->c / v;
     P.strips = (wo + tx - 1) / tx;
     // Rows ahead, where a call is long enough for bandwidth to count and accesses are 8 bytes or more (a copy of 4 bytes
-    // costs as much), us without and with: fp16 32x56x56x128 (51 MB) 16.2, 14.7; 123x188x336 (31 MB) 11.6, 11.0;
+    // costs as much), later for pairs of fp32, whose copies carry half of what those of four do.  us without and with: fp16 32x56x56x128 (51 MB) 16.2, 14.7; 123x188x336 (31 MB) 11.6, 11.0;
     // fp32 16x56x56x128 12.8, 10.0; but 11x49x39x112 (9 MB) 5.5, 6.0; 20x14x14x512 4.5, 5.0; single fp32 channels 8x42x42x881 25.0, 27.0;
     // pairs of fp16 8x42x42x882 17.5, 21.5; stride 2, two rows ahead in registers, 8x112x112x64 3.7, 5.0.
-    const bool ahead = h->stride == 1 && v * (int)eb >= 8 && (xe + ye) * (int64_t)eb >= 24000000;
+    // Around 24 MB fp16 15x56x56x128 9.0, 8.8, 13x56x56x128 (21 MB) 7.3 without; fp32 15x28x28x256 6.5, 5.8; fp32 pairs 36 MB 11x56x56x130
+    // 9.8, 10.7; 70 MB 6x75x75x250 16.6, 16.7, 21x56x56x130 17.0, 17.6; 100 MB 9x75x75x250 23.6, 22.6, 31x28x28x510 22.5, 21.0.
+    const bool ahead = h->stride == 1 && v * (int)eb >= 8 && (xe + ye) * (int64_t)eb >= (eb == 4 && v == 2 ? 90000000 : 24000000);
     const void *const kern = kernel_for(h->dtype, h->stride, v, ahead);
     // Pieces of an image's rows: a piece loads (and at stride 1 adds up) two rows besides its own and costs
     // about two more to start, so pieces want to be long; but the blocks run in waves of what the GPU holds,

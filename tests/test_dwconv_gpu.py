@@ -84,6 +84,35 @@ def test_mobilenet_layers_sampled_images():
             _compare(d, got[i:i + 1], x=d.x[i:i + 1])
 
 
+@pytest.mark.parametrize("dtype,n,c,h,w", [
+    ("f16", 27, 36, 111, 113),      # four channels a thread; a last strip of one column, heights that no split into pieces divides
+    ("f16", 140, 512, 13, 14),
+    ("f32", 13, 36, 83, 91),
+    ("f32", 61, 256, 14, 15),
+    ("f32", 11, 882, 42, 31),       # two: from 90 MB on
+    ("f32", 300, 34, 35, 34),
+])
+@pytest.mark.parametrize("relu", [True, False])
+def test_rows_that_come_ahead(dtype, n, c, h, w, relu):
+    """Calls long enough for rows to be copied ahead of their use: the first, last and some other images against the oracle,
+    the others against themselves in a call too short for it."""
+    import torch
+    s = wl.DepthwiseSpec("t", n, c, h, w, 1, dtype, 0.25, 12, "upm1", 0.05, True, 9)
+    d = wl.make_depthwise(s)
+    assert 2 * d.x.nbytes >= (90e6 if dtype == "f32" and c % 4 else 24e6)
+    got, pk = _run(d, relu=relu, bias=relu)
+    for i in sorted({0, 1, n // 2, n - 1}):
+        _compare(d, got[i:i + 1], relu=relu, bias=relu, x=d.x[i:i + 1])
+    x, b = torch.from_numpy(d.x).cuda(), torch.from_numpy(d.bias).cuda()
+    y = torch.full(got.shape, 777.0, dtype=x.dtype, device="cuda")
+    short = max(1, int(20e6 / (2 * d.x[0].nbytes)))
+    for i in range(0, n, short):
+        k = min(short, n - i)
+        pk.run(x[i:].data_ptr(), k, h, w, b.data_ptr() if relu else 0, relu, y[i:].data_ptr(), torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    assert np.array_equal(y.cpu().numpy(), got)
+
+
 def test_argument_errors():
     import torch
     d = wl.make_depthwise(wl.DepthwiseSpec("t", 1, 8, 6, 6, 1, "f32", 0.0, 8, "upm1", 0.05, True, 8))
