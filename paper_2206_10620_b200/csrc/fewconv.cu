@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -260,6 +261,17 @@ template <int DT> static const void *few_kernel_of(int c_in, int px) {
     }
 }
 
+// Of the current device.
+static int sm_count() {
+    static std::atomic<int> known[64];
+    int device = 0, sms = 148;
+    if (cudaGetDevice(&device) != cudaSuccess || device < 0 || device >= 64) return sms;
+    if (const int k = known[device].load(std::memory_order_relaxed)) return k;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 148;
+    known[device].store(sms, std::memory_order_relaxed);
+    return sms;
+}
+
 cudaError_t few_launch(const FewWeights &fw, const void *x, int n, int h, int w, int stride, const void *bias, bool relu, void *y,
                        bool overlap, cudaStream_t st) {
     FewParams P{};
@@ -276,7 +288,8 @@ cudaError_t few_launch(const FewWeights &fw, const void *x, int n, int h, int w,
     // Four pixels a thread where that still gives every scheduler of the GPU two warps, else fewer, so that a small image
     // spreads over it (13 x 20x171, 3 -> 32, fp16: 10.3 us with four, 5.2 with two).
     const int64_t units = ((int64_t)P.pixels + 31) / 32 * ((fw.rows + 15) / 16);
-    const int px = units >= 4 * 148 * 8 ? 4 : units >= 2 * 148 * 8 ? 2 : 1;
+    const int64_t sms = sm_count();
+    const int px = units >= 4 * sms * 8 ? 4 : units >= 2 * sms * 8 ? 2 : 1;
     const int per_block = (kFewThreads >> P.log_groups) * px;
     const dim3 grid((unsigned)(((int64_t)P.pixels + per_block - 1) / per_block), (unsigned)((fw.rows + kFewFilters - 1) / kFewFilters));
     const void *kern = fw.dtype == XGEN_F32 ? few_kernel_of<XGEN_F32>(fw.c_in, px)

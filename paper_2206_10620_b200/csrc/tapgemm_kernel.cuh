@@ -538,10 +538,8 @@ template <int DT> __device__ __forceinline__ void tap_quad(const TapParams &P, c
             if constexpr (DT == XGEN_I8_I32) { a0 += b.x + res.v[4 * k + 2 * i]; a1 += b.y + res.v[4 * k + 2 * i + 1]; }
             else {
                 add2(a0, a1, b.x, b.y);
-                if constexpr (DT == XGEN_F16_F32ACC) {
-                    const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&res.v[2 * k + i]));
-                    add2(a0, a1, __float_as_uint(f.x), __float_as_uint(f.y));
-                } else add2(a0, a1, res.v[4 * k + 2 * i], res.v[4 * k + 2 * i + 1]);
+                const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&res.v[2 * k + i]));
+                add2(a0, a1, __float_as_uint(f.x), __float_as_uint(f.y));
             }
             if (P.relu) { a0 = tap_max<DT>(a0, 0u); a1 = tap_max<DT>(a1, 0u); }
             if (DT == XGEN_I8_I32 && P.rq_scale) {
@@ -1424,7 +1422,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
                 __syncwarp();
                 if (lane == 0) arrive_lead(acc_empty(buf));
             };
-            if (kF32) {
+            if constexpr (kF32) {
                 uint32_t sum[2][32];                 // chunks `next` and `next` + kGroups
 #pragma unroll
                 for (int i = 0; i < 64; ++i) sum[i / 32][i % 32] = 0u;
