@@ -340,7 +340,7 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                     // shift into place: up to two stages of them on their way (three of a product).  The tiles of stride 2 (612
                     // pixels) leave no room for those: quarters or eighths of a stage, or one tile of x, whatever
                     // is weighed best, so that there is a plan whatever else takes room.  (Without one 32 images of 56x56x67 -> 93
-                    // fp16 took 176 us on the command stream, 42.6 now; 28x28x503 -> 256 1230, 59; int8 168, 21 and 1092, 33.)
+                    // fp16 took 176 us on the command stream, 40.6 now; 28x28x503 -> 256 1227, 57; int8 168, 20 and 1092, 33.)
                     size_t tables = sums;
                     const int raw_top = copied || dt == XGEN_F32 ? 0 : (int)std::min<int64_t>(uses, tw.taps == 1 ? 4 : 3);
                     const int two = (int)std::min<int64_t>(2, uses);

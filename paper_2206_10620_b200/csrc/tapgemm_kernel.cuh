@@ -503,7 +503,7 @@ __device__ __forceinline__ void tap_direct(const TapParams &P, const uint32_t *s
 // through shared memory.  Pixels px[2 h + r]: row 16 h + 8 r + lane / 4 of the warp's 32; sum v[8 h + 4 i + 2 r + e]:
 // channel c + 8 i + 2 (lane % 4) + e.  The residual is asked for before the sums are waited for.
 // (32 lanes a pixel each touched 32 lines an access; by way of shared memory 256 x 64 int32 residuals took 7000 cycles:
-// 64 images of 28x28x128 int8 20.5 us, 16.0 now.)
+// 64 images of 28x28x128 int8 20.9 us, 16.9 now.)
 template <int DT> struct QuadRes { uint32_t v[DT == XGEN_F16_F32ACC ? 8 : 16]; };
 template <int DT> __device__ __forceinline__ void quad_residual(const TapParams &P, QuadRes<DT> &res, const int (&px)[4], int c) {
     c += 2 * (threadIdx.x & 3);
@@ -1071,7 +1071,7 @@ tap_kernel(const __grid_constant__ TapParams P, const __grid_constant__ CUtensor
             // into one of raw_slots buffers, raw_slots - 1 of them ahead of their use, and shifted
             // into place from there.  A warp copies and shifts the same pixels, so warps need not meet.
             // Pieces are taken U at a time.  (The large tiles of stride 2 four: with two a stage waited for the latency of its
-            // shared memory, 32 images of 28x28x503 -> 256 fp16 60.4 us, 55.5 now; four that all lie outside the image, as most do
+            // shared memory, 32 images of 28x28x503 -> 256 fp16 60.4 us, 57.4 now; four that all lie outside the image, as most do
             // of a tile over small images, are neither copied nor shifted.)
             constexpr int U = STRIDE == 2 ? 4 : 2;
             constexpr uint32_t kNone = 0xFFFFFFFFu;      // (bytes from x on: it has fewer than 2^31 elements)
