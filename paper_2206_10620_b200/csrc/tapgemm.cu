@@ -333,6 +333,10 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                         p.grid = p.items * sp * ways;
                         waves = (p.items + cl - 1) / cl;
                     }
+                    // (no plan whose instructions alone take as long as the best so far: 512 -> 512 at 14x14 fp32 is planned in 24 us, 57 without)
+                    const double kk = (double)tw.planes / p.stages / 2, taps = tw.taps, per_tap = kk * mt * prod;
+                    const double mma = taps * std::max(per_tap * p.nt / 2.0, 90.0 + 46.0 * per_tap);
+                    if (3500.0 + (double)waves * p.per_split * mma >= best.cycles * 0.999) continue;
                     const size_t sums = sp > 1 ? (size_t)sp * ((8 * mt + sp - 1) / sp) * 64 * p.nt : s.staged ? (size_t)epi_warps(dt) * kStageBytes : 0;
                     const int64_t uses = (sp == 1 ? waves : 1) * p.per_split;      // stages one block goes through
                     // Shared memory: two tiles of x (more for a plain product, whose stages are short), the rest
@@ -379,11 +383,9 @@ bool tap_choose(const TapWeights &tw, const TapShape &s, int device, TapPlan &be
                         // (256 -> 256 at 14x14, batch 32, fp16: 12.8 us as pairs, 11.7 without); the
                         // short stages of a product wait 300 cycles for its other block (1842 filters x 5421 rows,
                         // fp32: 77 us as pairs, 57 us without).
-                        const double kk = (double)tw.planes / p.stages / 2, taps = tw.taps;
                         const double b_stage = taps * kk * 2 * parts * p.nt * 16.0 / ways, b_moved = p.resident && sp == 1 ? b_stage / waves : b_stage;
                         const double x_moved = (double)pixels * kk * 2 * cpp * xb, a_stage = (double)p.a_bytes * (swizzled ? 1 : 2);
-                        const double per_tap = kk * mt * prod, instr = taps * per_tap;
-                        const double mma = taps * std::max(per_tap * p.nt / 2.0, 90.0 + 46.0 * per_tap);
+                        const double instr = taps * per_tap;
                         const double shared = (instr * (4096.0 + p.nt * 32.0 / ways) + b_moved + a_stage) / 128.0;
                         const double move = (x_moved + b_moved) / 40.0 + (copied && p.straddle ? 60.0 * p.rows * (s.stride == 1 ? 1 : 4) : 0.0) * 0.5;
                         // cycles of the producer warps for a piece; no stage of x ahead
